@@ -1,6 +1,6 @@
 """In-tree build of libmbc.so (nvcc for sm_103a + g++ for the host builder).
 
-Three translation units compiled in parallel, then linked with nvcc; no cmake.
+Four translation units compiled in parallel, then linked with nvcc; no cmake.
 The result lands next to this file and is git-ignored.
 """
 from __future__ import annotations
@@ -45,12 +45,14 @@ def build(force: bool = False, verbose: bool = False) -> str:
     cu_obj = os.path.join(OUT, "contract.o")
     cpp_obj = os.path.join(OUT, "builder.o")
     io_obj = os.path.join(OUT, "list_io.o")
+    plan_obj = os.path.join(OUT, "plan.o")
     jobs = [
         [nvcc, "-O3", "-std=c++17", *ARCH, "-lineinfo", "-Xcompiler", "-fPIC", *inc, "-c",
          os.path.join(CSRC, "contract.cu"), "-o", cu_obj],
         ["g++", "-O3", "-std=c++17", "-fPIC", "-fopenmp", *inc, "-c", os.path.join(CSRC, "builder.cpp"), "-o",
          cpp_obj],
         ["g++", "-O2", "-std=c++17", "-fPIC", *inc, "-c", os.path.join(CSRC, "list_io.cpp"), "-o", io_obj],
+        ["g++", "-O2", "-std=c++17", "-fPIC", *inc, "-c", os.path.join(CSRC, "plan.cpp"), "-o", plan_obj],
     ]
 
     def run(cmd):
@@ -58,11 +60,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
             print(" ".join(cmd), file=sys.stderr)
         subprocess.check_call(cmd)
 
-    with ThreadPoolExecutor(max_workers=3) as ex:
+    with ThreadPoolExecutor(max_workers=4) as ex:
         for f in [ex.submit(run, j) for j in jobs]:
             f.result()
     tmp = LIB + f".{os.getpid()}.tmp"
-    run([nvcc, "-shared", *ARCH, "-o", tmp, cu_obj, cpp_obj, io_obj, "-Xcompiler", "-fopenmp", "-lgomp"])
+    run([nvcc, "-shared", *ARCH, "-o", tmp, cu_obj, cpp_obj, io_obj, plan_obj, "-Xcompiler", "-fopenmp", "-lgomp"])
     os.replace(tmp, LIB)
     return LIB
 

@@ -11,6 +11,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <memory>
 #include <tuple>
 #include <type_traits>
 #include <new>
@@ -18,6 +19,7 @@
 
 #include "large_kernel.cuh"
 #include "mbc_internal.h"
+#include "plan.h"
 
 #include <atomic>
 
@@ -154,6 +156,10 @@ struct DeviceCache {
     int64_t site_entries = 0;
     uint32_t *d_small_ops = nullptr;
     uint32_t *d_small_zops = nullptr;
+    int32_t *d_run_off = nullptr;      // minor form: runs of a component, terms of a run
+    int32_t *d_term_off = nullptr;
+    double *d_run_coef = nullptr;
+    uint32_t *d_terms = nullptr;
     // large path
     std::vector<uint32_t *> d_opx;
     std::vector<uint16_t *> d_opy;
@@ -178,6 +184,10 @@ void free_cache(DeviceCache *c) {
     if (c->device >= 0) cudaSetDevice(c->device);
     cudaFree(c->d_small_ops);
     cudaFree(c->d_small_zops);
+    cudaFree(c->d_run_off);
+    cudaFree(c->d_term_off);
+    cudaFree(c->d_run_coef);
+    cudaFree(c->d_terms);
     for (auto p : c->d_opx) cudaFree(p);
     for (auto p : c->d_opy) cudaFree(p);
     for (auto p : c->d_zrank) cudaFree(p);
@@ -210,11 +220,56 @@ mbc_status upload(T **dst, const T *src, size_t n) {
 // Nonzero entries of Gamma_2 (eq. def_g): 4 relativistic, 2 nonrelativistic.
 inline int n_g2(const mbc_term_list *L) { return L->dim == 4 ? 4 : 2; }
 
+// Shared-memory layout of one site for the minor form: the tile at offset 0
+// for the whole site (lists of a batch share it), then the minors of each
+// order from the step that makes them to their last use.
+bool plan_minors(const MinorPlan &mp, SmallPlan &P, int64_t &site_entries) {
+    const int ns = (int)mp.steps.size(), fin = 1 + ns;
+    if (ns > 16) return false;
+    Interval reg[8];
+    for (int o = 0; o < 8; ++o) reg[o] = {0, 0, mp.reg_size[o], 0};
+    reg[1].end = fin;
+    std::vector<Interval *> order{&reg[1]};
+    for (int i = 0; i < ns; ++i) {
+        const auto &st = mp.steps[(size_t)i];
+        reg[st.z_reg].start = reg[st.z_reg].end = 1 + i;
+        reg[st.x_reg].end = std::max(reg[st.x_reg].end, 1 + i);
+        reg[st.y_reg].end = std::max(reg[st.y_reg].end, 1 + i);
+        order.push_back(&reg[st.z_reg]);
+    }
+    for (const auto &t : mp.terms) reg[t.x_reg].end = reg[t.y_reg].end = fin;
+    place(order, 1);
+    int64_t top = 0;
+    for (auto *b : order) top = std::max(top, b->off + b->size);
+    site_entries = (top + 1) & ~int64_t(1);
+    P.site_entries = P.part_off = (int)site_entries;
+    P.bilinear = 1;
+    P.n_steps = ns;
+    P.s_off = (int)reg[1].off;
+    for (int i = 0; i < ns; ++i) {
+        const auto &st = mp.steps[(size_t)i];
+        SmallStepDesc &d = P.step[i];
+        d.n_z = st.n_z;
+        d.k = st.k;
+        split_groups(st.n_z, st.k, d.g, d.n_main, d.g2);
+        d.x_off = (int)reg[st.x_reg].off;
+        d.y_off = (int)reg[st.y_reg].off;
+        d.z_off = (int)reg[st.z_reg].off;
+    }
+    int64_t kmax = 1;
+    for (int c = 0; c < P.n_comp; ++c)
+        kmax = std::max<int64_t>(kmax, mp.term_off[(size_t)mp.run_off[(size_t)c + 1]] - mp.term_off[(size_t)mp.run_off[(size_t)c]]);
+    P.fin_g = pick_group(P.n_comp, kmax);
+    return true;
+}
+
 // Build the small-kernel plan (shared-memory layout of one site) on the host.
 // The shared-memory kernels hold square single-source tiles only.
+// A list with a minor form takes that one.
 // part_off receives, per nucleus of the list, the region offset of the stage
 // its components are contracted from (blocks for a single baryon).
-bool plan_small(const mbc_term_list *L, SmallPlan &P, int64_t &site_entries, std::vector<int> &part_off) {
+bool plan_small(const mbc_term_list *L, const MinorPlan *minor, SmallPlan &P, int64_t &site_entries,
+                std::vector<int> &part_off) {
     std::memset(&P, 0, sizeof(P));
     const int A = L->A;
     if (A > 16 || L->n_comp > kSmallMaxComp || L->n_comp < 1) return false;
@@ -228,6 +283,7 @@ bool plan_small(const mbc_term_list *L, SmallPlan &P, int64_t &site_entries, std
     P.n_comp = L->n_comp;
     P.n_steps = A - 1;
     P.path0 = L->path[0];
+    if (minor) return plan_minors(*minor, P, site_entries);
     P.block_size = (int)L->block_size;
     P.npair = (int)binom64(L->nxi, 2);
     if (L->block_size >= 32768) return false;
@@ -235,19 +291,15 @@ bool plan_small(const mbc_term_list *L, SmallPlan &P, int64_t &site_entries, std
         if (s.n_x >= 65536) return false;
     const int n_ph = 3 + A;  // phases: 0 load, 1 Q, 2 blocks, 3.. steps, 2 + A contraction
     Interval Sb{0, 2, (int64_t)L->nxi * L->nxi, 0}, Qb{1, 2, 3LL * L->nxi * L->nxi, 0};
-    Interval blk[2];
     std::vector<Interval> stage((size_t)A + 1);
-    // both blocks first, at fixed offsets [0, bs) and [bs, 2 bs), live to the
-    // end: lists with the same tile shape then share one block computation
-    // per site in a batch (blocks do not depend on the nucleus); the S tile,
-    // the diquark and the stages are placed after them by first fit
+    // the block of both species first, at offset 0, live to the end: lists
+    // with the same tile shape then share one block computation per site in a
+    // batch (blocks do not depend on the nucleus); the S tile, the diquark and
+    // the stages are placed after it by first fit
     const int last_phase = 2 + A;
     std::vector<Interval *> order;
-    for (int b = 0; b < 2; ++b) {
-        P.need_blk[b] = L->need_block[b] ? 1 : 0;
-        blk[b] = {2, last_phase, L->block_size, (int64_t)b * L->block_size};
-        order.push_back(&blk[b]);
-    }
+    Interval blk{2, last_phase, L->block_size, 0};
+    order.push_back(&blk);
     order.push_back(&Sb);
     order.push_back(&Qb);
     // a stage where a nucleus of the list ends stays live until the contraction
@@ -259,7 +311,7 @@ bool plan_small(const mbc_term_list *L, SmallPlan &P, int64_t &site_entries, std
         order.push_back(&stage[(size_t)m + 1]);
     }
     (void)n_ph;
-    place(order, 2);
+    place(order, 1);
     int64_t top = 0;
     for (auto *b : order) top = std::max(top, b->off + b->size);
     site_entries = (top + 1) & ~int64_t(1);
@@ -267,7 +319,7 @@ bool plan_small(const mbc_term_list *L, SmallPlan &P, int64_t &site_entries, std
     P.part_off = (int)site_entries;  // lanes-are-sites kernel: 64 partial rows after the site region
     P.s_off = (int)Sb.off;
     P.q_off = (int)Qb.off;
-    for (int b = 0; b < 2; ++b) P.blk_off[b] = (int)blk[b].off;
+    P.blk_off = (int)blk.off;
     int64_t op_off = 0;
     for (int m = 1; m < A; ++m) {
         const Step &s = L->steps[(size_t)m - 1];
@@ -275,15 +327,15 @@ bool plan_small(const mbc_term_list *L, SmallPlan &P, int64_t &site_entries, std
         d.n_z = (int)s.n_z;
         d.k = (int)s.k;
         split_groups(s.n_z, s.k, d.g, d.n_main, d.g2);
-        d.x_off = m == 1 ? P.blk_off[L->path[0]] : (int)stage[(size_t)m].off;
-        d.y_off = P.blk_off[s.baryon];
+        d.x_off = m == 1 ? P.blk_off : (int)stage[(size_t)m].off;
+        d.y_off = P.blk_off;
         d.z_off = (int)stage[(size_t)m + 1].off;
         d.op_off = op_off;
         op_off += s.n_z * s.k;
     }
     part_off.clear();
     for (const auto &pt : L->parts)
-        part_off.push_back(pt.A == 1 ? P.blk_off[L->path[0]] : (int)stage[(size_t)pt.A].off);
+        part_off.push_back(pt.A == 1 ? P.blk_off : (int)stage[(size_t)pt.A].off);
     int64_t kmax = 1;
     for (int c = 0; c < L->n_comp; ++c) kmax = std::max(kmax, L->fin_off[(size_t)c + 1] - L->fin_off[(size_t)c]);
     P.fin_g = pick_group(L->n_comp, kmax);
@@ -315,7 +367,8 @@ DeviceCache *get_cache(const mbc_term_list *Lc, int device, mbc_status &st) {
     }
     // small-kernel plan and packed ops
     std::vector<int> part_off;
-    c->small_ok = !L->pauli_forbidden && plan_small(L, c->sp, c->site_entries, part_off);
+    const std::shared_ptr<const MinorPlan> minor = minor_plan(L);
+    c->small_ok = !L->pauli_forbidden && plan_small(L, minor.get(), c->sp, c->site_entries, part_off);
     if (c->small_ok) {
         // contracted entries as offsets in the site region; per-component
         // normalisation and homogeneity degree of its nucleus
@@ -327,7 +380,7 @@ DeviceCache *get_cache(const mbc_term_list *Lc, int device, mbc_status &st) {
             for (int cc = pt.c0; cc < pt.c1; ++cc) {
                 inv[(size_t)cc] = 1.0 / pt.norm;
                 deg[(size_t)cc] = 3 * pt.A;
-                for (int64_t e = L->fin_off[(size_t)cc]; e < L->fin_off[(size_t)cc + 1]; ++e)
+                for (int64_t e = L->fin_off[(size_t)cc]; !minor && e < L->fin_off[(size_t)cc + 1]; ++e)
                     zs[(size_t)e] = L->fin_z[(size_t)e] + (uint32_t)part_off[j];
             }
         }
@@ -339,25 +392,36 @@ DeviceCache *get_cache(const mbc_term_list *Lc, int device, mbc_status &st) {
         }
         // per step and part (outputs [0, n_main) with g lanes, the rest with
         // g2): [round j][z][sub], padded to a whole number of rounds
-        std::vector<uint32_t> packed;
-        for (size_t m = 0; m < L->steps.size(); ++m) {
+        // operation i of step m: operand indices and sign, of the list's own
+        // steps or of the minor form's
+        struct Op {
+            uint32_t x, y, neg;
+        };
+        auto op_at = [&](size_t m, size_t i) {
+            if (minor) {
+                const auto &s = minor->steps[m];
+                return Op{s.x[i], s.y[i], s.neg[i]};
+            }
             const Step &s = L->steps[m];
+            return Op{s.x[i], s.ys[i] & 0x7fffu, (uint32_t)(s.ys[i] >> 15)};
+        };
+        std::vector<uint32_t> packed;
+        for (int m = 0; m < c->sp.n_steps; ++m) {
             SmallStepDesc &d = c->sp.step[m];
+            const int64_t k = d.k;
             auto pack = [&](int64_t z_begin, int64_t n, int64_t g) {
-                const int64_t off = (int64_t)packed.size(), kk = (s.k + g - 1) / g;
+                const int64_t off = (int64_t)packed.size(), kk = (k + g - 1) / g;
                 packed.resize(packed.size() + (size_t)(kk * n * g), 0u);
                 uint32_t *dst = packed.data() + off;
                 for (int64_t zl = 0; zl < n; ++zl)
-                    for (int64_t j = 0; j < s.k; ++j) {
-                        const size_t i = (size_t)((z_begin + zl) * s.k + j);
-                        const uint32_t op =
-                            s.x[i] | ((uint32_t)(s.ys[i] & 0x7fffu) << 16) | ((uint32_t)(s.ys[i] >> 15) << 31);
-                        dst[((j / g) * n + zl) * g + (j % g)] = op;
+                    for (int64_t j = 0; j < k; ++j) {
+                        const Op o = op_at((size_t)m, (size_t)((z_begin + zl) * k + j));
+                        dst[((j / g) * n + zl) * g + (j % g)] = o.x | o.y << 16 | o.neg << 31;
                     }
                 return off;
             };
             d.op_off = pack(0, d.n_main, d.g);
-            d.op_off2 = pack(d.n_main, s.n_z - d.n_main, d.g2);
+            d.op_off2 = pack(d.n_main, d.n_z - d.n_main, d.g2);
         }
         if ((st = upload(&c->d_small_ops, packed.data(), packed.size())) != MBC_OK) {
             free_cache(c);
@@ -372,18 +436,38 @@ DeviceCache *get_cache(const mbc_term_list *Lc, int device, mbc_status &st) {
         // records need no sign
         std::vector<uint32_t> zpk;
         c->ls_ok = true;
-        for (size_t m = 0; m < L->steps.size(); ++m) {
-            const Step &s = L->steps[m];
-            c->sp.step[m].zop_off = (int64_t)zpk.size();
-            for (int64_t z = 0; z < s.n_z; ++z)
+        for (int m = 0; m < c->sp.n_steps; ++m) {
+            SmallStepDesc &d = c->sp.step[m];
+            d.zop_off = (int64_t)zpk.size();
+            for (int64_t z = 0; z < d.n_z; ++z)
                 for (uint32_t want = 0; want < 2; ++want)
-                    for (int64_t j = 0; j < s.k; ++j) {
-                        const size_t i = (size_t)(z * s.k + j);
-                        const uint32_t x = s.x[i], y = s.ys[i] & 0x7fffu, sg = (uint32_t)(s.ys[i] >> 15);
-                        if (sg != want) continue;
-                        if (x >= 256 || y >= 256) c->ls_ok = false;
-                        zpk.push_back((x & 0xffu) << 8 | sg | (y & 0xffu) << 24);
+                    for (int64_t j = 0; j < d.k; ++j) {
+                        const Op o = op_at((size_t)m, (size_t)(z * d.k + j));
+                        if (o.neg != want) continue;
+                        if (o.x >= 256 || o.y >= 256) c->ls_ok = false;
+                        zpk.push_back((o.x & 0xffu) << 8 | o.neg | (o.y & 0xffu) << 24);
                     }
+        }
+        if (minor) {
+            // products of the contraction as entry offsets in the site region
+            int32_t reg_off[8] = {0};
+            reg_off[1] = c->sp.s_off;
+            for (size_t m = 0; m < minor->steps.size(); ++m) reg_off[minor->steps[m].z_reg] = c->sp.step[m].z_off;
+            std::vector<uint32_t> terms;
+            for (const auto &t : minor->terms)
+                terms.push_back((uint32_t)(reg_off[t.x_reg] + t.x) | (uint32_t)(reg_off[t.y_reg] + t.y) << 16 |
+                                (uint32_t)t.neg << 31);
+            if ((st = upload(&c->d_run_off, minor->run_off.data(), minor->run_off.size())) != MBC_OK ||
+                (st = upload(&c->d_term_off, minor->term_off.data(), minor->term_off.size())) != MBC_OK ||
+                (st = upload(&c->d_run_coef, minor->run_coef.data(), minor->run_coef.size())) != MBC_OK ||
+                (st = upload(&c->d_terms, terms.data(), terms.size())) != MBC_OK) {
+                free_cache(c);
+                return nullptr;
+            }
+            c->sp.run_off = c->d_run_off;
+            c->sp.term_off = c->d_term_off;
+            c->sp.run_coef = c->d_run_coef;
+            c->sp.terms = c->d_terms;
         }
         if ((st = upload(&c->d_small_zops, zpk.data(), zpk.size())) != MBC_OK) {
             free_cache(c);
@@ -1447,8 +1531,10 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
         if (regime == 1 && !small) return MBC_ERR_UNSUPPORTED;
         (small ? small_ids : large_ids).push_back(li);
     }
+    // minor-form lists first: lists of one form share their tile (and block)
     std::stable_sort(small_ids.begin(), small_ids.end(), [&](int a, int b) {
-        return lists[a]->stats.n_ops_total > lists[b]->stats.n_ops_total;
+        const int fa = caches[(size_t)a]->sp.bilinear, fb = caches[(size_t)b]->sp.bilinear;
+        return fa != fb ? fa > fb : lists[a]->stats.n_ops_total > lists[b]->stats.n_ops_total;
     });
     struct BatchRun {
         std::vector<int> ids;
@@ -1464,6 +1550,7 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
         while (i < small_ids.size() && (int)br.ids.size() < kMaxBatch) {
             std::vector<const DeviceCache *> trial = cs;
             trial.push_back(caches[(size_t)small_ids[i]]);
+            if (trial[0]->sp.bilinear != trial.back()->sp.bilinear) break;
             int32_t ss, cc;
             SmallLaunch l = size_small_batch(trial, F, opts->tune, mixed, ss, cc);
             if (!l.ok && !br.ids.empty()) break;
@@ -1493,13 +1580,11 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
         for (int j = 1; j < br.B.n_lists && share; ++j) {
             const SmallPlan &a = br.B.plan[0], &b = br.B.plan[j];
             share = a.nxi == b.nxi && a.dim == b.dim && a.n_g2 == b.n_g2 && a.block_size == b.block_size &&
-                    a.npair == b.npair && a.s_off == b.s_off && a.q_off == b.q_off && a.blk_off[0] == b.blk_off[0] &&
-                    a.blk_off[1] == b.blk_off[1];
+                    a.npair == b.npair && a.s_off == b.s_off && a.q_off == b.q_off && a.blk_off == b.blk_off &&
+                    a.bilinear == b.bilinear;
         }
         if (share) {
             br.B.shared = 1;
-            for (int j = 0; j < br.B.n_lists; ++j)
-                for (int b = 0; b < 2; ++b) br.B.need_union[b] |= br.B.plan[j].need_blk[b];
             br.B.total_items = n_slabs * br.sl.tiles_per_slab;
         }
         br.part_bytes = (size_t)poff * sizeof(double2);
@@ -1794,7 +1879,8 @@ extern "C" mbc_status mbc_contract_noalloc(const mbc_props *props, const mbc_ter
     SmallLaunch l;
     if (!zero) {
         std::vector<int> part_off;
-        if (!plan_small(list, hp, site_entries, part_off)) return MBC_ERR_UNSUPPORTED;  // relativistic lists: no static variant
+        const std::shared_ptr<const MinorPlan> minor = minor_plan(list);
+        if (!plan_small(list, minor.get(), hp, site_entries, part_off)) return MBC_ERR_UNSUPPORTED;  // relativistic lists: no static variant
         // the launch shape the kernel will run with, and from it the bytes
         // of the tile partials (one sizing, used for the check and the launch)
         l = size_small_tiles((int32_t)site_entries, hp.n_comp, F, opts->tune, false);

@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cstdint>
+#include <memory>
 #include <mutex>
 #include <vector>
 
@@ -36,6 +37,7 @@ struct Step {
 };
 
 struct DeviceCache;  // defined by the CUDA side
+struct MinorPlan;    // plan.h
 
 }  // namespace mbc
 
@@ -71,6 +73,10 @@ struct mbc_term_list {
     // device copies, one per device ordinal, created on first use
     std::mutex dev_mu;
     std::vector<mbc::DeviceCache *> dev;
+    // evaluation plans derived from the list (plan.h), made at first use
+    std::mutex plan_mu;
+    std::shared_ptr<const mbc::MinorPlan> minor;
+    bool minor_tried = false;
 };
 
 namespace mbc {

@@ -13,6 +13,10 @@
 //   3. every step F^(m+1)[z] = sum_j s_j F^(m)[x_j] f[y_j] (eq. recr_F) over
 //      the z-major lists; g lanes share one z and combine by xor shuffles;
 //   4. the contraction with L (eq. C_final) into FP64;
+// Lists whose minor form (plan.h) takes fewer operations - 3He and 4He: 1.8 K
+// complex multiply-adds per site for both instead of 19.6 K - skip 2., build
+// minors of the tile in 3. (the same step code on other operands) and sum
+// signed products of two minors in 4.;
 // then the CTA multiplies each site's components by the momentum phases and
 // sums its T sites in a fixed order into one partial per (tile, mom, comp).
 #pragma once
@@ -36,7 +40,7 @@ struct SmallStepDesc {
 struct SmallPlan {
     int32_t A, dim, nxi, n_g2, n_comp, n_steps;
     int32_t path0;
-    int32_t need_blk[2], blk_off[2];
+    int32_t blk_off;                    // the block of both species (u = d)
     int32_t s_off, q_off;               // entry offsets in the per-site region
     int32_t site_entries;               // per-site region size (entries)
     int32_t block_size, npair;
@@ -46,6 +50,11 @@ struct SmallPlan {
     const uint32_t *zops;               // the same ops, z-major
     int32_t part_off;                   // lanes-are-sites: split partials (64 entries)
     const int64_t *fin_off;             // n_comp + 1
+    int32_t bilinear;                   // minor form: the contraction sums products of two entries
+    const int32_t *run_off;             // minor form: runs of component c (n_comp + 1)
+    const int32_t *term_off;            // terms of run r (n_runs + 1)
+    const double *run_coef;             // coefficient of run r
+    const uint32_t *terms;              // entry offsets x | y << 16 | sign << 31
     const uint32_t *fin_z;              // entry offsets in the per-site region
     const double *fin_l;                // integer L values
     const double *comp_inv_norm;        // per component: 1 / (n_P! n_N!)^2 of its nucleus
@@ -57,8 +66,8 @@ struct SmallPlan {
 // puts the most expensive list first), handed out by an atomic counter. In a
 // shared batch (lists with the same tile shape and buffer offsets of the S
 // tile, diquark and blocks) an item is a tile and covers every list: the
-// tile and the blocks (of the baryons any list needs) are computed once per
-// site, then each list runs its steps and contraction.
+// tile and the block are computed once per site, then each list runs its
+// steps and contraction.
 constexpr int kMaxBatch = 8;
 struct SmallBatch {
     int32_t n_lists;
@@ -66,7 +75,6 @@ struct SmallBatch {
     int32_t comp_stride;      // warp-per-site kernel: components per site in the C area (max)
     int32_t tiles_per_slab;
     int32_t shared;           // items are tiles covering every list
-    int32_t need_union[2];    // shared: blocks some list needs
     int64_t total_items;
     int64_t item_base[kMaxBatch + 1];
     int64_t partial_off[kMaxBatch];  // in double2 units
@@ -180,39 +188,38 @@ __device__ __forceinline__ void small_step(const SmallPlan &P, const SmallStepDe
     __syncwarp();
 }
 
-// Blocks (Sec. 2) for one site: Q, then f_P and/or f_N antisymmetric parts.
+// Blocks (Sec. 2) for one site: Q, then the antisymmetric block. With u = d
+// one block serves both species: Q[c][x2][x3] is symmetric in (x2, x3) (Gamma_2
+// and epsilon are both antisymmetric), so the proton (pair u, single d) and the
+// neutron (pair d, single u) have the same numbers, and Q is computed for
+// x2 <= x3 only.
 template <class Tr>
-__device__ __forceinline__ void small_blocks(const SmallPlan &P, const int32_t *need, typename Tr::V *R, int lane) {
+__device__ __forceinline__ void small_blocks(const SmallPlan &P, typename Tr::V *R, int lane) {
     using V = typename Tr::V;
-    const int nxi = P.nxi;
+    const int nxi = P.nxi, ntri = P.npair + nxi;
     const V *S = R + P.s_off;
     V *Q = R + P.q_off;
-    for (int e = lane; e < 3 * nxi * nxi; e += 32) {
-        int c = e / (nxi * nxi), r = e % (nxi * nxi);
-        Q[e] = diquark(S, nxi, nxi, P.n_g2, c, r / nxi, r % nxi);
+    for (int e = lane; e < 3 * ntri; e += 32) {
+        const int c = e / ntri, r = e % ntri;
+        const int x2 = r < P.npair ? c_pair_i[r] : r - P.npair, x3 = r < P.npair ? c_pair_j[r] : r - P.npair;
+        const V q = diquark(S, nxi, nxi, P.n_g2, c, x2, x3);
+        Q[(c * nxi + x2) * nxi + x3] = q;
+        Q[(c * nxi + x3) * nxi + x2] = q;
     }
     __syncwarp();
     const int per_spin = P.npair * nxi;
-    for (int b = 0; b < 2; ++b) {
-        if (!need[b]) continue;
-        V *F = R + P.blk_off[b];
-        for (int e = lane; e < P.block_size; e += 32) {
-            int dl = e / per_spin, r = e % per_spin;
-            int pr = r / nxi, single = r % nxi;
-            int i = c_pair_i[pr], j = c_pair_j[pr];
-            V acc{0, 0};
-            for (int c = 0; c < 3; ++c) {
-                const V *Sr = S + (3 * dl + c) * nxi;
-                if (b == 0) {  // proton: u pair (i, j) at slots 1, 2; d = single at slot 3
-                    acc = cfma(Sr[i], Q[(c * nxi + j) * nxi + single], acc);
-                    acc = cfms(Sr[j], Q[(c * nxi + i) * nxi + single], acc);
-                } else {  // neutron: d pair (i, k=j) at slots 1, 3; u = single at slot 2
-                    acc = cfma(Sr[i], Q[(c * nxi + single) * nxi + j], acc);
-                    acc = cfms(Sr[j], Q[(c * nxi + single) * nxi + i], acc);
-                }
-            }
-            F[e] = acc;
+    V *F = R + P.blk_off;
+    for (int e = lane; e < P.block_size; e += 32) {
+        int dl = e / per_spin, r = e % per_spin;
+        int pr = r / nxi, single = r % nxi;
+        int i = c_pair_i[pr], j = c_pair_j[pr];
+        V acc{0, 0};
+        for (int c = 0; c < 3; ++c) {
+            const V *Sr = S + (3 * dl + c) * nxi;
+            acc = cfma(Sr[i], Q[(c * nxi + j) * nxi + single], acc);
+            acc = cfms(Sr[j], Q[(c * nxi + i) * nxi + single], acc);
         }
+        F[e] = acc;
     }
     __syncwarp();
 }
@@ -257,7 +264,7 @@ __global__ void __launch_bounds__(1024, 1)
             for (int e = lane; e < nent; e += 32) R[P0.s_off + e] = Tr::from_d(load_prop(F, base, (e / nxi) * 12 + (e % nxi)));
             __syncwarp();
             // 2. blocks, once for every list of the item
-            small_blocks<Tr>(P0, B.shared ? B.need_union : P0.need_blk, R, lane);
+            if (!P0.bilinear) small_blocks<Tr>(P0, R, lane);
         }
         for (int li = li0; li < l_end; ++li) {
             const SmallPlan &P = B.plan[li];
@@ -270,7 +277,20 @@ __global__ void __launch_bounds__(1024, 1)
                 for (int c0 = 0; c0 < P.n_comp; c0 += per) {
                     int c = c0 + lane / g;
                     double re = 0.0, im = 0.0;
-                    if (c < P.n_comp) {
+                    if (c < P.n_comp && P.bilinear) {
+                        for (int r = P.run_off[c]; r < P.run_off[c + 1]; ++r) {
+                            typename Tr::Acc acc;
+                            acc.zero();
+                            for (int e = P.term_off[r] + sub; e < P.term_off[r + 1]; e += g) {
+                                const uint32_t op = __ldg(P.terms + e);
+                                acc.fma(R[op & 0xffffu], R[(op >> 16) & 0x7fffu], op & 0x80000000u);
+                            }
+                            const double2 v = acc.value();
+                            const double coef = __ldg(P.run_coef + r);
+                            re = __fma_rn(coef, v.x, re);
+                            im = __fma_rn(coef, v.y, im);
+                        }
+                    } else if (c < P.n_comp) {
                         for (int64_t e = P.fin_off[c] + sub; e < P.fin_off[c + 1]; e += g) {
                             double2 f = Tr::to_d(R[__ldg(P.fin_z + e)]);
                             double l = __ldg(P.fin_l + e);

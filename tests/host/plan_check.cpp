@@ -1,0 +1,172 @@
+// Host check of the evaluation plans (plan.h): on random propagators the minor
+// form of a list gives the components that the list's own recursion gives,
+// with every operand inside its region.
+#include <complex>
+#include <cstdio>
+#include <cstring>
+#include <random>
+#include <vector>
+
+#include "../../paper_1301_4895_gb300/csrc/builder.cpp"
+#include "../../paper_1301_4895_gb300/csrc/plan.cpp"
+
+namespace mbc {
+void free_device_cache(mbc_term_list *) {}
+}  // namespace mbc
+
+using cd = std::complex<double>;
+
+// blocks [spin][pair][single] of a tile S[row][col] (u = d: one block for both species)
+static std::vector<cd> block(const mbc_term_list &L, const std::vector<cd> &S) {
+    const int n = L.nxi, ns = L.n_sources;
+    const int g2[4][3] = {{0, 1, -1}, {1, 0, 1}, {2, 3, -1}, {3, 2, 1}};
+    auto lc = [](int a, int b, int c) { return (a - b) * (b - c) * (c - a) / 2; };
+    (void)ns;
+    std::vector<cd> f;
+    for (int a = 0; a < L.dim; ++a)
+        for (int j = 1; j < n; ++j)
+            for (int i = 0; i < j; ++i)
+                for (int s = 0; s < n; ++s) {
+                    cd v = 0;
+                    for (int g = 0; g < L.dim; ++g)
+                        for (int c1 = 0; c1 < 3; ++c1)
+                            for (int c2 = 0; c2 < 3; ++c2)
+                                for (int c3 = 0; c3 < 3; ++c3) {
+                                    const double e = lc(c1, c2, c3) * g2[g][2];
+                                    if (e == 0) continue;
+                                    const cd *r1 = &S[(size_t)(3 * a + c1) * n], *r2 = &S[(size_t)(3 * g2[g][0] + c2) * n],
+                                             *r3 = &S[(size_t)(3 * g2[g][1] + c3) * n];
+                                    v += e * (r1[i] * r2[j] - r1[j] * r2[i]) * r3[s];
+                                }
+                    f.push_back(v);
+                }
+    return f;
+}
+
+// components and their magnitudes by the list's own operations
+static void chain(const mbc_term_list &L, const std::vector<cd> &f, std::vector<cd> &C, std::vector<double> &mag) {
+    C.assign((size_t)L.n_comp, 0);
+    mag.assign((size_t)L.n_comp, 0);
+    std::vector<cd> x = f;
+    for (int m = 1; m <= L.A; ++m) {
+        if (m > 1) {
+            const auto &s = L.steps[(size_t)m - 2];
+            std::vector<cd> z((size_t)s.n_z, 0);
+            for (int64_t i = 0; i < s.n_z; ++i)
+                for (int64_t j = 0; j < s.k; ++j) {
+                    const size_t o = (size_t)(i * s.k + j);
+                    const cd t = x[s.x[o]] * f[s.ys[o] & 0x7fff];
+                    z[(size_t)i] += s.ys[o] & 0x8000 ? -t : t;
+                }
+            x.swap(z);
+        }
+        for (const auto &pt : L.parts)
+            for (int c = pt.c0; pt.A == m && c < pt.c1; ++c)
+                for (int64_t e = L.fin_off[(size_t)c]; e < L.fin_off[(size_t)c + 1]; ++e) {
+                    const cd t = L.fin_l[(size_t)e] * x[L.fin_z[(size_t)e]];
+                    C[(size_t)c] += t;
+                    mag[(size_t)c] += std::abs(t);
+                }
+    }
+}
+
+static int bad_minors(const char *name, const mbc_term_list &L, bool expect, std::mt19937 &rng) {
+    const auto P = mbc::minor_plan(&L);
+    if (!!P != expect) {
+        std::printf("%s: minor form %s\n", name, P ? "made" : "not made");
+        return 1;
+    }
+    if (!P) return 0;
+    std::normal_distribution<double> nd;
+    std::vector<cd> S((size_t)L.nxi * L.nxi);
+    for (auto &v : S) v = cd(nd(rng), nd(rng));
+    std::vector<cd> C;
+    std::vector<double> mag;
+    chain(L, block(L, S), C, mag);
+    std::vector<cd> reg[8];
+    reg[1] = S;
+    for (const auto &s : P->steps) {
+        reg[s.z_reg].assign((size_t)s.n_z, 0);
+        for (int64_t o = 0; o < (int64_t)s.n_z * s.k; ++o) {
+            const cd t = reg[s.x_reg].at(s.x[(size_t)o]) * reg[s.y_reg].at(s.y[(size_t)o]);
+            reg[s.z_reg][(size_t)(o / s.k)] += s.neg[(size_t)o] ? -t : t;
+        }
+    }
+    double worst = 0;
+    for (int c = 0; c < L.n_comp; ++c) {
+        cd v = 0;
+        for (int r = P->run_off[(size_t)c]; r < P->run_off[(size_t)c + 1]; ++r)
+            for (int e = P->term_off[(size_t)r]; e < P->term_off[(size_t)r + 1]; ++e) {
+                const auto &t = P->terms[(size_t)e];
+                const cd p = reg[t.x_reg].at(t.x) * reg[t.y_reg].at(t.y);
+                v += (t.neg ? -1.0 : 1.0) * P->run_coef[(size_t)r] * p;
+            }
+        const double scale = mag[(size_t)c] > 0 ? mag[(size_t)c] : 1.0;
+        worst = std::max(worst, std::abs(v - C[(size_t)c]) / scale);
+    }
+    std::printf("%s: minor form, %zu products, worst difference %.1e\n", name, P->terms.size(), worst);
+    return worst > 1e-11;
+}
+
+static mbc_op_spec spec(int np, int nn, int D) {
+    mbc_op_spec s;
+    std::memset(&s, 0, sizeof(s));
+    s.n_p = np;
+    s.n_n = nn;
+    s.dirac_dim = D;
+    s.n_sources = s.n_sinks = 1;
+    return s;
+}
+
+int main() {
+    std::mt19937 rng(7);
+    int bad = 0;
+    auto build1 = [](const mbc_op_spec &s) {
+        mbc_term_list *L = nullptr;
+        mbc_build_term_list(&s, &L);
+        return L;
+    };
+    struct Case {
+        const char *name;
+        int np, nn, D, list_free;
+        bool minors;
+    };
+    for (const Case &c : {Case{"3He", 2, 1, 2, 0, true}, Case{"3H", 1, 2, 2, 0, true}, Case{"4He", 2, 2, 2, 0, true},
+                          Case{"pn", 1, 1, 2, 0, false}, Case{"pn rel", 1, 1, 4, 0, false}}) {
+        mbc_op_spec s = spec(c.np, c.nn, c.D);
+        s.list_free = c.list_free;
+        mbc_term_list *L = build1(s);
+        bad += bad_minors(c.name, *L, c.minors, rng);
+        mbc_free_term_list(L);
+    }
+    {  // a projection: several sink and source sets with weights in one output
+        const int8_t snk[9] = {1, 0, 0, 0, 1, 1, 0, 1, 0}, src[9] = {0, 1, 0, 0, 1, 1, 1, 0, 1};
+        const int32_t to[3] = {0, 0, 1};
+        const double w[3] = {0.5, -0.25, 1.5};
+        mbc_op_spec s = spec(2, 1, 2);
+        s.spin_mode = MBC_SPIN_PROJECTED;
+        s.n_spin_sel = 3;
+        s.n_proj = 2;
+        s.snk_spins = snk;
+        s.src_spins = src;
+        s.term_proj = to;
+        s.term_coef = w;
+        mbc_term_list *L = build1(s);
+        bad += bad_minors("3He projections", *L, true, rng);
+        mbc_free_term_list(L);
+    }
+    {  // two nuclei on one path, both orders of adding baryons
+        for (int o = 0; o < 2; ++o) {
+            const int8_t path[2][4] = {{0, 0, 1, 1}, {0, 1, 0, 1}};
+            mbc_op_spec s[2] = {spec(2, 1, 2), spec(2, 2, 2)};
+            s[1].path = path[o];
+            s[1].path_len = 4;
+            mbc_term_list *L = nullptr;
+            mbc_build_combined(s, 2, &L);
+            bad += bad_minors("3He and 4He on one path", *L, true, rng);
+            mbc_free_term_list(L);
+        }
+    }
+    std::printf("%s\n", bad ? "FAIL" : "OK");
+    return bad ? 1 : 0;
+}
