@@ -30,6 +30,7 @@ inline void note_launch() { g_kernel_launches.fetch_add(1, std::memory_order_rel
 }  // namespace mbc
 #include "probe.cuh"
 #include "project_kernel.cuh"
+#include "saturated_kernel.cuh"
 #include "small_kernel.cuh"
 #include "small_ls_kernel.cuh"
 
@@ -173,6 +174,8 @@ struct DeviceCache {
     int32_t *d_comp_deg = nullptr;
     int64_t max_stage = 0;
     std::vector<YRuns> yruns;          // per step, made on first mixed use
+    bool wave_ready = false;           // d_opx .. d_xmap uploaded
+    double *d_sat_coef = nullptr;      // saturated form: coefficient per component
 };
 
 namespace {
@@ -184,6 +187,7 @@ void free_cache(DeviceCache *c) {
     if (c->device >= 0) cudaSetDevice(c->device);
     cudaFree(c->d_small_ops);
     cudaFree(c->d_small_zops);
+    cudaFree(c->d_sat_coef);
     cudaFree(c->d_run_off);
     cudaFree(c->d_term_off);
     cudaFree(c->d_run_coef);
@@ -213,7 +217,12 @@ mbc_status upload(T **dst, const T *src, size_t n) {
     *dst = nullptr;
     if (n == 0) return MBC_OK;
     MBC_CUDA_TRY(cudaMalloc((void **)dst, n * sizeof(T)));
-    MBC_CUDA_TRY(cudaMemcpy(*dst, src, n * sizeof(T), cudaMemcpyHostToDevice));
+    if (cudaMemcpy(*dst, src, n * sizeof(T), cudaMemcpyHostToDevice) != cudaSuccess) {
+        (void)cudaGetLastError();
+        cudaFree(*dst);
+        *dst = nullptr;
+        return MBC_ERR_CUDA;
+    }
     return MBC_OK;
 }
 
@@ -340,6 +349,33 @@ bool plan_small(const mbc_term_list *L, const MinorPlan *minor, SmallPlan &P, in
     for (int c = 0; c < L->n_comp; ++c) kmax = std::max(kmax, L->fin_off[(size_t)c + 1] - L->fin_off[(size_t)c]);
     P.fin_g = pick_group(L->n_comp, kmax);
     return true;
+}
+
+// Operation arrays up to this size go to the device with the list's first use;
+// larger ones (8Be 2.7 GB, 4He with all components 3.2 GB) with the first call
+// that runs them, since other routes never read them.
+constexpr size_t kEagerOpBytes = (size_t)64 << 20;
+
+// The wave kernels' arrays of a list (caller holds the list's device lock).
+mbc_status upload_wave(const mbc_term_list *L, DeviceCache *c) {
+    if (c->wave_ready) return MBC_OK;
+    const size_t n = L->steps.size();
+    c->d_opx.resize(n, nullptr);
+    c->d_opy.resize(n, nullptr);
+    c->d_zrank.resize(n, nullptr);
+    c->d_xmap.resize(n, nullptr);
+    mbc_status st;
+    for (size_t m = 0; m < n; ++m) {
+        const Step &s = L->steps[m];
+        // what an earlier attempt uploaded before it ran out of memory stays
+        if ((!c->d_opx[m] && (st = upload(&c->d_opx[m], s.x.data(), s.x.size())) != MBC_OK) ||
+            (!c->d_opy[m] && (st = upload(&c->d_opy[m], s.ys.data(), s.ys.size())) != MBC_OK) ||
+            (!c->d_zrank[m] && (st = upload(&c->d_zrank[m], s.zrank.data(), s.zrank.size())) != MBC_OK) ||
+            (!c->d_xmap[m] && (st = upload(&c->d_xmap[m], s.xmap.data(), s.xmap.size())) != MBC_OK))
+            return st;
+    }
+    c->wave_ready = true;
+    return MBC_OK;
 }
 
 DeviceCache *get_cache(const mbc_term_list *Lc, int device, mbc_status &st) {
@@ -481,24 +517,32 @@ DeviceCache *get_cache(const mbc_term_list *Lc, int device, mbc_status &st) {
         c->sp.comp_inv_norm = c->d_comp_inv_norm;
         c->sp.comp_deg = c->d_comp_deg;
     }
-    // large-path op arrays
-    c->d_opx.assign(L->steps.size(), nullptr);
-    c->d_opy.assign(L->steps.size(), nullptr);
-    c->d_zrank.assign(L->steps.size(), nullptr);
-    c->d_xmap.assign(L->steps.size(), nullptr);
-    for (size_t m = 0; m < L->steps.size(); ++m) {
-        const Step &s = L->steps[m];
-        c->max_stage = std::max(c->max_stage, s.n_z);
-        if ((st = upload(&c->d_opx[m], s.x.data(), s.x.size())) != MBC_OK ||
-            (st = upload(&c->d_opy[m], s.ys.data(), s.ys.size())) != MBC_OK ||
-            (st = upload(&c->d_zrank[m], s.zrank.data(), s.zrank.size())) != MBC_OK ||
-            (st = upload(&c->d_xmap[m], s.xmap.data(), s.xmap.size())) != MBC_OK) {
+    if (const auto sat = saturated_plan(L)) {
+        if ((st = upload(&c->d_sat_coef, sat->coef.data(), sat->coef.size())) != MBC_OK) {
             free_cache(c);
             return nullptr;
         }
     }
+    size_t op_bytes = 0;
+    for (const auto &s : L->steps) {
+        c->max_stage = std::max(c->max_stage, s.n_z);
+        op_bytes += s.x.size() * sizeof(uint32_t) + s.ys.size() * sizeof(uint16_t);
+    }
+    if (op_bytes <= kEagerOpBytes && (st = upload_wave(L, c)) != MBC_OK) {
+        free_cache(c);
+        return nullptr;
+    }
     L->dev[(size_t)device] = c;
     return c;
+}
+
+// The list's device copy with the wave kernels' arrays.
+DeviceCache *get_wave_cache(const mbc_term_list *L, int device, mbc_status &st) {
+    DeviceCache *c = get_cache(L, device, st);
+    if (!c) return nullptr;
+    std::lock_guard<std::mutex> g(const_cast<mbc_term_list *>(L)->dev_mu);
+    st = upload_wave(L, c);
+    return st == MBC_OK ? c : nullptr;
 }
 
 // ---- scratch ---------------------------------------------------------------
@@ -1471,8 +1515,11 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
     for (int q = 0; q < opts->n_mom; ++q)
         for (int d = 0; d < 3; ++d) M.mom[q][d] = opts->mom[3 * q + d];
 
-    cudaError_t ce = cudaMemsetAsync(dev_out, 0, out_bytes, stream);
-    if (ce != cudaSuccess) return MBC_ERR_CUDA;
+    // entries no kernel writes are zero: the tails of lists with fewer
+    // components than the largest, and lists that vanish identically
+    bool whole = true;
+    for (int i = 0; i < n_lists; ++i) whole = whole && !lists[i]->pauli_forbidden && lists[i]->n_comp == comp_max;
+    if (!whole && cudaMemsetAsync(dev_out, 0, out_bytes, stream) != cudaSuccess) return MBC_ERR_CUDA;
     const int64_t n_slabs = (int64_t)props->n_cfg * n_t;
     const bool mixed = opts->precision == MBC_MIXED;
 
@@ -1485,7 +1532,7 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
         for (int li = 0; li < n_lists; ++li) {
             const mbc_term_list *L = lists[li];
             if (L->pauli_forbidden || L->n_comp == 0) continue;
-            cs[(size_t)li] = get_cache(L, device, st);
+            cs[(size_t)li] = get_wave_cache(L, device, st);
             if (!cs[(size_t)li]) return st;
             lsz[(size_t)li] = mixed ? large_sizes<MixedTraits>(L, cs[(size_t)li], opts->tune, n_items_p)
                                     : large_sizes<FP64Traits>(L, cs[(size_t)li], opts->tune, n_items_p);
@@ -1517,18 +1564,23 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
     const int64_t n_items = n_slabs * v3p;
     const int regime = opts->tune ? opts->tune->regime : 0;
     std::vector<DeviceCache *> caches((size_t)n_lists, nullptr);
-    std::vector<int> small_ids, large_ids;
+    std::vector<int> small_ids, large_ids, sat_ids;
     for (int li = 0; li < n_lists; ++li) {
         const mbc_term_list *L = lists[li];
         if (L->pauli_forbidden || L->n_comp == 0) continue;  // identically zero
         caches[(size_t)li] = get_cache(L, device, st);
         if (!caches[(size_t)li]) return st;
+        if (regime == 0 && caches[(size_t)li]->d_sat_coef) {
+            sat_ids.push_back(li);
+            continue;
+        }
         bool small = caches[(size_t)li]->small_ok && (!mixed || caches[(size_t)li]->ls_ok) && regime != 2;
         if (small) {  // the list alone must fit the shared-memory kernel
             int32_t ss, cs;
             small = size_small_batch({caches[(size_t)li]}, F, opts->tune, mixed, ss, cs).ok;
         }
         if (regime == 1 && !small) return MBC_ERR_UNSUPPORTED;
+        if (!small && !get_wave_cache(L, device, st)) return st;
         (small ? small_ids : large_ids).push_back(li);
     }
     // minor-form lists first: lists of one form share their tile (and block)
@@ -1593,6 +1645,11 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
     size_t small_bytes = 0;
     for (auto &br : batches) small_bytes += 256 + align256(br.part_bytes);
     size_t large_bytes = 0;
+    // 8Be: 8-site tiles only where 2-site ones would fill every SM several times
+    const int sat_sites = n_slabs * v3 > 16LL * kSatNarrow * sm_count(device) ? kSatWide : kSatNarrow;
+    const int sat_tiles = (int)((v3 + sat_sites - 1) / sat_sites);  // per slab
+    for (int li : sat_ids)
+        large_bytes = std::max(large_bytes, (size_t)(n_slabs * sat_tiles) * M.n_mom * lists[li]->n_comp * sizeof(double2));
     std::vector<LargeSizes> lsz((size_t)n_lists);
     for (int li : large_ids) {
         const mbc_term_list *L = lists[li];
@@ -1609,7 +1666,7 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
     void *scr = nullptr;
     if ((st = scratch_get(device, stream, phase_bytes + small_bytes + large_bytes, &scr)) != MBC_OK) return st;
     double2 *phase = reinterpret_cast<double2 *>(scr);
-    {
+    if (!small_ids.empty() || !large_ids.empty()) {  // the saturated kernel makes its own phases
         unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((v3 * M.n_mom + 255) / 256, 4096));
         note_launch();
         k_phase_table<<<grid, 256, 0, stream>>>(F, M, phase);
@@ -1636,6 +1693,19 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
         for (int j = 0; j < br.B.n_lists; ++j)
             if ((st = reduce(br.ids[(size_t)j], partial + br.B.partial_off[j], br.sl.tiles_per_slab)) != MBC_OK)
                 return st;
+    }
+    for (int li : sat_ids) {
+        double2 *partial = reinterpret_cast<double2 *>(cur);
+        if (n_slabs * sat_tiles > 0x7fffffff) return MBC_ERR_INVALID_ARG;
+        {
+            TimedLaunch tl(stream);
+            note_launch();
+            auto kern = sat_sites == kSatWide ? k_saturated<kSatWide> : k_saturated<kSatNarrow>;
+            kern<<<(unsigned)(n_slabs * sat_tiles), 16 * sat_sites, 0, stream>>>(
+                F, M, caches[(size_t)li]->d_sat_coef, lists[li]->n_comp, sat_tiles, partial);
+        }
+        MBC_CUDA_TRY(cudaGetLastError());
+        if ((st = reduce(li, partial, sat_tiles)) != MBC_OK) return st;
     }
     for (int li : large_ids) {
         const mbc_term_list *L = lists[li];

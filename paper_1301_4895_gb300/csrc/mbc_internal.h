@@ -38,6 +38,7 @@ struct Step {
 
 struct DeviceCache;  // defined by the CUDA side
 struct MinorPlan;    // plan.h
+struct SaturatedPlan;
 
 }  // namespace mbc
 
@@ -76,7 +77,8 @@ struct mbc_term_list {
     // evaluation plans derived from the list (plan.h), made at first use
     std::mutex plan_mu;
     std::shared_ptr<const mbc::MinorPlan> minor;
-    bool minor_tried = false;
+    std::shared_ptr<const mbc::SaturatedPlan> saturated;
+    bool minor_tried = false, saturated_tried = false;
 };
 
 namespace mbc {

@@ -250,7 +250,55 @@ std::shared_ptr<const MinorPlan> make_minor_plan(const mbc_term_list &L) {
     return minor < chain ? P : nullptr;
 }
 
+std::shared_ptr<const SaturatedPlan> make_saturated_plan(const mbc_term_list &L) {
+    if (L.dim != 4 || L.n_sources != 1 || L.n_sinks != 1 || L.n_comp < 1 || L.parts.size() != 1) return nullptr;
+    const auto &pt = L.parts[0];
+    if (2 * pt.n_p + pt.n_n != L.nxi || pt.n_p + 2 * pt.n_n != L.nxi || pt.c0 != 0 || pt.c1 != L.n_comp) return nullptr;
+    std::vector<std::vector<PlanEntry>> comp;
+    if (!list_entries(L, comp)) return nullptr;
+    const uint32_t all = (1u << L.nxi) - 1;
+    auto P = std::make_shared<SaturatedPlan>();
+    std::map<std::pair<uint32_t, uint32_t>, double> sink;
+    for (const auto &entries : comp) {
+        double v = 0.0;
+        for (const auto &e : entries) {
+            auto it = sink.find({e.z.dp, e.z.dn});
+            if (it == sink.end()) {
+                std::map<std::pair<uint32_t, uint32_t>, int64_t> neutron;
+                for (const auto &n : species_tensor(L.dim, e.z.dn)) neutron[{n.single, n.pair}] = n.v;
+                double t = 0.0;
+                for (const auto &p : species_tensor(L.dim, e.z.dp)) {
+                    const auto n = neutron.find({all ^ p.pair, all ^ p.single});
+                    if (n == neutron.end()) continue;
+                    const int neg = parity(p.pair, n->first.first) ^ parity(p.single, n->first.second);
+                    t += (double)p.v * (double)n->second * (neg ? -1.0 : 1.0);
+                }
+                // full signed sums: n_P! n_N! times the ordered product
+                t *= std::tgamma(pt.n_p + 1.0) * std::tgamma(pt.n_n + 1.0);
+                it = sink.insert({{e.z.dp, e.z.dn}, t}).first;
+            }
+            v += e.l * it->second;
+        }
+        P->coef.push_back(v / pt.norm);
+    }
+    return P;
+}
+
 }  // namespace
+
+std::shared_ptr<const SaturatedPlan> saturated_plan(const mbc_term_list *Lc) {
+    mbc_term_list *L = const_cast<mbc_term_list *>(Lc);
+    std::lock_guard<std::mutex> g(L->plan_mu);
+    if (!L->saturated_tried) {
+        try {
+            L->saturated = make_saturated_plan(*L);
+            L->saturated_tried = true;
+        } catch (const std::bad_alloc &) {
+            return nullptr;
+        }
+    }
+    return L->saturated;
+}
 
 std::shared_ptr<const MinorPlan> minor_plan(const mbc_term_list *Lc) {
     mbc_term_list *L = const_cast<mbc_term_list *>(Lc);

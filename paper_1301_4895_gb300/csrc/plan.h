@@ -76,4 +76,13 @@ struct MinorPlan {
 // and 4He on 16^3 x 32 sites: FP64 18.42 -> 2.69 ms, mixed 2.05 -> 0.86 ms.
 std::shared_ptr<const MinorPlan> minor_plan(const mbc_term_list *L);
 
+// Saturated form of a relativistic point-sink list: where every contracted
+// component takes all 12 u and all 12 d indices (8Be), the only minors left are
+// the determinants, C_c = coef[c] det S_u det S_d (Sec. 8), coef[c] the
+// contraction of the two tensors' single entries.
+struct SaturatedPlan {
+    std::vector<double> coef;
+};
+std::shared_ptr<const SaturatedPlan> saturated_plan(const mbc_term_list *L);
+
 }  // namespace mbc

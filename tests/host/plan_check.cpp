@@ -167,6 +167,26 @@ int main() {
             mbc_free_term_list(L);
         }
     }
+    {  // 8Be: L^2 = 1,814,400^2; an odd order of the sink spins flips the sign
+        const int8_t snk[16] = {0, 1, 2, 3, 0, 1, 2, 3, 1, 0, 2, 3, 0, 1, 2, 3};
+        const int8_t src[16] = {0, 1, 2, 3, 0, 1, 2, 3, 0, 1, 2, 3, 0, 1, 2, 3};
+        mbc_op_spec s = spec(4, 4, 4);
+        s.spin_mode = MBC_SPIN_LISTED;
+        s.n_spin_sel = 2;
+        s.snk_spins = snk;
+        s.src_spins = src;
+        s.list_free = 1;
+        mbc_term_list *L = build1(s);
+        const auto P = mbc::saturated_plan(L);
+        const double K = 1814400.0 * 1814400.0;
+        const bool ok = P && P->coef.size() == 2 && P->coef[0] == K && P->coef[1] == -K;
+        std::printf("8Be: saturated form %s\n", ok ? "as expected" : "wrong");
+        bad += !ok;
+        mbc_free_term_list(L);
+        L = build1(spec(2, 2, 2));
+        bad += mbc::saturated_plan(L) != nullptr;
+        mbc_free_term_list(L);
+    }
     std::printf("%s\n", bad ? "FAIL" : "OK");
     return bad ? 1 : 0;
 }
