@@ -52,7 +52,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         ["g++", "-O3", "-std=c++17", "-fPIC", "-fopenmp", *inc, "-c", os.path.join(CSRC, "builder.cpp"), "-o",
          cpp_obj],
         ["g++", "-O2", "-std=c++17", "-fPIC", *inc, "-c", os.path.join(CSRC, "list_io.cpp"), "-o", io_obj],
-        ["g++", "-O2", "-std=c++17", "-fPIC", *inc, "-c", os.path.join(CSRC, "plan.cpp"), "-o", plan_obj],
+        ["g++", "-O3", "-std=c++17", "-fPIC", "-fopenmp", *inc, "-c", os.path.join(CSRC, "plan.cpp"), "-o", plan_obj],
     ]
 
     def run(cmd):

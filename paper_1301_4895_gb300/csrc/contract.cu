@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "large_kernel.cuh"
+#include "pair_kernel.cuh"
 #include "mbc_internal.h"
 #include "plan.h"
 
@@ -176,6 +177,18 @@ struct DeviceCache {
     std::vector<YRuns> yruns;          // per step, made on first mixed use
     bool wave_ready = false;           // d_opx .. d_xmap uploaded
     double *d_sat_coef = nullptr;      // saturated form: coefficient per component
+    // pair form (plan.h), one launch per tile shape of its units
+    std::shared_ptr<const PairPlan> pair;
+    uint32_t *d_pair_x = nullptr;      // two-baryon products
+    uint16_t *d_pair_ys = nullptr;
+    uint32_t *d_pair_row = nullptr, *d_pair_col = nullptr;
+    double *d_pair_val = nullptr;
+    PairUnit *d_pair_units[2] = {nullptr, nullptr};  // FP64 and mixed tiles
+    int32_t n_pair_units[2] = {0, 0};
+    int32_t *d_pair_comp_off = nullptr, *d_pair_comp_eval = nullptr;
+    int32_t *d_pair_slot_off[2] = {nullptr, nullptr};
+    int32_t pair_slots[2] = {0, 0};
+    int pair_shape[2] = {0, 0};        // index into kPairShapes
 };
 
 namespace {
@@ -188,6 +201,17 @@ void free_cache(DeviceCache *c) {
     cudaFree(c->d_small_ops);
     cudaFree(c->d_small_zops);
     cudaFree(c->d_sat_coef);
+    cudaFree(c->d_pair_x);
+    cudaFree(c->d_pair_ys);
+    cudaFree(c->d_pair_row);
+    cudaFree(c->d_pair_col);
+    cudaFree(c->d_pair_val);
+    cudaFree(c->d_pair_comp_off);
+    cudaFree(c->d_pair_comp_eval);
+    for (int m = 0; m < 2; ++m) {
+        cudaFree(c->d_pair_units[m]);
+        cudaFree(c->d_pair_slot_off[m]);
+    }
     cudaFree(c->d_run_off);
     cudaFree(c->d_term_off);
     cudaFree(c->d_run_coef);
@@ -545,6 +569,113 @@ DeviceCache *get_wave_cache(const mbc_term_list *L, int device, mbc_status &st) 
     return st == MBC_OK ? c : nullptr;
 }
 
+// Tile shapes (proton x neutron elements per unit) of the pair kernels: one
+// component, a few, all. With more accumulators a warp reuses a row sum y for
+// more components; mixed sums carry a compensation word each, so its largest
+// tile is 6 x 2 (96 accumulator registers) against FP64's 6 x 6 (144).
+constexpr int kPairShapes[2][3][2] = {{{1, 1}, {2, 2}, {6, 6}}, {{1, 1}, {2, 2}, {6, 2}}};
+// Units per SM: enough that the last ones finish together, few enough that
+// their partial sums stay small beside the products; a unit has at least
+// kPairUnitRows rows.
+constexpr int kPairUnitsPerSm = 16;
+constexpr int kPairUnitRows = 16;
+
+// Units of a pair plan for one tile shape: the groups' rows cut into chunks of
+// about equal work.
+void pair_units(const PairPlan &P, const int shape[2], int n_sm, std::vector<PairUnit> &units,
+                std::vector<int32_t> &slot_off) {
+    const int MP = shape[0], MN = shape[1];
+    // cost of rows: entries x neutron elements (2 multiply-adds) + products (4)
+    auto cost = [&](int64_t nnz, int64_t rows, int64_t na, int64_t nb) { return nnz * nb * 2 + rows * na * nb * 4; };
+    int64_t total = 0;
+    for (const auto &g : P.groups)
+        total += cost(P.row_ptr[(size_t)g.row1] - P.row_ptr[(size_t)g.row0], g.row1 - g.row0, (int64_t)g.mp.size(),
+                      (int64_t)g.mn.size());
+    const int64_t target = std::max<int64_t>(1, total / std::max(1, n_sm * kPairUnitsPerSm));
+    slot_off.assign((size_t)P.n_evals + 1, 0);
+    int32_t slot = 0;
+    for (const auto &g : P.groups) {
+        // row chunks of the group, the same for each of its tiles
+        const int64_t ta = std::min<int64_t>(MP, (int64_t)g.mp.size()), tb = std::min<int64_t>(MN, (int64_t)g.mn.size());
+        std::vector<int64_t> cut{g.row0};
+        int64_t acc = 0;
+        for (int64_t r = g.row0; r < g.row1; ++r) {
+            acc += cost(P.row_ptr[(size_t)r + 1] - P.row_ptr[(size_t)r], 1, ta, tb);
+            if (acc >= target && r + 1 - cut.back() >= kPairUnitRows && r + 1 < g.row1) {
+                cut.push_back(r + 1);
+                acc = 0;
+            }
+        }
+        cut.push_back(g.row1);
+        const int32_t nc = (int32_t)cut.size() - 1, nb = (int32_t)g.mn.size(), na = (int32_t)g.mp.size();
+        for (int32_t a = 0; a < na; ++a)
+            for (int32_t b = 0; b < nb; ++b) {
+                slot_off[(size_t)(g.eval0 + (int64_t)a * nb + b)] = slot + (a * nb + b) * nc;
+                slot_off[(size_t)(g.eval0 + (int64_t)a * nb + b) + 1] = slot + (a * nb + b + 1) * nc;
+            }
+        for (int32_t a0 = 0; a0 < na; a0 += MP)
+            for (int32_t b0 = 0; b0 < nb; b0 += MN)
+                for (int32_t k = 0; k < nc; ++k) {
+                    PairUnit u;
+                    std::memset(&u, 0, sizeof(u));
+                    u.row0 = (int32_t)cut[(size_t)k];
+                    u.e0 = P.row_ptr[(size_t)cut[(size_t)k]];
+                    u.e1 = P.row_ptr[(size_t)cut[(size_t)k + 1]];
+                    u.na = std::min(MP, na - a0);
+                    u.nb = std::min(MN, nb - b0);
+                    for (int i = 0; i < u.na; ++i) u.mp[i] = g.mp[(size_t)(a0 + i)];
+                    for (int i = 0; i < u.nb; ++i) u.mn[i] = g.mn[(size_t)(b0 + i)];
+                    u.stride_b = nc;
+                    u.stride_a = nb * nc;
+                    u.slot = slot + (a0 * nb + b0) * nc + k;
+                    units.push_back(u);
+                }
+        slot += na * nb * nc;
+    }
+}
+
+int sm_count(int device);
+
+// The list's device copy with its pair form (regime 0, one or two baryons per
+// species); c->pair stays empty where the list has none. Built and uploaded
+// with the first call that can use it.
+mbc_status ensure_pair(const mbc_term_list *Lc, DeviceCache *c, bool mixed) {
+    const std::shared_ptr<const PairPlan> P = pair_plan(Lc);
+    if (!P || (mixed && !P->val_fp32)) return MBC_OK;
+    std::lock_guard<std::mutex> lock(const_cast<mbc_term_list *>(Lc)->dev_mu);
+    const int m = mixed ? 1 : 0;
+    mbc_status st = MBC_OK;
+    auto put = [&](auto **dst, const auto *src, size_t n) {
+        if (st == MBC_OK && !*dst) st = upload(dst, src, n);
+    };
+    if (!c->pair) {
+        std::vector<uint32_t> col(P->col);
+        for (size_t r = 0; r + 1 < P->row_ptr.size(); ++r) col[(size_t)P->row_ptr[r + 1] - 1] |= 0x80000000u;
+        put(&c->d_pair_x, P->sx.data(), P->sx.size());
+        put(&c->d_pair_ys, P->sys.data(), P->sys.size());
+        put(&c->d_pair_row, P->row_id.data(), P->row_id.size());
+        put(&c->d_pair_col, col.data(), col.size());
+        put(&c->d_pair_val, P->val.data(), P->val.size());
+        put(&c->d_pair_comp_off, P->comp_off.data(), P->comp_off.size());
+        put(&c->d_pair_comp_eval, P->comp_eval.data(), P->comp_eval.size());
+        if (st != MBC_OK) return st;
+        c->pair = P;
+    }
+    if (!c->d_pair_units[m]) {
+        size_t most = 0;
+        for (const auto &g : P->groups) most = std::max({most, g.mp.size(), g.mn.size()});
+        c->pair_shape[m] = most <= 1 ? 0 : most <= 2 ? 1 : 2;
+        std::vector<PairUnit> units;
+        std::vector<int32_t> slot_off;
+        pair_units(*P, kPairShapes[m][c->pair_shape[m]], sm_count(c->device), units, slot_off);
+        put(&c->d_pair_slot_off[m], slot_off.data(), slot_off.size());
+        put(&c->d_pair_units[m], units.data(), units.size());
+        c->n_pair_units[m] = (int32_t)units.size();
+        c->pair_slots[m] = slot_off.empty() ? 0 : slot_off.back();
+    }
+    return st;
+}
+
 // ---- scratch ---------------------------------------------------------------
 struct Scratch {
     void *p = nullptr;
@@ -718,19 +849,51 @@ mbc_status launch_small_batch(const SmallBatch &B, const FieldDesc &F, const Mom
     return MBC_OK;
 }
 
+size_t align256(size_t n) { return (n + 255) & ~size_t(255); }
+
 // Site-operations (operations x sites) a wave needs at least.
 constexpr int64_t kWaveSiteOps = 20000000000LL;
 
 struct LargeSizes {
     int W;
-    size_t blk_bytes, stage_bytes, c_bytes, sexp_bytes;
+    bool pair;  // pair form: one stage buffer (the products) and the units' partial sums
+    size_t blk_bytes, stage_bytes, part_bytes, c_bytes, sexp_bytes;
+    size_t buffers() const {
+        return align256(blk_bytes) + (pair ? 1 : 2) * align256(stage_bytes) + align256(part_bytes) + align256(c_bytes) +
+               align256(sexp_bytes);
+    }
 };
+
+// Wave of the pair form: its products of 64 sites are what concurrent warps
+// gather from (site groups are the items' slow index), so the wave only has to
+// amortise its launches: up to 1024 sites (512 in FP64) within 1 GB.
+template <class Tr>
+LargeSizes pair_sizes(const mbc_term_list *L, const DeviceCache *c, const mbc_tune *tune, int64_t n_items) {
+    using V = typename Tr::V;
+    const bool mixed = sizeof(V) == sizeof(float2);
+    const PairPlan &P = *c->pair;
+    LargeSizes s{};
+    s.pair = true;
+    const int64_t prod = (int64_t)P.masks2.size() * P.n_rows2, slots = c->pair_slots[mixed ? 1 : 0];
+    const int64_t per_site = (int64_t)sizeof(V) * (L->block_size + prod) + 16 * (slots + L->n_comp) + 4;
+    int64_t W = std::min<int64_t>(mixed ? 1024 : 512, ((int64_t)1 << 30) / per_site);
+    if (tune && tune->wave_sites > 0) W = std::min(tune->wave_sites, 4096);
+    W = std::min<int64_t>(W, (n_items + 63) / 64 * 64);
+    W = std::max<int64_t>(64, W / 64 * 64);
+    s.W = (int)W;
+    s.blk_bytes = (size_t)(L->block_size * W) * sizeof(V);
+    s.stage_bytes = (size_t)(prod * W) * sizeof(V);
+    s.part_bytes = (size_t)(slots * W) * sizeof(double2);
+    s.c_bytes = (size_t)L->n_comp * W * sizeof(double2);
+    s.sexp_bytes = (size_t)W * sizeof(int32_t);
+    return s;
+}
 
 template <class Tr>
 LargeSizes large_sizes(const mbc_term_list *L, const DeviceCache *c, const mbc_tune *tune, int64_t n_items) {
     using V = typename Tr::V;
     LargeSizes s{};
-    int64_t per_site = (int64_t)sizeof(V) * (2 * L->block_size + 2 * std::max<int64_t>(c->max_stage, 1)) +
+    int64_t per_site = (int64_t)sizeof(V) * (L->block_size + 2 * std::max<int64_t>(c->max_stage, 1)) +
                        16LL * L->n_comp + 4;
     const int64_t budget = 8LL << 30;
     int64_t W = budget / per_site;
@@ -765,7 +928,26 @@ LargeSizes large_sizes(const mbc_term_list *L, const DeviceCache *c, const mbc_t
     return s;
 }
 
-size_t align256(size_t n) { return (n + 255) & ~size_t(255); }
+// A list takes its pair form unless the call forces the wave kernels or asks
+// them to regenerate operations.
+bool wants_pair(const mbc_tune *tune) { return !tune || (tune->regime == 0 && tune->list_free == 0); }
+bool has_pair(const DeviceCache *c, const mbc_tune *tune, bool mixed) {
+    return wants_pair(tune) && c->pair && c->d_pair_units[mixed ? 1 : 0];
+}
+
+// The list's device copy with what its large route reads.
+DeviceCache *get_large_cache(const mbc_term_list *L, int device, const mbc_tune *tune, bool mixed, mbc_status &st) {
+    DeviceCache *c = get_cache(L, device, st);
+    if (!c) return nullptr;
+    if (wants_pair(tune) && (st = ensure_pair(L, c, mixed)) != MBC_OK) return nullptr;
+    return has_pair(c, tune, mixed) ? c : get_wave_cache(L, device, st);
+}
+
+LargeSizes wave_sizes(const mbc_term_list *L, const DeviceCache *c, const mbc_tune *tune, int64_t n_items, bool mixed) {
+    if (has_pair(c, tune, mixed))
+        return mixed ? pair_sizes<MixedTraits>(L, c, tune, n_items) : pair_sizes<FP64Traits>(L, c, tune, n_items);
+    return mixed ? large_sizes<MixedTraits>(L, c, tune, n_items) : large_sizes<FP64Traits>(L, c, tune, n_items);
+}
 
 // Device description of step m (0-based) for regenerating its operations.
 GenStep gen_step(const mbc_term_list *L, const DeviceCache *c, size_t m) {
@@ -1067,6 +1249,64 @@ mbc_status contract_parts(const mbc_term_list *L, const DeviceCache *c, int stag
     return MBC_OK;
 }
 
+// The pair form of a wave from its blocks f: products of two baryons (a step
+// of 12 terms per output), the bilinear contraction, the sum over units.
+// deg_per_baryon as in contract_parts.
+template <class Tr>
+mbc_status pair_wave(const mbc_term_list *L, const DeviceCache *c, int W, const typename Tr::V *f,
+                     typename Tr::V *prod, double2 *part, const int32_t *sexp, int deg_per_baryon, double2 *Cb, int nsm,
+                     cudaStream_t stream) {
+    using V = typename Tr::V;
+    constexpr bool mixed = sizeof(V) == sizeof(float2);
+    constexpr int m = mixed ? 1 : 0;
+    const PairPlan &P = *c->pair;
+    const int64_t n_z = (int64_t)P.masks2.size() * P.n_rows2;
+    if (n_z > 0) {
+        TimedLaunch tl(stream);
+        note_launch();
+        if constexpr (mixed) {
+            const int64_t items = (n_z * (W / 64) + 31) / 32;
+            k_large_step_split<32, 4><<<(unsigned)std::min<int64_t>(items, nsm), 1024, 0, stream>>>(
+                c->d_pair_x, c->d_pair_ys, n_z, 12, 1, W, f, f, prod);
+        } else {
+            const int64_t ngroups = W / 32;
+            int64_t zchunk = std::max<int64_t>(1, std::min<int64_t>(256, n_z * ngroups / ((int64_t)nsm * 512)));
+            const int64_t items = ((n_z + zchunk - 1) / zchunk) * ngroups;
+            const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((items + 7) / 8, (int64_t)nsm * 8));
+            k_large_step<Tr, false><<<(unsigned)grid, 256, 0, stream>>>(c->d_pair_x, c->d_pair_ys, GenStep{}, n_z, 12,
+                                                                        zchunk, W, 0, f, f, prod);
+        }
+    }
+    MBC_CUDA_TRY(cudaGetLastError());
+    const int64_t block_rows = L->block_size / L->dim_snk;
+    const PairArgs A{c->d_pair_units[m], c->n_pair_units[m], c->d_pair_row,          c->d_pair_col,
+                     c->d_pair_val,      P.p_rows(block_rows), P.n_rows(block_rows)};
+    const V *Pb = P.np == 2 ? prod : f, *Nb = P.nn == 2 ? prod : f;
+    if (A.n_units > 0) {
+        const int shape = c->pair_shape[m];
+        const int threads = mixed ? 128 : 256;
+        const int64_t items = (int64_t)A.n_units * (W / (mixed ? 64 : 32));
+        const void *kern;
+        if constexpr (mixed)
+            kern = shape == 0 ? (const void *)k_pair_mx<1, 1> : shape == 1 ? (const void *)k_pair_mx<2, 2> : (const void *)k_pair_mx<6, 2>;
+        else
+            kern = shape == 0 ? (const void *)k_pair_fp64<1, 1> : shape == 1 ? (const void *)k_pair_fp64<2, 2> : (const void *)k_pair_fp64<6, 6>;
+        int per_sm = 0;
+        mbc_status st = prepare_kernel(kern, c->device, threads, 0, &per_sm);
+        if (st != MBC_OK) return st;
+        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((items * 32 + threads - 1) / threads, (int64_t)nsm * std::max(per_sm, 1)));
+        void *args[] = {(void *)&A, (void *)&W, (void *)&Pb, (void *)&Nb, (void *)&part};
+        TimedLaunch tl(stream);
+        note_launch();
+        MBC_CUDA_TRY(cudaLaunchKernel(kern, dim3((unsigned)grid), dim3(threads), args, 0, stream));
+    }
+    note_launch();
+    k_pair_sum<<<dim3((unsigned)L->n_comp, (unsigned)(W / 32)), 1024, 0, stream>>>(
+        c->d_pair_comp_off, c->d_pair_comp_eval, c->d_pair_slot_off[m], W, part, sexp, deg_per_baryon * L->A, P.scale, Cb);
+    MBC_CUDA_TRY(cudaGetLastError());
+    return MBC_OK;
+}
+
 template <class Tr>
 mbc_status run_large(const mbc_term_list *L, const DeviceCache *c, const FieldDesc &F, const MomDesc &M,
                      const mbc_tune *tune, int device, cudaStream_t stream, char *scratch, double2 *partial,
@@ -1074,15 +1314,15 @@ mbc_status run_large(const mbc_term_list *L, const DeviceCache *c, const FieldDe
     using V = typename Tr::V;
     const int W = ls.W;
     char *p = scratch;
-    V *fP = reinterpret_cast<V *>(p);
-    p += align256(ls.blk_bytes);
-    V *fN = reinterpret_cast<V *>(p);
+    V *f = reinterpret_cast<V *>(p);  // the block of both species (u = d)
     p += align256(ls.blk_bytes);
     V *buf[2];
     buf[0] = reinterpret_cast<V *>(p);
     p += align256(ls.stage_bytes);
     buf[1] = reinterpret_cast<V *>(p);
-    p += align256(ls.stage_bytes);
+    if (!ls.pair) p += align256(ls.stage_bytes);
+    double2 *ppart = reinterpret_cast<double2 *>(p);
+    p += align256(ls.part_bytes);
     double2 *Cb = reinterpret_cast<double2 *>(p);
     p += align256(ls.c_bytes);
     int32_t *sexp = reinterpret_cast<int32_t *>(p);
@@ -1108,21 +1348,26 @@ mbc_status run_large(const mbc_term_list *L, const DeviceCache *c, const FieldDe
         note_launch();
         if (ns_blk == 4)
             k_large_blocks<Tr, 4><<<W / 4, 512, blk_smem, stream>>>(F, wv, nrow, nxi, n_g2(L), (int)L->block_size,
-                                                                    (int)binom64(nxi, 2), L->need_block[0],
-                                                                    L->need_block[1], fP, fN, sexp);
+                                                                    (int)binom64(nxi, 2), f, sexp);
         else
             k_large_blocks<Tr, 16><<<W / 16, 512, blk_smem, stream>>>(F, wv, nrow, nxi, n_g2(L), (int)L->block_size,
-                                                                      (int)binom64(nxi, 2), L->need_block[0],
-                                                                      L->need_block[1], fP, fN, sexp);
+                                                                      (int)binom64(nxi, 2), f, sexp);
         MBC_CUDA_TRY(cudaGetLastError());
-        const V *X = L->path[0] == MBC_PROTON ? fP : fN;
+        if (ls.pair) {
+            mbc_status pst = pair_wave<Tr>(L, c, W, f, buf[0], ppart, sexp, 3, Cb, nsm, stream);
+            if (pst != MBC_OK) return pst;
+            const int64_t groups = std::min<int64_t>(W, n_items - item0) / 32;
+            note_launch();
+            k_large_sitesum<<<(unsigned)groups, 256, 0, stream>>>(F, wv, M, L->n_comp, phase, Cb, partial);
+            MBC_CUDA_TRY(cudaGetLastError());
+            continue;
+        }
+        const V *X = f;
         mbc_status cst = contract_parts<Tr>(L, c, 1, X, W, sexp, 3, Cb, nsm, stream);
         if (cst != MBC_OK) return cst;
         for (size_t m = 0; m < L->steps.size(); ++m) {
-            const Step &s = L->steps[m];
             V *Z = buf[(m + 1) & 1];
-            const V *Y = s.baryon == MBC_PROTON ? fP : fN;
-            if ((cst = launch_step<Tr>(L, c, m, tune, W, nsm, X, Y, Z, stream)) != MBC_OK) return cst;
+            if ((cst = launch_step<Tr>(L, c, m, tune, W, nsm, X, f, Z, stream)) != MBC_OK) return cst;
             X = Z;
             if ((cst = contract_parts<Tr>(L, c, (int)m + 2, X, W, sexp, 3, Cb, nsm, stream)) != MBC_OK) return cst;
         }
@@ -1157,15 +1402,15 @@ mbc_status run_projected(const mbc_term_list *L, const DeviceCache *c, const Fie
     double2 *Pf = reinterpret_cast<double2 *>(p);
     p += align256((size_t)n_slabs * M.n_mom * n_out * sizeof(double2));
     const int W = ls.W;
-    V *fP = reinterpret_cast<V *>(p);
-    p += align256(ls.blk_bytes);
-    V *fN = reinterpret_cast<V *>(p);
+    V *f = reinterpret_cast<V *>(p);  // the block of both species (u = d)
     p += align256(ls.blk_bytes);
     V *buf[2];
     buf[0] = reinterpret_cast<V *>(p);
     p += align256(ls.stage_bytes);
     buf[1] = reinterpret_cast<V *>(p);
-    p += align256(ls.stage_bytes);
+    if (!ls.pair) p += align256(ls.stage_bytes);
+    double2 *ppart = reinterpret_cast<double2 *>(p);
+    p += align256(ls.part_bytes);
     double2 *Cb = reinterpret_cast<double2 *>(p);
     p += align256(ls.c_bytes);
     int32_t *sexp = reinterpret_cast<int32_t *>(p);
@@ -1191,14 +1436,14 @@ mbc_status run_projected(const mbc_term_list *L, const DeviceCache *c, const Fie
             float2 *partial_mx = reinterpret_cast<float2 *>(partial);  // the mixed path's FP32 partials
             if (mx && nxi == 6)
                 k_project_blocks_mx<6><<<(unsigned)grid, 512, smem, stream>>>(
-                    F, M, phase, nrow, n_g2(L), bs, L->need_block[0], L->need_block[1], tps, n_tiles, partial_mx);
+                    F, M, phase, nrow, n_g2(L), bs, 1, 0, tps, n_tiles, partial_mx);
             else if (mx)
                 k_project_blocks_mx<12><<<(unsigned)grid, 512, smem, stream>>>(
-                    F, M, phase, nrow, n_g2(L), bs, L->need_block[0], L->need_block[1], tps, n_tiles, partial_mx);
+                    F, M, phase, nrow, n_g2(L), bs, 1, 0, tps, n_tiles, partial_mx);
             else
                 k_project_blocks<<<(unsigned)grid, 512, smem, stream>>>(F, M, phase, nrow, nxi, n_g2(L), bs,
-                                                                        (int)binom64(nxi, 2), L->need_block[0],
-                                                                        L->need_block[1], tps, n_tiles, partial);
+                                                                        (int)binom64(nxi, 2), 1, 0, tps, n_tiles,
+                                                                        partial);
         }
         MBC_CUDA_TRY(cudaGetLastError());
         // thousands of outputs per slab: one thread per output, coalesced
@@ -1219,16 +1464,15 @@ mbc_status run_projected(const mbc_term_list *L, const DeviceCache *c, const Fie
     for (int64_t item0 = 0; item0 < n_items; item0 += W) {
         note_launch();
         k_load_proj_blocks<Tr><<<(unsigned)((W + 7) / 8), 256, 0, stream>>>(Pf, n_items, item0, W, bs, per_spin, n_k,
-                                                                            M.n_mom, fP, fN, sexp);
+                                                                            M.n_mom, f, sexp);
         MBC_CUDA_TRY(cudaGetLastError());
-        const V *X = L->path[0] == MBC_PROTON ? fP : fN;
-        mbc_status cst = contract_parts<Tr>(L, c, 1, X, W, sexp, 1, Cb, nsm, stream);
+        const V *X = f;
+        mbc_status cst = ls.pair ? pair_wave<Tr>(L, c, W, f, buf[0], ppart, sexp, 1, Cb, nsm, stream)
+                                 : contract_parts<Tr>(L, c, 1, X, W, sexp, 1, Cb, nsm, stream);
         if (cst != MBC_OK) return cst;
-        for (size_t m = 0; m < L->steps.size(); ++m) {
-            const Step &s = L->steps[m];
+        for (size_t m = 0; !ls.pair && m < L->steps.size(); ++m) {
             V *Z = buf[(m + 1) & 1];
-            const V *Y = s.baryon == MBC_PROTON ? fP : fN;
-            if ((cst = launch_step<Tr>(L, c, m, tune, W, nsm, X, Y, Z, stream)) != MBC_OK) return cst;
+            if ((cst = launch_step<Tr>(L, c, m, tune, W, nsm, X, f, Z, stream)) != MBC_OK) return cst;
             X = Z;
             if ((cst = contract_parts<Tr>(L, c, (int)m + 2, X, W, sexp, 1, Cb, nsm, stream)) != MBC_OK) return cst;
         }
@@ -1248,8 +1492,7 @@ size_t projected_bytes(const mbc_term_list *L, const MomDesc &M, int v3, int64_t
     const int tps = (v3 + 15) / 16;
     const int64_t n_out = 2 * (L->block_size / L->n_sinks);
     return align256((size_t)n_slabs * tps * M.n_mom * n_out * sizeof(double2)) +
-           align256((size_t)n_slabs * M.n_mom * n_out * sizeof(double2)) + 2 * align256(ls.blk_bytes) +
-           2 * align256(ls.stage_bytes) + align256(ls.c_bytes) + align256(ls.sexp_bytes);
+           align256((size_t)n_slabs * M.n_mom * n_out * sizeof(double2)) + ls.buffers();
 }
 
 }  // namespace
@@ -1532,10 +1775,9 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
         for (int li = 0; li < n_lists; ++li) {
             const mbc_term_list *L = lists[li];
             if (L->pauli_forbidden || L->n_comp == 0) continue;
-            cs[(size_t)li] = get_wave_cache(L, device, st);
+            cs[(size_t)li] = get_large_cache(L, device, opts->tune, mixed, st);
             if (!cs[(size_t)li]) return st;
-            lsz[(size_t)li] = mixed ? large_sizes<MixedTraits>(L, cs[(size_t)li], opts->tune, n_items_p)
-                                    : large_sizes<FP64Traits>(L, cs[(size_t)li], opts->tune, n_items_p);
+            lsz[(size_t)li] = wave_sizes(L, cs[(size_t)li], opts->tune, n_items_p, mixed);
             need = std::max(need, projected_bytes(L, M, (int)v3, n_slabs, lsz[(size_t)li]));
         }
         const size_t phase_bytes_p = align256((size_t)v3 * M.n_mom * sizeof(double2));
@@ -1580,7 +1822,7 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
             small = size_small_batch({caches[(size_t)li]}, F, opts->tune, mixed, ss, cs).ok;
         }
         if (regime == 1 && !small) return MBC_ERR_UNSUPPORTED;
-        if (!small && !get_wave_cache(L, device, st)) return st;
+        if (!small && !get_large_cache(L, device, opts->tune, mixed, st)) return st;
         (small ? small_ids : large_ids).push_back(li);
     }
     // minor-form lists first: lists of one form share their tile (and block)
@@ -1654,13 +1896,10 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
     for (int li : large_ids) {
         const mbc_term_list *L = lists[li];
         DeviceCache *c = caches[(size_t)li];
-        lsz[(size_t)li] = mixed ? large_sizes<MixedTraits>(L, c, opts->tune, n_items)
-                                : large_sizes<FP64Traits>(L, c, opts->tune, n_items);
+        lsz[(size_t)li] = wave_sizes(L, c, opts->tune, n_items, mixed);
         const LargeSizes &ls = lsz[(size_t)li];
         const size_t pbytes = (size_t)(n_items / 32) * M.n_mom * L->n_comp * sizeof(double2);
-        large_bytes = std::max(large_bytes, align256(pbytes) + 2 * align256(ls.blk_bytes) +
-                                                2 * align256(ls.stage_bytes) + align256(ls.c_bytes) +
-                                                align256(ls.sexp_bytes));
+        large_bytes = std::max(large_bytes, align256(pbytes) + ls.buffers());
     }
     const size_t phase_bytes = align256((size_t)v3 * M.n_mom * sizeof(double2));
     void *scr = nullptr;

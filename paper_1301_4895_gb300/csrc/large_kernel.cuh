@@ -41,8 +41,8 @@ __device__ __forceinline__ bool item_site(const FieldDesc &F, const WaveDesc &wv
 __host__ __device__ constexpr int tile_stride(int nrow, int nxi) { return nrow * nxi + 1; }
 __host__ __device__ constexpr int diquark_stride(int nxi) { return 3 * nxi * nxi + 1; }
 
-// Blocks for NS sites per CTA (512 threads): thread = (site lane, entry
-// slice). The tile of a site has nrow sink rows (3 x Dirac dimension) and nxi
+// The block of both species (u = d, see small_blocks) for NS sites per CTA (512
+// threads): thread = (site lane, entry slice). The tile of a site has nrow sink rows (3 x Dirac dimension) and nxi
 // source columns (quark index over all sources, up to 24: two relativistic
 // sources, Sec. 6); NS = 4 for 24 columns keeps the tiles and diquarks in
 // shared memory.
@@ -50,8 +50,8 @@ constexpr int kTileLoads = 9;  // tile entries per lane: 12 x 24 / 32
 
 template <class Tr, int NS>
 __global__ void __launch_bounds__(512) k_large_blocks(FieldDesc F, WaveDesc wv, int nrow, int nxi, int n_g2,
-                                                      int block_size, int npair, int need_p, int need_n,
-                                                      typename Tr::V *fP, typename Tr::V *fN, int32_t *sexp_out) {
+                                                      int block_size, int npair, typename Tr::V *f,
+                                                      int32_t *sexp_out) {
     using V = typename Tr::V;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int sst = tile_stride(nrow, nxi), qst = diquark_stride(nxi);
@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(512) k_large_blocks(FieldDesc F, WaveDesc wv, 
     V *Q = S + NS * sst;                     // [NS][qst]: 3*nxi*nxi entries each
     const int sl = threadIdx.x % NS, slice = threadIdx.x / NS, nslice = blockDim.x / NS;
     const int w0 = blockIdx.x * NS;  // first site of this CTA within the wave
-    const int nent = nrow * nxi, nq = nxi * nxi;
+    const int nent = nrow * nxi;
     // load + scale: one warp per site
     for (int s = threadIdx.x >> 5; s < NS; s += blockDim.x >> 5) {
         int lane = threadIdx.x & 31;
@@ -90,34 +90,29 @@ __global__ void __launch_bounds__(512) k_large_blocks(FieldDesc F, WaveDesc wv, 
         if (lane == 0) sexp_out[w0 + s] = se;
     }
     __syncthreads();
-    for (int e = slice; e < 3 * nq; e += nslice) {
-        int c = e / nq, r = e % nq;
-        Q[sl * qst + e] = diquark(S + sl * sst, nxi, nxi, n_g2, c, r / nxi, r % nxi);
+    const int ntri = npair + nxi;  // Q is symmetric (small_blocks)
+    for (int e = slice; e < 3 * ntri; e += nslice) {
+        const int c = e / ntri, r = e % ntri;
+        const int x2 = r < npair ? c_pair_i[r] : r - npair, x3 = r < npair ? c_pair_j[r] : r - npair;
+        const V q = diquark(S + sl * sst, nxi, nxi, n_g2, c, x2, x3);
+        Q[sl * qst + (c * nxi + x2) * nxi + x3] = q;
+        Q[sl * qst + (c * nxi + x3) * nxi + x2] = q;
     }
     __syncthreads();
     const V *Ss = S + sl * sst;
     const V *Qs = Q + sl * qst;
     const int per_spin = npair * nxi;
-    for (int b = 0; b < 2; ++b) {
-        if (b == 0 ? !need_p : !need_n) continue;
-        V *out = b == 0 ? fP : fN;
-        for (int e = slice; e < block_size; e += nslice) {
-            int dl = e / per_spin, r = e % per_spin;
-            int pr = r / nxi, single = r % nxi;
-            int i = c_pair_i[pr], j = c_pair_j[pr];
-            V acc{0, 0};
-            for (int c = 0; c < 3; ++c) {
-                const V *Sr = Ss + (3 * dl + c) * nxi;
-                if (b == 0) {
-                    acc = cfma(Sr[i], Qs[(c * nxi + j) * nxi + single], acc);
-                    acc = cfms(Sr[j], Qs[(c * nxi + i) * nxi + single], acc);
-                } else {
-                    acc = cfma(Sr[i], Qs[(c * nxi + single) * nxi + j], acc);
-                    acc = cfms(Sr[j], Qs[(c * nxi + single) * nxi + i], acc);
-                }
-            }
-            Tr::wave_st(out, (int64_t)e * wv.W + w0 + sl, acc);
+    for (int e = slice; e < block_size; e += nslice) {
+        int dl = e / per_spin, r = e % per_spin;
+        int pr = r / nxi, single = r % nxi;
+        int i = c_pair_i[pr], j = c_pair_j[pr];
+        V acc{0, 0};
+        for (int c = 0; c < 3; ++c) {
+            const V *Sr = Ss + (3 * dl + c) * nxi;
+            acc = cfma(Sr[i], Qs[(c * nxi + j) * nxi + single], acc);
+            acc = cfms(Sr[j], Qs[(c * nxi + i) * nxi + single], acc);
         }
+        Tr::wave_st(f, (int64_t)e * wv.W + w0 + sl, acc);
     }
 }
 

@@ -39,6 +39,7 @@ struct Step {
 struct DeviceCache;  // defined by the CUDA side
 struct MinorPlan;    // plan.h
 struct SaturatedPlan;
+struct PairPlan;
 
 }  // namespace mbc
 
@@ -78,7 +79,8 @@ struct mbc_term_list {
     std::mutex plan_mu;
     std::shared_ptr<const mbc::MinorPlan> minor;
     std::shared_ptr<const mbc::SaturatedPlan> saturated;
-    bool minor_tried = false, saturated_tried = false;
+    std::shared_ptr<const mbc::PairPlan> pair;
+    bool minor_tried = false, saturated_tried = false, pair_tried = false;
 };
 
 namespace mbc {

@@ -284,7 +284,225 @@ std::shared_ptr<const SaturatedPlan> make_saturated_plan(const mbc_term_list &L)
     return P;
 }
 
+int64_t rank_of(uint32_t m) {
+    int64_t r = 0;
+    for (int t = 1; m; m &= m - 1, ++t) r += binom_p(__builtin_ctz(m), t);
+    return r;
+}
+
+// (subset, rest, sign of subset | rest) for every k-subset of a set
+struct Split {
+    uint32_t sub, rest;
+    int neg;
+};
+std::vector<Split> splits_of(uint32_t set, int k) {
+    std::vector<Split> out;
+    for (uint32_t c = (0u - set) & set; c; c = (c - set) & set)
+        if (__builtin_popcount(c) == k) out.push_back({c, set ^ c, parity(c, set ^ c)});
+    return out;
+}
+
+constexpr int64_t kMaxPairEntries = (int64_t)1 << 26;  // 12 B each on the device
+
+std::shared_ptr<const PairPlan> make_pair_plan(const mbc_term_list &L) {
+    if (L.parts.size() != 1 || L.nxi > 12 || L.n_comp < 1) return nullptr;
+    const auto &pt = L.parts[0];
+    const int np = pt.n_p, nn = pt.n_n, nxi = L.nxi;
+    if (np < 1 || np > 2 || nn < 1 || nn > 2 || pt.c0 != 0 || pt.c1 != L.n_comp) return nullptr;
+    for (const auto &s : L.steps)
+        if (s.generated) return nullptr;  // list-free lists keep no tables
+    std::vector<std::vector<PlanEntry>> comp;
+    if (!list_entries(L, comp)) return nullptr;
+    // evaluations: (sink spin sets, tensor), the tensor a list of (U, D, l)
+    using UD = std::pair<uint32_t, uint32_t>;
+    using Tensor = std::map<UD, double>;
+    struct Group {
+        Tensor t;
+        std::map<uint32_t, int> mp, mn;  // spin sets -> position
+    };
+    std::map<Tensor, int> ids;
+    std::vector<Group> groups;
+    struct Eval {
+        int group;
+        uint32_t dp, dn;
+    };
+    std::vector<std::vector<Eval>> evals((size_t)L.n_comp);
+    for (int c = 0; c < L.n_comp; ++c) {
+        std::map<UD, Tensor> by_sink;
+        for (const auto &e : comp[(size_t)c])
+            if (e.l != 0.0) by_sink[{e.z.dp, e.z.dn}][{e.z.u, e.z.d}] += e.l;
+        for (auto &sk : by_sink) {
+            uint32_t dp = sk.first.first, dn = sk.first.second;
+            if (np == nn) {  // of the two flavour-exchanged forms the first one seen
+                auto it = ids.find(sk.second);
+                if (it == ids.end()) {
+                    Tensor ex;
+                    for (const auto &t : sk.second) ex[{t.first.second, t.first.first}] = t.second;
+                    it = ids.find(ex);
+                    if (it != ids.end()) {
+                        sk.second.swap(ex);
+                        std::swap(dp, dn);
+                    }
+                }
+            }
+            auto ins = ids.insert({sk.second, (int)groups.size()});
+            if (ins.second) groups.push_back({sk.second, {}, {}});
+            const int g = ins.first->second;
+            groups[(size_t)g].mp[dp] = groups[(size_t)g].mn[dn] = 0;
+            evals[(size_t)c].push_back({g, dp, dn});
+        }
+    }
+    int64_t total = 0;
+    const int64_t per_z = binom_p(2 * np + nn, 2 * np) * binom_p(np + 2 * nn, np);
+    for (const auto &g : groups) total += (int64_t)g.t.size() * per_z;
+    if (total > kMaxPairEntries) return nullptr;
+    auto P = std::make_shared<PairPlan>();
+    P->np = np;
+    P->nn = nn;
+    // rows: block entries [pair][single] for one baryon; for two the (4-set,
+    // 2-set) keys some entry names, in rank order
+    const int64_t nset2 = binom_p(nxi, 2), wide = binom_p(nxi, 4) * nset2;
+    std::vector<int32_t> row_of((size_t)((np == 2 || nn == 2) ? wide : 0), -1);
+    auto full_row = [&](uint32_t pair, uint32_t single, int n) {
+        return rank_of(pair) * (n == 2 ? nset2 : nxi) + rank_of(single);
+    };
+    struct Entry {
+        uint32_t i, j;
+        double v;
+    };
+    std::vector<std::vector<Entry>> lam(groups.size());
+#pragma omp parallel for schedule(dynamic, 1)
+    for (size_t g = 0; g < groups.size(); ++g) {
+        auto &out = lam[g];
+        out.reserve(groups[g].t.size() * (size_t)per_z);
+        // a symmetric tensor with equal sink sets: upper triangle, doubled
+        bool sym = np == nn && groups[g].mp.size() == 1 && groups[g].mn.size() == 1 &&
+                   groups[g].mp.begin()->first == groups[g].mn.begin()->first;
+        if (sym)
+            for (const auto &t : groups[g].t) {
+                const auto o = groups[g].t.find({t.first.second, t.first.first});
+                sym = sym && o != groups[g].t.end() && o->second == t.second;
+            }
+        for (const auto &t : groups[g].t) {
+            const auto us = splits_of(t.first.first, 2 * np), ds = splits_of(t.first.second, np);
+            for (const auto &u : us)
+                for (const auto &d : ds) {
+                    const uint32_t i = (uint32_t)full_row(u.sub, d.sub, np), j = (uint32_t)full_row(d.rest, u.rest, nn);
+                    const double v = (u.neg ^ d.neg) ? -t.second : t.second;
+                    if (!sym)
+                        out.push_back({i, j, v});
+                    else if (i <= j)
+                        out.push_back({i, j, i == j ? v : 2.0 * v});
+                }
+        }
+        std::sort(out.begin(), out.end(), [](const Entry &a, const Entry &b) { return a.i != b.i ? a.i < b.i : a.j < b.j; });
+    }
+    for (const auto &out : lam)
+        for (const auto &e : out) {
+            if (np == 2) row_of[e.i] = 0;
+            if (nn == 2) row_of[e.j] = 0;
+            P->val_fp32 = P->val_fp32 && (double)(float)e.v == e.v;
+        }
+    std::vector<UD> rows2;
+    for (int64_t r = 0; r < (int64_t)row_of.size(); ++r)
+        if (row_of[(size_t)r] == 0) {
+            row_of[(size_t)r] = P->n_rows2++;
+            rows2.push_back({unrank(r / nset2, 4, nxi), unrank(r % nset2, 2, nxi)});
+        }
+    // elements: spin values for one baryon, used two-spin sets for two
+    std::map<uint32_t, int32_t> elem2;
+    for (const auto &g : groups) {
+        if (np == 2)
+            for (const auto &m : g.mp) elem2[m.first] = 0;
+        if (nn == 2)
+            for (const auto &m : g.mn) elem2[m.first] = 0;
+    }
+    for (auto &m : elem2) {
+        m.second = (int32_t)P->masks2.size();
+        P->masks2.push_back(m.first);
+    }
+    auto elem = [&](uint32_t mask, int n) { return n == 2 ? elem2[mask] : (int32_t)__builtin_ctz(mask); };
+    int64_t work = 0;
+    P->row_ptr.push_back(0);
+    for (size_t g = 0; g < groups.size(); ++g) {
+        PairPlan::Group G;
+        G.row0 = (int64_t)P->row_id.size();
+        for (size_t k = 0; k < lam[g].size();) {
+            const uint32_t i = lam[g][k].i;
+            for (; k < lam[g].size() && lam[g][k].i == i; ++k) {
+                const uint32_t j = lam[g][k].j;
+                P->col.push_back(nn == 2 ? (uint32_t)row_of[j] : j);
+                P->val.push_back(lam[g][k].v);
+            }
+            P->row_id.push_back(np == 2 ? (uint32_t)row_of[i] : i);
+            P->row_ptr.push_back((int64_t)P->col.size());
+        }
+        std::vector<Entry>().swap(lam[g]);
+        G.row1 = (int64_t)P->row_id.size();
+        for (auto &m : groups[g].mp) {
+            m.second = (int)G.mp.size();
+            G.mp.push_back(elem(m.first, np));
+        }
+        for (auto &m : groups[g].mn) {
+            m.second = (int)G.mn.size();
+            G.mn.push_back(elem(m.first, nn));
+        }
+        G.eval0 = P->n_evals;
+        P->n_evals += (int64_t)(G.mp.size() * G.mn.size());
+        const int64_t nnz = P->row_ptr[(size_t)G.row1] - P->row_ptr[(size_t)G.row0];
+        work += nnz * (int64_t)G.mn.size() / 2 + (G.row1 - G.row0) * (int64_t)(G.mp.size() * G.mn.size());
+        P->groups.push_back(std::move(G));
+    }
+    if (P->n_evals > (int64_t)1 << 20) return nullptr;
+    work += 12LL * (int64_t)P->masks2.size() * P->n_rows2;
+    // complex multiply-adds of the list's own recursion; both forms share blocks
+    int64_t chain = 0;
+    for (const auto &s : L.steps) chain += s.n_z * s.k;
+    if (work * 5 > chain * 4) return nullptr;
+    P->comp_off.push_back(0);
+    for (int c = 0; c < L.n_comp; ++c) {
+        for (const auto &e : evals[(size_t)c]) {
+            const auto &g = groups[(size_t)e.group];
+            const auto &G = P->groups[(size_t)e.group];
+            P->comp_eval.push_back(
+                (int32_t)(G.eval0 + (int64_t)g.mp.at(e.dp) * (int64_t)G.mn.size() + g.mn.at(e.dn)));
+        }
+        P->comp_off.push_back((int32_t)P->comp_eval.size());
+    }
+    P->scale = std::tgamma(np + 1.0) * std::tgamma(nn + 1.0) / pt.norm;
+    // the two-baryon products
+    const int64_t npair = nset2;
+    P->sx.reserve(12 * P->masks2.size() * rows2.size());
+    P->sys.reserve(P->sx.capacity());
+    if (L.block_size > 32768) return nullptr;
+    for (uint32_t m : P->masks2) {
+        const int s1 = __builtin_ctz(m), s2 = __builtin_ctz(m & (m - 1));
+        for (const auto &r : rows2)
+            for (const auto &a : splits_of(r.first, 2))
+                for (const auto &e : splits_of(r.second, 1)) {
+                    P->sx.push_back((uint32_t)((s1 * npair + rank_of(a.sub)) * nxi + __builtin_ctz(e.sub)));
+                    P->sys.push_back((uint16_t)(((s2 * npair + rank_of(a.rest)) * nxi + __builtin_ctz(e.rest)) |
+                                                ((a.neg ^ e.neg) ? 0x8000 : 0)));
+                }
+    }
+    return P;
+}
+
 }  // namespace
+
+std::shared_ptr<const PairPlan> pair_plan(const mbc_term_list *Lc) {
+    mbc_term_list *L = const_cast<mbc_term_list *>(Lc);
+    std::lock_guard<std::mutex> g(L->plan_mu);
+    if (!L->pair_tried) {
+        try {
+            L->pair = make_pair_plan(*L);
+            L->pair_tried = true;
+        } catch (const std::bad_alloc &) {
+            return nullptr;
+        }
+    }
+    return L->pair;
+}
 
 std::shared_ptr<const SaturatedPlan> saturated_plan(const mbc_term_list *Lc) {
     mbc_term_list *L = const_cast<mbc_term_list *>(Lc);

@@ -85,4 +85,44 @@ struct SaturatedPlan {
 };
 std::shared_ptr<const SaturatedPlan> saturated_plan(const mbc_term_list *L);
 
+// Pair form of a nucleus with one or two baryons of each species. The protons'
+// product P[sigma; a, e] (a: u set, e: d set) and the neutrons' N (the same
+// numbers for u = d, with the flavours exchanged) are formed once per spin set,
+// ordered (f_{s1} ^ f_{s2}, s1 < s2: the recursion adds both orders, which are
+// equal), and a component is bilinear in them,
+//   C = sum_z L(z) F(z) = sum_{i, j} P_i Lambda_ij N_j,
+// Lambda_ij = +-L(a_i + g_j, b_j + e_i) real, sparse and the same for every
+// site. Components with the same L share a group: y_j-sums of a row are formed
+// once per neutron set and multiplied by every proton set's row. Exchanging the
+// flavours maps (sigma_p, sigma_n, L(U, D)) to (sigma_n, sigma_p, L(D, U)) with
+// the same value, so only one of the two is computed, and Lambda of a single
+// symmetric component keeps its upper triangle.
+struct PairPlan {
+    int np = 0, nn = 0;  // baryons per species: 1 or 2
+    // two-baryon rows: element m (spin set masks2[m]), row r at m * n_rows2 + r,
+    // 12 products each: x, y block entries, sign in bit 15 of ys (as Step)
+    std::vector<uint32_t> masks2;
+    int32_t n_rows2 = 0;
+    std::vector<uint32_t> sx;
+    std::vector<uint16_t> sys;
+    struct Group {
+        int64_t row0, row1;             // its rows in row_id / row_ptr
+        std::vector<int32_t> mp, mn;    // element indices; every (mp, mn) is evaluated
+        int64_t eval0;                  // evaluation (mp_i, mn_j) at eval0 + i * mn.size() + j
+    };
+    std::vector<Group> groups;
+    std::vector<uint32_t> row_id;       // P row of each Lambda row
+    std::vector<int64_t> row_ptr;       // its entries (one more than row_id)
+    std::vector<uint32_t> col;          // N row
+    std::vector<double> val;
+    bool val_fp32 = true;               // every value is an FP32 number
+    int64_t n_evals = 0;
+    std::vector<int32_t> comp_off;      // evaluations a component sums (n_comp + 1)
+    std::vector<int32_t> comp_eval;
+    double scale = 1.0;                 // n_P! n_N! / norm
+    int64_t p_rows(int64_t block_rows) const { return np == 2 ? n_rows2 : block_rows; }
+    int64_t n_rows(int64_t block_rows) const { return nn == 2 ? n_rows2 : block_rows; }
+};
+std::shared_ptr<const PairPlan> pair_plan(const mbc_term_list *L);
+
 }  // namespace mbc

@@ -108,6 +108,58 @@ static int bad_minors(const char *name, const mbc_term_list &L, bool expect, std
     return worst > 1e-11;
 }
 
+static int bad_pairs(const char *name, const mbc_term_list &L, bool expect, std::mt19937 &rng) {
+    const auto P = mbc::pair_plan(&L);
+    if (!!P != expect) {
+        std::printf("%s: pair form %s\n", name, P ? "made" : "not made");
+        return 1;
+    }
+    if (!P) return 0;
+    // any blocks will do: projected blocks are sums of blocks over sites
+    std::normal_distribution<double> nd;
+    std::vector<cd> f((size_t)L.block_size);
+    for (auto &v : f) v = cd(nd(rng), nd(rng));
+    std::vector<cd> C, prod;
+    std::vector<double> mag;
+    chain(L, f, C, mag);
+    for (size_t o = 0; o < P->sx.size(); o += 12) {
+        cd v = 0;
+        for (size_t j = o; j < o + 12; ++j) {
+            const cd t = f.at(P->sx[j]) * f.at(P->sys[j] & 0x7fff);
+            v += P->sys[j] & 0x8000 ? -t : t;
+        }
+        prod.push_back(v);
+    }
+    if (prod.size() != P->masks2.size() * (size_t)P->n_rows2) return 1;
+    const int64_t brows = L.block_size / L.dim_snk;
+    const int64_t pr = P->p_rows(brows), nr = P->n_rows(brows);
+    std::vector<cd> ev((size_t)P->n_evals, 0);
+    for (const auto &g : P->groups)
+        for (int64_t r = g.row0; r < g.row1; ++r)
+            for (size_t b = 0; b < g.mn.size(); ++b) {
+                cd y = 0;
+                for (int64_t e = P->row_ptr[(size_t)r]; e < P->row_ptr[(size_t)r + 1]; ++e) {
+                    if (P->col[(size_t)e] >= nr) return 1;
+                    y += P->val[(size_t)e] * (P->nn == 2 ? prod : f).at((size_t)(g.mn[b] * nr + P->col[(size_t)e]));
+                }
+                if (P->row_id[(size_t)r] >= pr) return 1;
+                for (size_t a = 0; a < g.mp.size(); ++a)
+                    ev.at((size_t)g.eval0 + a * g.mn.size() + b) +=
+                        y * (P->np == 2 ? prod : f).at((size_t)(g.mp[a] * pr + P->row_id[(size_t)r]));
+            }
+    double worst = 0;
+    for (int c = 0; c < L.n_comp; ++c) {
+        cd v = 0;
+        for (int e = P->comp_off[(size_t)c]; e < P->comp_off[(size_t)c + 1]; ++e) v += ev.at((size_t)P->comp_eval[(size_t)e]);
+        v *= P->scale * L.parts[0].norm;  // the chain's sums are not normalised
+        const double scale = mag[(size_t)c] > 0 ? mag[(size_t)c] : 1.0;
+        worst = std::max(worst, std::abs(v - C[(size_t)c]) / scale);
+    }
+    std::printf("%s: pair form, %zu groups, %zu entries, %zu x %d products, worst difference %.1e\n", name,
+                P->groups.size(), P->col.size(), P->masks2.size(), P->n_rows2, worst);
+    return worst > 1e-10;
+}
+
 static mbc_op_spec spec(int np, int nn, int D) {
     mbc_op_spec s;
     std::memset(&s, 0, sizeof(s));
@@ -137,6 +189,45 @@ int main() {
         s.list_free = c.list_free;
         mbc_term_list *L = build1(s);
         bad += bad_minors(c.name, *L, c.minors, rng);
+        bad += bad_pairs(c.name, *L, true, rng);
+        mbc_free_term_list(L);
+    }
+    {  // pair forms: listed components, odd spin orders, sinks and sources, paths
+        struct Listed {
+            const char *name;
+            int np, nn, D, ns, nk, n;
+            std::vector<int8_t> snk, src;
+            std::vector<int8_t> path;
+        };
+        for (const Listed &c : {
+                 Listed{"4He rel", 2, 2, 4, 1, 1, 1, {0, 1, 0, 1}, {0, 1, 0, 1}, {}},
+                 Listed{"4He rel, two listed", 2, 2, 4, 1, 1, 2, {0, 1, 0, 1, 2, 0, 1, 3}, {0, 1, 0, 1, 0, 1, 0, 1}, {}},
+                 Listed{"4He rel, exchanged", 2, 2, 4, 1, 1, 2, {0, 1, 0, 2, 0, 2, 0, 1}, {0, 1, 1, 3, 1, 3, 0, 1}, {0, 1, 0, 1}},
+                 Listed{"3He rel", 2, 1, 4, 1, 1, 2, {0, 1, 2, 0, 3, 1}, {0, 1, 0, 0, 1, 2}, {}},
+                 Listed{"3H rel", 1, 2, 4, 1, 1, 1, {2, 0, 1}, {0, 0, 1}, {1, 0, 1}},
+                 Listed{"4He two sources, two sinks", 2, 2, 2, 2, 2, 2, {0, 1, 2, 3, 0, 2, 0, 2}, {0, 2, 0, 2, 0, 2, 0, 2}, {}},
+                 Listed{"3He two sources", 2, 1, 2, 2, 1, 2, {0, 1, 0, 0, 1, 1}, {0, 1, 2, 1, 3, 0}, {}}}) {
+            mbc_op_spec s = spec(c.np, c.nn, c.D);
+            s.n_sources = c.ns;
+            s.n_sinks = c.nk;
+            s.spin_mode = MBC_SPIN_LISTED;
+            s.n_spin_sel = c.n;
+            s.snk_spins = c.snk.data();
+            s.src_spins = c.src.data();
+            s.path = c.path.empty() ? nullptr : c.path.data();
+            s.path_len = (int)c.path.size();
+            mbc_term_list *L = build1(s);
+            bad += bad_pairs(c.name, *L, true, rng);
+            mbc_free_term_list(L);
+        }
+        mbc_op_spec s = spec(2, 0, 4);  // one species alone
+        mbc_term_list *L = build1(s);
+        bad += bad_pairs("pp", *L, false, rng);
+        mbc_free_term_list(L);
+        s = spec(2, 2, 2);
+        s.list_free = 1;
+        L = build1(s);
+        bad += bad_pairs("4He list-free", *L, false, rng);
         mbc_free_term_list(L);
     }
     {  // a projection: several sink and source sets with weights in one output
@@ -153,6 +244,7 @@ int main() {
         s.term_coef = w;
         mbc_term_list *L = build1(s);
         bad += bad_minors("3He projections", *L, true, rng);
+        bad += bad_pairs("3He projections", *L, true, rng);
         mbc_free_term_list(L);
     }
     {  // two nuclei on one path, both orders of adding baryons
