@@ -177,18 +177,23 @@ struct DeviceCache {
     std::vector<YRuns> yruns;          // per step, made on first mixed use
     bool wave_ready = false;           // d_opx .. d_xmap uploaded
     double *d_sat_coef = nullptr;      // saturated form: coefficient per component
-    // pair form (plan.h), one launch per tile shape of its units
+    // pair form (plan.h)
     std::shared_ptr<const PairPlan> pair;
-    uint32_t *d_pair_x = nullptr;      // two-baryon products
-    uint16_t *d_pair_ys = nullptr;
-    uint32_t *d_pair_row = nullptr, *d_pair_col = nullptr;
+    uint32_t *d_prod_ops = nullptr, *d_masks2 = nullptr;  // two-baryon products
+    int32_t *d_range_off = nullptr;
+    uint16_t *d_range_e = nullptr;
+    // packs of the rows (PairArgs)
+    PairPack *d_pair_packs = nullptr;
+    PairRow *d_pair_rows = nullptr;
+    uint32_t *d_pair_cols = nullptr;
+    uint16_t *d_pair_slot = nullptr;
     double *d_pair_val = nullptr;
-    PairUnit *d_pair_units[2] = {nullptr, nullptr};  // FP64 and mixed tiles
-    int32_t n_pair_units[2] = {0, 0};
+    PairUnit *d_pair_units = nullptr;
+    int32_t n_pair_units = 0;
     int32_t *d_pair_comp_off = nullptr, *d_pair_comp_eval = nullptr;
-    int32_t *d_pair_slot_off[2] = {nullptr, nullptr};
-    int32_t pair_slots[2] = {0, 0};
-    int pair_shape[2] = {0, 0};        // index into kPairShapes
+    int32_t *d_pair_slot_off = nullptr;
+    int32_t pair_slots = 0;
+    int pair_shape = 0;                // index into kPairShapes
 };
 
 namespace {
@@ -201,17 +206,19 @@ void free_cache(DeviceCache *c) {
     cudaFree(c->d_small_ops);
     cudaFree(c->d_small_zops);
     cudaFree(c->d_sat_coef);
-    cudaFree(c->d_pair_x);
-    cudaFree(c->d_pair_ys);
-    cudaFree(c->d_pair_row);
-    cudaFree(c->d_pair_col);
+    cudaFree(c->d_prod_ops);
+    cudaFree(c->d_masks2);
+    cudaFree(c->d_range_off);
+    cudaFree(c->d_range_e);
+    cudaFree(c->d_pair_packs);
+    cudaFree(c->d_pair_rows);
+    cudaFree(c->d_pair_cols);
+    cudaFree(c->d_pair_slot);
     cudaFree(c->d_pair_val);
     cudaFree(c->d_pair_comp_off);
     cudaFree(c->d_pair_comp_eval);
-    for (int m = 0; m < 2; ++m) {
-        cudaFree(c->d_pair_units[m]);
-        cudaFree(c->d_pair_slot_off[m]);
-    }
+    cudaFree(c->d_pair_units);
+    cudaFree(c->d_pair_slot_off);
     cudaFree(c->d_run_off);
     cudaFree(c->d_term_off);
     cudaFree(c->d_run_coef);
@@ -569,69 +576,121 @@ DeviceCache *get_wave_cache(const mbc_term_list *L, int device, mbc_status &st) 
     return st == MBC_OK ? c : nullptr;
 }
 
-// Tile shapes (proton x neutron elements per unit) of the pair kernels: one
-// component, a few, all. With more accumulators a warp reuses a row sum y for
-// more components; mixed sums carry a compensation word each, so its largest
-// tile is 6 x 2 (96 accumulator registers) against FP64's 6 x 6 (144).
-constexpr int kPairShapes[2][3][2] = {{{1, 1}, {2, 2}, {6, 6}}, {{1, 1}, {2, 2}, {6, 2}}};
-// Units per SM: enough that the last ones finish together, few enough that
-// their partial sums stay small beside the products; a unit has at least
-// kPairUnitRows rows.
-constexpr int kPairUnitsPerSm = 16;
-constexpr int kPairUnitRows = 16;
+// Tile shapes (row-side x gathered elements per unit) of the pair kernel: one
+// component, a few, all.
+constexpr int kPairShapes[3][2] = {{1, 1}, {2, 2}, {6, 2}};
+// Units per SM and tile: enough that the last ones finish together, few enough
+// that their partial sums stay small beside the products; a unit's work is at
+// least kPairUnitCost multiply-adds per site, so that its warps have a dozen rows
+// each for one copy of the gathered ones.
+constexpr int kPairUnitsPerSm = 8;
+constexpr int64_t kPairUnitCost = 8192;
 
-// Units of a pair plan for one tile shape: the groups' rows cut into chunks of
-// about equal work.
-void pair_units(const PairPlan &P, const int shape[2], int n_sm, std::vector<PairUnit> &units,
-                std::vector<int32_t> &slot_off) {
-    const int MP = shape[0], MN = shape[1];
-    // cost of rows: entries x neutron elements (2 multiply-adds) + products (4)
-    auto cost = [&](int64_t nnz, int64_t rows, int64_t na, int64_t nb) { return nnz * nb * 2 + rows * na * nb * 4; };
-    int64_t total = 0;
+// Packs of a pair plan's rows (k_pair), group by group and side by side, and the
+// units: consecutive packs of about equal work for one tile of elements.
+struct PairLayout {
+    std::vector<PairPack> packs;
+    std::vector<PairRow> rows;
+    std::vector<uint32_t> cols;
+    std::vector<uint16_t> slot;
+    std::vector<PairUnit> units;
+    std::vector<int32_t> slot_off;
+};
+PairLayout pair_layout(const PairPlan &P, const int shape[2], int n_sm) {
+    PairLayout Q;
+    // cost of rows: entries x gathered elements (2 multiply-adds) + products (4)
+    auto cost = [&](int64_t nnz, int64_t rows, int64_t nr, int64_t ng) { return nnz * ng * 2 + rows * nr * ng * 4; };
+    int64_t total = 0, n_cols = 0;
     for (const auto &g : P.groups)
-        total += cost(P.row_ptr[(size_t)g.row1] - P.row_ptr[(size_t)g.row0], g.row1 - g.row0, (int64_t)g.mp.size(),
-                      (int64_t)g.mn.size());
-    const int64_t target = std::max<int64_t>(1, total / std::max(1, n_sm * kPairUnitsPerSm));
-    slot_off.assign((size_t)P.n_evals + 1, 0);
+        for (int s = 0; s < 2; ++s)
+            total += cost(P.row_ptr[(size_t)g.row1[s]] - P.row_ptr[(size_t)g.row0[s]], g.row1[s] - g.row0[s],
+                          (int64_t)(s ? g.mn : g.mp).size(), (int64_t)(s ? g.mp : g.mn).size());
+    const int64_t target = std::max<int64_t>(kPairUnitCost, total / std::max(1, n_sm * kPairUnitsPerSm));
+    for (uint32_t c : P.col) n_cols = std::max<int64_t>(n_cols, (int64_t)c + 1);
+    std::vector<int32_t> seen((size_t)n_cols, -1);  // pack that holds a gathered row, its position
+    std::vector<uint16_t> pos((size_t)n_cols, 0);
+    Q.slot.resize(P.col.size());
+    for (size_t r = 0; r < P.row_id.size(); ++r)
+        Q.rows.push_back({P.row_id[r], (uint32_t)(P.row_ptr[r + 1] - P.row_ptr[r]), P.row_ptr[r]});
+    Q.slot_off.assign((size_t)P.n_evals + 1, 0);
+    std::vector<uint16_t> cls;
     int32_t slot = 0;
     for (const auto &g : P.groups) {
-        // row chunks of the group, the same for each of its tiles
-        const int64_t ta = std::min<int64_t>(MP, (int64_t)g.mp.size()), tb = std::min<int64_t>(MN, (int64_t)g.mn.size());
-        std::vector<int64_t> cut{g.row0};
-        int64_t acc = 0;
-        for (int64_t r = g.row0; r < g.row1; ++r) {
-            acc += cost(P.row_ptr[(size_t)r + 1] - P.row_ptr[(size_t)r], 1, ta, tb);
-            if (acc >= target && r + 1 - cut.back() >= kPairUnitRows && r + 1 < g.row1) {
-                cut.push_back(r + 1);
-                acc = 0;
+        std::vector<int32_t> cut[2];  // unit bounds in packs, per side
+        for (int s = 0; s < 2; ++s) {
+            const auto &re = s ? g.mn : g.mp, &ge = s ? g.mp : g.mn;
+            const int64_t tr = std::min<int64_t>(shape[0], (int64_t)re.size()), tg = std::min<int64_t>(shape[1], (int64_t)ge.size());
+            cut[s].push_back((int32_t)Q.packs.size());
+            int64_t acc = 0;
+            for (int64_t r = g.row0[s]; r < g.row1[s];) {
+                PairPack pk{r, (int64_t)Q.cols.size(), 0, 0};
+                const int32_t id = (int32_t)Q.packs.size();
+                // rows while their gathered rows fit the pack and the unit is not full
+                for (; r < g.row1[s]; ++r) {
+                    const int64_t e0 = P.row_ptr[(size_t)r], e1 = P.row_ptr[(size_t)r + 1];
+                    int32_t fresh = 0;
+                    for (int64_t e = e0; e < e1; ++e) fresh += seen[P.col[(size_t)e]] != id;
+                    if (pk.n_rows > 0 && (pk.n_cols + fresh > kPackCols || acc >= target)) break;
+                    for (int64_t e = e0; e < e1; ++e) {
+                        const uint32_t c = P.col[(size_t)e];
+                        if (seen[c] != id) {
+                            seen[c] = id;
+                            pos[c] = (uint16_t)pk.n_cols++;
+                            Q.cols.push_back(c);
+                        }
+                        Q.slot[(size_t)e] = pos[c];
+                    }
+                    ++pk.n_rows;
+                    acc += cost(e1 - e0, 1, tr, tg);
+                }
+                Q.packs.push_back(pk);
+                if (acc >= target || r >= g.row1[s]) {
+                    cut[s].push_back((int32_t)Q.packs.size());
+                    acc = 0;
+                }
             }
         }
-        cut.push_back(g.row1);
-        const int32_t nc = (int32_t)cut.size() - 1, nb = (int32_t)g.mn.size(), na = (int32_t)g.mp.size();
-        for (int32_t a = 0; a < na; ++a)
-            for (int32_t b = 0; b < nb; ++b) {
-                slot_off[(size_t)(g.eval0 + (int64_t)a * nb + b)] = slot + (a * nb + b) * nc;
-                slot_off[(size_t)(g.eval0 + (int64_t)a * nb + b) + 1] = slot + (a * nb + b + 1) * nc;
-            }
-        for (int32_t a0 = 0; a0 < na; a0 += MP)
-            for (int32_t b0 = 0; b0 < nb; b0 += MN)
-                for (int32_t k = 0; k < nc; ++k) {
-                    PairUnit u;
-                    std::memset(&u, 0, sizeof(u));
-                    u.row0 = (int32_t)cut[(size_t)k];
-                    u.e0 = P.row_ptr[(size_t)cut[(size_t)k]];
-                    u.e1 = P.row_ptr[(size_t)cut[(size_t)k + 1]];
-                    u.na = std::min(MP, na - a0);
-                    u.nb = std::min(MN, nb - b0);
-                    for (int i = 0; i < u.na; ++i) u.mp[i] = g.mp[(size_t)(a0 + i)];
-                    for (int i = 0; i < u.nb; ++i) u.mn[i] = g.mn[(size_t)(b0 + i)];
-                    u.stride_b = nc;
-                    u.stride_a = nb * nc;
-                    u.slot = slot + (a0 * nb + b0) * nc + k;
-                    units.push_back(u);
-                }
+        const int32_t n0 = (int32_t)cut[0].size() - 1, nc = n0 + (int32_t)cut[1].size() - 1;
+        const int32_t nb = (int32_t)g.mn.size(), na = (int32_t)g.mp.size();
+        for (int64_t ev = 0; ev < (int64_t)na * nb; ++ev) {
+            Q.slot_off[(size_t)(g.eval0 + ev)] = slot + (int32_t)ev * nc;
+            Q.slot_off[(size_t)(g.eval0 + ev) + 1] = slot + (int32_t)(ev + 1) * nc;
+        }
+        for (int s = 0; s < 2; ++s) {
+            const auto &re = s ? g.mn : g.mp, &ge = s ? g.mp : g.mn;
+            const int32_t sr = s ? nc : nb * nc, sg = s ? nb * nc : nc;
+            for (size_t a0 = 0; a0 < re.size(); a0 += (size_t)shape[0])
+                for (size_t b0 = 0; b0 < ge.size(); b0 += (size_t)shape[1])
+                    for (size_t k = 0; k + 1 < cut[s].size(); ++k) {
+                        PairUnit u;
+                        std::memset(&u, 0, sizeof(u));
+                        u.swap = s;
+                        u.pack0 = cut[s][k];
+                        u.pack1 = cut[s][k + 1];
+                        cls.push_back(P.row_class[(size_t)Q.packs[(size_t)u.pack0].row0]);
+                        u.nr = (int32_t)std::min<size_t>((size_t)shape[0], re.size() - a0);
+                        u.ng = (int32_t)std::min<size_t>((size_t)shape[1], ge.size() - b0);
+                        for (int i = 0; i < u.nr; ++i) u.re[i] = re[a0 + (size_t)i];
+                        for (int i = 0; i < u.ng; ++i) u.ge[i] = ge[b0 + (size_t)i];
+                        u.stride_r = sr;
+                        u.stride_g = sg;
+                        u.slot = slot + (int32_t)a0 * sr + (int32_t)b0 * sg + (s ? n0 : 0) + (int32_t)k;
+                        Q.units.push_back(u);
+                    }
+        }
         slot += na * nb * nc;
     }
+    // all groups' units of one colour content together: what they read (a few MB
+    // of a tile's products, 100 MB for 4He with all components) then stays in
+    // L2, where the groups one after the other sweep all of it
+    std::vector<size_t> order(Q.units.size());
+    for (size_t i = 0; i < order.size(); ++i) order[i] = i;
+    std::stable_sort(order.begin(), order.end(), [&](size_t a, size_t b) { return cls[a] < cls[b]; });
+    std::vector<PairUnit> sorted;
+    sorted.reserve(Q.units.size());
+    for (size_t i : order) sorted.push_back(Q.units[i]);
+    Q.units.swap(sorted);
+    return Q;
 }
 
 int sm_count(int device);
@@ -643,37 +702,33 @@ mbc_status ensure_pair(const mbc_term_list *Lc, DeviceCache *c, bool mixed) {
     const std::shared_ptr<const PairPlan> P = pair_plan(Lc);
     if (!P || (mixed && !P->val_fp32)) return MBC_OK;
     std::lock_guard<std::mutex> lock(const_cast<mbc_term_list *>(Lc)->dev_mu);
-    const int m = mixed ? 1 : 0;
+    if (c->pair) return MBC_OK;
     mbc_status st = MBC_OK;
     auto put = [&](auto **dst, const auto *src, size_t n) {
         if (st == MBC_OK && !*dst) st = upload(dst, src, n);
     };
-    if (!c->pair) {
-        std::vector<uint32_t> col(P->col);
-        for (size_t r = 0; r + 1 < P->row_ptr.size(); ++r) col[(size_t)P->row_ptr[r + 1] - 1] |= 0x80000000u;
-        put(&c->d_pair_x, P->sx.data(), P->sx.size());
-        put(&c->d_pair_ys, P->sys.data(), P->sys.size());
-        put(&c->d_pair_row, P->row_id.data(), P->row_id.size());
-        put(&c->d_pair_col, col.data(), col.size());
-        put(&c->d_pair_val, P->val.data(), P->val.size());
-        put(&c->d_pair_comp_off, P->comp_off.data(), P->comp_off.size());
-        put(&c->d_pair_comp_eval, P->comp_eval.data(), P->comp_eval.size());
-        if (st != MBC_OK) return st;
-        c->pair = P;
-    }
-    if (!c->d_pair_units[m]) {
-        size_t most = 0;
-        for (const auto &g : P->groups) most = std::max({most, g.mp.size(), g.mn.size()});
-        c->pair_shape[m] = most <= 1 ? 0 : most <= 2 ? 1 : 2;
-        std::vector<PairUnit> units;
-        std::vector<int32_t> slot_off;
-        pair_units(*P, kPairShapes[m][c->pair_shape[m]], sm_count(c->device), units, slot_off);
-        put(&c->d_pair_slot_off[m], slot_off.data(), slot_off.size());
-        put(&c->d_pair_units[m], units.data(), units.size());
-        c->n_pair_units[m] = (int32_t)units.size();
-        c->pair_slots[m] = slot_off.empty() ? 0 : slot_off.back();
-    }
-    return st;
+    size_t most = 0;
+    for (const auto &g : P->groups) most = std::max({most, g.mp.size(), g.mn.size()});
+    c->pair_shape = most <= 1 ? 0 : most <= 2 ? 1 : 2;
+    const PairLayout Q = pair_layout(*P, kPairShapes[c->pair_shape], sm_count(c->device));
+    put(&c->d_prod_ops, P->prod_ops.data(), P->prod_ops.size());
+    put(&c->d_masks2, P->masks2.data(), P->masks2.size());
+    put(&c->d_range_off, P->range_off.data(), P->range_off.size());
+    put(&c->d_range_e, P->range_e.data(), P->range_e.size());
+    put(&c->d_pair_packs, Q.packs.data(), Q.packs.size());
+    put(&c->d_pair_rows, Q.rows.data(), Q.rows.size());
+    put(&c->d_pair_cols, Q.cols.data(), Q.cols.size());
+    put(&c->d_pair_slot, Q.slot.data(), Q.slot.size());
+    put(&c->d_pair_val, P->val.data(), P->val.size());
+    put(&c->d_pair_comp_off, P->comp_off.data(), P->comp_off.size());
+    put(&c->d_pair_comp_eval, P->comp_eval.data(), P->comp_eval.size());
+    put(&c->d_pair_slot_off, Q.slot_off.data(), Q.slot_off.size());
+    put(&c->d_pair_units, Q.units.data(), Q.units.size());
+    if (st != MBC_OK) return st;
+    c->n_pair_units = (int32_t)Q.units.size();
+    c->pair_slots = Q.slot_off.back();
+    c->pair = P;
+    return MBC_OK;
 }
 
 // ---- scratch ---------------------------------------------------------------
@@ -874,7 +929,7 @@ LargeSizes pair_sizes(const mbc_term_list *L, const DeviceCache *c, const mbc_tu
     const PairPlan &P = *c->pair;
     LargeSizes s{};
     s.pair = true;
-    const int64_t prod = (int64_t)P.masks2.size() * P.n_rows2, slots = c->pair_slots[mixed ? 1 : 0];
+    const int64_t prod = (int64_t)P.masks2.size() * P.n_rows2, slots = c->pair_slots;
     const int64_t per_site = (int64_t)sizeof(V) * (L->block_size + prod) + 16 * (slots + L->n_comp) + 4;
     int64_t W = std::min<int64_t>(mixed ? 1024 : 512, ((int64_t)1 << 30) / per_site);
     if (tune && tune->wave_sites > 0) W = std::min(tune->wave_sites, 4096);
@@ -932,7 +987,7 @@ LargeSizes large_sizes(const mbc_term_list *L, const DeviceCache *c, const mbc_t
 // them to regenerate operations.
 bool wants_pair(const mbc_tune *tune) { return !tune || (tune->regime == 0 && tune->list_free == 0); }
 bool has_pair(const DeviceCache *c, const mbc_tune *tune, bool mixed) {
-    return wants_pair(tune) && c->pair && c->d_pair_units[mixed ? 1 : 0];
+    return wants_pair(tune) && c->pair && (!mixed || c->pair->val_fp32);
 }
 
 // The list's device copy with what its large route reads.
@@ -1258,51 +1313,51 @@ mbc_status pair_wave(const mbc_term_list *L, const DeviceCache *c, int W, const 
                      cudaStream_t stream) {
     using V = typename Tr::V;
     constexpr bool mixed = sizeof(V) == sizeof(float2);
-    constexpr int m = mixed ? 1 : 0;
     const PairPlan &P = *c->pair;
-    const int64_t n_z = (int64_t)P.masks2.size() * P.n_rows2;
-    if (n_z > 0) {
+    const int64_t prod_rows = (int64_t)P.masks2.size() * P.n_rows2;
+    const int tiles = W / (mixed ? kTileMx : kTile64);
+    if (prod_rows > 0) {
+        const int npair = (int)binom64(L->nxi, 2), n_ranges = (int)P.range_e.size(), n_masks = (int)P.masks2.size();
+        const size_t smem = (size_t)4 * npair * 512;
+        const void *kern = (const void *)k_pair_prod<mixed>;
+        int per_sm = 0;
+        mbc_status st = prepare_kernel(kern, c->device, 32 * kProdWarps, smem, &per_sm);
+        if (st != MBC_OK) return st;
         TimedLaunch tl(stream);
         note_launch();
-        if constexpr (mixed) {
-            const int64_t items = (n_z * (W / 64) + 31) / 32;
-            k_large_step_split<32, 4><<<(unsigned)std::min<int64_t>(items, nsm), 1024, 0, stream>>>(
-                c->d_pair_x, c->d_pair_ys, n_z, 12, 1, W, f, f, prod);
-        } else {
-            const int64_t ngroups = W / 32;
-            int64_t zchunk = std::max<int64_t>(1, std::min<int64_t>(256, n_z * ngroups / ((int64_t)nsm * 512)));
-            const int64_t items = ((n_z + zchunk - 1) / zchunk) * ngroups;
-            const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((items + 7) / 8, (int64_t)nsm * 8));
-            k_large_step<Tr, false><<<(unsigned)grid, 256, 0, stream>>>(c->d_pair_x, c->d_pair_ys, GenStep{}, n_z, 12,
-                                                                        zchunk, W, 0, f, f, prod);
-        }
+        k_pair_prod<mixed><<<(unsigned)(tiles * n_ranges * n_masks), 32 * kProdWarps, smem, stream>>>(
+            reinterpret_cast<const uint4 *>(c->d_prod_ops), c->d_range_off, c->d_range_e, n_ranges, c->d_masks2, n_masks,
+            npair, L->nxi, L->block_size, P.n_rows2, reinterpret_cast<const ulonglong2 *>(f),
+            reinterpret_cast<ulonglong2 *>(prod));
     }
     MBC_CUDA_TRY(cudaGetLastError());
     const int64_t block_rows = L->block_size / L->dim_snk;
-    const PairArgs A{c->d_pair_units[m], c->n_pair_units[m], c->d_pair_row,          c->d_pair_col,
-                     c->d_pair_val,      P.p_rows(block_rows), P.n_rows(block_rows)};
+    const PairArgs A{c->d_pair_units, c->n_pair_units, tiles,         c->d_pair_packs,
+                     c->d_pair_rows,  c->d_pair_cols,  c->d_pair_slot, c->d_pair_val,
+                     P.p_rows(block_rows), P.n_rows(block_rows),
+                     P.np == 2 ? prod_rows : L->block_size, P.nn == 2 ? prod_rows : L->block_size};
     const V *Pb = P.np == 2 ? prod : f, *Nb = P.nn == 2 ? prod : f;
     if (A.n_units > 0) {
-        const int shape = c->pair_shape[m];
-        const int threads = mixed ? 128 : 256;
-        const int64_t items = (int64_t)A.n_units * (W / (mixed ? 64 : 32));
-        const void *kern;
-        if constexpr (mixed)
-            kern = shape == 0 ? (const void *)k_pair_mx<1, 1> : shape == 1 ? (const void *)k_pair_mx<2, 2> : (const void *)k_pair_mx<6, 2>;
-        else
-            kern = shape == 0 ? (const void *)k_pair_fp64<1, 1> : shape == 1 ? (const void *)k_pair_fp64<2, 2> : (const void *)k_pair_fp64<6, 6>;
+        using T = std::conditional_t<mixed, PairMx, Pair64>;
+        // warps per CTA: what the accumulators' registers allow
+        constexpr int kW[3] = {16, 16, 12};
+        const int shape = c->pair_shape, threads = 32 * kW[shape];
+        const void *kern = shape == 0   ? (const void *)k_pair<T, 1, 1, kW[0]>
+                           : shape == 1 ? (const void *)k_pair<T, 2, 2, kW[1]>
+                                        : (const void *)k_pair<T, 6, 2, kW[2]>;
+        const size_t smem = shape == 0 ? pair_smem<1, kW[0]>() : shape == 1 ? pair_smem<2, kW[1]>() : pair_smem<2, kW[2]>();
         int per_sm = 0;
-        mbc_status st = prepare_kernel(kern, c->device, threads, 0, &per_sm);
+        mbc_status st = prepare_kernel(kern, c->device, threads, smem, &per_sm);
         if (st != MBC_OK) return st;
-        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((items * 32 + threads - 1) / threads, (int64_t)nsm * std::max(per_sm, 1)));
+        const int64_t grid = std::min<int64_t>((int64_t)A.n_units * tiles, (int64_t)nsm * std::max(per_sm, 1));
         void *args[] = {(void *)&A, (void *)&W, (void *)&Pb, (void *)&Nb, (void *)&part};
         TimedLaunch tl(stream);
         note_launch();
-        MBC_CUDA_TRY(cudaLaunchKernel(kern, dim3((unsigned)grid), dim3(threads), args, 0, stream));
+        MBC_CUDA_TRY(cudaLaunchKernel(kern, dim3((unsigned)grid), dim3(threads), args, smem, stream));
     }
     note_launch();
     k_pair_sum<<<dim3((unsigned)L->n_comp, (unsigned)(W / 32)), 1024, 0, stream>>>(
-        c->d_pair_comp_off, c->d_pair_comp_eval, c->d_pair_slot_off[m], W, part, sexp, deg_per_baryon * L->A, P.scale, Cb);
+        c->d_pair_comp_off, c->d_pair_comp_eval, c->d_pair_slot_off, W, part, sexp, deg_per_baryon * L->A, P.scale, Cb);
     MBC_CUDA_TRY(cudaGetLastError());
     return MBC_OK;
 }
@@ -1338,6 +1393,7 @@ mbc_status run_large(const mbc_term_list *L, const DeviceCache *c, const FieldDe
         if (pst != MBC_OK) return pst;
         if (per_sm < 1) return MBC_ERR_UNSUPPORTED;
     }
+    const int T = !ls.pair ? W : sizeof(V) == sizeof(float2) ? kTileMx : kTile64;
     for (int64_t item0 = 0; item0 < n_items; item0 += W) {
         WaveDesc wv;
         wv.item0 = item0;
@@ -1348,10 +1404,10 @@ mbc_status run_large(const mbc_term_list *L, const DeviceCache *c, const FieldDe
         note_launch();
         if (ns_blk == 4)
             k_large_blocks<Tr, 4><<<W / 4, 512, blk_smem, stream>>>(F, wv, nrow, nxi, n_g2(L), (int)L->block_size,
-                                                                    (int)binom64(nxi, 2), f, sexp);
+                                                                    (int)binom64(nxi, 2), T, f, sexp);
         else
             k_large_blocks<Tr, 16><<<W / 16, 512, blk_smem, stream>>>(F, wv, nrow, nxi, n_g2(L), (int)L->block_size,
-                                                                      (int)binom64(nxi, 2), f, sexp);
+                                                                      (int)binom64(nxi, 2), T, f, sexp);
         MBC_CUDA_TRY(cudaGetLastError());
         if (ls.pair) {
             mbc_status pst = pair_wave<Tr>(L, c, W, f, buf[0], ppart, sexp, 3, Cb, nsm, stream);
@@ -1461,10 +1517,11 @@ mbc_status run_projected(const mbc_term_list *L, const DeviceCache *c, const Fie
     // 2. recursion and contraction per item, a wave of W items at a time
     const int64_t n_items = n_slabs * n_groups;
     const int per_spin = (int)(binom64(nxi, 2) * nxi);
+    const int T = !ls.pair ? W : mx ? kTileMx : kTile64;
     for (int64_t item0 = 0; item0 < n_items; item0 += W) {
         note_launch();
         k_load_proj_blocks<Tr><<<(unsigned)((W + 7) / 8), 256, 0, stream>>>(Pf, n_items, item0, W, bs, per_spin, n_k,
-                                                                            M.n_mom, f, sexp);
+                                                                            M.n_mom, T, f, sexp);
         MBC_CUDA_TRY(cudaGetLastError());
         const V *X = f;
         mbc_status cst = ls.pair ? pair_wave<Tr>(L, c, W, f, buf[0], ppart, sexp, 1, Cb, nsm, stream)

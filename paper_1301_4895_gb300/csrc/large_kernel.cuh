@@ -35,6 +35,14 @@ __device__ __forceinline__ bool item_site(const FieldDesc &F, const WaveDesc &wv
     return site < wv.v3;
 }
 
+// Entry of component e at wave site w in a buffer of tiles of T sites,
+// [tile][component][site]. The recursion's buffers are one tile of the whole
+// wave; the pair form's are tiles of one warp's sites (512 B rows): gathers from
+// rows a power of two apart would share a few cache sets and L2 slices.
+__device__ __forceinline__ int64_t wave_index(int64_t e, int w, int T, int64_t n_comp) {
+    return (int64_t)(w / T) * T * n_comp + e * T + w % T;
+}
+
 // Per-site regions of the block kernels' shared memory are padded by one
 // element: the 16 sites of a warp then read the same entry from 16 distinct
 // banks (an unpadded 12 x 12 tile puts all of them in one bank).
@@ -48,9 +56,10 @@ __host__ __device__ constexpr int diquark_stride(int nxi) { return 3 * nxi * nxi
 // shared memory.
 constexpr int kTileLoads = 9;  // tile entries per lane: 12 x 24 / 32
 
+// T: sites per tile of the output buffer (wave_index).
 template <class Tr, int NS>
 __global__ void __launch_bounds__(512) k_large_blocks(FieldDesc F, WaveDesc wv, int nrow, int nxi, int n_g2,
-                                                      int block_size, int npair, typename Tr::V *f,
+                                                      int block_size, int npair, int T, typename Tr::V *f,
                                                       int32_t *sexp_out) {
     using V = typename Tr::V;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -112,7 +121,7 @@ __global__ void __launch_bounds__(512) k_large_blocks(FieldDesc F, WaveDesc wv, 
             acc = cfma(Sr[i], Qs[(c * nxi + j) * nxi + single], acc);
             acc = cfms(Sr[j], Qs[(c * nxi + i) * nxi + single], acc);
         }
-        Tr::wave_st(f, (int64_t)e * wv.W + w0 + sl, acc);
+        Tr::wave_st(f, wave_index(e, w0 + sl, T, block_size), acc);
     }
 }
 

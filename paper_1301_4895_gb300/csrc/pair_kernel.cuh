@@ -2,229 +2,313 @@
 // C = sum_ij P_i Lambda_ij N_j with P and N the ordered products of a species'
 // blocks, one sparse real Lambda per group of components.
 //
-//   k_pair      a warp takes a unit - a chunk of a group's Lambda rows for up to
-//               MP proton and MN neutron spin sets - and a site group (32
-//               sites; 64 in mixed precision, two per lane). Per row it sums
-//               y_b = sum_j Lambda_ij N_b[j] over the row's entries, then adds
-//               P_a[i] y_b to MP x MN accumulators. Site groups are the slow
-//               index of the items, so the warps of the GPU gather from one
-//               group's products at a time and those stay in L2.
+// Blocks and products lie in tiles of a warp's sites, [tile][row][32 sites of
+// FP64 or 64 of FP32], 512 B a row.
+//   k_pair_prod a CTA copies the 4 x n_pairs block rows that the products with
+//               two given singles name into shared memory (135 KB) and forms the
+//               range's products from there: their 24 operands a row would
+//               otherwise come from L2, at its bandwidth in mixed precision.
+//   k_pair      a CTA takes a unit - packs of rows of one group for up to MR spin
+//               sets of the row side and MG of the gathered side (a P row
+//               gathers N, an N row gathers P) - and a tile. A pack is rows that
+//               name at most kPackCols distinct gathered entries; the CTA copies
+//               those into shared memory, then a warp takes a row at a time: y_b
+//               = sum_j Lambda_ij G_b[j] from shared memory, then R_a[i] y_b into
+//               MR x MG accumulators, R_a[i] loaded while y is summed. Gathering
+//               from L2 instead left the warps waiting (11 cycles an
+//               instruction, L1 hits 57 %).
 //   k_pair_sum  adds the units' partial sums of every component in a fixed
 //               order and undoes the mixed path's scaling.
-// FP64 is bound by the FP64 pipe, mixed by the L2 gathers of N. Whole calls on
-// GB300 against the recursion (8.5 M complex multiply-adds per site for one
-// component, here 0.37 M for the products and 0.31 M real-complex ones; 531 M
-// for all 1296): one component mixed, 16^3 x 4, 125.2 -> 12.1 ms; all, FP64, 64
-// sites, 233.7 -> 26.9 ms; all, mixed, 512 sites, 227.7 -> 70.8 ms.
+// FP64 is bound by the FP64 pipe, mixed by shared-memory wavefronts (53-66 % of
+// the pipe) and its few warps' latencies. Whole calls on GB300 against the
+// recursion (8.5 M complex multiply-adds per site for one component, here 0.37 M
+// for the products and 0.31 M real-complex ones; 531 M for all 1296): one
+// component mixed, 16^3 x 4, 125.2 -> 9.3 ms (12.1 with L2 gathers, rows in rank
+// order); all, FP64, 64 sites, 233.7 -> 20.4 ms (26.9); all, mixed, 512 sites,
+// 227.7 -> 25.5 ms (70.8).
 #pragma once
 
 #include "large_kernel.cuh"
 
 namespace mbc {
 
-// One unit: rows [row0, row1) of Lambda (entries [e0, e1)), proton elements
-// mp[0, na), neutron elements mn[0, nb); the partial of (a, b) goes to slot
-// slot + a * stride_a + b * stride_b.
+constexpr int kTile64 = 32, kTileMx = 64;  // sites per tile
+constexpr int kProdWarps = 24;
+
+// Products of one (tile, spin set, singles range) per CTA; grid = tiles x sets x ranges.
+template <bool MX>
+__global__ void __launch_bounds__(32 * kProdWarps, 1)
+    k_pair_prod(const uint4 *__restrict__ ops, const int32_t *__restrict__ range_off,
+                const uint16_t *__restrict__ range_e, int n_ranges, const uint32_t *__restrict__ masks, int n_masks,
+                int npair, int nxi, int64_t block_rows, int n_rows, const ulonglong2 *__restrict__ f,
+                ulonglong2 *__restrict__ prod) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    ulonglong2 *rows = reinterpret_cast<ulonglong2 *>(smem_raw);  // [f | g][single][pair][lane]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int k = blockIdx.x % n_ranges, m = blockIdx.x / n_ranges % n_masks;
+    const int64_t tile = blockIdx.x / n_ranges / n_masks;
+    const uint32_t mask = __ldg(masks + m);
+    const int spin[2] = {__ffs(mask) - 1, 31 - __clz(mask)};
+    const int e[2] = {range_e[k] & 255, range_e[k] >> 8};
+    const ulonglong2 *ft = f + tile * block_rows * 32;
+    for (int r = warp; r < 4 * npair; r += kProdWarps) {
+        const int s = r / (2 * npair), i = r / npair & 1, p = r % npair;
+        rows[r * 32 + lane] = __ldg(ft + ((int64_t)(spin[s] * npair + p) * nxi + e[i]) * 32 + lane);
+    }
+    __syncthreads();
+    const ulonglong2 *F = rows + lane, *G = rows + 2 * npair * 32 + lane;
+    ulonglong2 *out = prod + ((tile * n_masks + m) * n_rows) * 32 + lane;
+    const int r1 = range_off[k + 1];
+    for (int r = range_off[k] + warp; r < r1; r += kProdWarps) {
+        uint32_t op[12];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const uint4 v = __ldg(ops + 3 * r + q);
+            op[4 * q] = v.x;
+            op[4 * q + 1] = v.y;
+            op[4 * q + 2] = v.z;
+            op[4 * q + 3] = v.w;
+        }
+        if constexpr (MX) {
+            PairAcc acc;
+            acc.zero();
+#pragma unroll
+            for (int j = 0; j < 12; ++j)
+                acc.fma(F[(op[j] & 0x7fffu) * 32], G[(op[j] >> 15 & 0x7fffu) * 32], f2_sign_pair((int32_t)op[j] < 0));
+            out[(int64_t)r * 32] = acc.store();
+        } else {
+            FP64Traits::Acc acc;
+            acc.zero();
+#pragma unroll
+            for (int j = 0; j < 12; ++j) {
+                const double2 x = reinterpret_cast<const double2 *>(F)[(op[j] & 0x7fffu) * 32];
+                const double2 y = reinterpret_cast<const double2 *>(G)[(op[j] >> 15 & 0x7fffu) * 32];
+                acc.fma(x, y, op[j] & 0x80000000u);
+            }
+            reinterpret_cast<double2 *>(out)[(int64_t)r * 32] = acc.store();
+        }
+    }
+}
+
+// Gathered entries a pack names at most: with two spin sets 208 rows of 512 B
+// fill an SM's shared memory; one set takes half of it, so two CTAs overlap one's
+// copies with the other's sums.
+constexpr int kPackCols = 208;
+
+struct PairPack {
+    int64_t row0;    // rows [row0, row0 + n_rows)
+    int64_t col0;    // gathered rows cols[col0 .. col0 + n_cols)
+    int32_t n_rows, n_cols;
+};
+// One unit: packs [pack0, pack1), row-side elements re[0, nr), gathered
+// elements ge[0, ng) (swap: rows of N gathering P); the partial of (a, b) goes
+// to slot + a * stride_r + b * stride_g.
 struct PairUnit {
-    int64_t e0, e1;
-    int32_t row0;
-    int32_t na, nb;
-    int32_t mp[6], mn[6];
-    int32_t slot, stride_a, stride_b;
+    int32_t pack0, pack1, swap;
+    int32_t nr, ng;
+    int32_t re[6], ge[6];
+    int32_t slot, stride_r, stride_g;
+};
+struct __align__(16) PairRow {
+    uint32_t row, n;  // row-side row, entries [e0, e0 + n)
+    int64_t e0;
 };
 
 struct PairArgs {
     const PairUnit *units;
-    int32_t n_units;
-    const uint32_t *row_id;
-    const uint32_t *col;   // N row, bit 31: last entry of its Lambda row
+    int32_t n_units, n_tiles;
+    const PairPack *packs;
+    const PairRow *rows;
+    const uint32_t *cols;
+    const uint16_t *slot;      // entries: position of the gathered row in its pack
     const double *val;
-    int64_t p_rows, n_rows;  // rows per element
+    int64_t p_rows, n_rows;    // rows per element
+    int64_t p_tile, n_tile;    // rows per tile of P's and N's buffer
+};
+
+// y += v x with a real factor v, and acc += x y; values of 16 B per lane: one
+// site in FP64, two in mixed precision. Mixed terms of y enter the Kahan step as
+// fma(x, v, n): one rounding each, as PairAcc's signed step with a factor in the
+// place of the sign.
+struct Pair64 {
+    static constexpr int kSites = 1;
+    struct Y {
+        double re, im;
+        __device__ __forceinline__ void zero() { re = im = 0.0; }
+        __device__ __forceinline__ void add(ulonglong2 x, double v) {
+            re = __fma_rn(v, __longlong_as_double((long long)x.x), re);
+            im = __fma_rn(v, __longlong_as_double((long long)x.y), im);
+        }
+    };
+    struct Acc {
+        FP64Traits::Acc a;
+        __device__ __forceinline__ void zero() { a.zero(); }
+        __device__ __forceinline__ void fma(ulonglong2 x, const Y &y) {
+            a.fma(make_double2(__longlong_as_double((long long)x.x), __longlong_as_double((long long)x.y)),
+                  make_double2(y.re, y.im), 0u);
+        }
+        __device__ __forceinline__ void values(double2 (&v)[1]) const { v[0] = a.value(); }
+    };
+    __device__ __forceinline__ static double factor(double v) { return v; }
+};
+struct PairMx {
+    static constexpr int kSites = 2;
+    struct Y {
+        uint64_t sr, si, nr, ni;
+        __device__ __forceinline__ void zero() { sr = si = nr = ni = 0ull; }
+        __device__ __forceinline__ void add(ulonglong2 x, uint64_t v) {
+            f2_kahan_signed(sr, nr, x.x, v);
+            f2_kahan_signed(si, ni, x.y, v);
+        }
+    };
+    struct Acc {
+        PairAcc a;
+        __device__ __forceinline__ void zero() { a.zero(); }
+        __device__ __forceinline__ void fma(ulonglong2 x, const Y &y) {
+            a.fma(x, make_ulonglong2(f2_add(y.sr, y.nr), f2_add(y.si, y.ni)), f2_sign_pair(false));
+        }
+        __device__ __forceinline__ void values(double2 (&v)[2]) const {
+            const float2 sr = f2_unpack(a.sr), si = f2_unpack(a.si), nr = f2_unpack(a.nr), ni = f2_unpack(a.ni);
+            v[0] = make_double2((double)sr.x + (double)nr.x, (double)si.x + (double)ni.x);
+            v[1] = make_double2((double)sr.y + (double)nr.y, (double)si.y + (double)ni.y);
+        }
+    };
+    __device__ __forceinline__ static uint64_t factor(double v) { return f2_pack((float)v, (float)v); }
 };
 
 struct __align__(16) PairRec {
-    uint32_t col, last;
-    double val;
+    uint32_t off, pad;
+    uint64_t v;  // FP64: the value; mixed: its FP32 pair
 };
 
-// y += v x with a real factor, complex FP64
-struct RealAcc64 {
-    double re, im;
-    __device__ __forceinline__ void zero() { re = im = 0.0; }
-    __device__ __forceinline__ void add(double2 x, double v) {
-        re = __fma_rn(v, x.x, re);
-        im = __fma_rn(v, x.y, im);
-    }
-    __device__ __forceinline__ double2 store() const { return make_double2(re, im); }
-};
-
-template <int MP, int MN>
-__global__ void __launch_bounds__(256) k_pair_fp64(PairArgs A, int W, const double2 *__restrict__ P,
-                                                   const double2 *__restrict__ N, double2 *__restrict__ part) {
-    __shared__ PairRec recs[8][32];
-    const int lane = threadIdx.x & 31;
-    PairRec *rec = recs[threadIdx.x >> 5];
-    const int64_t n_items = (int64_t)A.n_units * (W >> 5);
-    for (int64_t item = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); item < n_items; item += (int64_t)gridDim.x * 8) {
-        const PairUnit &u = A.units[item % A.n_units];
-        const int col0 = (int)(item / A.n_units) * 32 + lane;
-        const double2 *Nb[MN];
-#pragma unroll
-        for (int b = 0; b < MN; ++b) Nb[b] = N + (int64_t)u.mn[min(b, u.nb - 1)] * A.n_rows * W + col0;
-        const double2 *Pb[MP];
-#pragma unroll
-        for (int a = 0; a < MP; ++a) Pb[a] = P + (int64_t)u.mp[min(a, u.na - 1)] * A.p_rows * W + col0;
-        RealAcc64 y[MN];
-        FP64Traits::Acc acc[MP][MN];
-#pragma unroll
-        for (int b = 0; b < MN; ++b) {
-            y[b].zero();
-#pragma unroll
-            for (int a = 0; a < MP; ++a) acc[a][b].zero();
-        }
-        const uint32_t *row = A.row_id + u.row0;
-        for (int64_t e0 = u.e0; e0 < u.e1; e0 += 32) {
-            const int n = (int)min((int64_t)32, u.e1 - e0);
-            __syncwarp();
-            if (lane < n) {
-                const uint32_t c = __ldg(A.col + e0 + lane);
-                rec[lane] = PairRec{c & 0x7fffffffu, c >> 31, __ldg(A.val + e0 + lane)};
-            }
-            __syncwarp();
-            constexpr int G = MN > 2 ? 1 : 4;
-            for (int t = 0; t < n; t += G) {
-                double2 x[G][MN];
-#pragma unroll
-                for (int g = 0; g < G; ++g)
-                    if (t + g < n) {
-                        const int64_t o = (int64_t)rec[t + g].col * W;
-#pragma unroll
-                        for (int b = 0; b < MN; ++b) x[g][b] = __ldg(Nb[b] + o);
-                    }
-#pragma unroll
-                for (int g = 0; g < G; ++g) {
-                    if (t + g >= n) break;
-                    const PairRec r = rec[t + g];
-#pragma unroll
-                    for (int b = 0; b < MN; ++b) y[b].add(x[g][b], r.val);
-                    if (r.last) {
-                        const int64_t o = (int64_t)__ldg(row++) * W;
-#pragma unroll
-                        for (int a = 0; a < MP; ++a) {
-                            const double2 p = __ldg(Pb[a] + o);
-#pragma unroll
-                            for (int b = 0; b < MN; ++b) acc[a][b].fma(p, y[b].store(), 0u);
-                        }
-#pragma unroll
-                        for (int b = 0; b < MN; ++b) y[b].zero();
-                    }
-                }
-            }
-        }
-#pragma unroll
-        for (int a = 0; a < MP; ++a)
-#pragma unroll
-            for (int b = 0; b < MN; ++b)
-                if (a < u.na && b < u.nb)
-                    part[(int64_t)(u.slot + a * u.stride_a + b * u.stride_b) * W + col0] = acc[a][b].value();
-    }
+// dynamic shared memory: the pack's rows [MG][kPackCols][32 lanes], then 32
+// records per warp; the partial sums of a unit reuse the rows' room
+template <int MG, int WARPS>
+__host__ __device__ constexpr size_t pair_smem() {
+    return (size_t)MG * kPackCols * 512 + (size_t)WARPS * 32 * sizeof(PairRec);
 }
 
-// The mixed form: two sites per lane, compensated FP32 sums (PairAcc). A row
-// sum's terms enter the Kahan step as fma(x, v, n): one rounding each, as the
-// signed step of PairAcc with a factor in the place of the sign.
-struct RealAccPair {
-    uint64_t sr, si, nr, ni;
-    __device__ __forceinline__ void zero() { sr = si = nr = ni = 0ull; }
-    __device__ __forceinline__ void add(ulonglong2 x, uint64_t v) {
-        f2_kahan_signed(sr, nr, x.x, v);
-        f2_kahan_signed(si, ni, x.y, v);
-    }
-    __device__ __forceinline__ ulonglong2 store() const { return make_ulonglong2(f2_add(sr, nr), f2_add(si, ni)); }
-};
-
-template <int MP, int MN>
-__global__ void __launch_bounds__(128, MP * MN > 4 ? 3 : 6)
-    k_pair_mx(PairArgs A, int W, const float2 *__restrict__ P, const float2 *__restrict__ N,
-              double2 *__restrict__ part) {
-    __shared__ OpRec recs[4][32];  // x: N row, y: last, sg: the value twice
-    const int lane = threadIdx.x & 31;
-    OpRec *rec = recs[threadIdx.x >> 5];
-    const int64_t n_items = (int64_t)A.n_units * (W >> 6);
-    const uint32_t row_bytes = (uint32_t)W * (uint32_t)sizeof(float2);
-    for (int64_t item = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5); item < n_items; item += (int64_t)gridDim.x * 4) {
+template <class T, int MR, int MG, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, MG == 1 ? 2 : 1)
+    k_pair(PairArgs A, int W, const ulonglong2 *__restrict__ P, const ulonglong2 *__restrict__ N,
+           double2 *__restrict__ part) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    ulonglong2 *stage = reinterpret_cast<ulonglong2 *>(smem_raw);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    PairRec *rec = reinterpret_cast<PairRec *>(smem_raw + (size_t)MG * kPackCols * 512) + warp * 32;
+    const int64_t n_items = (int64_t)A.n_units * A.n_tiles;
+    for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
         const PairUnit &u = A.units[item % A.n_units];
-        const int grp = (int)(item / A.n_units);
-        const unsigned char *Nb[MN], *Pb[MP];
+        const int64_t tile = item / A.n_units;
+        const ulonglong2 *Pt = P + tile * A.p_tile * 32 + lane, *Nt = N + tile * A.n_tile * 32 + lane;
+        const ulonglong2 *Rs = u.swap ? Nt : Pt, *Gs = u.swap ? Pt : Nt;
+        const int64_t r_rows = u.swap ? A.n_rows : A.p_rows, g_rows = u.swap ? A.p_rows : A.n_rows;
+        const ulonglong2 *Rb[MR];
 #pragma unroll
-        for (int b = 0; b < MN; ++b)
-            Nb[b] = reinterpret_cast<const unsigned char *>(N + (int64_t)u.mn[min(b, u.nb - 1)] * A.n_rows * W) +
-                    grp * 512 + lane * 16;
+        for (int a = 0; a < MR; ++a) Rb[a] = Rs + (int64_t)u.re[min(a, u.nr - 1)] * r_rows * 32;
+        typename T::Acc acc[MR][MG];
 #pragma unroll
-        for (int a = 0; a < MP; ++a)
-            Pb[a] = reinterpret_cast<const unsigned char *>(P + (int64_t)u.mp[min(a, u.na - 1)] * A.p_rows * W) +
-                    grp * 512 + lane * 16;
-        RealAccPair y[MN];
-        PairAcc acc[MP][MN];
+        for (int a = 0; a < MR; ++a)
 #pragma unroll
-        for (int b = 0; b < MN; ++b) {
-            y[b].zero();
+            for (int b = 0; b < MG; ++b) acc[a][b].zero();
+        for (int k = u.pack0; k < u.pack1; ++k) {
+            const PairPack pk = A.packs[k];
+            __syncthreads();  // the previous pack (or unit) is done with the rows
+            for (int c = warp; c < pk.n_cols; c += WARPS) {
+                const int64_t row = (int64_t)__ldg(A.cols + pk.col0 + c) * 32;
 #pragma unroll
-            for (int a = 0; a < MP; ++a) acc[a][b].zero();
-        }
-        const uint64_t one = f2_sign_pair(false);
-        const uint32_t *row = A.row_id + u.row0;
-        for (int64_t e0 = u.e0; e0 < u.e1; e0 += 32) {
-            const int n = (int)min((int64_t)32, u.e1 - e0);
-            __syncwarp();
-            if (lane < n) {
-                const uint32_t c = __ldg(A.col + e0 + lane);
-                const float v = (float)__ldg(A.val + e0 + lane);
-                rec[lane] = OpRec{c & 0x7fffffffu, c >> 31, f2_pack(v, v)};
+                for (int b = 0; b < MG; ++b)
+                    stage[(b * kPackCols + c) * 32 + lane] = __ldg(Gs + (int64_t)u.ge[min(b, u.ng - 1)] * g_rows * 32 + row);
             }
-            __syncwarp();
-            constexpr int G = MN > 2 ? 2 : 8 / MN;
-            for (int t = 0; t < n; t += G) {
-                ulonglong2 x[G][MN];
+            __syncthreads();
+            const ulonglong2 *G = stage + lane;
+            // two rows ahead: the next row's records are loaded while this one is
+            // worked off, and the row after gives their place
+            const PairRow none{0u, 0u, 0};
+            const PairRow *rows = A.rows + pk.row0;
+            PairRow row = warp < pk.n_rows ? rows[warp] : none;
+            PairRow next = warp + WARPS < pk.n_rows ? rows[warp + WARPS] : none;
+            auto load = [&](const PairRow &w, uint32_t e0, double &v, uint32_t &o) {
+                if (e0 + lane < w.n) {
+                    v = __ldg(A.val + w.e0 + e0 + lane);
+                    o = __ldg(A.slot + w.e0 + e0 + lane);
+                }
+            };
+            double rv = 0.0;
+            uint32_t ro = 0;
+            load(row, 0, rv, ro);
+            for (int r = warp; r < pk.n_rows; r += WARPS) {
+                ulonglong2 x[MR];
 #pragma unroll
-                for (int g = 0; g < G; ++g)
-                    if (t + g < n) {
-                        const size_t o = (size_t)rec[t + g].x * row_bytes;
+                for (int a = 0; a < MR; ++a) x[a] = __ldg(Rb[a] + row.row * 32u);
+                const PairRow after = r + 2 * WARPS < pk.n_rows ? rows[r + 2 * WARPS] : none;
+                typename T::Y y[MG];
 #pragma unroll
-                        for (int b = 0; b < MN; ++b) x[g][b] = __ldg(reinterpret_cast<const ulonglong2 *>(Nb[b] + o));
+                for (int b = 0; b < MG; ++b) y[b].zero();
+                for (uint32_t e0 = 0; e0 < row.n; e0 += 32) {
+                    const int n = (int)min(32u, row.n - e0);
+                    __syncwarp();
+                    {
+                        const auto f = T::factor(rv);
+                        PairRec v{ro * 32u, 0u, 0ull};
+                        memcpy(&v.v, &f, 8);
+                        rec[lane] = v;
                     }
+                    __syncwarp();
+                    if (e0 + 32 < row.n)
+                        load(row, e0 + 32, rv, ro);
+                    else
+                        load(next, 0, rv, ro);
+                    int t = 0;
+                    for (; t + 4 <= n; t += 4) {
 #pragma unroll
-                for (int g = 0; g < G; ++g) {
-                    if (t + g >= n) break;
-                    const OpRec r = rec[t + g];
+                        for (int g = 0; g < 4; ++g) {
+                            const PairRec v = rec[t + g];
+                            decltype(T::factor(0.0)) f;
+                            memcpy(&f, &v.v, 8);
 #pragma unroll
-                    for (int b = 0; b < MN; ++b) y[b].add(x[g][b], r.sg);
-                    if (r.y) {
-                        const size_t o = (size_t)__ldg(row++) * row_bytes;
-#pragma unroll
-                        for (int a = 0; a < MP; ++a) {
-                            const ulonglong2 p = __ldg(reinterpret_cast<const ulonglong2 *>(Pb[a] + o));
-#pragma unroll
-                            for (int b = 0; b < MN; ++b) acc[a][b].fma(p, y[b].store(), one);
+                            for (int b = 0; b < MG; ++b) y[b].add(G[b * kPackCols * 32 + v.off], f);
                         }
+                    }
+                    for (; t < n; ++t) {
+                        const PairRec v = rec[t];
+                        decltype(T::factor(0.0)) f;
+                        memcpy(&f, &v.v, 8);
 #pragma unroll
-                        for (int b = 0; b < MN; ++b) y[b].zero();
+                        for (int b = 0; b < MG; ++b) y[b].add(G[b * kPackCols * 32 + v.off], f);
                     }
                 }
+#pragma unroll
+                for (int a = 0; a < MR; ++a)
+#pragma unroll
+                    for (int b = 0; b < MG; ++b) acc[a][b].fma(x[a], y[b]);
+                row = next;
+                next = after;
             }
         }
-        const int col0 = grp * 64 + 2 * lane;
+        // the unit's partial: the warps' sums added in warp order, a pair (a, b)
+        // per round of MG
+        constexpr int S = T::kSites;
+        double2 *sums = reinterpret_cast<double2 *>(smem_raw);  // [MG][WARPS][32 S]
 #pragma unroll
-        for (int a = 0; a < MP; ++a)
+        for (int a = 0; a < MR; ++a) {
+            __syncthreads();
 #pragma unroll
-            for (int b = 0; b < MN; ++b)
-                if (a < u.na && b < u.nb) {
-                    double2 *dst = part + (int64_t)(u.slot + a * u.stride_a + b * u.stride_b) * W + col0;
-                    const float2 sr = f2_unpack(acc[a][b].sr), si = f2_unpack(acc[a][b].si);
-                    const float2 nr = f2_unpack(acc[a][b].nr), ni = f2_unpack(acc[a][b].ni);
-                    dst[0] = make_double2((double)sr.x + (double)nr.x, (double)si.x + (double)ni.x);
-                    dst[1] = make_double2((double)sr.y + (double)nr.y, (double)si.y + (double)ni.y);
-                }
+            for (int b = 0; b < MG; ++b) {
+                double2 v[S];
+                acc[a][b].values(v);
+#pragma unroll
+                for (int q = 0; q < S; ++q) sums[(b * WARPS + warp) * 32 * S + lane * S + q] = v[q];
+            }
+            __syncthreads();
+            for (int o = threadIdx.x; o < MG * 32 * S; o += 32 * WARPS) {
+                const int b = o / (32 * S), site = o % (32 * S);
+                if (a >= u.nr || b >= u.ng) continue;
+                double2 t = sums[b * WARPS * 32 * S + site];
+                for (int w = 1; w < WARPS; ++w) t = cadd(t, sums[(b * WARPS + w) * 32 * S + site]);
+                part[(int64_t)(u.slot + a * u.stride_r + b * u.stride_g) * W + tile * 32 * S + site] = t;
+            }
+        }
     }
 }
 

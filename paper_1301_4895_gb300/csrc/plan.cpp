@@ -3,6 +3,7 @@
 #include "plan.h"
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <map>
 #include <new>
@@ -302,6 +303,100 @@ std::vector<Split> splits_of(uint32_t set, int k) {
     return out;
 }
 
+struct PairEntry {
+    uint32_t i, j;
+    double v;
+};
+// Rows of one group's matrix: [0] P rows gathering N, [1] N rows gathering P.
+struct PairRows {
+    struct Row {
+        uint32_t id;
+        int64_t e0, e1;
+        int32_t block;
+        uint16_t cls;
+    };
+    std::vector<Row> rows[2];
+    std::vector<uint32_t> col;
+    std::vector<double> val;
+};
+
+// Assign every entry to its P row or its N row by a greedy vertex cover (the
+// vertex with the most unassigned entries next) and order the rows by
+// connected block, then by their columns. n_n = 0: one vertex set for both
+// sides (symmetric matrix), P rows only.
+template <class ClassOf>
+void pair_rows(const std::vector<PairEntry> &all, int64_t n_p, int64_t n_n, ClassOf &&class_of, PairRows &R) {
+    const bool sym = n_n == 0;
+    const size_t nv = (size_t)(n_p + n_n);
+    auto vert = [&](const PairEntry &e, int s) { return s == 0 || sym ? (s ? e.j : e.i) : (uint32_t)(n_p + e.j); };
+    std::vector<int64_t> off(nv + 1, 0);
+    std::vector<int32_t> up(nv);
+    for (size_t v = 0; v < nv; ++v) up[v] = (int32_t)v;
+    auto find = [&](uint32_t v) {
+        while (up[v] != (int32_t)v) v = (uint32_t)(up[v] = up[(size_t)up[v]]);
+        return v;
+    };
+    for (const auto &e : all) {
+        const uint32_t a = vert(e, 0), b = vert(e, 1);
+        ++off[a + 1];
+        if (b != a) ++off[b + 1];
+        const uint32_t x = find(a), y = find(b);
+        if (x != y) up[std::max(x, y)] = (int32_t)std::min(x, y);
+    }
+    for (size_t v = 0; v < nv; ++v) off[v + 1] += off[v];
+    std::vector<int64_t> at(off.begin(), off.end() - 1), deg(nv);
+    std::vector<int32_t> adj((size_t)off[nv]);
+    for (size_t k = 0; k < all.size(); ++k) {
+        const uint32_t a = vert(all[k], 0), b = vert(all[k], 1);
+        adj[(size_t)at[a]++] = (int32_t)k;
+        if (b != a) adj[(size_t)at[b]++] = (int32_t)k;
+    }
+    std::vector<uint8_t> taken(all.size(), 0);
+    std::vector<std::vector<uint32_t>> bucket;
+    for (size_t v = 0; v < nv; ++v) {
+        deg[v] = off[v + 1] - off[v];
+        if (deg[v] >= (int64_t)bucket.size()) bucket.resize((size_t)deg[v] + 1);
+        if (deg[v]) bucket[(size_t)deg[v]].push_back((uint32_t)v);
+    }
+    R.col.reserve(all.size());
+    R.val.reserve(all.size());
+    for (int64_t d = (int64_t)bucket.size() - 1; d > 0; --d)
+        for (size_t q = 0; q < bucket[(size_t)d].size(); ++q) {
+            const uint32_t v = bucket[(size_t)d][q];
+            if (deg[v] != d) {  // lost entries since it was filed
+                if (deg[v] > 0 && deg[v] < d) bucket[(size_t)deg[v]].push_back(v);
+                continue;
+            }
+            const bool n_row = !sym && (int64_t)v >= n_p;
+            PairRows::Row row{n_row ? (uint32_t)(v - n_p) : v, (int64_t)R.col.size(), 0, (int32_t)find(v), 0};
+            row.cls = class_of(row.id, n_row ? 1 : 0);
+            std::vector<std::pair<uint32_t, double>> entries;
+            for (int64_t k = off[v]; k < off[v + 1]; ++k) {
+                const int32_t e = adj[(size_t)k];
+                if (taken[(size_t)e]) continue;
+                taken[(size_t)e] = 1;
+                const uint32_t a = vert(all[(size_t)e], 0), b = vert(all[(size_t)e], 1), o = a == v ? b : a;
+                entries.push_back({n_row || sym ? o : all[(size_t)e].j, all[(size_t)e].v});
+                if (o != v) --deg[o];
+            }
+            deg[v] = 0;
+            std::sort(entries.begin(), entries.end());
+            for (const auto &e : entries) {
+                R.col.push_back(e.first);
+                R.val.push_back(e.second);
+            }
+            row.e1 = (int64_t)R.col.size();
+            R.rows[n_row ? 1 : 0].push_back(row);
+        }
+    for (auto &rows : R.rows)
+        std::sort(rows.begin(), rows.end(), [&](const PairRows::Row &a, const PairRows::Row &b) {
+            if (a.cls != b.cls) return a.cls < b.cls;
+            if (a.block != b.block) return a.block < b.block;
+            return std::lexicographical_compare(R.col.begin() + a.e0, R.col.begin() + a.e1, R.col.begin() + b.e0,
+                                                R.col.begin() + b.e1);
+        });
+}
+
 constexpr int64_t kMaxPairEntries = (int64_t)1 << 26;  // 12 B each on the device
 
 std::shared_ptr<const PairPlan> make_pair_plan(const mbc_term_list &L) {
@@ -313,11 +408,13 @@ std::shared_ptr<const PairPlan> make_pair_plan(const mbc_term_list &L) {
         if (s.generated) return nullptr;  // list-free lists keep no tables
     std::vector<std::vector<PlanEntry>> comp;
     if (!list_entries(L, comp)) return nullptr;
-    // evaluations: (sink spin sets, tensor), the tensor a list of (U, D, l)
+    // evaluations: (sink spin sets, tensor), the tensor a list of (U, D, l) in
+    // key order (the list's contraction entries are sorted by key)
     using UD = std::pair<uint32_t, uint32_t>;
-    using Tensor = std::map<UD, double>;
+    using Tensor = std::vector<std::pair<UD, double>>;
     struct Group {
         Tensor t;
+        bool sym = false;
         std::map<uint32_t, int> mp, mn;  // spin sets -> position
     };
     std::map<Tensor, int> ids;
@@ -326,88 +423,133 @@ std::shared_ptr<const PairPlan> make_pair_plan(const mbc_term_list &L) {
         int group;
         uint32_t dp, dn;
     };
+    auto exchanged = [](const Tensor &t) {
+        Tensor x;
+        x.reserve(t.size());
+        for (const auto &e : t) x.push_back({{e.first.second, e.first.first}, e.second});
+        std::sort(x.begin(), x.end());
+        return x;
+    };
     std::vector<std::vector<Eval>> evals((size_t)L.n_comp);
     for (int c = 0; c < L.n_comp; ++c) {
         std::map<UD, Tensor> by_sink;
         for (const auto &e : comp[(size_t)c])
-            if (e.l != 0.0) by_sink[{e.z.dp, e.z.dn}][{e.z.u, e.z.d}] += e.l;
+            if (e.l != 0.0) by_sink[{e.z.dp, e.z.dn}].push_back({{e.z.u, e.z.d}, e.l});
+        std::vector<PlanEntry>().swap(comp[(size_t)c]);
         for (auto &sk : by_sink) {
             uint32_t dp = sk.first.first, dn = sk.first.second;
-            if (np == nn) {  // of the two flavour-exchanged forms the first one seen
-                auto it = ids.find(sk.second);
-                if (it == ids.end()) {
-                    Tensor ex;
-                    for (const auto &t : sk.second) ex[{t.first.second, t.first.first}] = t.second;
-                    it = ids.find(ex);
-                    if (it != ids.end()) {
-                        sk.second.swap(ex);
-                        std::swap(dp, dn);
-                    }
-                }
+            std::sort(sk.second.begin(), sk.second.end());
+            auto it = ids.find(sk.second);
+            if (it == ids.end() && np == nn) {  // of the two flavour-exchanged forms the first one seen
+                Tensor ex = exchanged(sk.second);
+                it = ids.find(ex);
+                if (it != ids.end())
+                    std::swap(dp, dn);
+                else if (ex == sk.second)
+                    groups.push_back({{}, true, {}, {}});
             }
-            auto ins = ids.insert({sk.second, (int)groups.size()});
-            if (ins.second) groups.push_back({sk.second, {}, {}});
-            const int g = ins.first->second;
+            if (it == ids.end()) {
+                if (groups.size() == ids.size()) groups.push_back({});
+                it = ids.insert({sk.second, (int)ids.size()}).first;
+                groups.back().t = sk.second;
+            }
+            const int g = it->second;
             groups[(size_t)g].mp[dp] = groups[(size_t)g].mn[dn] = 0;
             evals[(size_t)c].push_back({g, dp, dn});
         }
     }
+    ids.clear();
     int64_t total = 0;
     const int64_t per_z = binom_p(2 * np + nn, 2 * np) * binom_p(np + 2 * nn, np);
-    for (const auto &g : groups) total += (int64_t)g.t.size() * per_z;
+    for (auto &g : groups) {
+        total += (int64_t)g.t.size() * per_z;
+        if (g.sym) {  // both orders of a pair of sets are evaluated
+            g.mp.insert(g.mn.begin(), g.mn.end());
+            g.mn = g.mp;
+        }
+    }
     if (total > kMaxPairEntries) return nullptr;
     auto P = std::make_shared<PairPlan>();
     P->np = np;
     P->nn = nn;
     // rows: block entries [pair][single] for one baryon; for two the (4-set,
-    // 2-set) keys some entry names, in rank order
-    const int64_t nset2 = binom_p(nxi, 2), wide = binom_p(nxi, 4) * nset2;
+    // 2-set) keys some entry names, 2-set slowest
+    const int64_t nset2 = binom_p(nxi, 2), nset4 = binom_p(nxi, 4), wide = nset4 * nset2;
+    const int64_t n_of[2] = {np == 2 ? wide : nset2 * nxi, nn == 2 ? wide : nset2 * nxi};
     std::vector<int32_t> row_of((size_t)((np == 2 || nn == 2) ? wide : 0), -1);
     auto full_row = [&](uint32_t pair, uint32_t single, int n) {
-        return rank_of(pair) * (n == 2 ? nset2 : nxi) + rank_of(single);
+        return n == 2 ? rank_of(single) * nset4 + rank_of(pair) : rank_of(pair) * nxi + rank_of(single);
     };
-    struct Entry {
-        uint32_t i, j;
-        double v;
-    };
-    std::vector<std::vector<Entry>> lam(groups.size());
+    // colour content of a full row: how many of its quarks have colours 0 and 1
+    std::vector<uint16_t> cls[2];
+    for (int s = 0; s < 2; ++s) {
+        const int n = s ? nn : np;
+        if (s == 1 && nn == np) {
+            cls[1] = cls[0];
+            break;
+        }
+        auto colours = [&](uint32_t m) {
+            uint16_t v = 0;
+            for (; m; m &= m - 1) {
+                const int col = (__builtin_ctz(m) / L.n_sources) % 3;
+                v = (uint16_t)(v + (col == 0 ? 16 : col == 1 ? 1 : 0));
+            }
+            return v;
+        };
+        const int64_t second = n == 2 ? nset4 : nxi;  // fastest index: 4-set or single
+        std::vector<uint16_t> slow, fast;
+        for (int64_t r = 0; r < n_of[s] / second; ++r) slow.push_back(colours(unrank(r, 2, nxi)));
+        for (int64_t r = 0; r < second; ++r) fast.push_back(colours(unrank(r, n == 2 ? 4 : 1, nxi)));
+        for (int64_t r = 0; r < n_of[s]; ++r)
+            cls[s].push_back((uint16_t)(slow[(size_t)(r / second)] + fast[(size_t)(r % second)]));
+    }
+    auto class_of = [&](uint32_t row, int side) { return cls[side][row]; };
+    std::vector<PairRows> lam(groups.size());
+    std::atomic<bool> failed{false};
 #pragma omp parallel for schedule(dynamic, 1)
     for (size_t g = 0; g < groups.size(); ++g) {
-        auto &out = lam[g];
-        out.reserve(groups[g].t.size() * (size_t)per_z);
-        // a symmetric tensor with equal sink sets: upper triangle, doubled
-        bool sym = np == nn && groups[g].mp.size() == 1 && groups[g].mn.size() == 1 &&
-                   groups[g].mp.begin()->first == groups[g].mn.begin()->first;
-        if (sym)
+        try {
+            std::vector<PairEntry> all;
+            all.reserve(groups[g].t.size() * (size_t)per_z);
+            std::map<uint32_t, std::vector<Split>> us, ds;
             for (const auto &t : groups[g].t) {
-                const auto o = groups[g].t.find({t.first.second, t.first.first});
-                sym = sym && o != groups[g].t.end() && o->second == t.second;
+                const double l = t.second;
+                auto &u = us[t.first.first], &d = ds[t.first.second];
+                if (u.empty()) u = splits_of(t.first.first, 2 * np);
+                if (d.empty()) d = splits_of(t.first.second, np);
+                for (const auto &a : u)
+                    for (const auto &e : d) {
+                        const uint32_t i = (uint32_t)full_row(a.sub, e.sub, np), j = (uint32_t)full_row(e.rest, a.rest, nn);
+                        const double v = (a.neg ^ e.neg) ? -l : l;
+                        if (!groups[g].sym || i < j)
+                            all.push_back({i, j, v});
+                        else if (i == j)
+                            all.push_back({i, j, 0.5 * v});
+                    }
             }
-        for (const auto &t : groups[g].t) {
-            const auto us = splits_of(t.first.first, 2 * np), ds = splits_of(t.first.second, np);
-            for (const auto &u : us)
-                for (const auto &d : ds) {
-                    const uint32_t i = (uint32_t)full_row(u.sub, d.sub, np), j = (uint32_t)full_row(d.rest, u.rest, nn);
-                    const double v = (u.neg ^ d.neg) ? -t.second : t.second;
-                    if (!sym)
-                        out.push_back({i, j, v});
-                    else if (i <= j)
-                        out.push_back({i, j, i == j ? v : 2.0 * v});
-                }
+            pair_rows(all, n_of[0], groups[g].sym ? 0 : n_of[1], class_of, lam[g]);
+        } catch (const std::bad_alloc &) {
+            failed = true;
         }
-        std::sort(out.begin(), out.end(), [](const Entry &a, const Entry &b) { return a.i != b.i ? a.i < b.i : a.j < b.j; });
     }
-    for (const auto &out : lam)
-        for (const auto &e : out) {
-            if (np == 2) row_of[e.i] = 0;
-            if (nn == 2) row_of[e.j] = 0;
-            P->val_fp32 = P->val_fp32 && (double)(float)e.v == e.v;
+    if (failed) throw std::bad_alloc();
+    const int n_side[2] = {np, nn};
+    for (const auto &R : lam)
+        for (int s = 0; s < 2; ++s) {
+            const auto &rows = R.rows[s];
+            for (const auto &r : rows) {
+                if (n_side[s] == 2) row_of[r.id] = 0;
+                for (int64_t e = r.e0; e < r.e1; ++e) {
+                    if (n_side[1 - s] == 2) row_of[R.col[(size_t)e]] = 0;
+                    P->val_fp32 = P->val_fp32 && (double)(float)R.val[(size_t)e] == R.val[(size_t)e];
+                }
+            }
         }
     std::vector<UD> rows2;
     for (int64_t r = 0; r < (int64_t)row_of.size(); ++r)
         if (row_of[(size_t)r] == 0) {
             row_of[(size_t)r] = P->n_rows2++;
-            rows2.push_back({unrank(r / nset2, 4, nxi), unrank(r % nset2, 2, nxi)});
+            rows2.push_back({unrank(r % nset4, 4, nxi), unrank(r / nset4, 2, nxi)});
         }
     // elements: spin values for one baryon, used two-spin sets for two
     std::map<uint32_t, int32_t> elem2;
@@ -426,19 +568,22 @@ std::shared_ptr<const PairPlan> make_pair_plan(const mbc_term_list &L) {
     P->row_ptr.push_back(0);
     for (size_t g = 0; g < groups.size(); ++g) {
         PairPlan::Group G;
-        G.row0 = (int64_t)P->row_id.size();
-        for (size_t k = 0; k < lam[g].size();) {
-            const uint32_t i = lam[g][k].i;
-            for (; k < lam[g].size() && lam[g][k].i == i; ++k) {
-                const uint32_t j = lam[g][k].j;
-                P->col.push_back(nn == 2 ? (uint32_t)row_of[j] : j);
-                P->val.push_back(lam[g][k].v);
+        const int64_t nnz0 = (int64_t)P->col.size(), rows0 = (int64_t)P->row_id.size();
+        for (int s = 0; s < 2; ++s) {
+            G.row0[s] = (int64_t)P->row_id.size();
+            for (const auto &r : lam[g].rows[s]) {
+                for (int64_t e = r.e0; e < r.e1; ++e) {
+                    const uint32_t j = lam[g].col[(size_t)e];
+                    P->col.push_back(n_side[1 - s] == 2 ? (uint32_t)row_of[j] : j);
+                    P->val.push_back(lam[g].val[(size_t)e]);
+                }
+                P->row_class.push_back(r.cls);
+                P->row_id.push_back(n_side[s] == 2 ? (uint32_t)row_of[r.id] : r.id);
+                P->row_ptr.push_back((int64_t)P->col.size());
             }
-            P->row_id.push_back(np == 2 ? (uint32_t)row_of[i] : i);
-            P->row_ptr.push_back((int64_t)P->col.size());
+            G.row1[s] = (int64_t)P->row_id.size();
         }
-        std::vector<Entry>().swap(lam[g]);
-        G.row1 = (int64_t)P->row_id.size();
+        lam[g] = PairRows();
         for (auto &m : groups[g].mp) {
             m.second = (int)G.mp.size();
             G.mp.push_back(elem(m.first, np));
@@ -449,8 +594,8 @@ std::shared_ptr<const PairPlan> make_pair_plan(const mbc_term_list &L) {
         }
         G.eval0 = P->n_evals;
         P->n_evals += (int64_t)(G.mp.size() * G.mn.size());
-        const int64_t nnz = P->row_ptr[(size_t)G.row1] - P->row_ptr[(size_t)G.row0];
-        work += nnz * (int64_t)G.mn.size() / 2 + (G.row1 - G.row0) * (int64_t)(G.mp.size() * G.mn.size());
+        work += ((int64_t)P->col.size() - nnz0) * (int64_t)G.mn.size() / 2 +
+                ((int64_t)P->row_id.size() - rows0) * (int64_t)(G.mp.size() * G.mn.size());
         P->groups.push_back(std::move(G));
     }
     if (P->n_evals > (int64_t)1 << 20) return nullptr;
@@ -464,27 +609,30 @@ std::shared_ptr<const PairPlan> make_pair_plan(const mbc_term_list &L) {
         for (const auto &e : evals[(size_t)c]) {
             const auto &g = groups[(size_t)e.group];
             const auto &G = P->groups[(size_t)e.group];
-            P->comp_eval.push_back(
-                (int32_t)(G.eval0 + (int64_t)g.mp.at(e.dp) * (int64_t)G.mn.size() + g.mn.at(e.dn)));
+            auto ev = [&](uint32_t a, uint32_t b) {
+                return (int32_t)(G.eval0 + (int64_t)g.mp.at(a) * (int64_t)G.mn.size() + g.mn.at(b));
+            };
+            P->comp_eval.push_back(ev(e.dp, e.dn));
+            if (g.sym) P->comp_eval.push_back(ev(e.dn, e.dp));
         }
         P->comp_off.push_back((int32_t)P->comp_eval.size());
     }
     P->scale = std::tgamma(np + 1.0) * std::tgamma(nn + 1.0) / pt.norm;
-    // the two-baryon products
-    const int64_t npair = nset2;
-    P->sx.reserve(12 * P->masks2.size() * rows2.size());
-    P->sys.reserve(P->sx.capacity());
-    if (L.block_size > 32768) return nullptr;
-    for (uint32_t m : P->masks2) {
-        const int s1 = __builtin_ctz(m), s2 = __builtin_ctz(m & (m - 1));
-        for (const auto &r : rows2)
-            for (const auto &a : splits_of(r.first, 2))
-                for (const auto &e : splits_of(r.second, 1)) {
-                    P->sx.push_back((uint32_t)((s1 * npair + rank_of(a.sub)) * nxi + __builtin_ctz(e.sub)));
-                    P->sys.push_back((uint16_t)(((s2 * npair + rank_of(a.rest)) * nxi + __builtin_ctz(e.rest)) |
-                                                ((a.neg ^ e.neg) ? 0x8000 : 0)));
-                }
+    // the two-baryon products, f before g: splits of the pairs' set and of the singles
+    P->prod_ops.reserve(12 * rows2.size());
+    for (size_t r = 0; r < rows2.size(); ++r) {
+        const uint32_t e = rows2[r].second;
+        if (r == 0 || e != rows2[r - 1].second) {
+            P->range_off.push_back((int32_t)r);
+            P->range_e.push_back((uint16_t)(__builtin_ctz(e) | __builtin_ctz(e & (e - 1)) << 8));
+        }
+        for (const auto &a : splits_of(rows2[r].first, 2))
+            for (uint32_t i = 0; i < 2; ++i)  // f takes single e_i, g the other: e1 | e0 is odd
+                P->prod_ops.push_back((uint32_t)(i * nset2 + rank_of(a.sub)) |
+                                      (uint32_t)((1 - i) * nset2 + rank_of(a.rest)) << 15 |
+                                      (uint32_t)(a.neg ^ (int)i) << 31);
     }
+    if (!rows2.empty()) P->range_off.push_back((int32_t)rows2.size());
     return P;
 }
 

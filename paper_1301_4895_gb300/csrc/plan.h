@@ -92,28 +92,41 @@ std::shared_ptr<const SaturatedPlan> saturated_plan(const mbc_term_list *L);
 // equal), and a component is bilinear in them,
 //   C = sum_z L(z) F(z) = sum_{i, j} P_i Lambda_ij N_j,
 // Lambda_ij = +-L(a_i + g_j, b_j + e_i) real, sparse and the same for every
-// site. Components with the same L share a group: y_j-sums of a row are formed
-// once per neutron set and multiplied by every proton set's row. Exchanging the
-// flavours maps (sigma_p, sigma_n, L(U, D)) to (sigma_n, sigma_p, L(D, U)) with
-// the same value, so only one of the two is computed, and Lambda of a single
-// symmetric component keeps its upper triangle.
+// site. Components with the same L share a group. Exchanging the flavours maps
+// (sigma_p, sigma_n, L(U, D)) to (sigma_n, sigma_p, L(D, U)) with the same
+// value, so only one of the two is computed, and a symmetric Lambda keeps each
+// pair (i, j) once, <P_a, T P_b> + <P_b, T P_a>.
+//   Every entry belongs to a row: a P row i that gathers N_b[j] (y_b = sum_j
+// Lambda_ij N_b[j], then P_a[i] y_b for every proton set a), or an N row j that
+// gathers P_a[i]. A row costs sets_p x sets_n products however few entries it
+// has, so a greedy vertex cover picks the rows (half of them in 4He with all
+// components). Lambda splits into about a thousand blocks of at most 285 rows
+// that share no column; rows are ordered by colour content (28 classes, which a
+// row's entries share), block and columns, so that the rows of neighbouring
+// warps gather the same entries.
 struct PairPlan {
     int np = 0, nn = 0;  // baryons per species: 1 or 2
-    // two-baryon rows: element m (spin set masks2[m]), row r at m * n_rows2 + r,
-    // 12 products each: x, y block entries, sign in bit 15 of ys (as Step)
+    // two-baryon products: element m (spin set masks2[m]), row r at m * n_rows2 +
+    // r. Rows with the same two singles (e0, e1) are consecutive: range k is
+    // rows [range_off[k], range_off[k + 1]) with singles range_e[k] = e0 | e1 << 8.
+    // A row is 12 products of a lower-spin block f and an upper-spin block g, the
+    // same for every spin set: prod_ops[12 r + j] = x | y << 15 | sign << 31 with
+    // x = i * n_pairs + pair for f[pair; e_i] and y likewise for g.
     std::vector<uint32_t> masks2;
     int32_t n_rows2 = 0;
-    std::vector<uint32_t> sx;
-    std::vector<uint16_t> sys;
+    std::vector<uint32_t> prod_ops;
+    std::vector<int32_t> range_off;
+    std::vector<uint16_t> range_e;
     struct Group {
-        int64_t row0, row1;             // its rows in row_id / row_ptr
+        int64_t row0[2], row1[2];       // its rows in row_id / row_ptr: P rows, N rows
         std::vector<int32_t> mp, mn;    // element indices; every (mp, mn) is evaluated
         int64_t eval0;                  // evaluation (mp_i, mn_j) at eval0 + i * mn.size() + j
     };
     std::vector<Group> groups;
-    std::vector<uint32_t> row_id;       // P row of each Lambda row
+    std::vector<uint32_t> row_id;       // P (or N) row of each Lambda row
+    std::vector<uint16_t> row_class;    // colour content of the row
     std::vector<int64_t> row_ptr;       // its entries (one more than row_id)
-    std::vector<uint32_t> col;          // N row
+    std::vector<uint32_t> col;          // N (or P) row of each entry
     std::vector<double> val;
     bool val_fp32 = true;               // every value is an FP32 number
     int64_t n_evals = 0;

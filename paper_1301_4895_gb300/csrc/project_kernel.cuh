@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(256) k_reduce_tiles_cols_mx(const float2 *__re
 template <class Tr>
 __global__ void __launch_bounds__(256) k_load_proj_blocks(const double2 *__restrict__ Pf, int64_t n_items,
                                                           int64_t item0, int W, int bs_site, int per_spin, int n_k,
-                                                          int n_mom, typename Tr::V *__restrict__ f,
+                                                          int n_mom, int T, typename Tr::V *__restrict__ f,
                                                           int32_t *__restrict__ sexp) {
     const int lane = threadIdx.x & 31;
     const int col = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(256) k_load_proj_blocks(const double2 *__restr
         const int k = psi % n_k, alpha = psi / n_k;
         const double2 *s_k = src + (int64_t)k * 2 * bs_site + alpha * per_spin + r;
         const double2 p = live ? s_k[0] : make_double2(0, 0);
-        Tr::wave_st(f, (int64_t)e * W + col, Tr::from_d(make_double2(scalbn(p.x, se), scalbn(p.y, se))));
+        Tr::wave_st(f, wave_index(e, col, T, block_size), Tr::from_d(make_double2(scalbn(p.x, se), scalbn(p.y, se))));
     }
     if (lane == 0) sexp[col] = se;
 }

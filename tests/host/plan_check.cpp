@@ -122,30 +122,48 @@ static int bad_pairs(const char *name, const mbc_term_list &L, bool expect, std:
     std::vector<cd> C, prod;
     std::vector<double> mag;
     chain(L, f, C, mag);
-    for (size_t o = 0; o < P->sx.size(); o += 12) {
-        cd v = 0;
-        for (size_t j = o; j < o + 12; ++j) {
-            const cd t = f.at(P->sx[j]) * f.at(P->sys[j] & 0x7fff);
-            v += P->sys[j] & 0x8000 ? -t : t;
-        }
-        prod.push_back(v);
+    const int64_t npair = (int64_t)L.nxi * (L.nxi - 1) / 2;
+    for (uint32_t m : P->masks2) {
+        const int s1 = __builtin_ctz(m), s2 = __builtin_ctz(m & (m - 1));
+        for (size_t k = 0; k + 1 < P->range_off.size(); ++k)
+            for (int r = P->range_off[k]; r < P->range_off[k + 1]; ++r) {
+                const int e[2] = {P->range_e[k] & 255, P->range_e[k] >> 8};
+                cd v = 0;
+                for (int j = 0; j < 12; ++j) {
+                    const uint32_t op = P->prod_ops.at((size_t)(12 * r + j)), x = op & 0x7fff, y = op >> 15 & 0x7fff;
+                    if (x >= 2 * npair || y >= 2 * npair) return 1;
+                    const cd t = f.at((size_t)((s1 * npair + x % npair) * L.nxi + e[x / npair])) *
+                                 f.at((size_t)((s2 * npair + y % npair) * L.nxi + e[y / npair]));
+                    v += op >> 31 ? -t : t;
+                }
+                prod.push_back(v);
+            }
     }
     if (prod.size() != P->masks2.size() * (size_t)P->n_rows2) return 1;
     const int64_t brows = L.block_size / L.dim_snk;
     const int64_t pr = P->p_rows(brows), nr = P->n_rows(brows);
     std::vector<cd> ev((size_t)P->n_evals, 0);
+    // rows of side 0 gather neutron products, rows of side 1 proton products
+    const std::vector<cd> &pv = P->np == 2 ? prod : f, &nv = P->nn == 2 ? prod : f;
     for (const auto &g : P->groups)
-        for (int64_t r = g.row0; r < g.row1; ++r)
-            for (size_t b = 0; b < g.mn.size(); ++b) {
-                cd y = 0;
-                for (int64_t e = P->row_ptr[(size_t)r]; e < P->row_ptr[(size_t)r + 1]; ++e) {
-                    if (P->col[(size_t)e] >= nr) return 1;
-                    y += P->val[(size_t)e] * (P->nn == 2 ? prod : f).at((size_t)(g.mn[b] * nr + P->col[(size_t)e]));
+        for (int side = 0; side < 2; ++side)
+            for (int64_t r = g.row0[side]; r < g.row1[side]; ++r) {
+                const auto &rows = side ? g.mn : g.mp, &cols = side ? g.mp : g.mn;
+                const std::vector<cd> &rv = side ? nv : pv, &cv = side ? pv : nv;
+                const int64_t n_row = side ? nr : pr, n_col = side ? pr : nr;
+                if (P->row_id[(size_t)r] >= n_row) return 1;
+                for (size_t b = 0; b < cols.size(); ++b) {
+                    cd y = 0;
+                    for (int64_t e = P->row_ptr[(size_t)r]; e < P->row_ptr[(size_t)r + 1]; ++e) {
+                        if (P->col[(size_t)e] >= n_col) return 1;
+                        y += P->val[(size_t)e] * cv.at((size_t)(cols[b] * n_col + P->col[(size_t)e]));
+                    }
+                    for (size_t a = 0; a < rows.size(); ++a) {
+                        const size_t ia = side ? b : a, ib = side ? a : b;
+                        ev.at((size_t)g.eval0 + ia * g.mn.size() + ib) +=
+                            y * rv.at((size_t)(rows[a] * n_row + P->row_id[(size_t)r]));
+                    }
                 }
-                if (P->row_id[(size_t)r] >= pr) return 1;
-                for (size_t a = 0; a < g.mp.size(); ++a)
-                    ev.at((size_t)g.eval0 + a * g.mn.size() + b) +=
-                        y * (P->np == 2 ? prod : f).at((size_t)(g.mp[a] * pr + P->row_id[(size_t)r]));
             }
     double worst = 0;
     for (int c = 0; c < L.n_comp; ++c) {
