@@ -1437,26 +1437,71 @@ mbc_status run_large(const mbc_term_list *L, const DeviceCache *c, const FieldDe
     return MBC_OK;
 }
 
-// Momentum-projected blocks: per-site blocks summed over sites with the phase
-// (FP64), then the recursion once per (slab, momentum group) item on the wave
-// kernels; a group holds the n_sinks momenta of the list's sink functions.
+// Chunks per slab of k_project: the walks of one slab's sites that keep every SM
+// busy with the fewest rounds of resident CTAs (a walk costs its sites and a few
+// more for its start and its sums).
+int project_chunks(int64_t n_slabs, int nrow, int nxi, int v3, int slots) {
+    const int64_t per = n_slabs * (nrow / 6);
+    int best = 1;
+    double best_cost = 1e300;
+    for (int n = 1; n <= 256 && n <= std::max(1, v3 / 8); ++n) {
+        const double rounds = (double)((per * n + slots - 1) / slots);
+        const double cost = rounds * ((v3 + n - 1) / n + 8.0);
+        if (cost < 0.98 * best_cost) {
+            best_cost = cost;
+            best = n;
+        }
+    }
+    return best;
+}
+
+struct ProjectSizes {
+    int n_chunks;
+    size_t tab_bytes, partial_bytes, pf_bytes, amax_bytes;
+    size_t bytes() const { return tab_bytes + partial_bytes + pf_bytes + amax_bytes; }
+};
+ProjectSizes project_sizes(const mbc_term_list *L, const FieldDesc &F, const MomDesc &M, int64_t n_slabs, int device) {
+    ProjectSizes z;
+    const int nxi = L->nxi, nrow = 3 * L->dim;
+    const int bs = (int)(L->block_size / L->n_sinks);
+    const int64_t G = (int64_t)L->dim * nxi * proj_njs(nxi);
+    z.n_chunks = project_chunks(n_slabs, nrow, nxi, F.lx * F.ly * F.lz, sm_count(device) * proj_ways(nxi));
+    z.tab_bytes = align256(((size_t)F.lx + (size_t)F.ly * F.lz) * M.n_mom * sizeof(double2));
+    z.partial_bytes = align256((size_t)n_slabs * z.n_chunks * M.n_mom * G * sizeof(double2));
+    z.pf_bytes = align256((size_t)n_slabs * M.n_mom * bs * sizeof(double2));
+    z.amax_bytes = align256((size_t)n_slabs * M.n_mom * sizeof(unsigned long long));
+    return z;
+}
+
+template <class Sum, int NXI>
+const void *project_kernel(int n_x) {
+    return n_x == 1 ? (const void *)k_project<Sum, NXI, 1>
+           : n_x == 2 ? (const void *)k_project<Sum, NXI, 2>
+                      : (const void *)k_project<Sum, NXI, 4>;
+}
+
+// Momentum-projected blocks: per-site blocks summed over sites with the phase,
+// then the recursion once per (slab, momentum group) item on the wave kernels; a
+// group holds the n_sinks momenta of the list's sink functions.
 template <class Tr>
 mbc_status run_projected(const mbc_term_list *L, const DeviceCache *c, const FieldDesc &F, const MomDesc &M,
-                         const mbc_tune *tune, int device, cudaStream_t stream, char *scratch, const double2 *phase,
-                         int li, int n_lists, int comp_max, double2 *out, int64_t n_slabs, const LargeSizes &ls) {
+                         const mbc_tune *tune, int device, cudaStream_t stream, char *scratch, int li, int n_lists,
+                         int comp_max, double2 *out, int64_t n_slabs, const LargeSizes &ls, const ProjectSizes &pz) {
     using V = typename Tr::V;
     const int nxi = L->nxi, nrow = 3 * L->dim, n_k = L->n_sinks;
     const int bs = (int)(L->block_size / n_k);  // one sink function: dirac_dim * C(nxi, 2) * nxi
     const int n_groups = M.n_mom / n_k;
-    const int v3 = F.lx * F.ly * F.lz;
-    const int tps = (v3 + 15) / 16;
-    const int64_t n_tiles = n_slabs * tps;
-    const int64_t n_out = 2LL * bs;
+    const bool mx = sizeof(V) == sizeof(float2);
+    if (nxi != 6 && nxi != 12) return MBC_ERR_UNSUPPORTED;  // 3 x Dirac dimension x sources
     char *p = scratch;
+    double2 *xtab = reinterpret_cast<double2 *>(p), *ytab = xtab + (size_t)F.lx * M.n_mom;
+    p += pz.tab_bytes;
     double2 *partial = reinterpret_cast<double2 *>(p);
-    p += align256((size_t)n_tiles * M.n_mom * n_out * sizeof(double2));
+    p += pz.partial_bytes;
     double2 *Pf = reinterpret_cast<double2 *>(p);
-    p += align256((size_t)n_slabs * M.n_mom * n_out * sizeof(double2));
+    p += pz.pf_bytes;
+    unsigned long long *amax = mx ? reinterpret_cast<unsigned long long *>(p) : nullptr;
+    p += pz.amax_bytes;
     const int W = ls.W;
     V *f = reinterpret_cast<V *>(p);  // the block of both species (u = d)
     p += align256(ls.blk_bytes);
@@ -1471,47 +1516,69 @@ mbc_status run_projected(const mbc_term_list *L, const DeviceCache *c, const Fie
     p += align256(ls.c_bytes);
     int32_t *sexp = reinterpret_cast<int32_t *>(p);
     const int nsm = sm_count(device);
-    // 1. blocks of every site, phase-weighted tile sums, reduction over tiles
-    // FP64 blocks and sums for the FP64 path, FP32 products with compensated
-    // FP32 sums for the mixed path
-    const bool mx = sizeof(V) == sizeof(float2);
-    if (mx && nxi != 6 && nxi != 12) return MBC_ERR_UNSUPPORTED;  // 3 x Dirac dimension x sources
-    const void *pkern = !mx ? (const void *)k_project_blocks
-                            : nxi == 6 ? (const void *)k_project_blocks_mx<6> : (const void *)k_project_blocks_mx<12>;
-    const size_t smem = mx ? project_smem_bytes_mx(nrow, nxi, M.n_mom) : project_smem_bytes(nrow, nxi, M.n_mom);
-    {
-        int per_sm = 0;
-        mbc_status pst = prepare_kernel(pkern, device, 512, smem, &per_sm);
-        if (pst != MBC_OK) return pst;
+    // 1. blocks of every site summed with the phases. Passes of up to kProjMoms
+    // momenta; the columns of the x table are the distinct n_x modulo Lx
+    MomDesc D;
+    std::memset(&D, 0, sizeof(D));
+    auto reduced = [&](int q) { return ((M.mom[q][0] % F.lx) + F.lx) % F.lx; };
+    auto column = [&](int n) {
+        int d = 0;
+        while (d < D.n_mom && D.mom[d][0] != n) ++d;
+        if (d == D.n_mom) D.mom[D.n_mom++][0] = n;
+        return d;
+    };
+    std::vector<ProjPass> passes;
+    for (int q0 = 0; q0 < M.n_mom; q0 += kProjMoms) {
+        ProjPass ps;
+        std::memset(&ps, 0, sizeof(ps));
+        ps.q0 = q0;
+        ps.n_mom = std::min(kProjMoms, M.n_mom - q0);
+        for (int m = 0; m < ps.n_mom; ++m) {
+            const int col = column(reduced(q0 + m));
+            int k = 0;
+            while (k < ps.n_x && ps.xcol[k] != col) ++k;
+            if (k == ps.n_x) {
+                ps.xcol[k] = col;
+                ps.trivial[k] = D.mom[col][0] == 0;
+                ++ps.n_x;
+            }
+            ps.nx_of[m] = k;
+        }
+        passes.push_back(ps);
     }
     {
-        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(n_tiles, (int64_t)nsm * 8));
-        {
-            TimedLaunch tl(stream);
-            note_launch();
-            float2 *partial_mx = reinterpret_cast<float2 *>(partial);  // the mixed path's FP32 partials
-            if (mx && nxi == 6)
-                k_project_blocks_mx<6><<<(unsigned)grid, 512, smem, stream>>>(
-                    F, M, phase, nrow, n_g2(L), bs, 1, 0, tps, n_tiles, partial_mx);
-            else if (mx)
-                k_project_blocks_mx<12><<<(unsigned)grid, 512, smem, stream>>>(
-                    F, M, phase, nrow, n_g2(L), bs, 1, 0, tps, n_tiles, partial_mx);
-            else
-                k_project_blocks<<<(unsigned)grid, 512, smem, stream>>>(F, M, phase, nrow, nxi, n_g2(L), bs,
-                                                                        (int)binom64(nxi, 2), 1, 0, tps, n_tiles,
-                                                                        partial);
-        }
-        MBC_CUDA_TRY(cudaGetLastError());
-        // thousands of outputs per slab: one thread per output, coalesced
-        const int64_t outs = n_slabs * M.n_mom * n_out;
-        const unsigned rg = (unsigned)std::max<int64_t>(1, std::min<int64_t>((outs + 255) / 256, (int64_t)nsm * 16));
+        const int64_t n = (int64_t)F.lx * D.n_mom + (int64_t)F.ly * F.lz * M.n_mom;
         note_launch();
-        if (mx)
-            k_reduce_tiles_cols_mx<<<rg, 256, 0, stream>>>(reinterpret_cast<const float2 *>(partial), n_slabs, tps,
-                                                           (int64_t)M.n_mom * n_out, Pf);
-        else
-            k_reduce_tiles_cols<<<rg, 256, 0, stream>>>(partial, n_slabs, tps, M.n_mom, (int)n_out, F.n_t, 0, 1,
-                                                        (int)n_out, Pf);
+        k_line_phases<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 4096)), 256, 0, stream>>>(
+            F, M, D, xtab, ytab);
+        MBC_CUDA_TRY(cudaGetLastError());
+    }
+    int n_dx = D.n_mom, n_g2_ = n_g2(L), n_chunks = pz.n_chunks, n_mom = M.n_mom, nrow_ = nrow;
+    int64_t n_ways = n_slabs * (nrow / 6) * n_chunks;
+    const int64_t grid = (n_ways + proj_ways(nxi) - 1) / proj_ways(nxi);
+    for (const ProjPass &ps : passes) {
+        using Sum = std::conditional_t<std::is_same<Tr, FP64Traits>::value, ProjSum64, ProjSumMx>;
+        const void *kern = nxi == 6 ? project_kernel<Sum, 6>(ps.n_x) : project_kernel<Sum, 12>(ps.n_x);
+        const size_t smem = project_smem_bytes(nrow, nxi, ps.n_mom, mx);
+        int per_sm = 0;
+        mbc_status pst = prepare_kernel(kern, device, proj_threads(nxi), smem, &per_sm);
+        if (pst != MBC_OK) return pst;
+        if (per_sm < 1) return MBC_ERR_UNSUPPORTED;
+        void *args[] = {(void *)&F,     (void *)&ps,   (void *)&xtab, (void *)&n_dx,     (void *)&ytab,   (void *)&n_mom,
+                        (void *)&nrow_, (void *)&n_g2_, (void *)&n_chunks, (void *)&n_ways, (void *)&partial};
+        TimedLaunch tl(stream);
+        note_launch();
+        MBC_CUDA_TRY(cudaLaunchKernel(kern, dim3((unsigned)grid), dim3(proj_threads(nxi)), args, smem, stream));
+    }
+    if (mx) MBC_CUDA_TRY(cudaMemsetAsync(amax, 0, (size_t)n_slabs * n_groups * sizeof(unsigned long long), stream));
+    // slabs x momenta in the grid's y, at most 65535 at a time (whole slabs)
+    const int64_t slab_step = std::max<int64_t>(1, 65535 / M.n_mom), G = (int64_t)L->dim * nxi * proj_njs(nxi);
+    for (int64_t s0 = 0; s0 < n_slabs; s0 += slab_step) {
+        const int64_t ns = std::min(slab_step, n_slabs - s0);
+        note_launch();
+        k_project_sum<<<dim3((unsigned)((bs + 255) / 256), (unsigned)(ns * M.n_mom)), 256, 0, stream>>>(
+            partial + s0 * n_chunks * M.n_mom * G, ns, n_chunks, M.n_mom, n_k, nxi, bs, Pf + s0 * M.n_mom * bs,
+            amax ? amax + s0 * n_groups : nullptr);
         MBC_CUDA_TRY(cudaGetLastError());
     }
     // 2. recursion and contraction per item, a wave of W items at a time
@@ -1520,8 +1587,9 @@ mbc_status run_projected(const mbc_term_list *L, const DeviceCache *c, const Fie
     const int T = !ls.pair ? W : mx ? kTileMx : kTile64;
     for (int64_t item0 = 0; item0 < n_items; item0 += W) {
         note_launch();
-        k_load_proj_blocks<Tr><<<(unsigned)((W + 7) / 8), 256, 0, stream>>>(Pf, n_items, item0, W, bs, per_spin, n_k,
-                                                                            M.n_mom, T, f, sexp);
+        const int64_t n_load = L->block_size * W;
+        k_load_proj_blocks<Tr><<<(unsigned)std::min<int64_t>((n_load + 255) / 256, (int64_t)nsm * 32), 256, 0, stream>>>(
+            Pf, n_items, item0, W, bs, per_spin, n_k, M.n_mom, amax, T, f, sexp);
         MBC_CUDA_TRY(cudaGetLastError());
         const V *X = f;
         mbc_status cst = ls.pair ? pair_wave<Tr>(L, c, W, f, buf[0], ppart, sexp, 1, Cb, nsm, stream)
@@ -1543,13 +1611,6 @@ mbc_status run_projected(const mbc_term_list *L, const DeviceCache *c, const Fie
         }
     }
     return MBC_OK;
-}
-
-size_t projected_bytes(const mbc_term_list *L, const MomDesc &M, int v3, int64_t n_slabs, const LargeSizes &ls) {
-    const int tps = (v3 + 15) / 16;
-    const int64_t n_out = 2 * (L->block_size / L->n_sinks);
-    return align256((size_t)n_slabs * tps * M.n_mom * n_out * sizeof(double2)) +
-           align256((size_t)n_slabs * M.n_mom * n_out * sizeof(double2)) + ls.buffers();
 }
 
 }  // namespace
@@ -1828,6 +1889,7 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
         const int64_t n_items_p = n_slabs * n_out_mom;
         std::vector<DeviceCache *> cs((size_t)n_lists, nullptr);
         std::vector<LargeSizes> lsz((size_t)n_lists);
+        std::vector<ProjectSizes> psz((size_t)n_lists);
         size_t need = 0;
         for (int li = 0; li < n_lists; ++li) {
             const mbc_term_list *L = lists[li];
@@ -1835,25 +1897,16 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
             cs[(size_t)li] = get_large_cache(L, device, opts->tune, mixed, st);
             if (!cs[(size_t)li]) return st;
             lsz[(size_t)li] = wave_sizes(L, cs[(size_t)li], opts->tune, n_items_p, mixed);
-            need = std::max(need, projected_bytes(L, M, (int)v3, n_slabs, lsz[(size_t)li]));
+            psz[(size_t)li] = project_sizes(L, F, M, n_slabs, device);
+            need = std::max(need, psz[(size_t)li].bytes() + lsz[(size_t)li].buffers());
         }
-        const size_t phase_bytes_p = align256((size_t)v3 * M.n_mom * sizeof(double2));
         void *scr_p = nullptr;
-        if ((st = scratch_get(device, stream, phase_bytes_p + need, &scr_p)) != MBC_OK) return st;
-        double2 *phase_p = reinterpret_cast<double2 *>(scr_p);
-        unsigned pg = (unsigned)std::max<int64_t>(1, std::min<int64_t>((v3 * M.n_mom + 255) / 256, 4096));
-        note_launch();
-        k_phase_table<<<pg, 256, 0, stream>>>(F, M, phase_p);
-        MBC_CUDA_TRY(cudaGetLastError());
+        if ((st = scratch_get(device, stream, need, &scr_p)) != MBC_OK) return st;
         for (int li = 0; li < n_lists; ++li) {
             if (!cs[(size_t)li]) continue;
-            char *rest_p = reinterpret_cast<char *>(scr_p) + phase_bytes_p;
-            st = mixed ? run_projected<MixedTraits>(lists[li], cs[(size_t)li], F, M, opts->tune, device, stream,
-                                                    rest_p, phase_p, li, n_lists, comp_max,
-                                                    reinterpret_cast<double2 *>(dev_out), n_slabs, lsz[(size_t)li])
-                       : run_projected<FP64Traits>(lists[li], cs[(size_t)li], F, M, opts->tune, device, stream, rest_p,
-                                                   phase_p, li, n_lists, comp_max,
-                                                   reinterpret_cast<double2 *>(dev_out), n_slabs, lsz[(size_t)li]);
+            auto run = mixed ? run_projected<MixedTraits> : run_projected<FP64Traits>;
+            st = run(lists[li], cs[(size_t)li], F, M, opts->tune, device, stream, reinterpret_cast<char *>(scr_p), li,
+                     n_lists, comp_max, reinterpret_cast<double2 *>(dev_out), n_slabs, lsz[(size_t)li], psz[(size_t)li]);
             if (st != MBC_OK) return st;
         }
     } else {

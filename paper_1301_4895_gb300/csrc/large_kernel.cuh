@@ -621,48 +621,4 @@ __global__ void k_reduce_tiles(const double2 *__restrict__ partial, int64_t n_sl
     }
 }
 
-// The same reduction for slabs with many outputs (momentum-projected blocks:
-// n_mom x 2 x block entries each, a few hundred tiles per slab): one thread
-// per output adds the slab's tiles in a fixed order, tile tl into partial sum
-// tl mod 4, then ((s0 + s1) + (s2 + s3)). Plain FP64 additions: GB300 issues
-// few FP64 operations per clock, and with hundreds of thousands of outputs a
-// compensated sum (six FP64 operations a term) costs more than the rest of
-// the step; the error of this order is below (tiles/4 + 2) ulp of the sum of
-// the magnitudes. Consecutive threads take consecutive outputs, so every load
-// of a warp is one contiguous 512 B segment. out as in k_reduce_tiles.
-__global__ void __launch_bounds__(256) k_reduce_tiles_cols(const double2 *__restrict__ partial, int64_t n_slabs,
-                                                           int tiles_per_slab, int n_mom, int n_comp, int n_t,
-                                                           int list_idx, int n_lists, int comp_stride,
-                                                           double2 *out) {
-    const int64_t per_slab = (int64_t)n_mom * n_comp;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < n_slabs * per_slab; o += stride) {
-        const int64_t slab = o / per_slab;
-        const int r = (int)(o % per_slab);
-        const double2 *p = partial + slab * tiles_per_slab * per_slab + r;
-        double2 acc[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[j] = make_double2(0.0, 0.0);
-        int tl = 0;
-        for (; tl + 4 <= tiles_per_slab; tl += 4) {
-            double2 v[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) v[j] = __ldg(p + (int64_t)(tl + j) * per_slab);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[j] = make_double2(acc[j].x + v[j].x, acc[j].y + v[j].y);
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (tl + j < tiles_per_slab) {
-                const double2 v = __ldg(p + (int64_t)(tl + j) * per_slab);
-                acc[j] = make_double2(acc[j].x + v.x, acc[j].y + v.y);
-            }
-        const int cfg = (int)(slab / n_t), tt = (int)(slab % n_t);
-        const int q = r / n_comp, c = r % n_comp;
-        const int64_t oi = ((((int64_t)cfg * n_lists + list_idx) * n_t + tt) * n_mom + q) * comp_stride + c;
-        out[oi] = make_double2((acc[0].x + acc[1].x) + (acc[2].x + acc[3].x),
-                               (acc[0].y + acc[1].y) + (acc[2].y + acc[3].y));
-    }
-}
-
 }  // namespace mbc

@@ -2,290 +2,332 @@
 // every baryon uses s(x) = exp(-2 pi i n.x / L)), then one recursion per
 // (configuration, time slice, momentum) on the summed blocks.
 //
-//   k_project_blocks   per-site antisymmetric blocks in FP64, a chunk of
-//                      entries at a time through shared memory, multiplied
-//                      by the phase and summed over the 16 sites of a tile
-//                      in a fixed order by one thread per (block, momentum,
-//                      entry) -> tile partials, reduced over tiles by
-//                      k_reduce_tiles (compensated, fixed order);
-//   k_project_blocks_mx the same with FP32 products and compensated FP32
-//                      sums (mixed precision), FP32 tile partials reduced by
-//                      k_reduce_tiles_cols_mx;
+// The block is f[alpha; i j; s] = g[alpha, i; j s] - g[alpha, j; i s] with
+// g[alpha, i; j s] = sum_c S[alpha c, i] Q[c][j, s] and Q symmetric, so the site
+// sums are taken over g (48 x 78 entries of 3 multiply-adds each, against 6 for
+// each of f's 3168) and antisymmetrised once. Momentum phases factorise over a
+// lattice line: sum_x e^{-2 pi i n_x x / L_x} g first, one sum per distinct n_x
+// (plain additions for n_x = 0), then the line's phase per momentum.
+//
+//   k_line_phases   tables of the x phases and of the lines' phases;
+//   k_project       a CTA walks a chunk of a slab's sites with the sums of 2 spins
+//                   x 12 x 78 entries of g: the line's in registers (a thread: one
+//                   (j, s), two i, both spins), the momenta's (up to 4) in shared
+//                   memory, where the tiles and diquarks of a batch of sites pass
+//                   too. 15 warps. Only chunk sums are written, where 16-site
+//                   tiles wrote 0.2-0.4 GB;
+//   k_project_sum   adds the chunks in order and antisymmetrises: f per (slab,
+//                   momentum), and in mixed precision the largest entry per item;
 //   k_load_proj_blocks copies the summed blocks of a wave of items into the
-//                      [component][item] layout of the wave kernels (MIXED:
-//                      exact power-of-two scaling per item);
-//   k_write_items      writes each item's contracted components to out.
+//                   layout of the wave kernels (MIXED: exact power-of-two scaling
+//                   per item);
+//   k_write_items   writes each item's contracted components to out.
+// FP64 throughout in the FP64 path (bound by its pipe); FP32 products with
+// compensated FP32 sums over a line and over the lines in the mixed path.
 #pragma once
 
 #include "large_kernel.cuh"
 
 namespace mbc {
 
-// Entries of a block chunk held in shared memory between the block pass and
-// the phase-sum pass; the site index is padded to 17 so that the threads of
-// the phase sum (consecutive entries) read distinct banks.
-constexpr int kProjChunk = 128;
-constexpr int kProjPad = 17;
+constexpr int kProjMoms = 4;  // momenta per pass
 
-// Shared memory of k_project_blocks for tiles of 16 sites.
-inline size_t project_smem_bytes(int nrow, int nxi, int n_mom) {
-    return sizeof(double2) * (16 * (size_t)tile_stride(nrow, nxi) + 16 * (size_t)diquark_stride(nxi) +
-                              2 * (size_t)kProjChunk * kProjPad + 16 * (size_t)n_mom);
-}
+// One pass of k_project: momenta q0 .. q0 + n_mom, their n_x among n_x distinct
+// values; x phases in column xcol[k] of the x table (trivial: all ones).
+struct ProjPass {
+    int32_t q0, n_mom, n_x;
+    int32_t nx_of[kProjMoms], xcol[kProjMoms], trivial[kProjMoms];
+};
 
-__global__ void __launch_bounds__(512) k_project_blocks(FieldDesc F, MomDesc M, const double2 *__restrict__ phase,
-                                                        int nrow, int nxi, int n_g2, int block_size, int npair,
-                                                        int need_p,
-                                                        int need_n, int tiles_per_slab, int64_t n_tiles,
-                                                        double2 *__restrict__ partial) {
-    constexpr int NS = 16;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int sst = tile_stride(nrow, nxi), qst = diquark_stride(nxi);
-    double2 *S = reinterpret_cast<double2 *>(smem_raw);  // [NS][sst]
-    double2 *Q = S + NS * sst;                    // [NS][3*nxi*nxi]
-    double2 *Fb = Q + NS * qst;                          // [2][kProjChunk][kProjPad]: block values of the chunk
-    double2 *Ph = Fb + 2 * kProjChunk * kProjPad;        // [NS][n_mom]: the tile's phases
-    const int sl = threadIdx.x % NS, slice = threadIdx.x / NS, nslice = blockDim.x / NS;
-    const int nent = nrow * nxi, nq = nxi * nxi;
-    const int v3 = F.lx * F.ly * F.lz;
-    const int n_out = 2 * block_size;  // proton block, then neutron block
-    for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        const int64_t slab = tile / tiles_per_slab;
-        const int tin = (int)(tile % tiles_per_slab);
-        const int cfg = (int)(slab / F.n_t), t = F.t0 + (int)(slab % F.n_t);
-        __syncthreads();  // shared memory of the previous tile is free
-        for (int s = threadIdx.x >> 5; s < NS; s += blockDim.x >> 5) {
-            const int lane = threadIdx.x & 31;
-            const int site = tin * NS + s;
-            const bool live = site < v3;
-            const int64_t base = cfg * F.stride_cfg + t * F.stride_t + (int64_t)site * site_elems(F);
-            for (int e = lane; e < nent; e += 32)
-                S[s * sst + e] = live ? load_prop(F, base, tile_index(F, e, nxi)) : make_double2(0, 0);
-        }
-        for (int o = threadIdx.x; o < NS * M.n_mom; o += blockDim.x) {
-            const int site = tin * NS + o / M.n_mom;
-            Ph[o] = site < v3 ? __ldg(phase + (int64_t)site * M.n_mom + o % M.n_mom) : make_double2(0, 0);
-        }
-        __syncthreads();
-        for (int e = slice; e < 3 * nq; e += nslice) {
-            const int c = e / nq, r = e % nq;
-            Q[sl * qst + e] = diquark(S + sl * sst, nxi, nxi, n_g2, c, r / nxi, r % nxi);
-        }
-        __syncthreads();
-        const int site = tin * NS + sl;
-        const bool live = site < v3;
-        const double2 *Ss = S + sl * sst;
-        const double2 *Qs = Q + sl * qst;
-        const int per_spin = npair * nxi;
-        for (int e0 = 0; e0 < block_size; e0 += kProjChunk) {
-            // 1. block values of the chunk's entries for the tile's sites
-            for (int el = slice; el < kProjChunk; el += nslice) {
-                const int e = e0 + el;
-                const bool ok = live && e < block_size;
-                const int dl = e / per_spin, r = e % per_spin;
-                const int pr = r / nxi, single = r % nxi;
-                const int i = ok ? c_pair_i[pr] : 0, j = ok ? c_pair_j[pr] : 0;
-                for (int b = 0; b < 2; ++b) {
-                    double2 f = make_double2(0, 0);
-                    if (ok && (b == 0 ? need_p : need_n)) {
-                        for (int c = 0; c < 3; ++c) {
-                            const double2 *Sr = Ss + (3 * dl + c) * nxi;
-                            if (b == 0) {
-                                f = cfma(Sr[i], Qs[(c * nxi + j) * nxi + single], f);
-                                f = cfms(Sr[j], Qs[(c * nxi + i) * nxi + single], f);
-                            } else {
-                                f = cfma(Sr[i], Qs[(c * nxi + single) * nxi + j], f);
-                                f = cfms(Sr[j], Qs[(c * nxi + single) * nxi + i], f);
-                            }
-                        }
-                    }
-                    Fb[(b * kProjChunk + el) * kProjPad + sl] = f;
-                }
-            }
-            __syncthreads();
-            // 2. phase-weighted sums over the tile's 16 sites in a fixed order,
-            //    one (block, momentum, entry) per thread
-            for (int o = threadIdx.x; o < 2 * M.n_mom * kProjChunk; o += blockDim.x) {
-                const int el = o % kProjChunk, q = (o / kProjChunk) % M.n_mom, b = o / (kProjChunk * M.n_mom);
-                const int e = e0 + el;
-                if (e >= block_size) continue;
-                const double2 *fv = Fb + (b * kProjChunk + el) * kProjPad;
-                double re = 0.0, im = 0.0;
-                for (int w = 0; w < NS; ++w) {
-                    const double2 ph = Ph[w * M.n_mom + q], f = fv[w];
-                    re = __fma_rn(ph.x, f.x, __fma_rn(-ph.y, f.y, re));
-                    im = __fma_rn(ph.x, f.y, __fma_rn(ph.y, f.x, im));
-                }
-                partial[(tile * M.n_mom + q) * (int64_t)n_out + b * block_size + e] = make_double2(re, im);
-            }
-            __syncthreads();  // the chunk's values are consumed
+// xtab[x][d] = e^{-2 pi i D.mom[d][0] x / Lx}; ytab[y + Ly z][q] = the (y, z) phase
+// of momentum q. Column d of xtab belongs to the d-th distinct n_x.
+__global__ void k_line_phases(FieldDesc F, MomDesc M, MomDesc D, double2 *xtab, double2 *ytab) {
+    const int nl = F.ly * F.lz;
+    const int64_t total = (int64_t)F.lx * D.n_mom + (int64_t)nl * M.n_mom;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        if (i < (int64_t)F.lx * D.n_mom) {
+            const int n[3] = {D.mom[i % D.n_mom][0], 0, 0};
+            xtab[i] = mom_phase(n, (int)(i / D.n_mom), 0, 0, F.lx, F.ly, F.lz);
+        } else {
+            const int64_t k = i - (int64_t)F.lx * D.n_mom;
+            const int q = (int)(k % M.n_mom), line = (int)(k / M.n_mom);
+            const int n[3] = {0, M.mom[q][1], M.mom[q][2]};
+            ytab[k] = mom_phase(n, 0, line % F.ly, line / F.ly, F.lx, F.ly, F.lz);
         }
     }
 }
 
-// Shared memory of k_project_blocks_mx (FP32 values) for tiles of 16 sites.
-inline size_t project_smem_bytes_mx(int nrow, int nxi, int n_mom) {
-    return sizeof(float2) * (16 * (size_t)tile_stride(nrow, nxi) + 16 * (size_t)diquark_stride(nxi) +
-                             2 * (size_t)kProjChunk * kProjPad + 16 * (size_t)n_mom);
+// Sums over sites: acc += ph x (or += x), and acc += ph times a line's sum.
+struct ProjSum64 {
+    using V = double2;
+    double re, im;
+    __device__ __forceinline__ void zero() { re = im = 0.0; }
+    __device__ __forceinline__ void add(V x) {
+        re += x.x;
+        im += x.y;
+    }
+    __device__ __forceinline__ void add(V ph, V x) {
+        re = __fma_rn(ph.x, x.x, __fma_rn(-ph.y, x.y, re));
+        im = __fma_rn(ph.x, x.y, __fma_rn(ph.y, x.x, im));
+    }
+    __device__ __forceinline__ V line() const { return make_double2(re, im); }
+    __device__ __forceinline__ double2 value() const { return make_double2(re, im); }
+};
+struct ProjSumMx {
+    using V = float2;
+    MixedTraits::Acc a;
+    __device__ __forceinline__ void zero() { a.zero(); }
+    __device__ __forceinline__ void add(V x) { f2_kahan(a.s, a.n, f2_pack(x.x, x.y)); }
+    __device__ __forceinline__ void add(V ph, V x) { a.add_prod(ph, x); }
+    __device__ __forceinline__ V line() const { return a.store(); }
+    __device__ __forceinline__ double2 value() const { return a.value(); }
+};
+
+// (j, s) pairs, i values per thread, threads of one way (a walk over one chunk)
+// and ways of a CTA (six walks share a CTA for 6 columns).
+__host__ __device__ constexpr int proj_njs(int nxi) { return nxi * (nxi + 1) / 2; }
+__host__ __device__ constexpr int proj_ipt(int nxi) { return nxi == 12 ? 2 : 3; }
+__host__ __device__ constexpr int proj_way(int nxi) { return nxi / proj_ipt(nxi) * proj_njs(nxi); }
+__host__ __device__ constexpr int proj_ways(int nxi) { return nxi == 12 ? 1 : 6; }
+__host__ __device__ constexpr int proj_threads(int nxi) { return (proj_way(nxi) * proj_ways(nxi) + 31) / 32 * 32; }
+// sites in shared memory at a time (a multiple of 2: 16-byte rows)
+__host__ __device__ constexpr int proj_batch(bool mixed) { return mixed ? 8 : 4; }
+
+inline size_t project_smem_bytes(int nrow, int nxi, int n_mom, bool mixed) {
+    return (size_t)2 * proj_ipt(nxi) * n_mom * proj_threads(nxi) * 16 +
+           (size_t)proj_ways(nxi) * proj_batch(mixed) * (nrow * nxi + 3 * proj_njs(nxi) + kProjMoms) * (mixed ? 8 : 16);
 }
 
-// The same projection for the mixed path: the tile, the diquark and the
-// blocks in FP32 products, the phase-weighted sum over the tile's 16 sites
-// with compensated (two-word) FP32 accumulation in the same fixed order, the
-// tile partial rounded once to FP32 for the reduction over tiles. The number of
-// quark-index columns is a template parameter (6 or 12), so the decoding
-// of an entry into (spin, pair, single) divides by constants.
-template <int NXI>
-__global__ void __launch_bounds__(512) k_project_blocks_mx(FieldDesc F, MomDesc M, const double2 *__restrict__ phase,
-                                                           int nrow, int n_g2, int block_size, int need_p, int need_n,
-                                                           int tiles_per_slab, int64_t n_tiles,
-                                                           float2 *__restrict__ partial) {
-    constexpr int NS = 16;
-    constexpr int nxi = NXI, npair = NXI * (NXI - 1) / 2;
-    using Acc = MixedTraits::Acc;
+template <class Sum, int NXI, int NX>
+__global__ void __launch_bounds__(proj_threads(NXI), 1)
+    k_project(FieldDesc F, const __grid_constant__ ProjPass ps, const double2 *__restrict__ xtab, int n_dx,
+              const double2 *__restrict__ ytab, int n_mom, int nrow, int n_g2, int n_chunks, int64_t n_ways,
+              double2 *__restrict__ partial) {
+    using V = typename Sum::V;
+    using R = decltype(V::x);
+    constexpr int NJS = proj_njs(NXI), WAY = proj_way(NXI), WAYS = proj_ways(NXI);
+    constexpr int B = proj_batch(sizeof(V) == 8);
+    constexpr int I = proj_ipt(NXI), O = 2 * I;  // outputs of a thread: (spin, i)
+    constexpr int kProjThreads = proj_threads(NXI);
+    static_assert(sizeof(Sum) == 16, "sums in shared memory");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int sst = tile_stride(nrow, nxi), qst = diquark_stride(nxi);
-    float2 *S = reinterpret_cast<float2 *>(smem_raw);  // [NS][sst]
-    float2 *Q = S + NS * sst;                   // [NS][3*nxi*nxi]
-    float2 *Fb = Q + NS * qst;                         // [2][kProjChunk][kProjPad]
-    float2 *Ph = Fb + 2 * kProjChunk * kProjPad;       // [NS][n_mom]
-    const int sl = threadIdx.x % NS, slice = threadIdx.x / NS, nslice = blockDim.x / NS;
-    const int nent = nrow * nxi, nq = nxi * nxi;
+    Sum *out = reinterpret_cast<Sum *>(smem_raw) + threadIdx.x;  // [mom][O][thread]
+    const int nent = nrow * NXI, per_way = B * (nent + 3 * NJS + kProjMoms);
+    const int wy = threadIdx.x / WAY, tw = threadIdx.x % WAY;
+    const int64_t way = (int64_t)blockIdx.x * WAYS + wy;
+    const bool active = wy < WAYS && way < n_ways;
+    V *S = reinterpret_cast<V *>(smem_raw + (size_t)O * ps.n_mom * kProjThreads * 16) +
+           (wy < WAYS ? wy : 0) * per_way;  // [B][nrow][NXI]
+    V *Q = S + B * nent;                    // [B][3][NJS]
+    V *Ph = Q + B * 3 * NJS;                // [B][n_x]
+    const int asplit = nrow / 6;            // pairs of spins
+    const int ch = (int)(way % n_chunks), a2 = (int)(way / n_chunks % asplit);
+    const int64_t slab = way / n_chunks / asplit;
     const int v3 = F.lx * F.ly * F.lz;
-    const int n_out = 2 * block_size;
-    for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        const int64_t slab = tile / tiles_per_slab;
-        const int tin = (int)(tile % tiles_per_slab);
-        const int cfg = (int)(slab / F.n_t), t = F.t0 + (int)(slab % F.n_t);
-        __syncthreads();  // shared memory of the previous tile is free
-        for (int s = threadIdx.x >> 5; s < NS; s += blockDim.x >> 5) {
-            const int lane = threadIdx.x & 31;
-            const int site = tin * NS + s;
-            const bool live = site < v3;
-            const int64_t base = cfg * F.stride_cfg + t * F.stride_t + (int64_t)site * site_elems(F);
-            for (int e = lane; e < nent; e += 32) {
-                const double2 v = live ? load_prop(F, base, tile_index(F, e, nxi)) : make_double2(0, 0);
-                S[s * sst + e] = make_float2((float)v.x, (float)v.y);
+    const int c0 = (int)((int64_t)v3 * ch / n_chunks), c1 = active ? (int)((int64_t)v3 * (ch + 1) / n_chunks) : c0;
+    const int64_t base = slab / F.n_t * F.stride_cfg + (F.t0 + slab % F.n_t) * F.stride_t;
+    const int js = tw % NJS, i0 = tw / NJS * I;
+    Sum line[NX][O];
+#pragma unroll
+    for (int k = 0; k < NX; ++k)
+#pragma unroll
+        for (int o = 0; o < O; ++o) line[k][o].zero();
+    for (int o = 0; o < O * ps.n_mom; ++o) out[o * kProjThreads].zero();
+    const int n_batches = ((v3 + n_chunks - 1) / n_chunks + B - 1) / B;  // of the longest chunk
+    // a thread loads the same entries of every batch, one batch ahead
+    constexpr int NL = (B * (NXI == 12 ? 144 : 36) + WAY - 1) / WAY;
+    int ent_b[NL], ent_off[NL];
+    V pre[NL], pre_ph{0, 0};
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+        const int e = tw + l * WAY;
+        ent_b[l] = active && e < B * nent ? e / nent : B;
+        ent_off[l] = e < B * nent ? tile_index(F, e % nent, NXI) : 0;
+    }
+    const bool ph_lane = active && tw < B * ps.n_x;
+    const int ph_b = tw / ps.n_x, ph_col = ph_lane ? ps.xcol[tw % ps.n_x] : 0;
+    auto fetch = [&](int s0) {
+#pragma unroll
+        for (int l = 0; l < NL; ++l) {
+            const int site = s0 + ent_b[l];
+            double2 v = make_double2(0.0, 0.0);
+            if (ent_b[l] < B && site < c1) v = load_prop(F, base + (int64_t)site * site_elems(F), ent_off[l]);
+            pre[l] = V{(R)v.x, (R)v.y};
+        }
+        if (ph_lane && s0 + ph_b < c1) {
+            const double2 v = __ldg(xtab + (int64_t)((s0 + ph_b) % F.lx) * n_dx + ph_col);
+            pre_ph = V{(R)v.x, (R)v.y};
+        }
+    };
+    // the thread's diquark entries: pair (x2, x3) = js, colours and sites in turn
+    int x3 = 0;
+    while ((x3 + 1) * (x3 + 2) / 2 <= js) ++x3;
+    const int x2 = js - x3 * (x3 + 1) / 2;
+    fetch(c0);
+    int x = c0 % F.lx, ln = c0 / F.lx;  // of the next site
+    for (int bt = 0; bt < n_batches; ++bt) {
+        const int s0 = c0 + bt * B;
+        __syncthreads();  // the previous batch is consumed
+#pragma unroll
+        for (int l = 0; l < NL; ++l)
+            if (ent_b[l] < B) S[tw + l * WAY] = pre[l];
+        if (ph_lane) Ph[ph_b * kProjMoms + tw % ps.n_x] = pre_ph;
+        __syncthreads();
+        fetch(s0 + B);
+        if (active)
+            for (int q = tw / NJS; q < 3 * B; q += WAY / NJS) {
+                const int c = q % 3, r2 = (c + 1) % 3 * NXI, r3 = (c + 2) % 3 * NXI;
+                V acc{0, 0};
+                for (int g = 0; g < n_g2; g += 2) {  // spins (g, g + 1): entries -1 and +1 of C gamma_5
+                    const V *lo = S + q / 3 * nent + 3 * g * NXI, *hi = lo + 3 * NXI;
+                    acc = cfms(lo[r2 + x2], hi[r3 + x3], acc);
+                    acc = cfma(lo[r3 + x2], hi[r2 + x3], acc);
+                    acc = cfma(hi[r2 + x2], lo[r3 + x3], acc);
+                    acc = cfms(hi[r3 + x2], lo[r2 + x3], acc);
+                }
+                Q[q * NJS + js] = acc;
             }
-        }
-        for (int o = threadIdx.x; o < NS * M.n_mom; o += blockDim.x) {
-            const int site = tin * NS + o / M.n_mom;
-            const double2 p = site < v3 ? __ldg(phase + (int64_t)site * M.n_mom + o % M.n_mom) : make_double2(0, 0);
-            Ph[o] = make_float2((float)p.x, (float)p.y);
-        }
         __syncthreads();
-        for (int e = slice; e < 3 * nq; e += nslice) {
-            const int c = e / nq, r = e % nq;
-            Q[sl * qst + e] = diquark(S + sl * sst, nxi, nxi, n_g2, c, r / nxi, r % nxi);
-        }
-        __syncthreads();
-        const int site = tin * NS + sl;
-        const bool live = site < v3;
-        const float2 *Ss = S + sl * sst;
-        const float2 *Qs = Q + sl * qst;
-        const int per_spin = npair * nxi;
-        for (int e0 = 0; e0 < block_size; e0 += kProjChunk) {
-            for (int el = slice; el < kProjChunk; el += nslice) {
-                const int e = e0 + el;
-                const bool ok = live && e < block_size;
-                const int dl = e / per_spin, r = e % per_spin;
-                const int pr = r / nxi, single = r % nxi;
-                const int i = ok ? c_pair_i[pr] : 0, j = ok ? c_pair_j[pr] : 0;
-                for (int b = 0; b < 2; ++b) {
-                    float2 f = make_float2(0.f, 0.f);
-                    if (ok && (b == 0 ? need_p : need_n)) {
-                        for (int c = 0; c < 3; ++c) {
-                            const float2 *Sr = Ss + (3 * dl + c) * nxi;
-                            if (b == 0) {
-                                f = cfma(Sr[i], Qs[(c * nxi + j) * nxi + single], f);
-                                f = cfms(Sr[j], Qs[(c * nxi + i) * nxi + single], f);
-                            } else {
-                                f = cfma(Sr[i], Qs[(c * nxi + single) * nxi + j], f);
-                                f = cfms(Sr[j], Qs[(c * nxi + single) * nxi + i], f);
-                            }
-                        }
+        if (!active) continue;
+        for (int b = 0; b < B && s0 + b < c1; ++b) {
+            V g[O];
+#pragma unroll
+            for (int o = 0; o < O; ++o) g[o] = V{0, 0};
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const V q = Q[(b * 3 + c) * NJS + js];
+#pragma unroll
+                for (int al = 0; al < 2; ++al) {
+                    const V *row = S + b * nent + (3 * (2 * a2 + al) + c) * NXI + i0;
+                    V r[I];
+                    if constexpr (sizeof(V) == 8 && I == 2) {  // one 16-byte broadcast (rows of 96 B, i0 even)
+                        const float4 w = *reinterpret_cast<const float4 *>(row);
+                        r[0] = V{w.x, w.y};
+                        r[1] = V{w.z, w.w};
+                    } else {
+#pragma unroll
+                        for (int o = 0; o < I; ++o) r[o] = row[o];
                     }
-                    Fb[(b * kProjChunk + el) * kProjPad + sl] = f;
+#pragma unroll
+                    for (int o = 0; o < I; ++o) g[al * I + o] = cfma(r[o], q, g[al * I + o]);
                 }
             }
-            __syncthreads();
-            for (int o = threadIdx.x; o < 2 * M.n_mom * kProjChunk; o += blockDim.x) {
-                const int el = o % kProjChunk, q = (o / kProjChunk) % M.n_mom, b = o / (kProjChunk * M.n_mom);
-                const int e = e0 + el;
-                if (e >= block_size) continue;
-                const float2 *fv = Fb + (b * kProjChunk + el) * kProjPad;
-                Acc acc;
-                acc.zero();
-                for (int w = 0; w < NS; ++w) acc.fma(Ph[w * M.n_mom + q], fv[w], 0u);
-                partial[(tile * M.n_mom + q) * (int64_t)n_out + b * block_size + e] = acc.store();
+#pragma unroll
+            for (int k = 0; k < NX; ++k)
+                if (k < ps.n_x) {
+                    if (ps.trivial[k]) {
+#pragma unroll
+                        for (int o = 0; o < O; ++o) line[k][o].add(g[o]);
+                    } else {
+                        const V ph = Ph[b * kProjMoms + k];
+#pragma unroll
+                        for (int o = 0; o < O; ++o) line[k][o].add(ph, g[o]);
+                    }
+                }
+            if (++x == F.lx || s0 + b == c1 - 1) {  // end of a line: into the momenta
+                const double2 *yt = ytab + (int64_t)ln * n_mom + ps.q0;
+                x = 0;
+                ++ln;
+#pragma unroll
+                for (int k = 0; k < NX; ++k) {
+                    for (int m = 0; m < ps.n_mom; ++m) {
+                        if (ps.nx_of[m] != k) continue;
+                        const double2 p = __ldg(yt + m);
+                        const V ph{(R)p.x, (R)p.y};
+                        Sum *t = out + m * O * kProjThreads;
+#pragma unroll
+                        for (int o = 0; o < O; ++o) {
+                            Sum v = t[o * kProjThreads];
+                            v.add(ph, line[k][o].line());
+                            t[o * kProjThreads] = v;
+                        }
+                    }
+#pragma unroll
+                    for (int o = 0; o < O; ++o) line[k][o].zero();
+                }
             }
-            __syncthreads();
         }
     }
+    if (!active) return;
+    // partial[slab][chunk][mom][(alpha, i)][js]
+    const int64_t G = (int64_t)(nrow / 3) * NXI * NJS;
+    for (int m = 0; m < ps.n_mom; ++m)
+#pragma unroll
+        for (int o = 0; o < O; ++o)
+            partial[((slab * n_chunks + ch) * n_mom + ps.q0 + m) * G +
+                    (int64_t)((2 * a2 + o / I) * NXI + i0 + o % I) * NJS + js] =
+                out[(m * O + o) * kProjThreads].value();
 }
 
-// The reduction over tiles of the mixed projection: one thread per output
-// (consecutive threads, consecutive outputs: coalesced) adds the slab's FP32
-// tile partials in tile order with a packed Kahan step on (re, im); the sum
-// goes out in FP64, Pf[slab][per_slab].
-__global__ void __launch_bounds__(256) k_reduce_tiles_cols_mx(const float2 *__restrict__ partial, int64_t n_slabs,
-                                                              int tiles_per_slab, int64_t per_slab,
-                                                              double2 *__restrict__ out) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < n_slabs * per_slab; o += stride) {
-        const int64_t slab = o / per_slab, r = o % per_slab;
-        const float2 *p = partial + slab * tiles_per_slab * per_slab + r;
-        MixedTraits::Acc acc;
-        acc.zero();
+// Pf[slab][mom][block entry]: chunk sums in order, then f = g[i; j s] - g[j; i s].
+// amax (mixed): per (slab, group of n_k momenta) the bits of the largest |re| or
+// |im| (nonnegative doubles order as integers); cleared before.
+__global__ void __launch_bounds__(256) k_project_sum(const double2 *__restrict__ partial, int64_t n_slabs, int n_chunks,
+                                                     int n_mom, int n_k, int nxi, int bs, double2 *__restrict__ Pf,
+                                                     unsigned long long *__restrict__ amax) {
+    const int njs = proj_njs(nxi), npair = nxi * (nxi - 1) / 2;
+    const int64_t G = (int64_t)bs / (npair * nxi) * nxi * njs;
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t sm = blockIdx.y;  // slab * n_mom + mom
+    double big = 0.0;
+    if (e < bs) {
+        const int al = e / (npair * nxi), pr = e / nxi % npair, s = e % nxi;
+        const int i = c_pair_i[pr], j = c_pair_j[pr];
+        const int tj = j <= s ? s * (s + 1) / 2 + j : j * (j + 1) / 2 + s;
+        const int ti = i <= s ? s * (s + 1) / 2 + i : i * (i + 1) / 2 + s;
+        const double2 *p = partial + (sm / n_mom * n_chunks * n_mom + sm % n_mom) * G;
+        const double2 *pi = p + (int64_t)(al * nxi + i) * njs + tj, *pj = p + (int64_t)(al * nxi + j) * njs + ti;
+        double2 a = make_double2(0.0, 0.0), b = a;
 #pragma unroll 4
-        for (int tl = 0; tl < tiles_per_slab; ++tl) {
-            const float2 v = __ldg(p + (int64_t)tl * per_slab);
-            f2_kahan(acc.s, acc.n, f2_pack(v.x, v.y));
+        for (int k = 0; k < n_chunks; ++k) {
+            a = cadd(a, __ldg(pi + (int64_t)k * n_mom * G));
+            b = cadd(b, __ldg(pj + (int64_t)k * n_mom * G));
         }
-        out[o] = acc.value();
+        const double2 f = csub(a, b);
+        Pf[sm * bs + e] = f;
+        big = fmax(fabs(f.x), fabs(f.y));
+    }
+    if (!amax) return;
+    for (int off = 16; off > 0; off >>= 1) big = fmax(big, __shfl_xor_sync(0xffffffffu, big, off));
+    if ((threadIdx.x & 31) == 0) {
+        const int64_t item = sm / n_mom * (n_mom / n_k) + sm % n_mom / n_k;
+        atomicMax(amax + item, (unsigned long long)__double_as_longlong(big));
     }
 }
 
-// One warp per item of the wave: summed blocks -> wave layout. An item is
-// (slab, group of n_k momenta); with n_k sink functions (Sec. 6) the sink
-// index of the item's block is psi = n_k * alpha + k, and block entry
-// (psi; pair, single) is entry (alpha; pair, single) of the block projected
-// with momentum k of the group. Pf: [slab][momentum][P block, N block] with
-// bs_site entries per block (one sink function).
+// Summed blocks of the wave's items -> wave layout (wave_index); thread = (block
+// entry, item). An item is (slab, group of n_k momenta); with n_k sink functions
+// (Sec. 6) the sink index of the item's block is psi = n_k * alpha + k, and block
+// entry (psi; pair, single) is entry (alpha; pair, single) of the block projected
+// with momentum k of the group. Pf: [slab][momentum][block] with bs_site entries
+// (one sink function).
 template <class Tr>
 __global__ void __launch_bounds__(256) k_load_proj_blocks(const double2 *__restrict__ Pf, int64_t n_items,
                                                           int64_t item0, int W, int bs_site, int per_spin, int n_k,
-                                                          int n_mom, int T, typename Tr::V *__restrict__ f,
-                                                          int32_t *__restrict__ sexp) {
-    const int lane = threadIdx.x & 31;
-    const int col = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (col >= W) return;
-    const int64_t item = item0 + col;
-    const bool live = item < n_items;
-    const int n_groups = n_mom / n_k;
-    const int64_t it = live ? item : 0;
-    const int64_t slab = it / n_groups;
-    const int q0 = (int)(it % n_groups) * n_k;
-    const double2 *src = Pf + (slab * n_mom + q0) * 2 * (int64_t)bs_site;  // n_k consecutive momenta
+                                                          int n_mom, const unsigned long long *__restrict__ amax, int T,
+                                                          typename Tr::V *__restrict__ f, int32_t *__restrict__ sexp) {
     const int block_size = bs_site * n_k;
-    int se = 0;
-    if (sizeof(typename Tr::V) == sizeof(float2)) {
-        double amax = 0.0;
-        for (int e = lane; live && e < 2 * block_size; e += 32) {
-            const double2 v = src[e];
-            amax = fmax(amax, fmax(fabs(v.x), fabs(v.y)));
+    const int n_groups = n_mom / n_k;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (int64_t)block_size * W;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int e = (int)(i % block_size), col = (int)(i / block_size);
+        const int64_t item = item0 + col;
+        double2 v = make_double2(0.0, 0.0);
+        int se = 0;
+        if (item < n_items) {
+            const int64_t slab = item / n_groups;
+            const int q0 = (int)(item % n_groups) * n_k;
+            const int psi = e / per_spin, r = e % per_spin;
+            v = Pf[(slab * n_mom + q0 + psi % n_k) * bs_site + psi / n_k * per_spin + r];
+            if (amax) {
+                const double big = __longlong_as_double((long long)amax[item]);
+                se = big > 0.0 ? -ilogb(big) : 0;
+                v = make_double2(scalbn(v.x, se), scalbn(v.y, se));
+            }
         }
-        for (int off = 16; off > 0; off >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, off));
-        se = amax > 0.0 ? -ilogb(amax) : 0;
+        Tr::wave_st(f, wave_index(e, col, T, block_size), Tr::from_d(v));
+        if (e == 0) sexp[col] = se;
     }
-    for (int e = lane; e < block_size; e += 32) {
-        const int psi = e / per_spin, r = e % per_spin;
-        const int k = psi % n_k, alpha = psi / n_k;
-        const double2 *s_k = src + (int64_t)k * 2 * bs_site + alpha * per_spin + r;
-        const double2 p = live ? s_k[0] : make_double2(0, 0);
-        Tr::wave_st(f, wave_index(e, col, T, block_size), Tr::from_d(make_double2(scalbn(p.x, se), scalbn(p.y, se))));
-    }
-    if (lane == 0) sexp[col] = se;
 }
 
 // out[cfg][list][t - t0][mom][comp_stride] = C[comp][item] for the wave's items
