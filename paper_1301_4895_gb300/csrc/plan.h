@@ -73,7 +73,7 @@ struct MinorPlan {
 // where its own operations are fewer: 3He takes 2.4 K complex multiply-adds per
 // site as minors against 8.6 K (with both blocks), 4He 0.2 K against 13.6 K,
 // while pn's 7 K products exceed its recursion's 2.7 K. Measured on GB300, 3He
-// and 4He on 16^3 x 32 sites: FP64 18.42 -> 2.69 ms, mixed 2.05 -> 0.86 ms.
+// and 4He on 16^3 x 32 sites: FP64 18.42 -> 2.14 ms, mixed 2.05 -> 0.48 ms.
 std::shared_ptr<const MinorPlan> minor_plan(const mbc_term_list *L);
 
 // Saturated form of a relativistic point-sink list: where every contracted

@@ -123,39 +123,37 @@ __global__ void __launch_bounds__(1024, 1)
         __syncthreads();
         // 2. diquark (symmetric: upper triangle) and the block of both species
         //    (Sec. 2; see small_blocks); lane = site
-        if (!P.bilinear) {
-            const int npair = NXI > 0 ? NXI * (NXI - 1) / 2 : P.npair, ntri = npair + nxi;
-            for (int e = warp; e < 3 * ntri; e += NW) {
-                const int c = e / ntri, r = e % ntri;
-                const int x2 = r < npair ? c_pair_i[r] : r - npair, x3 = r < npair ? c_pair_j[r] : r - npair;
-                V acc{0, 0};
-                for (int gg = 0; gg < P.n_g2; ++gg) {
-                    const int s2 = c_g2[gg][0], s3 = c_g2[gg][1], v = c_g2[gg][2];
-                    for (int q = 0; q < 2; ++q) {
-                        const int c2 = c_eps[c][q][0], c3 = c_eps[c][q][1], sg = c_eps[c][q][2] * v;
-                        const V a = ROW(P.s_off + (3 * s2 + c2) * nxi + x2), b = ROW(P.s_off + (3 * s3 + c3) * nxi + x3);
-                        acc = sg > 0 ? cfma(a, b, acc) : cfms(a, b, acc);
-                    }
+        const int npair = NXI > 0 ? NXI * (NXI - 1) / 2 : P.npair, ntri = npair + nxi;
+        for (int e = warp; e < 3 * ntri; e += NW) {
+            const int c = e / ntri, r = e % ntri;
+            const int x2 = r < npair ? c_pair_i[r] : r - npair, x3 = r < npair ? c_pair_j[r] : r - npair;
+            V acc{0, 0};
+            for (int gg = 0; gg < P.n_g2; ++gg) {
+                const int s2 = c_g2[gg][0], s3 = c_g2[gg][1], v = c_g2[gg][2];
+                for (int q = 0; q < 2; ++q) {
+                    const int c2 = c_eps[c][q][0], c3 = c_eps[c][q][1], sg = c_eps[c][q][2] * v;
+                    const V a = ROW(P.s_off + (3 * s2 + c2) * nxi + x2), b = ROW(P.s_off + (3 * s3 + c3) * nxi + x3);
+                    acc = sg > 0 ? cfma(a, b, acc) : cfms(a, b, acc);
                 }
-                ROW(P.q_off + (c * nxi + x2) * nxi + x3) = acc;
-                ROW(P.q_off + (c * nxi + x3) * nxi + x2) = acc;
             }
-            __syncthreads();
-            const int per_spin = npair * nxi;
-            for (int e = warp; e < P.block_size; e += NW) {
-                const int dl = e / per_spin, r = e % per_spin;
-                const int pr = r / nxi, single = r % nxi;
-                const int i = c_pair_i[pr], j = c_pair_j[pr];
-                V acc{0, 0};
-                for (int c = 0; c < 3; ++c) {
-                    const int sr = P.s_off + (3 * dl + c) * nxi;
-                    acc = cfma(ROW(sr + i), ROW(P.q_off + (c * nxi + j) * nxi + single), acc);
-                    acc = cfms(ROW(sr + j), ROW(P.q_off + (c * nxi + i) * nxi + single), acc);
-                }
-                ROW(P.blk_off + e) = acc;
-            }
-            __syncthreads();
+            ROW(P.q_off + (c * nxi + x2) * nxi + x3) = acc;
+            ROW(P.q_off + (c * nxi + x3) * nxi + x2) = acc;
         }
+        __syncthreads();
+        const int per_spin = npair * nxi;
+        for (int e = warp; e < P.block_size; e += NW) {
+            const int dl = e / per_spin, r = e % per_spin;
+            const int pr = r / nxi, single = r % nxi;
+            const int i = c_pair_i[pr], j = c_pair_j[pr];
+            V acc{0, 0};
+            for (int c = 0; c < 3; ++c) {
+                const int sr = P.s_off + (3 * dl + c) * nxi;
+                acc = cfma(ROW(sr + i), ROW(P.q_off + (c * nxi + j) * nxi + single), acc);
+                acc = cfms(ROW(sr + j), ROW(P.q_off + (c * nxi + i) * nxi + single), acc);
+            }
+            ROW(P.blk_off + e) = acc;
+        }
+        __syncthreads();
         for (int li = li0; li < l_end; ++li) {
             const SmallPlan &P = B.plan[li];
             double2 *partial = partial_base + B.partial_off[li];
@@ -261,43 +259,11 @@ __global__ void __launch_bounds__(1024, 1)
             //    32 sites of the tile by a fixed xor tree
             const int site = site0 + lane;
             const bool live = site < V3;
-            // minor form: each run's products are split over several warps, the
-            // compensated partials go through the partial rows (n_runs <= 32)
-            const int n_runs = P.bilinear ? P.run_off[P.n_comp] : 0;
-            const int rparts = n_runs > 0 ? max(1, min(NW, 32) / n_runs) : 1;
-            if (P.bilinear) {
-                for (int u = warp; u < n_runs * rparts; u += NW) {
-                    const int r = u / rparts, part = u % rparts;
-                    const int t0 = P.term_off[r], nt = P.term_off[r + 1] - t0;
-                    typename Tr::Acc acc;
-                    acc.zero();
-                    for (int e = t0 + part * nt / rparts; e < t0 + (part + 1) * nt / rparts; ++e) {
-                        const uint32_t op = __ldg(P.terms + e);
-                        acc.fma(ROW(op & 0xffffu), ROW((op >> 16) & 0x7fffu), op & 0x80000000u);
-                    }
-                    ROW(P.part_off + 2 * u) = f2_unpack(acc.s);
-                    ROW(P.part_off + 2 * u + 1) = f2_unpack(acc.n);
-                }
-                __syncthreads();
-            }
             for (int c = warp; c < P.n_comp; c += NW) {
                 const int ue = -__ldg(P.comp_deg + c) * sexp_s[lane];
                 const double inv_norm = __ldg(P.comp_inv_norm + c);
                 double re = 0.0, im = 0.0;
-                if (P.bilinear)
-                    for (int r = P.run_off[c]; r < P.run_off[c + 1]; ++r) {
-                        typename Tr::Acc a;
-                        a.zero();
-                        for (int u = r * rparts; u < (r + 1) * rparts; ++u) {
-                            const V r0 = ROW(P.part_off + 2 * u), r1 = ROW(P.part_off + 2 * u + 1);
-                            a.add(r0.x, r1.x, r0.y, r1.y);
-                        }
-                        const double2 v = a.value();
-                        const double coef = __ldg(P.run_coef + r);
-                        re = __fma_rn(coef, v.x, re);
-                        im = __fma_rn(coef, v.y, im);
-                    }
-                for (int64_t e = P.bilinear ? 0 : P.fin_off[c]; e < (P.bilinear ? 0 : P.fin_off[c + 1]); ++e) {
+                for (int64_t e = P.fin_off[c]; e < P.fin_off[c + 1]; ++e) {
                     const double2 f = Tr::to_d(ROW(__ldg(P.fin_z + e)));
                     const double l = __ldg(P.fin_l + e);
                     re = __fma_rn(l, f.x, re);
