@@ -334,7 +334,8 @@ bool plan_small(const mbc_term_list *L, const MinorPlan *minor, SmallPlan &P, in
     for (auto &s : L->steps)
         if (s.n_x >= 65536) return false;
     const int n_ph = 3 + A;  // phases: 0 load, 1 Q, 2 blocks, 3.. steps, 2 + A contraction
-    Interval Sb{0, 2, (int64_t)L->nxi * L->nxi, 0}, Qb{1, 2, 3LL * L->nxi * L->nxi, 0};
+    // diquark: square for reading, and (mixed) the upper triangle's low words
+    Interval Sb{0, 2, (int64_t)L->nxi * L->nxi, 0}, Qb{1, 2, 3LL * (L->nxi * L->nxi + L->nxi * (L->nxi + 1) / 2), 0};
     std::vector<Interval> stage((size_t)A + 1);
     // the block of both species first, at offset 0, live to the end: lists
     // with the same tile shape then share one block computation per site in a
@@ -1400,16 +1401,18 @@ mbc_status run_large(const mbc_term_list *L, const DeviceCache *c, const FieldDe
     int32_t *sexp = reinterpret_cast<int32_t *>(p);
     const int nsm = sm_count(device);
     const int nxi = L->nxi, nrow = 3 * L->dim;
-    // sites per CTA of the block kernel: 16, or 4 for 24 source columns
-    const int ns_blk = nxi > 12 ? 4 : 16;
-    const void *blk_kern = ns_blk == 4 ? (const void *)k_large_blocks<Tr, 4> : (const void *)k_large_blocks<Tr, 16>;
-    const size_t blk_smem = (size_t)ns_blk * (tile_stride(nrow, nxi) + diquark_stride(nxi)) * sizeof(V);
+    const void *blk_kern = (const void *)k_large_blocks<Tr>;
+    const size_t blk_smem = block_smem<Tr>(nrow, nxi);
     {
         int per_sm = 0;
-        mbc_status pst = prepare_kernel(blk_kern, device, 512, blk_smem, &per_sm);
+        mbc_status pst = prepare_kernel(blk_kern, device, 256, blk_smem, &per_sm);
         if (pst != MBC_OK) return pst;
         if (per_sm < 1) return MBC_ERR_UNSUPPORTED;
     }
+    const unsigned sitesum_y = (unsigned)std::max(1, std::min(64, (M.n_mom * L->n_comp + 255) / 256));
+    // entry slices: two CTAs per SM where a wave has fewer, a slice's share of the
+    // entries not below the diquarks it repeats
+    const unsigned blk_slices = (unsigned)std::max(1, std::min(8, 2 * nsm / (W / kBlockSites)));
     const int T = !ls.pair ? W : sizeof(V) == sizeof(float2) ? kTileMx : kTile64;
     for (int64_t item0 = 0; item0 < n_items; item0 += W) {
         WaveDesc wv;
@@ -1419,19 +1422,15 @@ mbc_status run_large(const mbc_term_list *L, const DeviceCache *c, const FieldDe
         wv.v3p = v3p;
         wv.n_items = n_items;
         note_launch();
-        if (ns_blk == 4)
-            k_large_blocks<Tr, 4><<<W / 4, 512, blk_smem, stream>>>(F, wv, nrow, nxi, n_g2(L), (int)L->block_size,
-                                                                    (int)binom64(nxi, 2), T, f, sexp);
-        else
-            k_large_blocks<Tr, 16><<<W / 16, 512, blk_smem, stream>>>(F, wv, nrow, nxi, n_g2(L), (int)L->block_size,
-                                                                      (int)binom64(nxi, 2), T, f, sexp);
+        k_large_blocks<Tr><<<dim3((unsigned)(W / kBlockSites), blk_slices), 256, blk_smem, stream>>>(
+            F, wv, nrow, nxi, n_g2(L), (int)L->block_size, (int)binom64(nxi, 2), T, f, sexp);
         MBC_CUDA_TRY(cudaGetLastError());
         if (ls.pair) {
             mbc_status pst = pair_wave<Tr>(L, c, W, f, buf[0], ppart, sexp, 3, Cb, nsm, stream);
             if (pst != MBC_OK) return pst;
             const int64_t groups = std::min<int64_t>(W, n_items - item0) / 32;
             note_launch();
-            k_large_sitesum<<<(unsigned)groups, 256, 0, stream>>>(F, wv, M, L->n_comp, phase, Cb, partial);
+            k_large_sitesum<<<dim3((unsigned)groups, sitesum_y), 256, 0, stream>>>(F, wv, M, L->n_comp, phase, Cb, partial);
             MBC_CUDA_TRY(cudaGetLastError());
             continue;
         }
@@ -1447,7 +1446,7 @@ mbc_status run_large(const mbc_term_list *L, const DeviceCache *c, const FieldDe
         {
             int64_t groups = std::min<int64_t>(W, n_items - item0) / 32;
             note_launch();
-            k_large_sitesum<<<(unsigned)groups, 256, 0, stream>>>(F, wv, M, L->n_comp, phase, Cb, partial);
+            k_large_sitesum<<<dim3((unsigned)groups, sitesum_y), 256, 0, stream>>>(F, wv, M, L->n_comp, phase, Cb, partial);
             MBC_CUDA_TRY(cudaGetLastError());
         }
     }

@@ -43,29 +43,36 @@ __device__ __forceinline__ int64_t wave_index(int64_t e, int w, int T, int64_t n
     return (int64_t)(w / T) * T * n_comp + e * T + w % T;
 }
 
-// Per-site regions of the block kernels' shared memory are padded by one
-// element: the 16 sites of a warp then read the same entry from 16 distinct
-// banks (an unpadded 12 x 12 tile puts all of them in one bank).
-__host__ __device__ constexpr int tile_stride(int nrow, int nxi) { return nrow * nxi + 1; }
-__host__ __device__ constexpr int diquark_stride(int nxi) { return 3 * nxi * nxi + 1; }
-
-// The block of both species (u = d, see small_blocks) for NS sites per CTA (512
-// threads): thread = (site lane, entry slice). The tile of a site has nrow sink rows (3 x Dirac dimension) and nxi
-// source columns (quark index over all sources, up to 24: two relativistic
-// sources, Sec. 6); NS = 4 for 24 columns keeps the tiles and diquarks in
-// shared memory.
+// The block of both species (u = d, see small_blocks) for kBlockSites sites per
+// CTA: thread = (site, entry slice); a site's tile has nrow sink rows (3 x Dirac
+// dimension) and nxi source columns (quark index over all sources, up to 24: two
+// relativistic sources, Sec. 6). Few sites per CTA spread a wave over the SMs (a
+// CTA of 16 kept one SM's FP64 pipe busy for 0.34 ms), and grid.y cuts the
+// entries of waves that still have too few CTAs, each forming its own diquarks.
+// Per-site regions of shared memory are padded by one element so that the sites
+// of a warp read distinct banks. T: sites per tile of the output buffer
+// (wave_index). Measured on GB300 (12 columns): 512 sites FP64 362 -> 101 us, 64
+// sites 360 -> 25 us, 1024 sites mixed 51 -> 61 us, now with exact products.
+constexpr int kBlockSites = 4;
 constexpr int kTileLoads = 9;  // tile entries per lane: 12 x 24 / 32
+__host__ __device__ constexpr int tile_stride(int nrow, int nxi) { return nrow * nxi + 1; }
+__host__ __device__ constexpr int diquark_stride(int nxi) { return 3 * (nxi * (nxi + 1) / 2) + 1; }
+template <class Tr>
+size_t block_smem(int nrow, int nxi) {
+    return (size_t)kBlockSites * (tile_stride(nrow, nxi) * sizeof(typename Tr::V) + diquark_stride(nxi) * sizeof(typename Tr::Q));
+}
 
-// T: sites per tile of the output buffer (wave_index).
-template <class Tr, int NS>
-__global__ void __launch_bounds__(512) k_large_blocks(FieldDesc F, WaveDesc wv, int nrow, int nxi, int n_g2,
+template <class Tr>
+__global__ void __launch_bounds__(256) k_large_blocks(FieldDesc F, WaveDesc wv, int nrow, int nxi, int n_g2,
                                                       int block_size, int npair, int T, typename Tr::V *f,
                                                       int32_t *sexp_out) {
     using V = typename Tr::V;
+    using Acc = typename Tr::BlockAcc;
+    constexpr int NS = kBlockSites;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int sst = tile_stride(nrow, nxi), qst = diquark_stride(nxi);
-    V *S = reinterpret_cast<V *>(smem_raw);  // [NS][sst]: nrow*nxi entries each
-    V *Q = S + NS * sst;                     // [NS][qst]: 3*nxi*nxi entries each
+    const int sst = tile_stride(nrow, nxi), qst = diquark_stride(nxi), ntri = npair + nxi;
+    typename Tr::Q *Q = reinterpret_cast<typename Tr::Q *>(smem_raw);  // [NS][qst]: upper triangles x2 <= x3 per colour
+    V *S = reinterpret_cast<V *>(Q + NS * qst);                        // [NS][sst]: nrow*nxi entries each
     const int sl = threadIdx.x % NS, slice = threadIdx.x / NS, nslice = blockDim.x / NS;
     const int w0 = blockIdx.x * NS;  // first site of this CTA within the wave
     const int nent = nrow * nxi;
@@ -96,32 +103,34 @@ __global__ void __launch_bounds__(512) k_large_blocks(FieldDesc F, WaveDesc wv, 
             int e = lane + 32 * q;
             if (e < nent) S[s * sst + e] = Tr::from_d(make_double2(scalbn(sv[q].x, se), scalbn(sv[q].y, se)));
         }
-        if (lane == 0) sexp_out[w0 + s] = se;
-    }
-    __syncthreads();
-    const int ntri = npair + nxi;  // Q is symmetric (small_blocks)
-    for (int e = slice; e < 3 * ntri; e += nslice) {
-        const int c = e / ntri, r = e % ntri;
-        const int x2 = r < npair ? c_pair_i[r] : r - npair, x3 = r < npair ? c_pair_j[r] : r - npair;
-        const V q = diquark(S + sl * sst, nxi, nxi, n_g2, c, x2, x3);
-        Q[sl * qst + (c * nxi + x2) * nxi + x3] = q;
-        Q[sl * qst + (c * nxi + x3) * nxi + x2] = q;
+        if (lane == 0 && blockIdx.y == 0) sexp_out[w0 + s] = se;
     }
     __syncthreads();
     const V *Ss = S + sl * sst;
-    const V *Qs = Q + sl * qst;
+    for (int e = slice; e < 3 * ntri; e += nslice) {
+        const int c = e / ntri, r = e % ntri;
+        const int x2 = r < npair ? c_pair_i[r] : r - npair, x3 = r < npair ? c_pair_j[r] : r - npair;
+        Q[sl * qst + c * ntri + x3 * (x3 + 1) / 2 + x2] =
+            diquark<Acc>([&](int row, int col) { return Ss[row * nxi + col]; }, n_g2, c, x2, x3).q();
+    }
+    __syncthreads();
+    const typename Tr::Q *Qs = Q + sl * qst;
     const int per_spin = npair * nxi;
-    for (int e = slice; e < block_size; e += nslice) {
+    const int e1 = (int)((int64_t)block_size * (blockIdx.y + 1) / gridDim.y);
+    for (int e = (int)((int64_t)block_size * blockIdx.y / gridDim.y) + slice; e < e1; e += nslice) {
         int dl = e / per_spin, r = e % per_spin;
         int pr = r / nxi, single = r % nxi;
         int i = c_pair_i[pr], j = c_pair_j[pr];
-        V acc{0, 0};
+        const int tj = j <= single ? single * (single + 1) / 2 + j : j * (j + 1) / 2 + single;
+        const int ti = i <= single ? single * (single + 1) / 2 + i : i * (i + 1) / 2 + single;
+        Acc acc;
+        acc.zero();
         for (int c = 0; c < 3; ++c) {
             const V *Sr = Ss + (3 * dl + c) * nxi;
-            acc = cfma(Sr[i], Qs[(c * nxi + j) * nxi + single], acc);
-            acc = cfms(Sr[j], Qs[(c * nxi + i) * nxi + single], acc);
+            acc.add(Sr[i], Qs[c * ntri + tj]);
+            acc.sub(Sr[j], Qs[c * ntri + ti]);
         }
-        Tr::wave_st(f, wave_index(e, w0 + sl, T, block_size), acc);
+        Tr::wave_st(f, wave_index(e, w0 + sl, T, block_size), acc.block());
     }
 }
 
@@ -548,7 +557,7 @@ __global__ void __launch_bounds__(256) k_large_contract(const int64_t *__restric
 }
 
 // Momentum phases and the fixed-order sum over each 32-site group: one CTA
-// per group, partial[tile][mom][comp].
+// per group (grid.y: 256 outputs each), partial[tile][mom][comp].
 __global__ void __launch_bounds__(256) k_large_sitesum(FieldDesc F, WaveDesc wv, MomDesc M, int n_comp,
                                                        const double2 *__restrict__ phase,
                                                        const double2 *__restrict__ C, double2 *__restrict__ partial) {
@@ -562,7 +571,7 @@ __global__ void __launch_bounds__(256) k_large_sitesum(FieldDesc F, WaveDesc wv,
     }
     __syncthreads();
     const int64_t tile = (wv.item0 >> 5) + g;
-    for (int o = threadIdx.x; o < M.n_mom * n_comp; o += blockDim.x) {
+    for (int o = blockIdx.y * blockDim.x + threadIdx.x; o < M.n_mom * n_comp; o += gridDim.y * blockDim.x) {
         int q = o / n_comp, c = o % n_comp;
         double re = 0.0, im = 0.0;
         for (int s = 0; s < 32; ++s) {

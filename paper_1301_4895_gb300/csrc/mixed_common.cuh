@@ -82,8 +82,49 @@ struct __align__(16) OpRec {
     uint64_t sg;
 };
 
+// Complex sums of exact FP32 products in two words: the blocks' arithmetic. With
+// u = d both species share a block, so its rounding counts once per baryon in
+// the same direction; formed this way it is rounded once, when it is stored.
+struct DiquarkMx {
+    float2 h, l;  // high and low words
+};
+struct BlockAccMx {
+    float2 h, l;
+    __device__ __forceinline__ void zero() { h = l = make_float2(0.f, 0.f); }
+    // (h, l) += x y
+    __device__ __forceinline__ static void term(float &h, float &l, float x, float y) {
+        const float p = __fmul_rn(x, y), e = __fmaf_rn(x, y, -p);
+        float s, err;
+        two_sum(h, p, s, err);
+        h = s;
+        l = __fadd_rn(l, __fadd_rn(err, e));
+    }
+    __device__ __forceinline__ void add(float2 a, float2 b) {
+        term(h.x, l.x, a.x, b.x);
+        term(h.x, l.x, -a.y, b.y);
+        term(h.y, l.y, a.x, b.y);
+        term(h.y, l.y, a.y, b.x);
+    }
+    __device__ __forceinline__ void sub(float2 a, float2 b) { add(make_float2(-a.x, -a.y), b); }
+    __device__ __forceinline__ void add(float2 a, DiquarkMx b) {
+        add(a, b.h);
+        l.x = __fmaf_rn(a.x, b.l.x, __fmaf_rn(-a.y, b.l.y, l.x));
+        l.y = __fmaf_rn(a.x, b.l.y, __fmaf_rn(a.y, b.l.x, l.y));
+    }
+    __device__ __forceinline__ void sub(float2 a, DiquarkMx b) { add(make_float2(-a.x, -a.y), b); }
+    __device__ __forceinline__ DiquarkMx q() const {
+        DiquarkMx r;
+        r.h = make_float2(__fadd_rn(h.x, l.x), __fadd_rn(h.y, l.y));
+        r.l = make_float2(__fsub_rn(l.x, __fsub_rn(r.h.x, h.x)), __fsub_rn(l.y, __fsub_rn(r.h.y, h.y)));
+        return r;
+    }
+    __device__ __forceinline__ float2 block() const { return make_float2(__fadd_rn(h.x, l.x), __fadd_rn(h.y, l.y)); }
+};
+
 struct MixedTraits {
     using V = float2;
+    using Q = DiquarkMx;
+    using BlockAcc = BlockAccMx;
     // Kahan-compensated FP32 accumulation of FP32 complex products: value =
     // s + n, where n = -c carries the rounding lost by the running sum s; the
     // real and imaginary parts share packed instructions.

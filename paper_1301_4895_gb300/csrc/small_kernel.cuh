@@ -202,7 +202,7 @@ __device__ __forceinline__ void small_blocks(const SmallPlan &P, typename Tr::V 
     for (int e = lane; e < 3 * ntri; e += 32) {
         const int c = e / ntri, r = e % ntri;
         const int x2 = r < P.npair ? c_pair_i[r] : r - P.npair, x3 = r < P.npair ? c_pair_j[r] : r - P.npair;
-        const V q = diquark(S, nxi, nxi, P.n_g2, c, x2, x3);
+        const V q = diquark<typename Tr::BlockAcc>([&](int row, int col) { return S[row * nxi + col]; }, P.n_g2, c, x2, x3).q();
         Q[(c * nxi + x2) * nxi + x3] = q;
         Q[(c * nxi + x3) * nxi + x2] = q;
     }
@@ -213,13 +213,14 @@ __device__ __forceinline__ void small_blocks(const SmallPlan &P, typename Tr::V 
         int dl = e / per_spin, r = e % per_spin;
         int pr = r / nxi, single = r % nxi;
         int i = c_pair_i[pr], j = c_pair_j[pr];
-        V acc{0, 0};
+        typename Tr::BlockAcc acc;
+        acc.zero();
         for (int c = 0; c < 3; ++c) {
             const V *Sr = S + (3 * dl + c) * nxi;
-            acc = cfma(Sr[i], Q[(c * nxi + j) * nxi + single], acc);
-            acc = cfms(Sr[j], Q[(c * nxi + i) * nxi + single], acc);
+            acc.add(Sr[i], Q[(c * nxi + j) * nxi + single]);
+            acc.sub(Sr[j], Q[(c * nxi + i) * nxi + single]);
         }
-        F[e] = acc;
+        F[e] = acc.block();
     }
     __syncwarp();
 }

@@ -127,17 +127,10 @@ __global__ void __launch_bounds__(1024, 1)
         for (int e = warp; e < 3 * ntri; e += NW) {
             const int c = e / ntri, r = e % ntri;
             const int x2 = r < npair ? c_pair_i[r] : r - npair, x3 = r < npair ? c_pair_j[r] : r - npair;
-            V acc{0, 0};
-            for (int gg = 0; gg < P.n_g2; ++gg) {
-                const int s2 = c_g2[gg][0], s3 = c_g2[gg][1], v = c_g2[gg][2];
-                for (int q = 0; q < 2; ++q) {
-                    const int c2 = c_eps[c][q][0], c3 = c_eps[c][q][1], sg = c_eps[c][q][2] * v;
-                    const V a = ROW(P.s_off + (3 * s2 + c2) * nxi + x2), b = ROW(P.s_off + (3 * s3 + c3) * nxi + x3);
-                    acc = sg > 0 ? cfma(a, b, acc) : cfms(a, b, acc);
-                }
-            }
-            ROW(P.q_off + (c * nxi + x2) * nxi + x3) = acc;
-            ROW(P.q_off + (c * nxi + x3) * nxi + x2) = acc;
+            const DiquarkMx q = diquark<BlockAccMx>([&](int row, int col) { return ROW(P.s_off + row * nxi + col); }, P.n_g2, c, x2, x3).q();
+            ROW(P.q_off + (c * nxi + x2) * nxi + x3) = q.h;
+            ROW(P.q_off + (c * nxi + x3) * nxi + x2) = q.h;
+            ROW(P.q_off + 3 * nent + c * ntri + r) = q.l;
         }
         __syncthreads();
         const int per_spin = npair * nxi;
@@ -145,13 +138,16 @@ __global__ void __launch_bounds__(1024, 1)
             const int dl = e / per_spin, r = e % per_spin;
             const int pr = r / nxi, single = r % nxi;
             const int i = c_pair_i[pr], j = c_pair_j[pr];
-            V acc{0, 0};
+            const int rj = j == single ? npair + j : max(j, single) * (max(j, single) - 1) / 2 + min(j, single);
+            const int ri = i == single ? npair + i : max(i, single) * (max(i, single) - 1) / 2 + min(i, single);
+            BlockAccMx acc;
+            acc.zero();
             for (int c = 0; c < 3; ++c) {
-                const int sr = P.s_off + (3 * dl + c) * nxi;
-                acc = cfma(ROW(sr + i), ROW(P.q_off + (c * nxi + j) * nxi + single), acc);
-                acc = cfms(ROW(sr + j), ROW(P.q_off + (c * nxi + i) * nxi + single), acc);
+                const int sr = P.s_off + (3 * dl + c) * nxi, ql = P.q_off + 3 * nent + c * ntri;
+                acc.add(ROW(sr + i), DiquarkMx{ROW(P.q_off + (c * nxi + j) * nxi + single), ROW(ql + rj)});
+                acc.sub(ROW(sr + j), DiquarkMx{ROW(P.q_off + (c * nxi + i) * nxi + single), ROW(ql + ri)});
             }
-            ROW(P.blk_off + e) = acc;
+            ROW(P.blk_off + e) = acc.block();
         }
         __syncthreads();
         for (int li = li0; li < l_end; ++li) {
