@@ -648,6 +648,9 @@ PairLayout pair_layout(const PairPlan &P, const int shape[2], int n_sm) {
                     ++pk.n_rows;
                     acc += cost(e1 - e0, 1, tr, tg);
                 }
+                // longest rows first: the warps' rows of a round are then of one length
+                std::stable_sort(Q.rows.begin() + pk.row0, Q.rows.begin() + pk.row0 + pk.n_rows,
+                                 [](const PairRow &a, const PairRow &b) { return a.n > b.n; });
                 Q.packs.push_back(pk);
                 if (acc >= target || r >= g.row1[s]) {
                     cut[s].push_back((int32_t)Q.packs.size());
@@ -1363,7 +1366,9 @@ mbc_status pair_wave(const mbc_term_list *L, const DeviceCache *c, int W, const 
         const void *kern = shape == 0   ? (const void *)k_pair<T, 1, 1, kW[0]>
                            : shape == 1 ? (const void *)k_pair<T, 2, 2, kW[1]>
                                         : (const void *)k_pair<T, 6, 2, kW[2]>;
-        const size_t smem = shape == 0 ? pair_smem<1, kW[0]>() : shape == 1 ? pair_smem<2, kW[1]>() : pair_smem<2, kW[2]>();
+        const size_t smem = shape == 0   ? pair_smem<T, 1, kW[0]>()
+                            : shape == 1 ? pair_smem<T, 2, kW[1]>()
+                                         : pair_smem<T, 2, kW[2]>();
         int per_sm = 0;
         mbc_status st = prepare_kernel(kern, c->device, threads, smem, &per_sm);
         if (st != MBC_OK) return st;

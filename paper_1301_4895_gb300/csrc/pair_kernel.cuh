@@ -25,7 +25,7 @@
 // for the products and 0.31 M real-complex ones; 531 M for all 1296): one
 // component mixed, 16^3 x 4, 125.2 -> 9.3 ms (12.1 with L2 gathers, rows in rank
 // order); all, FP64, 64 sites, 233.7 -> 20.4 ms (26.9); all, mixed, 512 sites,
-// 227.7 -> 25.5 ms (70.8).
+// 227.7 -> 24.2 ms (70.8).
 #pragma once
 
 #include "large_kernel.cuh"
@@ -149,7 +149,19 @@ struct Pair64 {
         }
         __device__ __forceinline__ void values(double2 (&v)[1]) const { v[0] = a.value(); }
     };
-    __device__ __forceinline__ static double factor(double v) { return v; }
+    // record of an entry: place of the gathered row, value
+    struct __align__(16) Rec {
+        uint32_t off, pad;
+        double v;
+    };
+    __device__ __forceinline__ static Rec rec(uint32_t off, double v) { return Rec{off, 0u, v}; }
+    static constexpr int kRead = 1;  // records per load
+    __device__ __forceinline__ static void read(const Rec *r, uint32_t (&off)[1], double (&v)[1]) {
+        const Rec w = *r;
+        off[0] = w.off;
+        v[0] = w.v;
+    }
+    using Factor = double;
 };
 struct PairMx {
     static constexpr int kSites = 2;
@@ -173,19 +185,24 @@ struct PairMx {
             v[1] = make_double2((double)sr.y + (double)nr.y, (double)si.y + (double)ni.y);
         }
     };
-    __device__ __forceinline__ static uint64_t factor(double v) { return f2_pack((float)v, (float)v); }
-};
-
-struct __align__(16) PairRec {
-    uint32_t off, pad;
-    uint64_t v;  // FP64: the value; mixed: its FP32 pair
+    using Rec = uint2;  // 8 B, two in one broadcast load
+    static constexpr int kRead = 2;
+    __device__ __forceinline__ static Rec rec(uint32_t off, double v) { return make_uint2(off, __float_as_uint((float)v)); }
+    __device__ __forceinline__ static void read(const Rec *r, uint32_t (&off)[2], uint64_t (&v)[2]) {
+        const uint4 w = *reinterpret_cast<const uint4 *>(r);
+        off[0] = w.x;
+        v[0] = f2_pack(__uint_as_float(w.y), __uint_as_float(w.y));
+        off[1] = w.z;
+        v[1] = f2_pack(__uint_as_float(w.w), __uint_as_float(w.w));
+    }
+    using Factor = uint64_t;
 };
 
 // dynamic shared memory: the pack's rows [MG][kPackCols][32 lanes], then 32
 // records per warp; the partial sums of a unit reuse the rows' room
-template <int MG, int WARPS>
+template <class T, int MG, int WARPS>
 __host__ __device__ constexpr size_t pair_smem() {
-    return (size_t)MG * kPackCols * 512 + (size_t)WARPS * 32 * sizeof(PairRec);
+    return (size_t)MG * kPackCols * 512 + (size_t)WARPS * 32 * sizeof(typename T::Rec);
 }
 
 template <class T, int MR, int MG, int WARPS>
@@ -195,7 +212,7 @@ __global__ void __launch_bounds__(32 * WARPS, MG == 1 ? 2 : 1)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     ulonglong2 *stage = reinterpret_cast<ulonglong2 *>(smem_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    PairRec *rec = reinterpret_cast<PairRec *>(smem_raw + (size_t)MG * kPackCols * 512) + warp * 32;
+    typename T::Rec *rec = reinterpret_cast<typename T::Rec *>(smem_raw + (size_t)MG * kPackCols * 512) + warp * 32;
     const int64_t n_items = (int64_t)A.n_units * A.n_tiles;
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
         const PairUnit &u = A.units[item % A.n_units];
@@ -203,9 +220,11 @@ __global__ void __launch_bounds__(32 * WARPS, MG == 1 ? 2 : 1)
         const ulonglong2 *Pt = P + tile * A.p_tile * 32 + lane, *Nt = N + tile * A.n_tile * 32 + lane;
         const ulonglong2 *Rs = u.swap ? Nt : Pt, *Gs = u.swap ? Pt : Nt;
         const int64_t r_rows = u.swap ? A.n_rows : A.p_rows, g_rows = u.swap ? A.p_rows : A.n_rows;
-        const ulonglong2 *Rb[MR];
+        uint32_t Ro[MR];  // 16-byte words from Rs
 #pragma unroll
-        for (int a = 0; a < MR; ++a) Rb[a] = Rs + (int64_t)u.re[min(a, u.nr - 1)] * r_rows * 32;
+        for (int a = 0; a < MR; ++a) Ro[a] = (uint32_t)(u.re[min(a, u.nr - 1)] * r_rows) * 32u;
+        // row-side values on their way while y is summed; the others follow (mixed: registers)
+        constexpr int H = T::kSites == 1 ? MR : (MR + 1) / 2;
         typename T::Acc acc[MR][MG];
 #pragma unroll
         for (int a = 0; a < MR; ++a)
@@ -238,9 +257,10 @@ __global__ void __launch_bounds__(32 * WARPS, MG == 1 ? 2 : 1)
             uint32_t ro = 0;
             load(row, 0, rv, ro);
             for (int r = warp; r < pk.n_rows; r += WARPS) {
-                ulonglong2 x[MR];
+                const ulonglong2 *Rr = Rs + row.row * 32u;
+                ulonglong2 x[H];
 #pragma unroll
-                for (int a = 0; a < MR; ++a) x[a] = __ldg(Rb[a] + row.row * 32u);
+                for (int a = 0; a < H; ++a) x[a] = __ldg(Rr + Ro[a]);
                 const PairRow after = r + 2 * WARPS < pk.n_rows ? rows[r + 2 * WARPS] : none;
                 typename T::Y y[MG];
 #pragma unroll
@@ -248,40 +268,48 @@ __global__ void __launch_bounds__(32 * WARPS, MG == 1 ? 2 : 1)
                 for (uint32_t e0 = 0; e0 < row.n; e0 += 32) {
                     const int n = (int)min(32u, row.n - e0);
                     __syncwarp();
-                    {
-                        const auto f = T::factor(rv);
-                        PairRec v{ro * 32u, 0u, 0ull};
-                        memcpy(&v.v, &f, 8);
-                        rec[lane] = v;
-                    }
+                    rec[lane] = T::rec(ro * 32u, rv);
                     __syncwarp();
                     if (e0 + 32 < row.n)
                         load(row, e0 + 32, rv, ro);
                     else
                         load(next, 0, rv, ro);
+                    constexpr int K = T::kRead;
                     int t = 0;
                     for (; t + 4 <= n; t += 4) {
 #pragma unroll
-                        for (int g = 0; g < 4; ++g) {
-                            const PairRec v = rec[t + g];
-                            decltype(T::factor(0.0)) f;
-                            memcpy(&f, &v.v, 8);
+                        for (int g = 0; g < 4; g += K) {
+                            uint32_t off[K];
+                            typename T::Factor v[K];
+                            T::read(rec + t + g, off, v);
 #pragma unroll
-                            for (int b = 0; b < MG; ++b) y[b].add(G[b * kPackCols * 32 + v.off], f);
+                            for (int q = 0; q < K; ++q)
+#pragma unroll
+                                for (int b = 0; b < MG; ++b) y[b].add(G[b * kPackCols * 32 + off[q]], v[q]);
                         }
                     }
-                    for (; t < n; ++t) {
-                        const PairRec v = rec[t];
-                        decltype(T::factor(0.0)) f;
-                        memcpy(&f, &v.v, 8);
+                    for (; t < n; t += K) {  // a record beyond n is not used
+                        uint32_t off[K];
+                        typename T::Factor v[K];
+                        T::read(rec + t, off, v);
 #pragma unroll
-                        for (int b = 0; b < MG; ++b) y[b].add(G[b * kPackCols * 32 + v.off], f);
+                        for (int q = 0; q < K; ++q)
+                            if (t + q < n)
+#pragma unroll
+                                for (int b = 0; b < MG; ++b) y[b].add(G[b * kPackCols * 32 + off[q]], v[q]);
                     }
                 }
+                ulonglong2 x2[MR > H ? MR - H : 1];
 #pragma unroll
-                for (int a = 0; a < MR; ++a)
+                for (int a = H; a < MR; ++a) x2[a - H] = __ldg(Rr + Ro[a]);
+#pragma unroll
+                for (int a = 0; a < H; ++a)
 #pragma unroll
                     for (int b = 0; b < MG; ++b) acc[a][b].fma(x[a], y[b]);
+#pragma unroll
+                for (int a = H; a < MR; ++a)
+#pragma unroll
+                    for (int b = 0; b < MG; ++b) acc[a][b].fma(x2[a - H], y[b]);
                 row = next;
                 next = after;
             }
