@@ -912,7 +912,6 @@ mbc_status launch_small_batch(const SmallBatch &B, const FieldDesc &F, const Mom
     if (per_sm < 1) return MBC_ERR_UNSUPPORTED;
     int64_t grid = std::min<int64_t>(B.total_items, (int64_t)per_sm * sm_count(device));
     if (grid < 1) return MBC_OK;
-    if (!l.minors) MBC_CUDA_TRY(cudaMemsetAsync(B.counter, 0, sizeof(unsigned long long), stream));
     if (timed) {
         TimedLaunch tl(stream);
         note_launch();
@@ -926,6 +925,27 @@ mbc_status launch_small_batch(const SmallBatch &B, const FieldDesc &F, const Mom
 }
 
 size_t align256(size_t n) { return (n + 255) & ~size_t(255); }
+
+// k_reduce_tiles with warps per output from the tiles a lane would add: several
+// where the outputs are too few to fill the SMs.
+mbc_status launch_reduce(const double2 *partial, int64_t n_slabs, int tiles_per_slab, int n_mom, int n_comp, int n_t,
+                         int li, int n_lists, int comp_max, double2 *out, int nsm, cudaStream_t stream) {
+    const int64_t outs = n_slabs * n_mom * n_comp;
+    int warps = 1;
+    while (warps < 16 && tiles_per_slab > 16 * warps && outs * warps < 4LL * nsm) warps *= 2;
+    auto kern = warps == 1   ? k_reduce_tiles<1>
+                : warps == 2 ? k_reduce_tiles<2>
+                : warps == 4 ? k_reduce_tiles<4>
+                : warps == 8 ? k_reduce_tiles<8>
+                             : k_reduce_tiles<16>;
+    const int per_cta = warps > 4 ? 1 : 4 / warps;
+    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((outs + per_cta - 1) / per_cta, 65535));
+    note_launch();
+    kern<<<grid, warps > 4 ? 32 * warps : kReduceThreads, 0, stream>>>(partial, n_slabs, tiles_per_slab, n_mom, n_comp, n_t,
+                                                                      li, n_lists, comp_max, out);
+    MBC_CUDA_TRY(cudaGetLastError());
+    return MBC_OK;
+}
 
 // Site-operations (operations x sites) a wave needs at least.
 constexpr int64_t kWaveSiteOps = 20000000000LL;
@@ -2016,10 +2036,13 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
         batches.push_back(br);
     }
     size_t small_bytes = 0;
-    for (auto &br : batches) small_bytes += 256 + align256(br.part_bytes);
+    for (auto &br : batches) small_bytes += align256(br.part_bytes);
     size_t large_bytes = 0;
-    // 8Be: 8-site tiles only where 2-site ones would fill every SM several times
-    const int sat_sites = n_slabs * v3 > 16LL * kSatNarrow * sm_count(device) ? kSatWide : kSatNarrow;
+    // 8Be: four warps per site where one would leave FP64 units idle (512 sites
+    // mixed: 22 us against 36); half a warp per site from the lattice on where that
+    // fills them
+    const bool sat_few = n_slabs * v3 <= 16LL * sm_count(device);
+    const int sat_sites = sat_few ? 1 : kSatSites;
     const int sat_tiles = (int)((v3 + sat_sites - 1) / sat_sites);  // per slab
     for (int li : sat_ids)
         large_bytes = std::max(large_bytes, (size_t)(n_slabs * sat_tiles) * M.n_mom * lists[li]->n_comp * sizeof(double2));
@@ -2032,11 +2055,16 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
         const size_t pbytes = (size_t)(n_items / 32) * M.n_mom * L->n_comp * sizeof(double2);
         large_bytes = std::max(large_bytes, align256(pbytes) + ls.buffers());
     }
-    const size_t phase_bytes = align256((size_t)v3 * M.n_mom * sizeof(double2));
+    // the saturated kernels make their own phases; zero momenta need none
+    bool zero_mom = true;
+    for (int q = 0; q < M.n_mom; ++q)
+        for (int d = 0; d < 3; ++d) zero_mom = zero_mom && M.mom[q][d] == 0;
+    const bool need_phase = !zero_mom && !(small_ids.empty() && large_ids.empty());
+    const size_t phase_bytes = need_phase ? align256((size_t)v3 * M.n_mom * sizeof(double2)) : 0;
     void *scr = nullptr;
     if ((st = scratch_get(device, stream, phase_bytes + small_bytes + large_bytes, &scr)) != MBC_OK) return st;
-    double2 *phase = reinterpret_cast<double2 *>(scr);
-    if (!small_ids.empty() || !large_ids.empty()) {  // the saturated kernel makes its own phases
+    double2 *phase = need_phase ? reinterpret_cast<double2 *>(scr) : nullptr;
+    if (need_phase) {
         unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((v3 * M.n_mom + 255) / 256, 4096));
         note_launch();
         k_phase_table<<<grid, 256, 0, stream>>>(F, M, phase);
@@ -2044,20 +2072,12 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
     }
     char *cur = reinterpret_cast<char *>(scr) + phase_bytes;
     auto reduce = [&](int li, const double2 *partial, int tiles_per_slab) -> mbc_status {
-        const mbc_term_list *L = lists[li];
-        int64_t outs = n_slabs * M.n_mom * L->n_comp;
-        unsigned grid = (unsigned)std::min<int64_t>((outs + 7) / 8, 65535);
-        note_launch();
-        k_reduce_tiles<<<std::max(grid, 1u), 256, 0, stream>>>(partial, n_slabs, tiles_per_slab, M.n_mom, L->n_comp,
-                                                              n_t, li, n_lists, comp_max,
-                                                              reinterpret_cast<double2 *>(dev_out));
-        MBC_CUDA_TRY(cudaGetLastError());
-        return MBC_OK;
+        return launch_reduce(partial, n_slabs, tiles_per_slab, M.n_mom, lists[li]->n_comp, n_t, li, n_lists, comp_max,
+                             reinterpret_cast<double2 *>(dev_out), sm_count(device), stream);
     };
     for (auto &br : batches) {
-        br.B.counter = reinterpret_cast<unsigned long long *>(cur);
-        double2 *partial = reinterpret_cast<double2 *>(cur + 256);
-        cur += 256 + align256(br.part_bytes);
+        double2 *partial = reinterpret_cast<double2 *>(cur);
+        cur += align256(br.part_bytes);
         if ((st = launch_small_batch(br.B, F, M, br.sl, mixed, device, stream, phase, partial, true)) != MBC_OK)
             return st;
         for (int j = 0; j < br.B.n_lists; ++j)
@@ -2070,9 +2090,12 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
         {
             TimedLaunch tl(stream);
             note_launch();
-            auto kern = sat_sites == kSatWide ? k_saturated<kSatWide> : k_saturated<kSatNarrow>;
-            kern<<<(unsigned)(n_slabs * sat_tiles), 16 * sat_sites, 0, stream>>>(
-                F, M, caches[(size_t)li]->d_sat_coef, lists[li]->n_comp, sat_tiles, partial);
+            const unsigned grid = (unsigned)(n_slabs * sat_tiles);
+            const double *coef = caches[(size_t)li]->d_sat_coef;
+            if (sat_few)
+                k_saturated_few<<<grid, 128, 0, stream>>>(F, M, coef, lists[li]->n_comp, partial);
+            else
+                k_saturated<<<grid, 16 * kSatSites, 0, stream>>>(F, M, coef, lists[li]->n_comp, sat_tiles, partial);
         }
         MBC_CUDA_TRY(cudaGetLastError());
         if ((st = reduce(li, partial, sat_tiles)) != MBC_OK) return st;
@@ -2351,10 +2374,8 @@ extern "C" mbc_status mbc_contract_noalloc(const mbc_props *props, const mbc_ter
     for (int q = 0; q < opts->n_mom; ++q)
         for (int dd = 0; dd < 3; ++dd) M.mom[q][dd] = opts->mom[3 * q + dd];
     double2 *phase = reinterpret_cast<double2 *>(scr);
-    unsigned long long *counter = reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(scr) + phase_bytes);
     double2 *partial = reinterpret_cast<double2 *>(reinterpret_cast<char *>(scr) + phase_bytes + 256);
-    // every phase-table entry and every tile partial is written before it is
-    // read; the work counter is set to zero below
+    // every phase-table entry and every tile partial is written before it is read
     unsigned pgrid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((v3 * M.n_mom + 255) / 256, 4096));
     note_launch();
     k_phase_table<<<pgrid, 256, 0, stream>>>(F, M, phase);
@@ -2367,16 +2388,11 @@ extern "C" mbc_status mbc_contract_noalloc(const mbc_props *props, const mbc_ter
     B.tiles_per_slab = l.tiles_per_slab;
     B.total_items = n_slabs * l.tiles_per_slab;
     B.item_base[1] = B.total_items;
-    B.counter = counter;
     B.plan[0] = c->sp;
     if ((st = launch_small_batch(B, F, M, l, false, device, stream, phase, partial, false)) != MBC_OK) return st;
-    const int64_t outs = n_slabs * M.n_mom * list->n_comp;
-    const unsigned rgrid = (unsigned)std::min<int64_t>((outs + 7) / 8, 65535);
-    note_launch();
-    k_reduce_tiles<<<std::max(rgrid, 1u), 256, 0, stream>>>(partial, n_slabs, B.tiles_per_slab, M.n_mom,
-                                                            list->n_comp, n_t, 0, 1, comp_max,
-                                                            reinterpret_cast<double2 *>(out));
-    MBC_CUDA_TRY(cudaGetLastError());
+    if ((st = launch_reduce(partial, n_slabs, B.tiles_per_slab, M.n_mom, list->n_comp, n_t, 0, 1, comp_max,
+                            reinterpret_cast<double2 *>(out), sm_count(device), stream)) != MBC_OK)
+        return st;
     return MBC_OK;
 }
 

@@ -567,7 +567,7 @@ __global__ void __launch_bounds__(256) k_large_sitesum(FieldDesc F, WaveDesc wv,
         int s = i / M.n_mom, q = i % M.n_mom;
         int cfg, t, site;
         bool live = item_site(F, wv, wv.item0 + g * 32 + s, cfg, t, site);
-        ph[i] = live ? __ldg(phase + (int64_t)site * M.n_mom + q) : make_double2(0, 0);
+        ph[i] = live ? site_phase(phase, site, M.n_mom, q) : make_double2(0, 0);
     }
     __syncthreads();
     const int64_t tile = (wv.item0 >> 5) + g;
@@ -583,49 +583,73 @@ __global__ void __launch_bounds__(256) k_large_sitesum(FieldDesc F, WaveDesc wv,
     }
 }
 
-// Final reduction over the tiles of each slab: one warp per output, lanes
-// take tiles lane, lane + 32, ... with Neumaier compensation, then a fixed
-// xor tree combines the lanes' (sum, compensation) pairs - a fixed order, so
-// results are bitwise reproducible. out[cfg][list][t - t0][mom][comp_stride].
+// Final reduction over the tiles of each slab: WARPS warps per output, the lower
+// half of a warp adds real parts, the upper half imaginary ones, lane by lane over
+// strided tiles with Neumaier compensation; a fixed xor tree combines the lanes'
+// (sum, compensation) pairs and the warps' in turn - a fixed order, so results are
+// bitwise reproducible. An FP64 instruction of a warp holds one of the SM's four
+// units for 64 cycles however many lanes use it, hence the split halves, four
+// warps per CTA, and several warps for outputs of many tiles. 128 outputs of 16
+// tiles: 3.3 us (8.9 with both parts in every lane and 8 warps per CTA).
+// out[cfg][list][t - t0][mom][comp_stride].
 __device__ __forceinline__ void neumaier(double &s, double &c, double v) {
     const double t = s + v;
     c += fabs(s) >= fabs(v) ? (s - t) + v : (v - t) + s;
     s = t;
 }
-__global__ void k_reduce_tiles(const double2 *__restrict__ partial, int64_t n_slabs, int tiles_per_slab, int n_mom,
-                               int n_comp, int n_t, int list_idx, int n_lists, int comp_stride, double2 *out) {
+// (s, c) of this lane and of its partner `off` lanes away, both adding in the
+// same order so that they agree bit for bit
+__device__ __forceinline__ void neumaier_pair(double &s, double &c, int off, int lane) {
+    const double os = __shfl_xor_sync(0xffffffffu, s, off), oc = __shfl_xor_sync(0xffffffffu, c, off);
+    const double a = lane & off ? os : s, b = lane & off ? s : os;
+    c += oc;
+    s = a;
+    neumaier(s, c, b);
+}
+constexpr int kReduceThreads = 128;
+template <int WARPS>
+__global__ void __launch_bounds__(WARPS > 4 ? 32 * WARPS : kReduceThreads)
+    k_reduce_tiles(const double2 *__restrict__ partial, int64_t n_slabs, int tiles_per_slab, int n_mom, int n_comp,
+                   int n_t, int list_idx, int n_lists, int comp_stride, double2 *out) {
+    constexpr int OUTS = WARPS > 4 ? 1 : 4 / WARPS;  // outputs per CTA
+    __shared__ double part_s[4 > WARPS ? 4 : WARPS][2], part_c[4 > WARPS ? 4 : WARPS][2];
     const int64_t per_slab = (int64_t)n_mom * n_comp;
-    const int lane = threadIdx.x & 31;
-    const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t o = wid; o < n_slabs * per_slab; o += nw) {
-        const int64_t slab = o / per_slab;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, im = lane >> 4;
+    const int w = warp % WARPS;
+    const double *p = reinterpret_cast<const double *>(partial);
+    for (int64_t o0 = (int64_t)blockIdx.x * OUTS; o0 < n_slabs * per_slab; o0 += (int64_t)gridDim.x * OUTS) {
+        const int64_t o = o0 + warp / WARPS;
+        const bool live = o < n_slabs * per_slab;
+        const int64_t slab = live ? o / per_slab : 0;
         const int r = (int)(o % per_slab);
-        double sr = 0.0, cr = 0.0, si = 0.0, ci = 0.0;
-        for (int tl = lane; tl < tiles_per_slab; tl += 32) {
-            const double2 v = partial[(slab * tiles_per_slab + tl) * per_slab + r];
-            neumaier(sr, cr, v.x);
-            neumaier(si, ci, v.y);
+        double s = 0.0, c = 0.0;
+        int tl = w * 16 + (lane & 15);
+        if (live && tl < tiles_per_slab) {
+            s = p[2 * ((slab * tiles_per_slab + tl) * per_slab + r) + im];
+            for (tl += 16 * WARPS; tl < tiles_per_slab; tl += 16 * WARPS)
+                neumaier(s, c, p[2 * ((slab * tiles_per_slab + tl) * per_slab + r) + im]);
         }
-        for (int off = 16; off > 0; off >>= 1) {
-            const double osr = __shfl_xor_sync(0xffffffffu, sr, off), ocr = __shfl_xor_sync(0xffffffffu, cr, off);
-            const double osi = __shfl_xor_sync(0xffffffffu, si, off), oci = __shfl_xor_sync(0xffffffffu, ci, off);
-            // both partners add in the same order, so they agree bit for bit
-            double ar = lane & off ? osr : sr, br = lane & off ? sr : osr;
-            double ai = lane & off ? osi : si, bi = lane & off ? si : osi;
-            double ccr = cr + ocr, cci = ci + oci;
-            sr = ar;
-            cr = ccr;
-            neumaier(sr, cr, br);
-            si = ai;
-            ci = cci;
-            neumaier(si, ci, bi);
+        for (int off = 8; off > 0; off >>= 1)
+            if (off < tiles_per_slab) neumaier_pair(s, c, off, lane);
+        if (WARPS > 1) {
+            if ((lane & 15) == 0) {
+                part_s[warp][im] = s;
+                part_c[warp][im] = c;
+            }
+            __syncthreads();
+            if (w == 0) {
+                const int k = lane & 15;
+                s = k < WARPS ? part_s[warp + k][im] : 0.0;
+                c = k < WARPS ? part_c[warp + k][im] : 0.0;
+                for (int off = WARPS / 2; off > 0; off >>= 1) neumaier_pair(s, c, off, lane);
+            }
+            __syncthreads();  // read before the next output's
         }
-        if (lane == 0) {
+        if (live && w == 0 && (lane & 15) == 0) {
             const int cfg = (int)(slab / n_t), tt = (int)(slab % n_t);
-            const int q = r / n_comp, c = r % n_comp;
-            const int64_t oi = ((((int64_t)cfg * n_lists + list_idx) * n_t + tt) * n_mom + q) * comp_stride + c;
-            out[oi] = make_double2(sr + cr, si + ci);
+            const int q = r / n_comp, cc = r % n_comp;
+            const int64_t oi = ((((int64_t)cfg * n_lists + list_idx) * n_t + tt) * n_mom + q) * comp_stride + cc;
+            reinterpret_cast<double *>(out)[2 * oi + im] = s + c;
         }
     }
 }

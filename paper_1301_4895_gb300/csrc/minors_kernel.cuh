@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(32 * MinorRows<Tr>::kWarps, MinorRows<Tr>::kMx
                     im = scalbn(im, ue);
                 }
                 for (int q = 0; q < M.n_mom; ++q) {
-                    const double2 ph = live ? __ldg(phase + (int64_t)site * M.n_mom + q) : make_double2(0, 0);
+                    const double2 ph = live ? site_phase(phase, site, M.n_mom, q) : make_double2(0, 0);
                     double pr = live ? __fma_rn(ph.x, re, -ph.y * im) : 0.0, pi = live ? __fma_rn(ph.x, im, ph.y * re) : 0.0;
                     for (int off = 16; off > 0; off >>= 1) {
                         pr += __shfl_xor_sync(0xffffffffu, pr, off);

@@ -10,17 +10,30 @@
 // the permutation's sign is counted. The kernel is bound by the FP64 units (a
 // warp's FP64 instruction takes one of the SM's four for 64 cycles) through
 // 12 dependent steps. Measured on GB300 against the recursion, whole calls: 64
-// sites FP64 198.0 ms -> 43 us, 512 sites mixed 156.1 ms -> 57 us (the kernel
-// 36 us of it).
+// sites FP64 198.0 ms -> 33 us, 512 sites mixed 156.1 ms -> 58 us, the kernels 17
+// and 22 us of it.
 #pragma once
 
 #include "small_kernel.cuh"
 
 namespace mbc {
 
-// Sites per CTA and tile: the warps of an SM share its FP64 unit, so lattices
-// of few sites take one warp per CTA to reach every SM.
-constexpr int kSatWide = 8, kSatNarrow = 2;
+// Sites per CTA and tile.
+constexpr int kSatSites = 8;
+
+// a / piv; pivots whose square would overflow or vanish are scaled first (with a)
+// by their exponent. A zero pivot has a zero column below it and nothing to
+// eliminate.
+__device__ __forceinline__ double2 pivot_factor(double2 a, double2 piv) {
+    const double big = fmax(fabs(piv.x), fabs(piv.y));
+    if (!(big > 0x1p-480 && big < 0x1p480)) {
+        const int e = big > 0.0 ? -ilogb(big) : 0;
+        a = make_double2(scalbn(a.x, e), scalbn(a.y, e));
+        piv = make_double2(scalbn(piv.x, e), scalbn(piv.y, e));
+    }
+    const double inv = big == 0.0 ? 0.0 : 1.0 / __fma_rn(piv.x, piv.x, piv.y * piv.y);
+    return make_double2(__fma_rn(a.x, piv.x, a.y * piv.y) * inv, __fma_rn(a.y, piv.x, -a.x * piv.y) * inv);
+}
 
 // det of the 12 x 12 matrix whose row (lane & 15) this lane holds
 __device__ __forceinline__ double2 det12(double2 (&a)[12]) {
@@ -40,19 +53,7 @@ __device__ __forceinline__ double2 det12(double2 (&a)[12]) {
         left &= ~(1u << p);
         const double2 piv = make_double2(__shfl_sync(half, a[k].x, p, 16), __shfl_sync(half, a[k].y, p, 16));
         det = cmul(det, piv);
-        // factor = a[k] / piv; pivots whose square would overflow or vanish are
-        // scaled first (with the column) by their exponent. A zero pivot has a
-        // zero column below it and nothing to eliminate
-        const double big = fmax(fabs(piv.x), fabs(piv.y));
-        double2 num = a[k], den = piv;
-        if (!(big > 0x1p-480 && big < 0x1p480)) {
-            const int e = big > 0.0 ? -ilogb(big) : 0;
-            num = make_double2(scalbn(num.x, e), scalbn(num.y, e));
-            den = make_double2(scalbn(den.x, e), scalbn(den.y, e));
-        }
-        const double inv = big == 0.0 ? 0.0 : 1.0 / __fma_rn(den.x, den.x, den.y * den.y);
-        const double2 f = make_double2(__fma_rn(num.x, den.x, num.y * den.y) * inv,
-                                       __fma_rn(num.y, den.x, -num.x * den.y) * inv);
+        const double2 f = pivot_factor(a[k], piv);
 #pragma unroll
         for (int j = k + 1; j < 12; ++j) {
             const double2 q = make_double2(__shfl_sync(half, a[j].x, p, 16), __shfl_sync(half, a[j].y, p, 16));
@@ -64,7 +65,6 @@ __device__ __forceinline__ double2 det12(double2 (&a)[12]) {
 
 // partial[tile][mom][comp]: phase-weighted sums over the tile's sites in a
 // fixed order, scaled by the component's coefficient
-template <int kSatSites>
 __global__ void __launch_bounds__(16 * kSatSites)
     k_saturated(FieldDesc F, MomDesc M, const double *__restrict__ coef, int n_comp, int tiles_per_slab,
                 double2 *__restrict__ partial) {
@@ -99,6 +99,74 @@ __global__ void __launch_bounds__(16 * kSatSites)
     for (int o = threadIdx.x; o < M.n_mom * n_comp; o += blockDim.x) {
         const double c = __ldg(coef + o % n_comp);
         partial[tile * (int64_t)(M.n_mom * n_comp) + o] = make_double2(c * sum[o / n_comp].x, c * sum[o / n_comp].y);
+    }
+}
+
+// The same elimination with a CTA of four warps per site, for lattices of few
+// sites: a warp's FP64 instructions run on one of the SM's four FP64 units, so
+// one warp per site leaves three idle. Lanes are rows, twice; warp w holds columns
+// w, w + 4 (upper half) and w + 8. The warp that owns a step's column finds the
+// pivot and writes the rows' factors to shared memory; every warp then fetches its
+// columns' pivot elements by shuffles and eliminates. 64 sites: 17 us, one warp
+// for two sites 30.
+__global__ void __launch_bounds__(128) k_saturated_few(FieldDesc F, MomDesc M, const double *__restrict__ coef,
+                                                       int n_comp, double2 *__restrict__ partial) {
+    __shared__ double2 fac[2][12], pivots[12], dd;
+    __shared__ int prow[2];
+    const int v3 = F.lx * F.ly * F.lz;
+    const int64_t tile = blockIdx.x, slab = tile / v3;
+    const int site = (int)(tile % v3), lane = threadIdx.x & 31, w = threadIdx.x >> 5, half = lane >> 4, row = lane & 15;
+    double2 a[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};  // columns w + 4 half, w + 8 (lower half)
+    if (row < 12) {
+        const int64_t base = slab / F.n_t * F.stride_cfg + (F.t0 + slab % F.n_t) * F.stride_t + (int64_t)site * 144;
+        a[0] = load_prop(F, base, row * 12 + w + 4 * half);
+        if (half == 0) a[1] = load_prop(F, base, row * 12 + w + 8);
+    }
+    unsigned left = 0xfffu, odd = 0;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const int h = (k >> 2) & 1, q = k >> 3;  // column k: warp k % 4, half h, register q
+        if (w == (k & 3) && half == h) {
+            const unsigned mask = 0xffffu << (16 * h);
+            const uint32_t key =
+                (left >> row & 1u) ? (uint32_t)__double2hiint(fabs(a[q].x) + fabs(a[q].y)) + 1u : 0u;
+            const uint32_t best = __reduce_max_sync(mask, key);
+            const int p = __ffs((__ballot_sync(mask, key == best) >> (16 * h)) & 0xffffu) - 1;
+            const double2 piv = make_double2(__shfl_sync(mask, a[q].x, p, 16), __shfl_sync(mask, a[q].y, p, 16));
+            const double2 f = pivot_factor(a[q], piv);
+            if (row < 12) fac[k & 1][row] = (left >> row & 1u) && row != p ? f : make_double2(0.0, 0.0);
+            if (row == 0) {
+                prow[k & 1] = p;
+                pivots[k] = piv;
+            }
+        }
+        __syncthreads();  // double-buffered: a step's readers are done before the next but one writes
+        const int p = prow[k & 1];
+        odd ^= __popc(left & ((1u << p) - 1u)) & 1u;
+        left &= ~(1u << p);
+        const double2 f = row < 12 ? fac[k & 1][row] : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            if (g == 0 ? w + 4 <= k : w + 8 <= k) continue;  // no column of this group is left
+            const double2 x = make_double2(__shfl_sync(0xffffffffu, a[g].x, p, 16), __shfl_sync(0xffffffffu, a[g].y, p, 16));
+            if (w + 4 * half + 8 * g > k && (left >> row & 1u)) a[g] = cfms(f, x, a[g]);
+        }
+    }
+    if (w == 0) {  // product of the pivots, in a fixed tree
+        double2 d = lane < 12 ? pivots[lane] : make_double2(1.0, 0.0);
+        for (int off = 8; off > 0; off >>= 1) {
+            const double2 o = make_double2(__shfl_xor_sync(0xffffffffu, d.x, off), __shfl_xor_sync(0xffffffffu, d.y, off));
+            d = cmul(d, o);
+        }
+        if (lane == 0) dd = cmul(d, d);  // the permutation's sign squares away
+    }
+    __syncthreads();
+    for (int o = threadIdx.x; o < M.n_mom * n_comp; o += blockDim.x) {
+        const double2 ph = mom_phase(M.mom[o / n_comp], site % F.lx, (site / F.lx) % F.ly, site / (F.lx * F.ly), F.lx,
+                                     F.ly, F.lz);
+        const double c = __ldg(coef + o % n_comp);
+        partial[tile * (int64_t)(M.n_mom * n_comp) + o] =
+            make_double2(c * __fma_rn(ph.x, dd.x, -ph.y * dd.y), c * __fma_rn(ph.x, dd.y, ph.y * dd.x));
     }
 }
 

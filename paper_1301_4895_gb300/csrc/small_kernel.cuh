@@ -63,7 +63,7 @@ struct SmallPlan {
 
 // A batch of term lists contracted by one persistent launch: the work items
 // are (list, tile) pairs, numbered list by list in the order given (the host
-// puts the most expensive list first), handed out by an atomic counter. In a
+// puts the most expensive list first), dealt to the CTAs in turn. In a
 // shared batch (lists with the same tile shape and buffer offsets of the S
 // tile, diquark and blocks) an item is a tile and covers every list: the
 // tile and the block are computed once per site, then each list runs its
@@ -78,24 +78,13 @@ struct SmallBatch {
     int64_t total_items;
     int64_t item_base[kMaxBatch + 1];
     int64_t partial_off[kMaxBatch];  // in double2 units
-    unsigned long long *counter;     // zeroed before the launch
     SmallPlan plan[kMaxBatch];
 };
 
-// next work item of the CTA (thread 0 draws, everyone reads); returns the list
-__device__ __forceinline__ int next_item(const SmallBatch &B, int64_t &tile) {
-    __shared__ long long s_item;
-    __syncthreads();
-    if (threadIdx.x == 0) s_item = (long long)atomicAdd(B.counter, 1ull);
-    __syncthreads();
-    const int64_t item = s_item;
-    if (item >= B.total_items) return -1;
-    if (B.shared) {
-        tile = item;
-        return 0;
-    }
+// list and tile of work item `item`
+__device__ __forceinline__ int item_list(const SmallBatch &B, int64_t item, int64_t &tile) {
     int l = 0;
-    while (l + 1 < B.n_lists && item >= B.item_base[l + 1]) ++l;
+    while (!B.shared && l + 1 < B.n_lists && item >= B.item_base[l + 1]) ++l;
     tile = item - B.item_base[l];
     return l;
 }
@@ -139,10 +128,16 @@ __device__ __forceinline__ double2 load_prop(const FieldDesc &f, int64_t base, i
 __device__ __forceinline__ double2 mom_phase(const int32_t *n, int x, int y, int z, int lx, int ly, int lz) {
     // reduce each product modulo its extent in integers, then one turn fraction
     int rx = ((n[0] * x) % lx + lx) % lx, ry = ((n[1] * y) % ly + ly) % ly, rz = ((n[2] * z) % lz + lz) % lz;
+    if ((rx | ry | rz) == 0) return make_double2(1.0, 0.0);
     double turns = (double)rx / lx + (double)ry / ly + (double)rz / lz;
     double s, c;
     sincospi(-2.0 * turns, &s, &c);
     return make_double2(c, s);
+}
+
+// entry of the phase table; no table: every momentum of the call is zero
+__device__ __forceinline__ double2 site_phase(const double2 *phase, int64_t site, int n_mom, int q) {
+    return phase ? __ldg(phase + site * n_mom + q) : make_double2(1.0, 0.0);
 }
 
 // Outputs [z_begin, z_begin + n) of a step with g lanes per output. Their ops
@@ -248,8 +243,10 @@ __global__ void __launch_bounds__(1024, 1)
     double2 *Cs = reinterpret_cast<double2 *>(reinterpret_cast<V *>(smem_raw) + (int64_t)T * B.site_stride);
     const int V3 = F.lx * F.ly * F.lz;
     const int tiles_per_slab = B.tiles_per_slab;
-    int64_t tile;
-    for (int li0; (li0 = next_item(B, tile)) >= 0;) {
+    for (int64_t item = blockIdx.x; item < B.total_items; item += gridDim.x) {
+        int64_t tile;
+        const int li0 = item_list(B, item, tile);
+        __syncthreads();  // the components of the previous item are read
         const int l_end = B.shared ? B.n_lists : li0 + 1;
         const SmallPlan &P0 = B.plan[li0];
         const int nxi = P0.nxi;
@@ -315,7 +312,7 @@ __global__ void __launch_bounds__(1024, 1)
                 int q = o / P.n_comp, c = o % P.n_comp;
                 double re = 0.0, im = 0.0;
                 for (int w = 0; w < T && site0 + w < V3; ++w) {
-                    double2 ph = __ldg(phase + (int64_t)(site0 + w) * M.n_mom + q), cv = Cs[w * B.comp_stride + c];
+                    double2 ph = site_phase(phase, site0 + w, M.n_mom, q), cv = Cs[w * B.comp_stride + c];
                     re = __fma_rn(ph.x, cv.x, __fma_rn(-ph.y, cv.y, re));
                     im = __fma_rn(ph.x, cv.y, __fma_rn(ph.y, cv.x, im));
                 }

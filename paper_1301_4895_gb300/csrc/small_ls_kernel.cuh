@@ -74,8 +74,10 @@ __global__ void __launch_bounds__(1024, 1)
     const int tiles_per_slab = B.tiles_per_slab;
 #define ROW(e) R[(int64_t)(e) * 32 + lane]
 
-    int64_t tile;
-    for (int li0; (li0 = next_item(B, tile)) >= 0;) {  // next_item synchronises the CTA
+    for (int64_t item = blockIdx.x; item < B.total_items; item += gridDim.x) {
+        int64_t tile;
+        const int li0 = item_list(B, item, tile);
+        __syncthreads();  // the previous item is done with the shared memory
         // a shared batch's item is a tile of every list: tile and blocks once
         const int l_end = B.shared ? B.n_lists : li0 + 1;
         const SmallPlan &P = B.plan[li0];
@@ -268,7 +270,7 @@ __global__ void __launch_bounds__(1024, 1)
                 re = live ? scalbn(re * inv_norm, ue) : 0.0;
                 im = live ? scalbn(im * inv_norm, ue) : 0.0;
                 for (int q = 0; q < M.n_mom; ++q) {
-                    const double2 ph = live ? __ldg(phase + (int64_t)site * M.n_mom + q) : make_double2(0, 0);
+                    const double2 ph = live ? site_phase(phase, site, M.n_mom, q) : make_double2(0, 0);
                     double pr = __fma_rn(ph.x, re, -ph.y * im), pi = __fma_rn(ph.x, im, ph.y * re);
                     for (int off = 16; off > 0; off >>= 1) {
                         pr += __shfl_xor_sync(full, pr, off);
