@@ -91,6 +91,8 @@ _lock = threading.Lock()
 def load(path: str | None = None):
     """Load libmbc.so (built by ``__graft_entry__.build()``); raises if absent."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -162,6 +164,13 @@ class TermList:
     @property
     def handle(self):
         return self._h
+
+    @property
+    def n_comp(self) -> int:
+        """Output components per site (a list never changes: read once)."""
+        if getattr(self, "_n_comp", None) is None:
+            self._n_comp = self.stats()["n_comp"]
+        return self._n_comp
 
     @property
     def pauli_forbidden(self) -> bool:
@@ -346,6 +355,16 @@ def _stream_ptr(stream):
 
 
 SINK_POINT, SINK_BLOCK_MOMENTUM = 0, 1
+_torch_module = None
+
+
+def _torch():
+    """torch, imported with the first device tensor (an import statement in a call costs it about a microsecond)."""
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def contract(field, lists, precision: int = FP64, moms=((0, 0, 0),), t0: int = 0, t1: int = 0, tune=None,
@@ -363,32 +382,40 @@ def contract(field, lists, precision: int = FP64, moms=((0, 0, 0),), t0: int = 0
     lists = list(lists)
     is_np = isinstance(field, np.ndarray)
     if is_np:
+        shape = field.shape
         if field.dtype not in (np.complex128, np.complex64) or not field.flags.c_contiguous:
             raise ValueError("field must be a C-contiguous complex128/complex64 array")
         dtype = C128 if field.dtype == np.complex128 else C64
         ptr = field.ctypes.data
-        shape = field.shape
     else:
-        import torch
-        if field.dtype not in (torch.complex128, torch.complex64) or not field.is_contiguous():
+        torch = _torch()
+        dt = field.dtype
+        if dt is torch.complex128:
+            dtype = C128
+        elif dt is torch.complex64:
+            dtype = C64
+        else:
+            dtype = None
+        if dtype is None or not field.is_contiguous():
             raise ValueError("field must be a contiguous complex128/complex64 tensor")
-        dtype = C128 if field.dtype == torch.complex128 else C64
         ptr = field.data_ptr()
-        shape = tuple(field.shape)
+        shape = field.shape
     if len(shape) not in (7, 8) or shape[-2:] != (12, 12):
         raise ValueError("field shape must be (n_cfg, nt, Lz, Ly, Lx, [n_src,] 12, 12)")
     n_cfg, nt, lz, ly, lx = shape[:5]
     n_src = shape[5] if len(shape) == 8 else 1
     t1e = nt if t1 == 0 else t1
-    moms = np.ascontiguousarray(np.array(moms, dtype=np.int32).reshape(-1, 3))
-    comp_max = max(1, max(tl.stats()["n_comp"] for tl in lists))
+    moms = np.array(moms, dtype=np.int32)
+    if moms.ndim != 2 or moms.shape[1] != 3 or not moms.flags.c_contiguous:
+        moms = np.ascontiguousarray(moms.reshape(-1, 3))
+    n_mom = len(moms)
+    comp_max = max(1, max([tl.n_comp for tl in lists]))
     n_k = max(1, int(lists[0].spec.get("n_sinks", 1) or 1)) if lists else 1
-    oshape = (n_cfg, len(lists), t1e - t0, moms.shape[0] // n_k, comp_max)
+    oshape = (n_cfg, len(lists), t1e - t0, n_mom // n_k, comp_max)
     if out is None:
         if is_np:
             out = np.zeros(oshape, dtype=np.complex128)
         else:
-            import torch
             out = torch.empty(oshape, dtype=torch.complex128, device=field.device)  # the library zero-fills
     optr = out.ctypes.data if is_np else out.data_ptr()
     pr = Props(ptr, ptr, dtype, MEM_HOST if is_np else MEM_DEVICE, n_cfg, nt, lx, ly, lz, 0, 0, n_src)
@@ -398,10 +425,12 @@ def contract(field, lists, precision: int = FP64, moms=((0, 0, 0),), t0: int = 0
         if unknown:
             raise ValueError(f"unknown tune fields {sorted(unknown)}")
         tn = Tune(*[int(tune.get(f, 0)) for f in Tune.FIELDS])
-    op = ContractOpts(precision, moms.shape[0], moms.ctypes.data, t0, t1, ctypes.addressof(tn) if tn else None, sink)
-    handles = (ctypes.c_void_p * len(lists))(*[tl.handle for tl in lists])
+    op = ContractOpts(precision, n_mom, moms.__array_interface__["data"][0], t0, t1,
+                      ctypes.addressof(tn) if tn else None, sink)
+    handles = (ctypes.c_void_p * len(lists))(*[tl._h for tl in lists])
     rc = lib.mbc_contract(ctypes.byref(pr), handles, len(lists), ctypes.byref(op), optr, _stream_ptr(stream))
-    _check(rc, "mbc_contract")
+    if rc:
+        raise MbcError(rc, "mbc_contract")
     return out
 
 

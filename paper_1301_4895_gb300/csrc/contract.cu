@@ -927,21 +927,18 @@ mbc_status launch_small_batch(const SmallBatch &B, const FieldDesc &F, const Mom
 size_t align256(size_t n) { return (n + 255) & ~size_t(255); }
 
 // k_reduce_tiles with warps per output from the tiles a lane would add: several
-// where the outputs are too few to fill the SMs.
+// where the outputs are too few to fill the SMs, at most one per FP64 unit (one
+// output of 512 tiles: 16 warps 9.0 us, 4 warps 6.0).
 mbc_status launch_reduce(const double2 *partial, int64_t n_slabs, int tiles_per_slab, int n_mom, int n_comp, int n_t,
                          int li, int n_lists, int comp_max, double2 *out, int nsm, cudaStream_t stream) {
     const int64_t outs = n_slabs * n_mom * n_comp;
     int warps = 1;
-    while (warps < 16 && tiles_per_slab > 16 * warps && outs * warps < 4LL * nsm) warps *= 2;
-    auto kern = warps == 1   ? k_reduce_tiles<1>
-                : warps == 2 ? k_reduce_tiles<2>
-                : warps == 4 ? k_reduce_tiles<4>
-                : warps == 8 ? k_reduce_tiles<8>
-                             : k_reduce_tiles<16>;
-    const int per_cta = warps > 4 ? 1 : 4 / warps;
+    while (warps < 4 && tiles_per_slab > 16 * warps && outs * warps < 4LL * nsm) warps *= 2;
+    auto kern = warps == 1 ? k_reduce_tiles<1> : warps == 2 ? k_reduce_tiles<2> : k_reduce_tiles<4>;
+    const int per_cta = 4 / warps;
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((outs + per_cta - 1) / per_cta, 65535));
     note_launch();
-    kern<<<grid, warps > 4 ? 32 * warps : kReduceThreads, 0, stream>>>(partial, n_slabs, tiles_per_slab, n_mom, n_comp, n_t,
+    kern<<<grid, kReduceThreads, 0, stream>>>(partial, n_slabs, tiles_per_slab, n_mom, n_comp, n_t,
                                                                       li, n_lists, comp_max, out);
     MBC_CUDA_TRY(cudaGetLastError());
     return MBC_OK;

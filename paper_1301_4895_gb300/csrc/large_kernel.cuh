@@ -608,11 +608,11 @@ __device__ __forceinline__ void neumaier_pair(double &s, double &c, int off, int
 }
 constexpr int kReduceThreads = 128;
 template <int WARPS>
-__global__ void __launch_bounds__(WARPS > 4 ? 32 * WARPS : kReduceThreads)
+__global__ void __launch_bounds__(kReduceThreads)
     k_reduce_tiles(const double2 *__restrict__ partial, int64_t n_slabs, int tiles_per_slab, int n_mom, int n_comp,
                    int n_t, int list_idx, int n_lists, int comp_stride, double2 *out) {
-    constexpr int OUTS = WARPS > 4 ? 1 : 4 / WARPS;  // outputs per CTA
-    __shared__ double part_s[4 > WARPS ? 4 : WARPS][2], part_c[4 > WARPS ? 4 : WARPS][2];
+    constexpr int OUTS = 4 / WARPS;  // outputs per CTA
+    __shared__ double part_s[4][2], part_c[4][2];
     const int64_t per_slab = (int64_t)n_mom * n_comp;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, im = lane >> 4;
     const int w = warp % WARPS;
