@@ -312,8 +312,9 @@ bool plan_minors(const MinorPlan &mp, SmallPlan &P, int64_t &site_entries) {
 // A list with a minor form takes that one.
 // part_off receives, per nucleus of the list, the region offset of the stage
 // its components are contracted from (blocks for a single baryon).
-bool plan_small(const mbc_term_list *L, const MinorPlan *minor, SmallPlan &P, int64_t &site_entries,
-                std::vector<int> &part_off) {
+// mirror: a pn list computes one output of each mirror pair.
+bool plan_small(const mbc_term_list *L, const MinorPlan *minor, const MirrorPlan *mirror, SmallPlan &P,
+                int64_t &site_entries, std::vector<int> &part_off) {
     std::memset(&P, 0, sizeof(P));
     const int A = L->A;
     if (A > 16 || L->n_comp > kSmallMaxComp || L->n_comp < 1) return false;
@@ -350,9 +351,9 @@ bool plan_small(const mbc_term_list *L, const MinorPlan *minor, SmallPlan &P, in
     // a stage where a nucleus of the list ends stays live until the contraction
     std::vector<bool> contracted((size_t)A + 1, false);
     for (const auto &pt : L->parts) contracted[(size_t)pt.A] = true;
+    auto outputs = [&](int m) { return mirror ? (int64_t)mirror->keep.size() : L->steps[(size_t)m - 1].n_z; };
     for (int m = 1; m < A; ++m) {
-        stage[(size_t)m + 1] = {3 + m - 1, contracted[(size_t)m + 1] ? last_phase : 3 + m,
-                                L->steps[(size_t)m - 1].n_z, 0};
+        stage[(size_t)m + 1] = {3 + m - 1, contracted[(size_t)m + 1] ? last_phase : 3 + m, outputs(m), 0};
         order.push_back(&stage[(size_t)m + 1]);
     }
     (void)n_ph;
@@ -369,9 +370,9 @@ bool plan_small(const mbc_term_list *L, const MinorPlan *minor, SmallPlan &P, in
     for (int m = 1; m < A; ++m) {
         const Step &s = L->steps[(size_t)m - 1];
         SmallStepDesc &d = P.step[m - 1];
-        d.n_z = (int)s.n_z;
+        d.n_z = (int)outputs(m);
         d.k = (int)s.k;
-        split_groups(s.n_z, s.k, d.g, d.n_main, d.g2);
+        split_groups(d.n_z, s.k, d.g, d.n_main, d.g2);
         d.x_off = m == 1 ? P.blk_off : (int)stage[(size_t)m].off;
         d.y_off = P.blk_off;
         d.z_off = (int)stage[(size_t)m + 1].off;
@@ -440,7 +441,8 @@ DeviceCache *get_cache(const mbc_term_list *Lc, int device, mbc_status &st) {
     // small-kernel plan and packed ops
     std::vector<int> part_off;
     const std::shared_ptr<const MinorPlan> minor = minor_plan(L);
-    c->small_ok = !L->pauli_forbidden && plan_small(L, minor.get(), c->sp, c->site_entries, part_off);
+    const std::shared_ptr<const MirrorPlan> mirror = mirror_plan(L);
+    c->small_ok = !L->pauli_forbidden && plan_small(L, minor.get(), mirror.get(), c->sp, c->site_entries, part_off);
     if (c->small_ok) {
         // contracted entries as offsets in the site region; per-component
         // normalisation and homogeneity degree of its nucleus
@@ -453,7 +455,8 @@ DeviceCache *get_cache(const mbc_term_list *Lc, int device, mbc_status &st) {
                 inv[(size_t)cc] = 1.0 / pt.norm;
                 deg[(size_t)cc] = 3 * pt.A;
                 for (int64_t e = L->fin_off[(size_t)cc]; !minor && e < L->fin_off[(size_t)cc + 1]; ++e)
-                    zs[(size_t)e] = L->fin_z[(size_t)e] + (uint32_t)part_off[j];
+                    zs[(size_t)e] = (mirror ? (uint32_t)mirror->rep[L->fin_z[(size_t)e]] : L->fin_z[(size_t)e]) +
+                                    (uint32_t)part_off[j];
             }
         }
         if ((st = upload(&c->d_fin_zs, zs.data(), zs.size())) != MBC_OK ||
@@ -475,6 +478,7 @@ DeviceCache *get_cache(const mbc_term_list *Lc, int device, mbc_status &st) {
                 return Op{s.x[i], s.y[i], s.neg[i]};
             }
             const Step &s = L->steps[m];
+            if (mirror) i = (size_t)mirror->keep[i / (size_t)s.k] * (size_t)s.k + i % (size_t)s.k;
             return Op{s.x[i], s.ys[i] & 0x7fffu, (uint32_t)(s.ys[i] >> 15)};
         };
         std::vector<uint32_t> packed;
@@ -2340,7 +2344,7 @@ extern "C" mbc_status mbc_contract_noalloc(const mbc_props *props, const mbc_ter
     if (!zero) {
         std::vector<int> part_off;
         const std::shared_ptr<const MinorPlan> minor = minor_plan(list);
-        if (!plan_small(list, minor.get(), hp, site_entries, part_off)) return MBC_ERR_UNSUPPORTED;  // relativistic lists: no static variant
+        if (!plan_small(list, minor.get(), mirror_plan(list).get(), hp, site_entries, part_off)) return MBC_ERR_UNSUPPORTED;  // relativistic lists: no static variant
         // the launch shape the kernel will run with, and from it the bytes
         // of the tile partials (one sizing, used for the check and the launch)
         l = size_small_tiles((int32_t)site_entries, hp.n_comp, F, opts->tune, false, minor != nullptr);

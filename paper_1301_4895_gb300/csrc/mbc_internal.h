@@ -40,6 +40,7 @@ struct DeviceCache;  // defined by the CUDA side
 struct MinorPlan;    // plan.h
 struct SaturatedPlan;
 struct PairPlan;
+struct MirrorPlan;
 
 }  // namespace mbc
 
@@ -80,7 +81,8 @@ struct mbc_term_list {
     std::shared_ptr<const mbc::MinorPlan> minor;
     std::shared_ptr<const mbc::SaturatedPlan> saturated;
     std::shared_ptr<const mbc::PairPlan> pair;
-    bool minor_tried = false, saturated_tried = false, pair_tried = false;
+    std::shared_ptr<const mbc::MirrorPlan> mirror;
+    bool minor_tried = false, saturated_tried = false, pair_tried = false, mirror_tried = false;
 };
 
 namespace mbc {

@@ -666,6 +666,45 @@ std::shared_ptr<const SaturatedPlan> saturated_plan(const mbc_term_list *Lc) {
     return L->saturated;
 }
 
+namespace {
+
+std::shared_ptr<const MirrorPlan> make_mirror_plan(const mbc_term_list &L) {
+    if (L.pauli_forbidden || L.A != 2 || L.parts.size() != 1 || L.parts[0].n_p != 1 || L.parts[0].n_n != 1 ||
+        L.parts[0].A != 2 || L.steps.size() != 1 || L.steps[0].generated || L.steps[0].n_z >= 65536)
+        return nullptr;
+    auto P = std::make_shared<MirrorPlan>();
+    std::map<std::vector<uint32_t>, int32_t> at;
+    for (int64_t z = 0; z < L.steps[0].n_z; ++z) {
+        PlanKey k;
+        if (!stage_key(L, 2, z, k)) return nullptr;
+        const auto m = at.find({k.dn, k.dp, k.d, k.u});
+        if (m != at.end()) {
+            P->rep.push_back(m->second);
+            continue;
+        }
+        at[{k.dp, k.dn, k.u, k.d}] = (int32_t)P->keep.size();
+        P->rep.push_back((int32_t)P->keep.size());
+        P->keep.push_back((int32_t)z);
+    }
+    return P;
+}
+
+}  // namespace
+
+std::shared_ptr<const MirrorPlan> mirror_plan(const mbc_term_list *Lc) {
+    mbc_term_list *L = const_cast<mbc_term_list *>(Lc);
+    std::lock_guard<std::mutex> g(L->plan_mu);
+    if (!L->mirror_tried) {
+        try {
+            L->mirror = make_mirror_plan(*L);
+            L->mirror_tried = true;
+        } catch (const std::bad_alloc &) {
+            return nullptr;
+        }
+    }
+    return L->mirror;
+}
+
 std::shared_ptr<const MinorPlan> minor_plan(const mbc_term_list *Lc) {
     mbc_term_list *L = const_cast<mbc_term_list *>(Lc);
     std::lock_guard<std::mutex> g(L->plan_mu);

@@ -138,4 +138,14 @@ struct PairPlan {
 };
 std::shared_ptr<const PairPlan> pair_plan(const mbc_term_list *L);
 
+// Mirror pairs of a pn list's outputs: exchanging the flavours maps the component
+// (sigma_p, sigma_n; U, D) to (sigma_n, sigma_p; D, U) of the same value (u = d),
+// so the step keeps one of each pair: 154 of 296 outputs for the nonrelativistic
+// list with all components (pn, 4^3 x 8: 41.0 -> 30.8 us).
+struct MirrorPlan {
+    std::vector<int32_t> keep;  // outputs computed
+    std::vector<int32_t> rep;   // per output, position in keep
+};
+std::shared_ptr<const MirrorPlan> mirror_plan(const mbc_term_list *L);
+
 }  // namespace mbc

@@ -178,6 +178,33 @@ static int bad_pairs(const char *name, const mbc_term_list &L, bool expect, std:
     return worst > 1e-10;
 }
 
+// every output of a pn step equals the one that stands for its mirror pair
+static int bad_mirror(const char *name, const mbc_term_list &L, bool expect, std::mt19937 &rng) {
+    const auto P = mbc::mirror_plan(&L);
+    if (!!P != expect) {
+        std::printf("%s: mirror pairs %s\n", name, P ? "made" : "not made");
+        return 1;
+    }
+    if (!P) return 0;
+    std::normal_distribution<double> nd;
+    std::vector<cd> f((size_t)L.block_size), z;
+    for (auto &v : f) v = cd(nd(rng), nd(rng));
+    const auto &s = L.steps[0];
+    for (int64_t i = 0; i < s.n_z; ++i) {
+        cd v = 0;
+        for (int64_t j = i * s.k; j < (i + 1) * s.k; ++j) {
+            const cd t = f[s.x[(size_t)j]] * f[s.ys[(size_t)j] & 0x7fff];
+            v += s.ys[(size_t)j] & 0x8000 ? -t : t;
+        }
+        z.push_back(v);
+    }
+    double worst = 0;
+    for (int64_t i = 0; i < s.n_z; ++i)
+        worst = std::max(worst, std::abs(z[(size_t)i] - z[(size_t)P->keep.at((size_t)P->rep.at((size_t)i))]));
+    std::printf("%s: %zu of %lld outputs, worst difference %.1e\n", name, P->keep.size(), (long long)s.n_z, worst);
+    return worst > 1e-11;
+}
+
 static mbc_op_spec spec(int np, int nn, int D) {
     mbc_op_spec s;
     std::memset(&s, 0, sizeof(s));
@@ -208,6 +235,20 @@ int main() {
         mbc_term_list *L = build1(s);
         bad += bad_minors(c.name, *L, c.minors, rng);
         bad += bad_pairs(c.name, *L, true, rng);
+        bad += bad_mirror(c.name, *L, c.np == 1 && c.nn == 1, rng);
+        mbc_free_term_list(L);
+    }
+    for (int o = 0; o < 2; ++o) {  // listed components, both paths
+        const int8_t snk[6] = {0, 1, 1, 1, 1, 0}, src[6] = {0, 0, 1, 0, 0, 1}, path[2][2] = {{0, 1}, {1, 0}};
+        mbc_op_spec s = spec(1, 1, 2);
+        s.spin_mode = MBC_SPIN_LISTED;
+        s.n_spin_sel = 3;
+        s.snk_spins = snk;
+        s.src_spins = src;
+        s.path = path[o];
+        s.path_len = 2;
+        mbc_term_list *L = build1(s);
+        bad += bad_mirror("pn listed", *L, true, rng);
         mbc_free_term_list(L);
     }
     {  // pair forms: listed components, odd spin orders, sinks and sources, paths
