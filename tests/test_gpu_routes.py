@@ -1,0 +1,128 @@
+"""GPU parity at the edges of the contraction's routes: tile remainders, the site
+counts where a launch rule changes kernel, and the forms (minors, determinant,
+pair products, line sums) on shapes where they can go wrong. Bounds as in
+test_gpu_parity (parity.check); closed forms as its full-slab test."""
+import numpy as np
+import pytest
+
+import parity
+import synth
+from gpu_helpers import EPS, legs, oracle_plan, oracle_slab
+from parity import TOL
+from test_gpu_parity import BE8, _be8_K, _check_sparse, check_legs, mbc, run  # noqa: F401  (mbc is the fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dims", [(1, 1, 1), (2, 3, 5), (14, 14, 13)])
+def test_saturated_few_and_many_sites(mbc, dims):
+    """8Be by one determinant per site, four warps per site (few sites) and half a
+    warp (more than 16 per SM: 2,548 sites), three momenta."""
+    from oracle import site_sum
+    field = synth.field(40, 1, 2, dims, 0.1, eps=0.02)
+    tl = mbc.build_term_list(4, 4, 4, spins=[(BE8, BE8)], list_free=True)
+    moms = ((0, 0, 0), (1, 0, 0), (0, 2, 1))
+    for p in (0, 1):
+        got = run(mbc, field, [tl], p, moms=moms)
+        for t in range(2):
+            C = _be8_K() * np.linalg.det(field[0, t].reshape(-1, 12, 12)) ** 2
+            ref = site_sum.site_sum(C[:, None], synth.site_coords(dims), tuple(dims[::-1]), list(moms))[:, 0]
+            # sum|terms| <= 10 |C| at eps = 0.02, as in the full-slab test
+            assert np.max(np.abs(got[0, 0, t, :, 0] - ref)) <= 10 * TOL[p] * np.sum(np.abs(C)), (p, t)
+
+
+@pytest.mark.parametrize("dims", [(1, 2, 3), (14, 14, 13)])
+def test_saturated_pivoting_and_singular_sites(mbc, dims):
+    """Row permutations (every pivot off the diagonal), a zero row, a zero matrix
+    and entries whose squares leave the exponent range."""
+    n = int(np.prod(dims))
+    rng = np.random.default_rng(41)
+    S = np.zeros((n, 12, 12), dtype=np.complex128)
+    perm = rng.permutation(12)
+    S[0] = np.eye(12)[perm] * 1.5
+    S[1] = rng.standard_normal((12, 12)) + 1j * rng.standard_normal((12, 12))
+    S[1, 7] = 0
+    S[2] = np.diag([1e-200, 1e200] + [1.0] * 10)
+    S[n - 1] = np.eye(12)[perm[::-1]] * 1j
+    tl = mbc.build_term_list(4, 4, 4, spins=[(BE8, BE8)], list_free=True)
+    ref = _be8_K() * (1.5 ** 24 + 0.0 + 1.0 + 1.0)  # det^2: 1.5^24, 0, 1, i^24
+    for p in (0, 1):
+        got = run(mbc, S.reshape((1, 1) + dims + (12, 12)), [tl], p)[0, 0, 0, 0, 0]
+        if p == 0:
+            assert abs(got - ref) <= 1e-12 * abs(ref)
+        assert np.isfinite(got.real)
+
+
+@pytest.mark.parametrize("dims", [(1, 1, 31), (3, 11, 1), (1, 5, 13)])
+def test_minor_form_tile_remainders(mbc, dims):
+    """31, 33 and 65 sites: 3He, 3H and 4He around the 32-site tiles."""
+    lists = [mbc.build_term_list(2, 1, 2), mbc.build_term_list(1, 2, 2), mbc.build_term_list(2, 2, 2)]
+    check_legs(mbc, 42, 1, 1, dims, 0.3, lists, [(2, 1, 2), (1, 2, 2), (2, 2, 2)], moms=((0, 0, 0), (1, 0, 2)))
+
+
+@pytest.mark.parametrize("n_p,n_n", [(2, 1), (2, 2), (1, 1)])
+def test_small_kernels_on_more_tiles_than_sms(mbc, n_p, n_n):
+    """17^3 sites (a ragged last tile, more tiles than SMs): FP64 minors with lanes
+    as sites, the tile sums of several warps."""
+    _check_sparse(mbc, 43, (17, 17, 17), 0.4, [0, 31, 32, 2500, 4912], mbc.build_term_list(n_p, n_n, 2), (n_p, n_n, 2))
+
+
+@pytest.mark.parametrize("n_p,n_n,spins", [
+    (1, 1, None),
+    (2, 1, [((0, 1, 2), (0, 1, 0)), ((0, 3, 1), (0, 1, 2))]),
+    (1, 2, [((2, 0, 1), (0, 0, 1))]),
+    (2, 2, [((0, 1, 0, 1), (0, 1, 0, 1)), ((0, 1, 0, 2), (0, 1, 0, 1))]),
+    (2, 2, [((0, 1, 0, 2), (0, 1, 1, 3)), ((0, 2, 0, 1), (1, 3, 0, 1)), ((2, 3, 0, 1), (0, 1, 1, 3))]),
+])
+def test_pair_form_relativistic(mbc, n_p, n_n, spins):
+    """Pair form with one and two baryons per species, one to six spin sets per
+    tile, exchanged flavours and a symmetric matrix; 65 sites (a tile and one)."""
+    dims = (1, 5, 13)
+    tl = mbc.build_term_list(n_p, n_n, 4, spins=spins)
+    check_legs(mbc, 44, 1, 1, dims, 0.3, [tl], [(n_p, n_n, 4)], moms=((0, 0, 0), (0, 1, 2)))
+
+
+@pytest.mark.parametrize("dims", [(1, 1, 1), (3, 2, 7), (2, 5, 3)])
+@pytest.mark.parametrize("n_p,n_n,D,spins", [(2, 1, 2, None), (1, 1, 4, [((0, 3), (1, 2)), ((2, 2), (0, 1))])])
+def test_projection_lines_and_passes(mbc, dims, n_p, n_n, D, spins):
+    """Line sums on odd extents with 7 momenta: two passes, up to four distinct n_x
+    in one, some equal modulo the extent."""
+    from oracle import projection
+    moms = ((0, 0, 0), (1, 0, 0), (2, 1, 0), (-1, 0, 3), (7, 1, 1), (0, 2, 1), (1, 1, 1))
+    tl = mbc.build_term_list(n_p, n_n, D, spins=spins)
+    comps = tl.components()
+    plan = oracle_plan(n_p, n_n, D, comps)
+    for field, precs in legs(45, 1, 2, dims, 0.3, gauss=False):
+        for p in precs:
+            got = run(mbc, field, [tl], p, moms=moms, sink=mbc.SINK_BLOCK_MOMENTUM)
+            for t in range(2):
+                C, sc = projection.projected_correlators(plan, field[0, t], dims, moms)
+                parity.check(got[0, 0, t, :, : len(comps)], C, sc, p, what=f"lines {dims} ({n_p},{n_n}) t {t}")
+
+
+def test_zero_momentum_without_phase_table(mbc):
+    """Calls at zero momentum alone use no phase table: the same bits as the zero
+    momentum of a call with others."""
+    dims = (3, 5, 7)
+    field = synth.field(46, 1, 2, dims, 0.3, eps=EPS)
+    sp = (0, 1, 0, 1)
+    lists = [mbc.build_term_list(1, 1, 2), mbc.build_term_list(2, 1, 2), mbc.build_term_list(2, 2, 4, spins=[(sp, sp)])]
+    for p in (0, 1):
+        one = run(mbc, field, lists, p)
+        two = run(mbc, field, lists, p, moms=((0, 0, 0), (1, 0, 2)))
+        assert np.array_equal(one[..., 0, :], two[..., 0, :]), p
+
+
+def test_block_slices_on_two_relativistic_sources(mbc):
+    """24-column tiles (triangular diquarks, entry slices) on pn, 5 sites."""
+    from oracle import gamma, recursion
+    dims = (1, 1, 5)
+    spins = [((0, 3), (1, 6)), ((2, 1), (0, 3))]
+    tl = mbc.build_term_list(1, 1, 4, spins=spins, n_sources=2)
+    comps = tl.components()
+    plan = recursion.Plan(1, 1, 4, requests=comps, G=gamma.g_tensor_sources(4, 2), G_sink=gamma.g_tensor(4))
+    for field, precs in legs(47, 1, 1, dims, 0.3, n_src=2):
+        ref, scale = oracle_slab(plan, recursion.source_columns(field[0, 0], 4), dims, [(0, 0, 0)])
+        for p in precs:
+            got = run(mbc, field, [tl], p)[0, 0, 0, :, : len(comps)]
+            parity.check(got, ref, scale[None, :], p, what="24 columns")
