@@ -29,6 +29,7 @@
 #pragma once
 
 #include "large_kernel.cuh"
+#include "plan.h"
 
 namespace mbc {
 
@@ -89,11 +90,6 @@ __global__ void __launch_bounds__(32 * kProdWarps, 1)
         }
     }
 }
-
-// Gathered entries a pack names at most: with two spin sets 208 rows of 512 B
-// fill an SM's shared memory; one set takes half of it, so two CTAs overlap one's
-// copies with the other's sums.
-constexpr int kPackCols = 208;
 
 struct PairPack {
     int64_t row0;    // rows [row0, row0 + n_rows)

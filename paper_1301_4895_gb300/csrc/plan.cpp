@@ -571,16 +571,17 @@ std::shared_ptr<const PairPlan> make_pair_plan(const mbc_term_list &L) {
         const int64_t nnz0 = (int64_t)P->col.size(), rows0 = (int64_t)P->row_id.size();
         for (int s = 0; s < 2; ++s) {
             G.row0[s] = (int64_t)P->row_id.size();
-            for (const auto &r : lam[g].rows[s]) {
-                for (int64_t e = r.e0; e < r.e1; ++e) {
-                    const uint32_t j = lam[g].col[(size_t)e];
-                    P->col.push_back(n_side[1 - s] == 2 ? (uint32_t)row_of[j] : j);
-                    P->val.push_back(lam[g].val[(size_t)e]);
+            for (const auto &r : lam[g].rows[s])
+                for (int64_t e0 = r.e0; e0 < r.e1; e0 += kPackCols) {  // a longer row goes in pieces
+                    for (int64_t e = e0; e < std::min(r.e1, e0 + kPackCols); ++e) {
+                        const uint32_t j = lam[g].col[(size_t)e];
+                        P->col.push_back(n_side[1 - s] == 2 ? (uint32_t)row_of[j] : j);
+                        P->val.push_back(lam[g].val[(size_t)e]);
+                    }
+                    P->row_class.push_back(r.cls);
+                    P->row_id.push_back(n_side[s] == 2 ? (uint32_t)row_of[r.id] : r.id);
+                    P->row_ptr.push_back((int64_t)P->col.size());
                 }
-                P->row_class.push_back(r.cls);
-                P->row_id.push_back(n_side[s] == 2 ? (uint32_t)row_of[r.id] : r.id);
-                P->row_ptr.push_back((int64_t)P->col.size());
-            }
             G.row1[s] = (int64_t)P->row_id.size();
         }
         lam[g] = PairRows();

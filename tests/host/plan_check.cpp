@@ -122,6 +122,8 @@ static int bad_pairs(const char *name, const mbc_term_list &L, bool expect, std:
     std::vector<cd> C, prod;
     std::vector<double> mag;
     chain(L, f, C, mag);
+    for (size_t r = 0; r < P->row_id.size(); ++r)
+        if (P->row_ptr[r + 1] - P->row_ptr[r] > mbc::kPackCols) return 1;
     const int64_t npair = (int64_t)L.nxi * (L.nxi - 1) / 2;
     for (uint32_t m : P->masks2) {
         const int s1 = __builtin_ctz(m), s2 = __builtin_ctz(m & (m - 1));
@@ -304,6 +306,30 @@ int main() {
         mbc_term_list *L = build1(s);
         bad += bad_minors("3He projections", *L, true, rng);
         bad += bad_pairs("3He projections", *L, true, rng);
+        mbc_free_term_list(L);
+    }
+    {  // a projection over every source set: rows of up to 1,311 entries
+        std::vector<int8_t> snk, src;
+        std::vector<int32_t> to;
+        std::vector<double> w;
+        for (int8_t a = 0; a < 4; ++a)
+            for (int8_t b = (int8_t)(a + 1); b < 4; ++b)
+                for (int8_t c = 0; c < 4; ++c) {
+                    for (int8_t v : {0, 1, 0}) snk.push_back(v);
+                    for (int8_t v : {a, b, c}) src.push_back(v);
+                    to.push_back(0);
+                    w.push_back(0.25 + 0.125 * (double)to.size());
+                }
+        mbc_op_spec s = spec(2, 1, 4);
+        s.spin_mode = MBC_SPIN_PROJECTED;
+        s.n_spin_sel = (int)to.size();
+        s.n_proj = 1;
+        s.snk_spins = snk.data();
+        s.src_spins = src.data();
+        s.term_proj = to.data();
+        s.term_coef = w.data();
+        mbc_term_list *L = build1(s);
+        bad += bad_pairs("3He rel, every source set", *L, true, rng);
         mbc_free_term_list(L);
     }
     {  // two nuclei on one path, both orders of adding baryons

@@ -9,7 +9,8 @@ import parity
 import synth
 from gpu_helpers import EPS, legs, oracle_plan, oracle_slab
 from parity import TOL
-from test_gpu_parity import BE8, _be8_K, _check_sparse, check_legs, mbc, run  # noqa: F401  (mbc is the fixture)
+from test_gpu_parity import (BE8, _be8_K, _check_sparse, check_legs, mbc, run,  # noqa: F401  (mbc is the fixture)
+                             test_spin_projection_outputs as check_projections)
 
 pytestmark = pytest.mark.gpu
 
@@ -80,6 +81,14 @@ def test_pair_form_relativistic(mbc, n_p, n_n, spins):
     dims = (1, 5, 13)
     tl = mbc.build_term_list(n_p, n_n, 4, spins=spins)
     check_legs(mbc, 44, 1, 1, dims, 0.3, [tl], [(n_p, n_n, 4)], moms=((0, 0, 0), (0, 1, 2)))
+
+
+def test_pair_form_long_rows(mbc):
+    """A projection over every source set: Lambda rows of up to 1,311 entries, more
+    than a pack of gathered rows holds (the weights exact in FP32)."""
+    sources = [(a, b, c) for a in range(4) for b in range(a + 1, 4) for c in range(4)]
+    terms = [((0, 1, 0), src, 0.25 + 0.125 * k) for k, src in enumerate(sources)]
+    check_projections(mbc, 2, 1, 4, [terms])
 
 
 @pytest.mark.parametrize("dims", [(1, 1, 1), (3, 2, 7), (2, 5, 3)])
