@@ -42,6 +42,15 @@ __device__ __forceinline__ void bulk_copy_g2s(void *dst, const void *src, uint32
         : "memory");
 }
 
+// one lane's 16 bytes, global to shared, both 16-byte aligned, without a register;
+// async_copy_wait_all: this thread's copies have landed
+__device__ __forceinline__ void async_copy16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void async_copy_wait_all() {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 // order this thread's earlier generic-proxy accesses of shared memory before
 // later async-proxy ones (a bulk copy overwriting what was just read)
 __device__ __forceinline__ void fence_proxy_async_smem() {

@@ -620,7 +620,7 @@ PairLayout pair_layout(const PairPlan &P, const int shape[2], int n_sm) {
     std::vector<uint16_t> pos((size_t)n_cols, 0);
     Q.slot.resize(P.col.size());
     for (size_t r = 0; r < P.row_id.size(); ++r)
-        Q.rows.push_back({P.row_id[r], (uint32_t)(P.row_ptr[r + 1] - P.row_ptr[r]), P.row_ptr[r]});
+        Q.rows.push_back({P.row_id[r] | (uint32_t)(P.row_ptr[r + 1] - P.row_ptr[r]) << 24, (uint32_t)P.row_ptr[r]});
     Q.slot_off.assign((size_t)P.n_evals + 1, 0);
     std::vector<uint16_t> cls;
     int32_t slot = 0;
@@ -654,7 +654,7 @@ PairLayout pair_layout(const PairPlan &P, const int shape[2], int n_sm) {
                 }
                 // longest rows first: the warps' rows of a round are then of one length
                 std::stable_sort(Q.rows.begin() + pk.row0, Q.rows.begin() + pk.row0 + pk.n_rows,
-                                 [](const PairRow &a, const PairRow &b) { return a.n > b.n; });
+                                 [](const PairRow &a, const PairRow &b) { return a.n() > b.n(); });
                 Q.packs.push_back(pk);
                 if (acc >= target || r >= g.row1[s]) {
                     cut[s].push_back((int32_t)Q.packs.size());
@@ -1387,9 +1387,9 @@ mbc_status pair_wave(const mbc_term_list *L, const DeviceCache *c, int W, const 
         const void *kern = shape == 0   ? (const void *)k_pair<T, 1, 1, kW[0]>
                            : shape == 1 ? (const void *)k_pair<T, 2, 2, kW[1]>
                                         : (const void *)k_pair<T, 6, 2, kW[2]>;
-        const size_t smem = shape == 0   ? pair_smem<T, 1, kW[0]>()
-                            : shape == 1 ? pair_smem<T, 2, kW[1]>()
-                                         : pair_smem<T, 2, kW[2]>();
+        const size_t smem = shape == 0   ? pair_smem<T, 1, 1, kW[0]>()
+                            : shape == 1 ? pair_smem<T, 2, 2, kW[1]>()
+                                         : pair_smem<T, 6, 2, kW[2]>();
         int per_sm = 0;
         mbc_status st = prepare_kernel(kern, c->device, threads, smem, &per_sm);
         if (st != MBC_OK) return st;

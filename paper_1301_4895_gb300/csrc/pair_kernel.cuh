@@ -23,9 +23,10 @@
 // the pipe) and its few warps' latencies. Whole calls on GB300 against the
 // recursion (8.5 M complex multiply-adds per site for one component, here 0.37 M
 // for the products and 0.31 M real-complex ones; 531 M for all 1296): one
-// component mixed, 16^3 x 4, 125.2 -> 9.3 ms (12.1 with L2 gathers, rows in rank
-// order); all, FP64, 64 sites, 233.7 -> 20.4 ms (26.9); all, mixed, 512 sites,
-// 227.7 -> 24.2 ms (70.8).
+// component mixed, 16^3 x 4, 125.2 -> 8.7 ms; all, FP64, 64 sites, 233.7 -> 19.5
+// ms; all, mixed, 512 sites, 210.1 -> 19.9 ms. With L2 gathers and rows in rank
+// order 12.1, 26.9 and 70.8; with rows staged through registers (one load's
+// latency per row and warp, 10 % of a pack's time) 9.35, 20.0 and 24.2.
 #pragma once
 
 #include "large_kernel.cuh"
@@ -54,8 +55,9 @@ __global__ void __launch_bounds__(32 * kProdWarps, 1)
     const ulonglong2 *ft = f + tile * block_rows * 32;
     for (int r = warp; r < 4 * npair; r += kProdWarps) {
         const int s = r / (2 * npair), i = r / npair & 1, p = r % npair;
-        rows[r * 32 + lane] = __ldg(ft + ((int64_t)(spin[s] * npair + p) * nxi + e[i]) * 32 + lane);
+        async_copy16(rows + r * 32 + lane, ft + ((int64_t)(spin[s] * npair + p) * nxi + e[i]) * 32 + lane);
     }
+    async_copy_wait_all();
     __syncthreads();
     const ulonglong2 *F = rows + lane, *G = rows + 2 * npair * 32 + lane;
     ulonglong2 *out = prod + ((tile * n_masks + m) * n_rows) * 32 + lane;
@@ -105,10 +107,13 @@ struct PairUnit {
     int32_t re[6], ge[6];
     int32_t slot, stride_r, stride_g;
 };
-struct __align__(16) PairRow {
-    uint32_t row, n;  // row-side row, entries [e0, e0 + n)
-    int64_t e0;
+struct __align__(8) PairRow {
+    uint32_t row_n;  // row-side row | entries << 24
+    uint32_t e0;     // first entry
+    __host__ __device__ uint32_t row() const { return row_n & 0xffffffu; }
+    __host__ __device__ uint32_t n() const { return row_n >> 24; }
 };
+static_assert(kPackCols < 256, "PairRow::n");
 
 struct PairArgs {
     const PairUnit *units;
@@ -194,11 +199,21 @@ struct PairMx {
     using Factor = uint64_t;
 };
 
-// dynamic shared memory: the pack's rows [MG][kPackCols][32 lanes], then 32
-// records per warp; the partial sums of a unit reuse the rows' room
-template <class T, int MG, int WARPS>
+// Row-side values a warp holds in registers while it sums y; the others of MR
+// (six spin sets, mixed: the accumulators leave no room) come by its own copies
+// through shared memory meanwhile (all components, mixed, 512 sites: 19.0 ms, 19.3
+// where they are loaded after y).
+template <class T, int MR>
+__host__ __device__ constexpr int pair_held() {
+    return T::kSites == 1 || MR <= 2 ? MR : MR / 2;
+}
+// dynamic shared memory: the pack's rows [MG][kPackCols][32 lanes], 32 records per
+// warp, its row-side values [MR - held][32 lanes]; the partial sums of a unit reuse
+// the pack's room
+template <class T, int MR, int MG, int WARPS>
 __host__ __device__ constexpr size_t pair_smem() {
-    return (size_t)MG * kPackCols * 512 + (size_t)WARPS * 32 * sizeof(typename T::Rec);
+    return (size_t)MG * kPackCols * 512 +
+           (size_t)WARPS * (32 * sizeof(typename T::Rec) + (MR - pair_held<T, MR>()) * 512);
 }
 
 template <class T, int MR, int MG, int WARPS>
@@ -209,6 +224,10 @@ __global__ void __launch_bounds__(32 * WARPS, MG == 1 ? 2 : 1)
     ulonglong2 *stage = reinterpret_cast<ulonglong2 *>(smem_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     typename T::Rec *rec = reinterpret_cast<typename T::Rec *>(smem_raw + (size_t)MG * kPackCols * 512) + warp * 32;
+    ulonglong2 *xs = reinterpret_cast<ulonglong2 *>(smem_raw + (size_t)MG * kPackCols * 512 +
+                                                    (size_t)WARPS * 32 * sizeof(typename T::Rec)) +
+                     warp * (MR - pair_held<T, MR>()) * 32 + lane;
+    __shared__ uint32_t Ro[MR];
     const int64_t n_items = (int64_t)A.n_units * A.n_tiles;
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
         const PairUnit &u = A.units[item % A.n_units];
@@ -216,11 +235,9 @@ __global__ void __launch_bounds__(32 * WARPS, MG == 1 ? 2 : 1)
         const ulonglong2 *Pt = P + tile * A.p_tile * 32 + lane, *Nt = N + tile * A.n_tile * 32 + lane;
         const ulonglong2 *Rs = u.swap ? Nt : Pt, *Gs = u.swap ? Pt : Nt;
         const int64_t r_rows = u.swap ? A.n_rows : A.p_rows, g_rows = u.swap ? A.p_rows : A.n_rows;
-        uint32_t Ro[MR];  // 16-byte words from Rs
-#pragma unroll
-        for (int a = 0; a < MR; ++a) Ro[a] = (uint32_t)(u.re[min(a, u.nr - 1)] * r_rows) * 32u;
-        // row-side values on their way while y is summed; the others follow (mixed: registers)
-        constexpr int H = T::kSites == 1 ? MR : (MR + 1) / 2;
+        // 16-byte words from Rs (shared memory: registers are short in the mixed form)
+        if (threadIdx.x < MR) Ro[threadIdx.x] = (uint32_t)(u.re[min((int)threadIdx.x, u.nr - 1)] * r_rows) * 32u;
+        constexpr int H = pair_held<T, MR>();
         typename T::Acc acc[MR][MG];
 #pragma unroll
         for (int a = 0; a < MR; ++a)
@@ -229,22 +246,26 @@ __global__ void __launch_bounds__(32 * WARPS, MG == 1 ? 2 : 1)
         for (int k = u.pack0; k < u.pack1; ++k) {
             const PairPack pk = A.packs[k];
             __syncthreads();  // the previous pack (or unit) is done with the rows
-            for (int c = warp; c < pk.n_cols; c += WARPS) {
-                const int64_t row = (int64_t)__ldg(A.cols + pk.col0 + c) * 32;
+            static_assert(kPackCols <= 32 * WARPS, "a lane holds one of its warp's columns");
+            const uint32_t mine = warp + WARPS * lane < pk.n_cols ? __ldg(A.cols + pk.col0 + warp + WARPS * lane) : 0u;
+            for (int c = warp, i = 0; c < pk.n_cols; c += WARPS, ++i) {
+                const int64_t row = (int64_t)__shfl_sync(0xffffffffu, mine, i) * 32;
 #pragma unroll
                 for (int b = 0; b < MG; ++b)
-                    stage[(b * kPackCols + c) * 32 + lane] = __ldg(Gs + (int64_t)u.ge[min(b, u.ng - 1)] * g_rows * 32 + row);
+                    async_copy16(stage + (b * kPackCols + c) * 32 + lane,
+                                 Gs + (int64_t)u.ge[min(b, u.ng - 1)] * g_rows * 32 + row);
             }
+            async_copy_wait_all();
             __syncthreads();
             const ulonglong2 *G = stage + lane;
             // two rows ahead: the next row's records are loaded while this one is
             // worked off, and the row after gives their place
-            const PairRow none{0u, 0u, 0};
+            const PairRow none{0u, 0u};
             const PairRow *rows = A.rows + pk.row0;
             PairRow row = warp < pk.n_rows ? rows[warp] : none;
             PairRow next = warp + WARPS < pk.n_rows ? rows[warp + WARPS] : none;
             auto load = [&](const PairRow &w, uint32_t e0, double &v, uint32_t &o) {
-                if (e0 + lane < w.n) {
+                if (e0 + lane < w.n()) {
                     v = __ldg(A.val + w.e0 + e0 + lane);
                     o = __ldg(A.slot + w.e0 + e0 + lane);
                 }
@@ -253,20 +274,22 @@ __global__ void __launch_bounds__(32 * WARPS, MG == 1 ? 2 : 1)
             uint32_t ro = 0;
             load(row, 0, rv, ro);
             for (int r = warp; r < pk.n_rows; r += WARPS) {
-                const ulonglong2 *Rr = Rs + row.row * 32u;
+                const ulonglong2 *Rr = Rs + row.row() * 32u;
                 ulonglong2 x[H];
 #pragma unroll
                 for (int a = 0; a < H; ++a) x[a] = __ldg(Rr + Ro[a]);
+#pragma unroll
+                for (int a = H; a < MR; ++a) async_copy16(xs + (a - H) * 32, Rr + Ro[a]);
                 const PairRow after = r + 2 * WARPS < pk.n_rows ? rows[r + 2 * WARPS] : none;
                 typename T::Y y[MG];
 #pragma unroll
                 for (int b = 0; b < MG; ++b) y[b].zero();
-                for (uint32_t e0 = 0; e0 < row.n; e0 += 32) {
-                    const int n = (int)min(32u, row.n - e0);
+                for (uint32_t e0 = 0; e0 < row.n(); e0 += 32) {
+                    const int n = (int)min(32u, row.n() - e0);
                     __syncwarp();
                     rec[lane] = T::rec(ro * 32u, rv);
                     __syncwarp();
-                    if (e0 + 32 < row.n)
+                    if (e0 + 32 < row.n())
                         load(row, e0 + 32, rv, ro);
                     else
                         load(next, 0, rv, ro);
@@ -295,17 +318,17 @@ __global__ void __launch_bounds__(32 * WARPS, MG == 1 ? 2 : 1)
                                 for (int b = 0; b < MG; ++b) y[b].add(G[b * kPackCols * 32 + off[q]], v[q]);
                     }
                 }
-                ulonglong2 x2[MR > H ? MR - H : 1];
-#pragma unroll
-                for (int a = H; a < MR; ++a) x2[a - H] = __ldg(Rr + Ro[a]);
 #pragma unroll
                 for (int a = 0; a < H; ++a)
 #pragma unroll
                     for (int b = 0; b < MG; ++b) acc[a][b].fma(x[a], y[b]);
+                if constexpr (H < MR) async_copy_wait_all();  // a lane reads what it copied
 #pragma unroll
-                for (int a = H; a < MR; ++a)
+                for (int a = H; a < MR; ++a) {
+                    const ulonglong2 v = xs[(a - H) * 32];
 #pragma unroll
-                    for (int b = 0; b < MG; ++b) acc[a][b].fma(x2[a - H], y[b]);
+                    for (int b = 0; b < MG; ++b) acc[a][b].fma(v, y[b]);
+                }
                 row = next;
                 next = after;
             }

@@ -105,10 +105,10 @@ std::shared_ptr<const SaturatedPlan> saturated_plan(const mbc_term_list *L);
 // row's entries share), block and columns, so that the rows of neighbouring
 // warps gather the same entries.
 // Gathered entries that a pack of rows names at most (k_pair): with two spin sets
-// 208 rows of 512 B fill an SM's shared memory; one set takes half of it, so two
+// 204 rows of 512 B fill an SM's shared memory; one set takes half of it, so two
 // CTAs overlap one's copies with the other's sums. No row is longer (88 entries in
 // 4He with all components; projections over many source sets reach 1,311, in pieces).
-constexpr int kPackCols = 208;
+constexpr int kPackCols = 204;
 struct PairPlan {
     int np = 0, nn = 0;  // baryons per species: 1 or 2
     // two-baryon products: element m (spin set masks2[m]), row r at m * n_rows2 +
