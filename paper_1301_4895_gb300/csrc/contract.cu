@@ -1400,7 +1400,12 @@ mbc_status pair_wave(const mbc_term_list *L, const DeviceCache *c, int W, const 
         MBC_CUDA_TRY(cudaLaunchKernel(kern, dim3((unsigned)grid), dim3(threads), args, smem, stream));
     }
     note_launch();
-    k_pair_sum<<<dim3((unsigned)L->n_comp, (unsigned)(W / 32)), 1024, 0, stream>>>(
+    // wide: too few CTAs of the other shape to fill the SMs, and the slots that a
+    // component sums on average make long chains for its four groups
+    const bool wide = (int64_t)L->n_comp * W < 32LL * nsm &&
+                      c->pair_slots * (int64_t)P.comp_eval.size() >= 32 * P.n_evals * (int64_t)L->n_comp;
+    auto *sum = wide ? k_pair_sum<8, 128> : k_pair_sum<32, 4>;
+    sum<<<dim3((unsigned)L->n_comp, (unsigned)(W / (wide ? 8 : 32))), wide ? 1024 : 128, 0, stream>>>(
         c->d_pair_comp_off, c->d_pair_comp_eval, c->d_pair_slot_off, W, part, sexp, deg_per_baryon * L->A, P.scale, Cb);
     MBC_CUDA_TRY(cudaGetLastError());
     return MBC_OK;

@@ -360,33 +360,50 @@ __global__ void __launch_bounds__(32 * WARPS, MG == 1 ? 2 : 1)
 }
 
 // Cout[comp][site]: the partials of the component's evaluations (slots
-// [slot_off[ev], slot_off[ev + 1])), warp w of the CTA adding slots w, w + 32,
-// ..., the warps' sums then in warp order. FP64: an SM's four FP64 units take a
-// warp's addition 64 cycles each, hence 32 warps per 32 sites.
-__global__ void __launch_bounds__(1024) k_pair_sum(const int32_t *__restrict__ comp_off,
-                                                   const int32_t *__restrict__ comp_eval,
-                                                   const int32_t *__restrict__ slot_off, int W,
-                                                   const double2 *__restrict__ part, const int32_t *__restrict__ sexp,
-                                                   int degree, double scale, double2 *__restrict__ Cout) {
-    __shared__ double2 sums[32][33];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.x;
-    const int col = blockIdx.y * 32 + lane;
+// [slot_off[ev], slot_off[ev + 1])) of S sites per CTA: group g of G adds slots g,
+// g + G, ..., the groups' sums then in a fixed order. An SM's four FP64 units take
+// a warp's addition 64 cycles each, so the shape follows the work. Enough CTAs
+// (all components): 32 sites, 4 groups, no tree - 0.09 ms for 512 sites, where 32
+// warps and a tree per CTA took 0.91. Else (one component): 8 sites and 128 groups,
+// which spreads the additions over the SMs - 6.2 us for 1,024 sites (10 with 4
+// groups, 12.5 with 32 warps on 32 sites).
+template <int S, int G>
+__global__ void __launch_bounds__(S * G) k_pair_sum(const int32_t *__restrict__ comp_off,
+                                                    const int32_t *__restrict__ comp_eval,
+                                                    const int32_t *__restrict__ slot_off, int W,
+                                                    const double2 *__restrict__ part, const int32_t *__restrict__ sexp,
+                                                    int degree, double scale, double2 *__restrict__ Cout) {
+    __shared__ double2 sums[G][S + 1];
+    const int site = threadIdx.x % S, g = threadIdx.x / S, c = blockIdx.x;
+    const int col = blockIdx.y * S + site;
     double2 s = make_double2(0.0, 0.0);
     for (int k = comp_off[c]; k < comp_off[c + 1]; ++k) {
         const int ev = comp_eval[k];
-        for (int t = slot_off[ev] + warp; t < slot_off[ev + 1]; t += 32) s = cadd(s, part[(int64_t)t * W + col]);
+        for (int t = slot_off[ev] + g; t < slot_off[ev + 1]; t += G) s = cadd(s, part[(int64_t)t * W + col]);
     }
-    sums[warp][lane] = s;
+    sums[g][site] = s;
     __syncthreads();
-    // transposed: warp w adds the 32 sums of site w by a fixed tree
-    s = sums[lane][warp];
-    for (int off = 16; off > 0; off >>= 1) {
-        s.x += __shfl_xor_sync(0xffffffffu, s.x, off);
-        s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
+    int out = -1;  // the site this thread writes
+    if constexpr (G <= 8) {
+        if (g == 0) {
+            for (int q = 1; q < G; ++q) s = cadd(s, sums[q][site]);
+            out = site;
+        }
+    } else {  // a warp per site: lane l adds groups l, l + 32, ..., then a fixed tree
+        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+        if (w < S) {
+            s = sums[lane][w];
+            for (int q = lane + 32; q < G; q += 32) s = cadd(s, sums[q][w]);
+            for (int off = 16; off > 0; off >>= 1) {
+                s.x += __shfl_xor_sync(0xffffffffu, s.x, off);
+                s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
+            }
+            if (lane == 0) out = w;
+        }
     }
-    if (lane == 0) {
-        const int site = blockIdx.y * 32 + warp, ue = -degree * sexp[site];
-        Cout[(int64_t)c * W + site] = make_double2(scalbn(s.x * scale, ue), scalbn(s.y * scale, ue));
+    if (out >= 0) {
+        const int at = blockIdx.y * S + out, ue = -degree * sexp[at];
+        Cout[(int64_t)c * W + at] = make_double2(scalbn(s.x * scale, ue), scalbn(s.y * scale, ue));
     }
 }
 
