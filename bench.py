@@ -99,18 +99,6 @@ def shared_path(nuclei):
     return path
 
 
-def site_flops(st, dirac_dim):
-    nxi = 3 * dirac_dim
-    n_g2 = 4 if dirac_dim == 4 else 2
-    n_blocks = len(set(st["path"]))
-    diquark = 3 * nxi * nxi * (2 * n_g2) * 8
-    blocks = n_blocks * st["block_size"] * 6 * 8
-    recursion = 8 * st["n_ops_total"]
-    contraction = 4 * st["n_l_total"]
-    return {"recursion": recursion, "blocks": diquark + blocks, "contraction": contraction,
-            "total": recursion + diquark + blocks + contraction}
-
-
 class ClockSampler:
     """nvidia-smi clock / throttle samples during the timed region."""
 
@@ -129,7 +117,7 @@ class ClockSampler:
         try:
             self.f = open(self.path, "w")
             self.proc = subprocess.Popen(["nvidia-smi", f"--id={self.index}", f"--query-gpu={q}",
-                                          "--format=csv,noheader,nounits", "-lms", "200"], stdout=self.f,
+                                          "--format=csv,noheader,nounits", "-lms", "20"], stdout=self.f,
                                          stderr=subprocess.DEVNULL)
         except OSError:
             self.proc = None
@@ -143,6 +131,20 @@ class ClockSampler:
             except subprocess.TimeoutExpired:
                 self.proc.kill()
             self.f.close()
+
+    def load(self, step, sync, limit_s=3.0):
+        """Untimed steps until three samples are in: a timed region of a few
+        milliseconds would else end before the first one."""
+        t_end = time.perf_counter() + (limit_s if self.proc is not None else 0.0)
+        while time.perf_counter() < t_end:
+            step()
+            sync()
+            try:
+                with open(self.path) as f:
+                    if sum(1 for _ in f) >= 3:
+                        return
+            except OSError:
+                return
 
     def summary(self):
         if self.proc is None or not os.path.exists(self.path):
@@ -374,23 +376,48 @@ def run_reference(args, wl):
     return 0
 
 
-def point_flops_per_site(stats, list_dims):
-    """Algorithmic flops per sink site of point-sink lists: recursion (8 per
-    operation) and contraction of every list, plus one diquark and one block
-    per species and operator type (the blocks of a site do not depend on the
-    nucleus, Sec. 2)."""
-    fl = [site_flops(st, d) for st, d in zip(stats, list_dims)]
-    per_site = sum(f["recursion"] + f["contraction"] for f in fl)
-    for d in sorted(set(list_dims)):
-        nxi = 3 * d
-        species = set()
-        bs = 0
-        for st, dd in zip(stats, list_dims):
-            if dd == d:
-                species |= set(st["path"])
-                bs = st["block_size"]
-        per_site += 3 * nxi * nxi * (2 * (4 if d == 4 else 2)) * 8 + len(species) * bs * 6 * 8
-    return per_site
+def point_flops_per_site(lists, precision):
+    """Flops per sink site of point-sink lists in the forms that a call with
+    default tuning evaluates (TermList.form; each list's blocks counted once)."""
+    return sum(tl.form(0, precision)[1] for tl in lists)
+
+
+def projected_flops(lists, list_dims, n_src, n_sinks, moms, lx, precision):
+    """(flops per site, flops per (configuration, time slice)) of projected
+    blocks: diquarks, the entries g of S Q and their sums per distinct n_x over a
+    line; recursion or pair form per momentum group."""
+    per_site = per_slab = 0.0
+    nx = {m[0] % lx for m in moms}
+    for tl, d in zip(lists, list_dims):
+        nxi = 3 * d * n_src
+        ntri = nxi * (nxi + 1) // 2
+        g = d * nxi * ntri
+        per_site += 3 * ntri * 2 * (4 if d == 4 else 2) * 8 + g * (3 * 8 + sum(2 if n == 0 else 8 for n in nx))
+        per_slab += tl.form(1, precision)[1] * (len(moms) // n_sinks)
+    return per_site, per_slab
+
+
+# kernels that take most of a form's time: FP64, mixed
+FORM_KERNELS = {"recursion": ("k_large_step", "k_large_step_split"), "minors": ("k_minors", "k_minors"),
+                "saturated": ("k_saturated", "k_saturated"), "pair": ("k_pair + k_pair_prod", "k_pair + k_pair_prod")}
+
+
+def form_kernels(lists, sink, precision):
+    names = []
+    for tl in lists:
+        form = tl.form(sink, precision)[0]
+        if form == "recursion" and sink == 0 and tl.spec.get("dirac_dim") == 2 and not tl.spec.get("list_free"):
+            names.append(("k_small", "k_small_ls")[precision])
+        else:
+            names.append(FORM_KERNELS[form][precision])
+    return " + ".join((["k_project"] if sink else []) + sorted(set(names)))
+
+
+def operand_bound(lists, sink, precision, n_sm, sm_max_mhz):
+    """l1_operand_bound where it applies: mixed lists that run the recursion."""
+    if precision == 1 and all(tl.form(sink, 1)[0] == "recursion" for tl in lists):
+        return l1_operand_bound(n_sm, sm_max_mhz)
+    return None
 
 
 def l1_operand_bound(n_sm, sm_max_mhz):
@@ -417,32 +444,28 @@ def roofline_entry(flops_step, steps, kms, ms, launches, peak, probe, kind, kern
             "peak": l1_peak / 1e12, "unit": "TFLOP/s", "frac": ach / l1_peak,
             "kind": "derived: SMs x 128 B/clk (one L1/shared-memory wavefront) x max SM clock / 16 B of FP32 "
                     "complex operands per site-operation x 8 flop; the data pipe, not the FP32 pipe, bounds the "
-                    "mixed recursion (ncu: 63 % of a wavefront per SM clock in k_small_ls on the default workload, "
-                    "81 % L1/shared throughput in k_large_step_split on 8Be's largest step)"}
+                    "mixed recursion"}
     return r
 
 
 # Configurations of the metric's headline nuclei reported beside the default
-# line: (workload, what the entry covers, oracle sample sites, profile of the
-# dominant kernels' DRAM traffic per site: FP64, mixed).
+# line: (workload, what the entry covers, oracle sample sites).
 PER_CONFIG = {
     "he4rel_all_components": (
         "he4rel", "4He relativistic, all 1296 spin components (Table 1: 531,321,120 operations per site), "
-        "one 16^3 slab (t = 0) of the 16^3x32 lattice, complex128, seed 2", 8,
-        ("k_large_step_fp64_he4rel_all_16x16x16x1.md", "k_large_step_split_mixed_he4rel_all_16x16x16x1.md")),
+        "one 16^3 slab (t = 0) of the 16^3x32 lattice, complex128, seed 2", 8),
     "be8": (
         "be8", "8Be relativistic (0,1,2,3,0,1,2,3) (Tables 1, 5: 448,496,928 operations per site), one 16^3 slab "
-        "(configuration 0, t = 0) of the 16^3x32 x 12 lattice, complex64 storage, seed 4", 8,
-        ("k_large_step_fp64_be8_16x16x16x1.md", "k_large_step_split_mixed_be8_16x16x16x1.md")),
+        "(configuration 0, t = 0) of the 16^3x32 x 12 lattice, complex64 storage, seed 4", 8),
 }
 
 
-def per_config_entry(mbc, torch, dev, name, peaks, n_sm, probes, warmup=3, steps64=1, steps_mx=3):
+def per_config_entry(mbc, torch, dev, name, peaks, n_sm, probes, warmup=3, steps64=5, steps_mx=5):
     """FP64 and mixed throughput of one headline configuration on one slab
     (the full lattices scale linearly in slabs: no work is shared between
     slabs), with its roofline, clocks, host-buffer e2e (mixed) and the oracle
     on a bounded sample of the same slab."""
-    key, what, cpu_sites, prof = PER_CONFIG[name]
+    key, what, cpu_sites = PER_CONFIG[name]
     wl = WORKLOADS[key]
     _, nuclei, dims, _, _, _, _ = wl
     nt = 1
@@ -453,39 +476,38 @@ def per_config_entry(mbc, torch, dev, name, peaks, n_sm, probes, warmup=3, steps
     stream = torch.cuda.Stream(dev)
     v3 = dims[0] * dims[1] * dims[2]
     units = v3 * nt * len(nuclei)
-    flops_step = point_flops_per_site(stats, [n[2] for n in nuclei]) * v3 * nt
+    flops_step = {p: point_flops_per_site(lists, p) * v3 * nt for p in (0, 1)}
     sm_max = float(peaks.get("sm_max_mhz", 2070.0))
     peak = {0: n_sm * 2 * 2 * sm_max * 1e6, 1: n_sm * 128 * 2 * sm_max * 1e6}
     kinds = {0: f"FP64 vector, derived: {n_sm} SMs x 2 DFMA/clk x max SM clock",
              1: f"FP32 vector, derived: {n_sm} SMs x 128 FFMA/clk x max SM clock"}
-    kernels = {0: "k_large_step<FP64>", 1: "k_large_step_split"}
-    # the launch shape changes the step kernels' traffic: the launch code is hashed too
-    src = ("large_kernel.cuh", "mixed_common.cuh", "device_common.cuh", "contract.cu")
+    kernels = {p: form_kernels(lists, 0, p) for p in (0, 1)}
+    # one slab fits L2: a buffer larger than it is written before every timed call
+    flush = torch.empty(256 << 20, dtype=torch.uint8, device=dev)
     entry = {"workload": what, "units_per_step": units, "sites_per_step": v3 * nt, "n_ops": [st["n_ops_total"] for st in stats],
-             "unit": "sink-site correlators/s", "warmup": warmup, "steps": {"fp64": steps64, "mixed": steps_mx}}
+             "unit": "sink-site correlators/s", "warmup": warmup, "steps": {"fp64": steps64, "mixed": steps_mx},
+             "l2": "256 MB written before every timed call"}
     with ClockSampler(dev.index if dev.index is not None else 0) as clk:
         for prec, steps in ((0, steps64), (1, steps_mx)):
             for _ in range(warmup):
                 mbc.contract(field, lists, precision=prec, stream=stream)
+            clk.load(lambda: mbc.contract(field, lists, precision=prec, stream=stream), lambda: torch.cuda.synchronize(dev))
             torch.cuda.synchronize(dev)
             mbc.timing_enable(True)
             mbc.timing_read()
-            e0 = torch.cuda.Event(enable_timing=True)
-            e1 = torch.cuda.Event(enable_timing=True)
-            e0.record(stream)
-            for _ in range(steps):
+            events = [[torch.cuda.Event(enable_timing=True) for _ in range(2)] for _ in range(steps)]
+            for e0, e1 in events:
+                with torch.cuda.stream(stream):
+                    flush.zero_()
+                e0.record(stream)
                 mbc.contract(field, lists, precision=prec, stream=stream)
-            e1.record(stream)
+                e1.record(stream)
             torch.cuda.synchronize(dev)
-            ms = e0.elapsed_time(e1)
+            ms = sum(e0.elapsed_time(e1) for e0, e1 in events)
             kms, launches = mbc.timing_read()
             mbc.timing_enable(False)
-            roof = roofline_entry(flops_step, steps, kms, ms, launches, peak[prec], probes[prec], kinds[prec],
-                                  kernels[prec], l1_operand_bound(n_sm, sm_max) if prec == 1 else None)
-            if roof is not None:
-                roof["traffic"] = profiled_traffic(prof[prec], v3 * nt, src)
-                roof["traffic_note"] = ("DRAM bytes of the step kernel per step (all its launches), from the "
-                                        "committed ncu summary scaled by sites; null if the kernel changed since")
+            roof = roofline_entry(flops_step[prec], steps, kms, ms, launches, peak[prec], probes[prec], kinds[prec],
+                                  kernels[prec], operand_bound(lists, 0, prec, n_sm, sm_max))
             entry["fp64" if prec == 0 else "mixed"] = {"value": units * steps / (ms * 1e-3), "ms_per_step": ms / steps,
                                                        "roofline": roof}
     entry["clocks"] = clk.summary()
@@ -505,7 +527,7 @@ def per_config_entry(mbc, torch, dev, name, peaks, n_sm, probes, warmup=3, steps
                                          budget_s=8.0, max_sites=cpu_sites)
     for tl in lists:
         tl.free()
-    del field
+    del field, flush
     torch.cuda.empty_cache()
     return entry
 
@@ -596,6 +618,7 @@ def main():
     def timed(precision, steps, warmup):
         for _ in range(warmup):
             step(precision)
+        clk.load(lambda: step(precision), lambda: torch.cuda.synchronize(dev))
         torch.cuda.synchronize(dev)
         mbc.timing_enable(True)
         mbc.timing_read()
@@ -674,20 +697,14 @@ def main():
     value64 = units_per_step * world * args.steps / (ms64 * 1e-3)
     value_mx = units_per_step * world * args.steps / (msmx * 1e-3)
     value = value64 if primary == 0 else value_mx
-    # roofline of the dominant kernel (the contraction kernel; FP64 pipe)
-    if sink == "block":
-        # per site: blocks of one sink function and their phase-weighted sums
-        # over the momenta; per (cfg, t, group): recursion and contraction
-        per_site = per_item = 0
-        for st, d in zip(stats, list_dims):
-            bs_site = st["block_size"] // n_sinks
-            nxi = 3 * d * n_src
-            n_blocks = len(set(st["path"]))
-            per_site += 3 * nxi * nxi * (2 * (4 if d == 4 else 2)) * 8 + n_blocks * bs_site * (6 * 8 + n_mom * 8)
-            per_item += 8 * st["n_ops_total"] + 4 * st["n_l_total"]
-        flops_step = (per_site * v3 + per_item * (n_mom // n_sinks)) * nt * args.cfgs
-    else:
-        flops_step = point_flops_per_site(stats, list_dims) * v3 * nt * args.cfgs
+    # roofline of the form that runs (the operations of its formula)
+    flops_step = {}
+    for p in (0, 1):
+        if sink == "block":
+            per_site, per_slab = projected_flops(lists, list_dims, n_src, n_sinks, moms, dims[2], p)
+            flops_step[p] = (per_site * v3 + per_slab) * nt * args.cfgs
+        else:
+            flops_step[p] = point_flops_per_site(lists, p) * v3 * nt * args.cfgs
     peaks = measured_peaks()
     probe64 = mbc.fma_probe(0)
     probe32 = mbc.fma_probe(1)
@@ -695,20 +712,12 @@ def main():
     n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
     nominal64 = n_sm * 2 * 2 * sm_max * 1e6  # 2 DFMA / clk / SM (1.25 TFLOP/s class), 2 flop each
     nominal32 = n_sm * 128 * 2 * sm_max * 1e6
-    has_small = any(n[2] == 2 for n in nuclei)
     has_large = any(n[2] == 4 for n in nuclei)
-    kname = {0: " + ".join(k for k, on in (("k_small<FP64>", has_small), ("k_large_step<FP64>", has_large)) if on),
-             1: " + ".join(k for k, on in (("k_small_ls<Mixed>", has_small),
-                                            ("k_large_step_gen" if args.list_free else "k_large_step_split", has_large))
-                           if on)}
-    if sink == "block" or n_src > 1 or args.list_free:  # wave kernels only
-        kname = {0: "k_large_step<FP64>", 1: "k_large_step_gen" if args.list_free else "k_large_step_split"}
-        if sink == "block":
-            kname = {p: "k_project_blocks + " + k for p, k in kname.items()}
+    kname = {p: form_kernels(lists, 1 if sink == "block" else 0, p) for p in (0, 1)}
 
     def roofline(kms, ms, launches, peak, probe, kind, prec):
-        return roofline_entry(flops_step, args.steps, kms, ms, launches, peak, probe, kind, kname[prec],
-                              l1_operand_bound(n_sm, sm_max) if prec == 1 else None)
+        return roofline_entry(flops_step[prec], args.steps, kms, ms, launches, peak, probe, kind, kname[prec],
+                              operand_bound(lists, 1 if sink == "block" else 0, prec, n_sm, sm_max))
 
     roof64 = roofline(k64, ms64, n64, nominal64, probe64,
                       f"FP64 vector, derived: {n_sm} SMs x 2 DFMA/clk x max SM clock", 0)
@@ -718,9 +727,8 @@ def main():
     if args.workload == "nonrel" and not has_large and not args.combined and not args.graph:
         note = ("DRAM bytes per launch (one launch per step) from the committed ncu summary, "
                 "scaled from 65,536 to the step's sites")
-        for r, name, srcs in ((roof64, "k_small_fp64_he3_he4_16x16x16x16.md", ("small_kernel.cuh", "device_common.cuh")),
-                              (roof_mx, "k_small_ls_mixed_he3_he4_16x16x16x16.md",
-                               ("small_ls_kernel.cuh", "mixed_common.cuh", "device_common.cuh"))):
+        srcs = ("minors_kernel.cuh", "mixed_common.cuh", "device_common.cuh")
+        for r, name in ((roof64, "k_minors_fp64_he3_he4_16x16x16x16.md"), (roof_mx, "k_minors_mixed_he3_he4_16x16x16x16.md")):
             if r is not None:
                 r["traffic"] = profiled_traffic(name, v3 * nt * args.cfgs, srcs)
                 r["traffic_note"] = note
@@ -740,7 +748,7 @@ def main():
         "roofline": roof,
         "fp64": {"value": value64, "ms_per_step": ms64 / args.steps, "roofline": roof64},
         "mixed": {"value": value_mx, "ms_per_step": msmx / args.steps, "speedup_vs_fp64": value_mx / value64,
-                  "dtype": "f32 products, Kahan-compensated f32 accumulation, f64 contraction and site sums", "roofline": roof_mx},
+                  "dtype": "f32 products, compensated f32 accumulation, f64 site sums", "roofline": roof_mx},
         "clocks": clocks,
         "e2e": e2e,
         # kernels the library launched in the timed region(s) (graph replays

@@ -235,6 +235,25 @@ mbc_status mbc_term_list_components(const mbc_term_list *list, int8_t *snk, int8
 /* Number of nonzero L entries of output component c (N_L, Tables 4-6). */
 int64_t mbc_term_list_n_l(const mbc_term_list *list, int32_t c);
 
+/*
+ * The form in which a contraction with default tuning evaluates a list, and its
+ * floating-point operations: the recursion over the list's operations, or a
+ * formula of the same components with fewer of them.
+ *   MBC_FORM_RECURSION  F_-^(m+1) = sum sgn(x|y) F_-^(m)[x] f[y] over the lists.
+ *   MBC_FORM_MINORS     3He, 4He and kin with nonrelativistic operators at a point
+ *                       sink: sums of products of two minors of the site's tile.
+ *   MBC_FORM_SATURATED  8Be at a point sink: C = K det S_u det S_d (Sec. 8).
+ *   MBC_FORM_PAIR       one or two baryons per species: the species' products,
+ *                       contracted with the sparse matrix that L defines.
+ * flops: per site with point sinks (blocks included), per (configuration, time
+ * slice, momentum group) with MBC_SINK_BLOCK_MOMENTUM (projection excluded); 8
+ * per complex multiply-add, 4 with a real factor. Either pointer may be NULL.
+ * Host only.
+ */
+enum { MBC_FORM_RECURSION = 0, MBC_FORM_MINORS = 1, MBC_FORM_SATURATED = 2, MBC_FORM_PAIR = 3 };
+mbc_status mbc_term_list_form(const mbc_term_list *list, int32_t sink_mode, int32_t precision, int32_t *form,
+                              double *flops);
+
 /* Release a list and its cached device copies (NULL is a no-op). Must not
  * race with an mbc_contract call still using the list. */
 void mbc_free_term_list(mbc_term_list *list);
@@ -281,7 +300,9 @@ typedef struct {
     int32_t n_src;
 } mbc_props;
 
-/* Launch tuning; zero fields select the library's choice. */
+/* Launch tuning; zero fields select the library's choice. The wave_* fields and
+ * zchunk shape the recursion on the large-stage kernels only; wave_sites also
+ * bounds the sites in flight of the pair form. */
 typedef struct {
     int32_t sites_per_cta;      /* FP64 small-stage kernel: sites per CTA      */
     int32_t threads_per_cta;    /* mixed small-stage kernel: threads per CTA   */
@@ -290,7 +311,9 @@ typedef struct {
                                    least 2e10 site-operations, within an 8 GB
                                    scratch budget; mixed list-free lists at least
                                    512, in multiples of 512)                      */
-    int32_t regime;             /* 0 auto, 1 force small-stage, 2 force large  */
+    int32_t regime;             /* 0 auto (the form of mbc_term_list_form), 1 force
+                                   small-stage, 2 force the recursion on the
+                                   large-stage kernels                            */
     int32_t zchunk;             /* large-stage step kernel: outputs per warp item
                                    (mixed default 1)                            */
     int32_t wave_order;         /* large-stage step kernels on stored lists. FP64:
@@ -319,9 +342,11 @@ typedef struct {
  * Options.
  *   precision    MBC_FP64: FP64 products and sums throughout.
  *                MBC_MIXED: per-site power-of-two input scaling, FP32 complex
- *                products with compensated (two-sum) float-float
- *                accumulation of every component, FP64 for the contraction
- *                with L and for the site/momentum sum.
+ *                products with compensated FP32 accumulation of every sum,
+ *                FP64 for the site/momentum sum. The contraction with L is FP64
+ *                in the recursion and the minor form; the pair form, which mixed
+ *                calls take only where every coefficient is exact in FP32, sums
+ *                it compensated in FP32. 8Be's determinants are FP64 in both.
  *   n_mom, mom   n_mom >= 1 momenta, mom[3 * i + {0, 1, 2}] = (n_x, n_y, n_z)
  *                integers (host pointer, read during the call).
  *   t0, t1       time slices [t0, t1) are evaluated; t1 == 0 means nt.
@@ -333,10 +358,8 @@ typedef struct {
  *                (Sec. 2 sink function s(x)), and the recursion runs once
  *                per (configuration, time slice, momentum) on those blocks.
  *                The blocks and their site sums are FP64 in the FP64 path;
- *                the mixed path forms them with FP32 products, sums each
- *                16-site tile with compensated FP32 accumulation, rounds the
- *                tile sum once to FP32 and adds the tiles with compensated
- *                FP32 accumulation, the result in FP64. Lists built
+ *                the mixed path forms and sums them in FP32 with compensated
+ *                accumulation, the result in FP64. Lists built
  *                with n_sinks = N_k > 1 (Sec. 6 sink functions s_1 .. s_N_k)
  *                take the momenta in groups of N_k (n_mom a multiple of N_k,
  *                all lists of the call with the same N_k): sink function k
@@ -402,9 +425,7 @@ mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *const *list
  *     capture begins;
  *   - no cudaMalloc, cudaFree or other allocating routine is called;
  *   - every call shares the one array and leaves the last call's contents in
- *     it. The one word that must start at zero (the work counter of the
- *     persistent kernel) is zeroed by each call on its stream; every other
- *     entry is written before it is read. Calls that overlap on the GPU - on
+ *     it; every entry is written before it is read. Calls that overlap on the GPU - on
  *     different streams, or from several host threads - race on the array and
  *     give wrong results: serialise them.
  */

@@ -119,6 +119,9 @@ def load(path: str | None = None):
         lib.mbc_term_list_components.restype = ctypes.c_int
         lib.mbc_term_list_n_l.argtypes = [V, ctypes.c_int32]
         lib.mbc_term_list_n_l.restype = ctypes.c_int64
+        lib.mbc_term_list_form.argtypes = [V, ctypes.c_int32, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32),
+                                           ctypes.POINTER(ctypes.c_double)]
+        lib.mbc_term_list_form.restype = ctypes.c_int
         lib.mbc_free_term_list.argtypes = [V]
         lib.mbc_free_term_list.restype = None
         lib.mbc_contract.argtypes = [ctypes.POINTER(Props), ctypes.POINTER(V), ctypes.c_int32,
@@ -220,6 +223,14 @@ class TermList:
 
     def n_l(self, c: int) -> int:
         return int(self._lib.mbc_term_list_n_l(self._h, c))
+
+    def form(self, sink: int = 0, precision: int = 0):
+        """``mbc_term_list_form``: ("recursion" | "minors" | "saturated" | "pair",
+        flops per site or per projected item)."""
+        kind, flops = ctypes.c_int32(), ctypes.c_double()
+        _check(self._lib.mbc_term_list_form(self._h, sink, precision, ctypes.byref(kind), ctypes.byref(flops)),
+               "mbc_term_list_form")
+        return ("recursion", "minors", "saturated", "pair")[kind.value], flops.value
 
     def free(self):
         if self._h:

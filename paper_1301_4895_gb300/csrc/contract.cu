@@ -327,7 +327,6 @@ bool plan_small(const mbc_term_list *L, const MinorPlan *minor, const MirrorPlan
     P.n_g2 = n_g2(L);
     P.n_comp = L->n_comp;
     P.n_steps = A - 1;
-    P.path0 = L->path[0];
     if (minor) return plan_minors(*minor, P, site_entries);
     P.block_size = (int)L->block_size;
     P.npair = (int)binom64(L->nxi, 2);
@@ -2127,6 +2126,52 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
         MBC_CUDA_TRY(cudaStreamSynchronize(stream));
         return take_device_status(stream);  // synchronous call: report a latched timeout
     }
+    return MBC_OK;
+}
+
+extern "C" mbc_status mbc_term_list_form(const mbc_term_list *L, int32_t sink_mode, int32_t precision, int32_t *form,
+                                         double *flops) {
+    if (!L || (sink_mode != MBC_SINK_POINT && sink_mode != MBC_SINK_BLOCK_MOMENTUM) ||
+        (precision != MBC_FP64 && precision != MBC_MIXED))
+        return MBC_ERR_INVALID_ARG;
+    const bool point = sink_mode == MBC_SINK_POINT;
+    int32_t kind = MBC_FORM_RECURSION;
+    double ops = 0.0;  // complex multiply-adds
+    const int64_t ntri = (int64_t)L->nxi * (L->nxi + 1) / 2;
+    const double blocks = point ? 3.0 * ntri * 2 * n_g2(L) + 6.0 * L->block_size : 0.0;
+    const std::shared_ptr<const SaturatedPlan> sat = point ? saturated_plan(L) : nullptr;
+    const std::shared_ptr<const MinorPlan> minor = point && !sat ? minor_plan(L) : nullptr;
+    SmallPlan sp;
+    int64_t entries = 0;
+    std::vector<int> part_off;
+    const std::shared_ptr<const MirrorPlan> mirror = mirror_plan(L);
+    const bool small = point && !L->pauli_forbidden && plan_small(L, minor.get(), mirror.get(), sp, entries, part_off) &&
+                       (int64_t)(entries + L->n_comp) * 16 <= kSmemLimit;
+    const std::shared_ptr<const PairPlan> pair = small ? nullptr : pair_plan(L);
+    if (L->pauli_forbidden || L->n_comp == 0) {
+        ops = 0.0;
+    } else if (sat) {
+        kind = MBC_FORM_SATURATED;
+        ops = (double)(L->nxi * L->nxi * L->nxi - L->nxi) / 3;
+    } else if (minor && small) {
+        kind = MBC_FORM_MINORS;
+        ops = (double)minor->terms.size();
+        for (const auto &st : minor->steps) ops += (double)st.n_z * st.k;
+    } else if (pair && (precision == MBC_FP64 || pair->val_fp32)) {
+        kind = MBC_FORM_PAIR;
+        ops = blocks + 12.0 * pair->masks2.size() * pair->n_rows2;
+        for (const auto &g : pair->groups)
+            for (int s = 0; s < 2; ++s)
+                ops += (double)(pair->row_ptr[(size_t)g.row1[s]] - pair->row_ptr[(size_t)g.row0[s]]) *
+                           (double)(s ? g.mp : g.mn).size() / 2 +
+                       (double)(g.row1[s] - g.row0[s]) * (double)(g.mp.size() * g.mn.size());
+    } else {
+        ops = blocks + L->stats.n_l_total / 2.0;
+        for (size_t m = 0; m < L->steps.size(); ++m)
+            ops += (double)L->steps[m].k * (small && mirror ? (double)mirror->keep.size() : (double)L->steps[m].n_z);
+    }
+    if (form) *form = kind;
+    if (flops) *flops = 8.0 * ops;
     return MBC_OK;
 }
 

@@ -39,7 +39,6 @@ struct SmallStepDesc {
 
 struct SmallPlan {
     int32_t A, dim, nxi, n_g2, n_comp, n_steps;
-    int32_t path0;
     int32_t blk_off;                    // the block of both species (u = d)
     int32_t s_off, q_off;               // entry offsets in the per-site region
     int32_t site_entries;               // per-site region size (entries)

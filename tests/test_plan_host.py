@@ -17,3 +17,15 @@ def test_plans_match_the_recursion(tmp_path):
     subprocess.check_call(["g++", "-O2", "-std=c++17", "-fopenmp", "-I", os.path.join(ROOT, "include"), src, "-o", exe])
     res = subprocess.run([exe], capture_output=True, text=True, timeout=600)
     assert res.returncode == 0 and res.stdout.strip().endswith("OK"), res.stdout + res.stderr
+
+
+@pytest.mark.parametrize("spec,kind", [
+    (dict(n_p=2, n_n=2, dirac_dim=2), "minors"), (dict(n_p=1, n_n=1, dirac_dim=2), "recursion"),
+    (dict(n_p=2, n_n=2, dirac_dim=2, list_free=True), "recursion"),
+    (dict(n_p=2, n_n=1, dirac_dim=4, spins=[((0, 1, 0), (0, 1, 0))]), "pair"),
+])
+def test_form_of_a_list(spec, kind):
+    import paper_1301_4895_gb300 as mbc
+    tl = mbc.build_term_list(**spec)
+    assert tl.form()[0] == kind and tl.form()[1] > 0
+    assert tl.form(mbc.SINK_BLOCK_MOMENTUM)[0] == ("recursion" if spec.get("list_free") else "pair")
