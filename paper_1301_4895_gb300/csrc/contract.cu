@@ -180,8 +180,9 @@ struct DeviceCache {
     double *d_sat_coef = nullptr;      // saturated form: coefficient per component
     // pair form (plan.h)
     std::shared_ptr<const PairPlan> pair;
-    uint32_t *d_prod_ops = nullptr, *d_masks2 = nullptr;  // two-baryon products
-    int32_t *d_range_off = nullptr;
+    PairPlan::ProdRun *d_prod_runs = nullptr;  // two-baryon products
+    uint32_t *d_prod_rec = nullptr, *d_masks2 = nullptr;
+    int32_t *d_range_off = nullptr, *d_prod_run_off = nullptr;
     uint16_t *d_range_e = nullptr;
     // packs of the rows (PairArgs)
     PairPack *d_pair_packs = nullptr;
@@ -207,7 +208,9 @@ void free_cache(DeviceCache *c) {
     cudaFree(c->d_small_ops);
     cudaFree(c->d_small_zops);
     cudaFree(c->d_sat_coef);
-    cudaFree(c->d_prod_ops);
+    cudaFree(c->d_prod_runs);
+    cudaFree(c->d_prod_rec);
+    cudaFree(c->d_prod_run_off);
     cudaFree(c->d_masks2);
     cudaFree(c->d_range_off);
     cudaFree(c->d_range_e);
@@ -722,7 +725,9 @@ mbc_status ensure_pair(const mbc_term_list *Lc, DeviceCache *c, bool mixed) {
     for (const auto &g : P->groups) most = std::max({most, g.mp.size(), g.mn.size()});
     c->pair_shape = most <= 1 ? 0 : most <= 2 ? 1 : 2;
     const PairLayout Q = pair_layout(*P, kPairShapes[c->pair_shape], sm_count(c->device));
-    put(&c->d_prod_ops, P->prod_ops.data(), P->prod_ops.size());
+    put(&c->d_prod_runs, P->prod_runs.data(), P->prod_runs.size());
+    put(&c->d_prod_rec, P->prod_rec.data(), P->prod_rec.size());
+    put(&c->d_prod_run_off, P->run_off.data(), P->run_off.size());
     put(&c->d_masks2, P->masks2.data(), P->masks2.size());
     put(&c->d_range_off, P->range_off.data(), P->range_off.size());
     put(&c->d_range_e, P->range_e.data(), P->range_e.size());
@@ -1360,15 +1365,15 @@ mbc_status pair_wave(const mbc_term_list *L, const DeviceCache *c, int W, const 
     if (prod_rows > 0) {
         const int npair = (int)binom64(L->nxi, 2), n_ranges = (int)P.range_e.size(), n_masks = (int)P.masks2.size();
         const size_t smem = (size_t)4 * npair * 512;
-        const void *kern = (const void *)k_pair_prod<mixed>;
+        auto *kern = npair == 66 ? k_pair_prod<mixed, 66> : k_pair_prod<mixed, 15>;
         int per_sm = 0;
-        mbc_status st = prepare_kernel(kern, c->device, 32 * kProdWarps, smem, &per_sm);
+        mbc_status st = prepare_kernel((const void *)kern, c->device, 32 * kProdWarps<mixed>, smem, &per_sm);
         if (st != MBC_OK) return st;
         TimedLaunch tl(stream);
         note_launch();
-        k_pair_prod<mixed><<<(unsigned)(tiles * n_ranges * n_masks), 32 * kProdWarps, smem, stream>>>(
-            reinterpret_cast<const uint4 *>(c->d_prod_ops), c->d_range_off, c->d_range_e, n_ranges, c->d_masks2, n_masks,
-            npair, L->nxi, L->block_size, P.n_rows2, reinterpret_cast<const ulonglong2 *>(f),
+        kern<<<(unsigned)(tiles * n_ranges * n_masks), 32 * kProdWarps<mixed>, smem, stream>>>(
+            reinterpret_cast<const uint2 *>(c->d_prod_runs), c->d_prod_run_off, c->d_prod_rec, c->d_range_off, c->d_range_e,
+            n_ranges, c->d_masks2, n_masks, L->nxi, L->block_size, P.n_rows2, reinterpret_cast<const ulonglong2 *>(f),
             reinterpret_cast<ulonglong2 *>(prod));
     }
     MBC_CUDA_TRY(cudaGetLastError());

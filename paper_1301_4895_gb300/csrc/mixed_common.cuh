@@ -211,6 +211,13 @@ struct PairAcc {
         f2_kahan_signed(sr, nr, pr, sg);
         f2_kahan_signed(si, ni, pi, sg);
     }
+    // the same with -Im y given
+    __device__ __forceinline__ void fma(ulonglong2 x, ulonglong2 y, uint64_t neg_yi, uint64_t sg) {
+        const uint64_t pr = f2_fma(x.x, y.x, f2_mul(x.y, neg_yi));
+        const uint64_t pi = f2_fma(x.x, y.y, f2_mul(x.y, y.x));
+        f2_kahan_signed(sr, nr, pr, sg);
+        f2_kahan_signed(si, ni, pi, sg);
+    }
     __device__ __forceinline__ ulonglong2 store() const {
         return make_ulonglong2(f2_add(sr, nr), f2_add(si, ni));
     }

@@ -6,8 +6,8 @@
 // FP64 or 64 of FP32], 512 B a row.
 //   k_pair_prod a CTA copies the 4 x n_pairs block rows that the products with
 //               two given singles name into shared memory (135 KB) and forms the
-//               range's products from there: their 24 operands a row would
-//               otherwise come from L2, at its bandwidth in mixed precision.
+//               range's products from there; from L2 their operands would need
+//               its whole bandwidth in mixed precision.
 //   k_pair      a CTA takes a unit - packs of rows of one group for up to MR spin
 //               sets of the row side and MG of the gathered side (a P row
 //               gathers N, an N row gathers P) - and a tile. A pack is rows that
@@ -35,60 +35,92 @@
 namespace mbc {
 
 constexpr int kTile64 = 32, kTileMx = 64;  // sites per tile
-constexpr int kProdWarps = 24;
-
-// Products of one (tile, spin set, singles range) per CTA; grid = tiles x sets x ranges.
+// warps per CTA of k_pair_prod: what its registers allow
 template <bool MX>
-__global__ void __launch_bounds__(32 * kProdWarps, 1)
-    k_pair_prod(const uint4 *__restrict__ ops, const int32_t *__restrict__ range_off,
-                const uint16_t *__restrict__ range_e, int n_ranges, const uint32_t *__restrict__ masks, int n_masks,
-                int npair, int nxi, int64_t block_rows, int n_rows, const ulonglong2 *__restrict__ f,
-                ulonglong2 *__restrict__ prod) {
+constexpr int kProdWarps = MX ? 16 : 24;
+
+// Products of one (tile, spin set, singles range) per CTA; grid = tiles x sets x
+// ranges. A warp takes runs of rows that share a quark triple: the triple's pairs
+// (12 of a row's 24 operands) stay in registers, and a row's other pairs are at
+// fixed distances from three addresses. With 24 operands read and 24 addresses
+// decoded for each row the mixed kernel was held by issue and the shared-memory
+// pipe: 3.68 -> 2.97 ms of a one-component 4He call on 16^3 x 4 sites (3.06 with 20
+// warps and the negated imaginary parts formed per term). FP64 is bound by its pipe
+// either way.
+template <bool MX, int NPAIR>
+__global__ void __launch_bounds__(32 * kProdWarps<MX>, 1)
+    k_pair_prod(const uint2 *__restrict__ runs, const int32_t *__restrict__ run_off, const uint32_t *__restrict__ recs,
+                const int32_t *__restrict__ range_off, const uint16_t *__restrict__ range_e, int n_ranges,
+                const uint32_t *__restrict__ masks, int n_masks, int nxi, int64_t block_rows, int n_rows,
+                const ulonglong2 *__restrict__ f, ulonglong2 *__restrict__ prod) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    using V = std::conditional_t<MX, ulonglong2, double2>;
     ulonglong2 *rows = reinterpret_cast<ulonglong2 *>(smem_raw);  // [f | g][single][pair][lane]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int k = blockIdx.x % n_ranges, m = blockIdx.x / n_ranges % n_masks;
     const int64_t tile = blockIdx.x / n_ranges / n_masks;
     const uint32_t mask = __ldg(masks + m);
-    const int spin[2] = {__ffs(mask) - 1, 31 - __clz(mask)};
-    const int e[2] = {range_e[k] & 255, range_e[k] >> 8};
+    const int s0 = __ffs(mask) - 1, s1 = 31 - __clz(mask), e0 = range_e[k] & 255, e1 = range_e[k] >> 8;
     const ulonglong2 *ft = f + tile * block_rows * 32;
-    for (int r = warp; r < 4 * npair; r += kProdWarps) {
-        const int s = r / (2 * npair), i = r / npair & 1, p = r % npair;
-        async_copy16(rows + r * 32 + lane, ft + ((int64_t)(spin[s] * npair + p) * nxi + e[i]) * 32 + lane);
+    for (int r = warp; r < 4 * NPAIR; r += kProdWarps<MX>) {
+        const int s = r / (2 * NPAIR), i = r / NPAIR & 1, p = r % NPAIR;
+        async_copy16(rows + r * 32 + lane, ft + ((int64_t)((s ? s1 : s0) * NPAIR + p) * nxi + (i ? e1 : e0)) * 32 + lane);
     }
     async_copy_wait_all();
     __syncthreads();
-    const ulonglong2 *F = rows + lane, *G = rows + 2 * npair * 32 + lane;
-    ulonglong2 *out = prod + ((tile * n_masks + m) * n_rows) * 32 + lane;
-    const int r1 = range_off[k + 1];
-    for (int r = range_off[k] + warp; r < r1; r += kProdWarps) {
-        uint32_t op[12];
+    const V *R = reinterpret_cast<const V *>(rows) + lane;
+    // f (s = 0) or g (s = 1) with single i
+    auto at = [](const V *pair, int s, int i) { return pair[(2 * s + i) * NPAIR * 32]; };
+    ulonglong2 *out = prod + ((tile * n_masks + m) * n_rows + range_off[k]) * 32 + lane;
+    // a run goes to one warp; in FP64 row by row, since its pipe wants equal warps
+    // and not fewer operands (5.07 against 5.11 ms in a batch on 24^3 sites)
+    constexpr int kPart = MX ? PairPlan::kProdRun : 1;
+    const int n_runs = run_off[k + 1] - run_off[k];
+    runs += run_off[k];
+    for (int u = warp; u < n_runs * ((PairPlan::kProdRun + kPart - 1) / kPart); u += kProdWarps<MX>) {
+        const uint2 run = __ldg(runs + u % n_runs);
+        const int t0 = u / n_runs * kPart, n = min((int)(run.y & 255u), t0 + kPart);
+        if (t0 >= n) continue;
+        const uint32_t mine = lane < n ? __ldg(recs + run.x + lane) : 0u;
+        V held[3][2][2];
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            const uint4 v = __ldg(ops + 3 * r + q);
-            op[4 * q] = v.x;
-            op[4 * q + 1] = v.y;
-            op[4 * q + 2] = v.z;
-            op[4 * q + 3] = v.w;
-        }
+        for (int q = 0; q < 3; ++q)
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+#pragma unroll
+                for (int i = 0; i < 2; ++i) held[q][s][i] = at(R + (run.y >> (8 * q + 8) & 255u) * 32, s, i);
+        uint64_t neg_im[MX ? 3 : 1][2][2];  // -Im held
         if constexpr (MX) {
-            PairAcc acc;
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+#pragma unroll
+                for (int s = 0; s < 2; ++s)
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) neg_im[q][s][i] = f2_neg(held[q][s][i].y);
+        }
+        for (int t = t0; t < n; ++t) {
+            const uint32_t rec = __shfl_sync(0xffffffffu, mine, t), odd = rec >> 30;
+            ulonglong2 *to = out + (int64_t)(rec >> 21 & 511u) * 32;
+            std::conditional_t<MX, PairAcc, FP64Traits::Acc> acc;
             acc.zero();
 #pragma unroll
-            for (int j = 0; j < 12; ++j)
-                acc.fma(F[(op[j] & 0x7fffu) * 32], G[(op[j] >> 15 & 0x7fffu) * 32], f2_sign_pair((int32_t)op[j] < 0));
-            out[(int64_t)r * 32] = acc.store();
-        } else {
-            FP64Traits::Acc acc;
-            acc.zero();
+            for (int q = 0; q < 3; ++q) {
+                const V *pair = R + (rec >> (7 * q) & 127u) * 32;
 #pragma unroll
-            for (int j = 0; j < 12; ++j) {
-                const double2 x = reinterpret_cast<const double2 *>(F)[(op[j] & 0x7fffu) * 32];
-                const double2 y = reinterpret_cast<const double2 *>(G)[(op[j] >> 15 & 0x7fffu) * 32];
-                acc.fma(x, y, op[j] & 0x80000000u);
+                for (int i = 0; i < 2; ++i) {  // f takes single i, g the other: e1 | e0 is odd
+                    const bool neg = (odd == (uint32_t)q) != (i == 1);
+                    if constexpr (MX) {
+                        const uint64_t sg = f2_sign_pair(neg);
+                        acc.fma(at(pair, 1, 1 - i), held[q][0][i], neg_im[q][0][i], sg);
+                        acc.fma(at(pair, 0, i), held[q][1][1 - i], neg_im[q][1][1 - i], sg);
+                    } else {
+                        const uint32_t sg = neg ? 0x80000000u : 0u;
+                        acc.fma(held[q][0][i], at(pair, 1, 1 - i), sg);
+                        acc.fma(at(pair, 0, i), held[q][1][1 - i], sg);
+                    }
+                }
             }
-            reinterpret_cast<double2 *>(out)[(int64_t)r * 32] = acc.store();
+            *reinterpret_cast<V *>(to) = acc.store();
         }
     }
 }

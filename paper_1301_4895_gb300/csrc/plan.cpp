@@ -397,6 +397,43 @@ void pair_rows(const std::vector<PairEntry> &all, int64_t n_p, int64_t n_n, Clas
         });
 }
 
+// Runs of one range's rows (quark sets of four): the triple that most of the
+// remaining sets contain, up to kProdRun of them, and so on - the longest first.
+bool prod_runs(const std::vector<uint32_t> &sets, int nxi, PairPlan &P) {
+    if (sets.size() > 512) return false;  // a record's row field; C(12, 4) = 495
+    std::vector<uint8_t> done(sets.size(), 0);
+    std::vector<int> count((size_t)1 << nxi);
+    for (size_t left = sets.size(); left > 0;) {
+        std::fill(count.begin(), count.end(), 0);
+        uint32_t triple = 0;
+        for (size_t r = 0; r < sets.size(); ++r)
+            for (uint32_t s = done[r] ? 0u : sets[r]; s; s &= s - 1) {
+                const uint32_t t = sets[r] ^ (s & (0u - s));
+                if (++count[t] > (triple ? count[triple] : 0)) triple = t;
+            }
+        const uint32_t a = triple & (0u - triple), c = 1u << (31 - __builtin_clz(triple)), b = triple ^ a ^ c;
+        const uint32_t held[3] = {a | b, a | c, b | c};
+        PairPlan::ProdRun run{(uint32_t)P.prod_rec.size(), 0, {}};
+        for (int k = 0; k < 3; ++k) run.pair[k] = (uint8_t)rank_of(held[k]);
+        for (size_t r = 0; r < sets.size() && run.n < PairPlan::kProdRun; ++r) {
+            if (done[r] || (sets[r] & triple) != triple) continue;
+            uint32_t rec = (uint32_t)r << 21, odd = 3;
+            for (int k = 0; k < 3; ++k) {
+                const uint32_t other = sets[r] ^ held[k];
+                rec |= (uint32_t)rank_of(other) << (7 * k);
+                if (parity(held[k], other)) odd = odd == 3 ? (uint32_t)k : 4u;
+            }
+            if (odd > 2) return false;  // one of the three splits interleaves
+            P.prod_rec.push_back(rec | odd << 30);
+            done[r] = 1;
+            ++run.n;
+            --left;
+        }
+        P.prod_runs.push_back(run);
+    }
+    return true;
+}
+
 constexpr int64_t kMaxPairEntries = (int64_t)1 << 26;  // 12 B each on the device
 
 std::shared_ptr<const PairPlan> make_pair_plan(const mbc_term_list &L) {
@@ -619,21 +656,20 @@ std::shared_ptr<const PairPlan> make_pair_plan(const mbc_term_list &L) {
         P->comp_off.push_back((int32_t)P->comp_eval.size());
     }
     P->scale = std::tgamma(np + 1.0) * std::tgamma(nn + 1.0) / pt.norm;
-    // the two-baryon products, f before g: splits of the pairs' set and of the singles
-    P->prod_ops.reserve(12 * rows2.size());
-    for (size_t r = 0; r < rows2.size(); ++r) {
-        const uint32_t e = rows2[r].second;
-        if (r == 0 || e != rows2[r - 1].second) {
-            P->range_off.push_back((int32_t)r);
-            P->range_e.push_back((uint16_t)(__builtin_ctz(e) | __builtin_ctz(e & (e - 1)) << 8));
-        }
-        for (const auto &a : splits_of(rows2[r].first, 2))
-            for (uint32_t i = 0; i < 2; ++i)  // f takes single e_i, g the other: e1 | e0 is odd
-                P->prod_ops.push_back((uint32_t)(i * nset2 + rank_of(a.sub)) |
-                                      (uint32_t)((1 - i) * nset2 + rank_of(a.rest)) << 15 |
-                                      (uint32_t)(a.neg ^ (int)i) << 31);
+    for (size_t r0 = 0, r1; r0 < rows2.size(); r0 = r1) {
+        const uint32_t e = rows2[r0].second;
+        for (r1 = r0; r1 < rows2.size() && rows2[r1].second == e;) ++r1;
+        P->range_off.push_back((int32_t)r0);
+        P->range_e.push_back((uint16_t)(__builtin_ctz(e) | __builtin_ctz(e & (e - 1)) << 8));
+        std::vector<uint32_t> sets;
+        for (size_t r = r0; r < r1; ++r) sets.push_back(rows2[r].first);
+        P->run_off.push_back((int32_t)P->prod_runs.size());
+        if (!prod_runs(sets, nxi, *P)) return nullptr;
     }
-    if (!rows2.empty()) P->range_off.push_back((int32_t)rows2.size());
+    if (!rows2.empty()) {
+        P->range_off.push_back((int32_t)rows2.size());
+        P->run_off.push_back((int32_t)P->prod_runs.size());
+    }
     return P;
 }
 

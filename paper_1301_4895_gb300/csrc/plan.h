@@ -114,12 +114,24 @@ struct PairPlan {
     // two-baryon products: element m (spin set masks2[m]), row r at m * n_rows2 +
     // r. Rows with the same two singles (e0, e1) are consecutive: range k is
     // rows [range_off[k], range_off[k + 1]) with singles range_e[k] = e0 | e1 << 8.
-    // A row is 12 products of a lower-spin block f and an upper-spin block g, the
-    // same for every spin set: prod_ops[12 r + j] = x | y << 15 | sign << 31 with
-    // x = i * n_pairs + pair for f[pair; e_i] and y likewise for g.
+    // A row of quark set {a, b, c, d} is the sum over its splits into two pairs and
+    // both orders of the singles of a lower-spin block f times an upper-spin block
+    // g, the same for every spin set: 12 products. Rows of a range that share a
+    // triple {a, b, c} form runs (ProdRun): the pairs within the triple are operands
+    // of all of them. Range k has runs [run_off[k], run_off[k + 1]); a run's rows are
+    // prod_rec[rec0 .. rec0 + n): cd | bd << 7 | ad << 14 (the pairs opposite to
+    // ab, ac and bc) | row within the range << 21 | odd split << 30, the one of the
+    // three splits whose sign is negative.
+    static constexpr int kProdRun = 9;  // rows of a run at most: the other quark states
+    struct ProdRun {
+        uint32_t rec0;
+        uint8_t n, pair[3];  // ab, ac, bc
+    };
     std::vector<uint32_t> masks2;
     int32_t n_rows2 = 0;
-    std::vector<uint32_t> prod_ops;
+    std::vector<ProdRun> prod_runs;
+    std::vector<uint32_t> prod_rec;
+    std::vector<int32_t> run_off;
     std::vector<int32_t> range_off;
     std::vector<uint16_t> range_e;
     struct Group {

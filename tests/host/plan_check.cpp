@@ -127,21 +127,30 @@ static int bad_pairs(const char *name, const mbc_term_list &L, bool expect, std:
     const int64_t npair = (int64_t)L.nxi * (L.nxi - 1) / 2;
     for (uint32_t m : P->masks2) {
         const int s1 = __builtin_ctz(m), s2 = __builtin_ctz(m & (m - 1));
+        const size_t base = prod.size();
+        prod.resize(base + (size_t)P->n_rows2, cd(NAN, NAN));  // every row is written
         for (size_t k = 0; k + 1 < P->range_off.size(); ++k)
-            for (int r = P->range_off[k]; r < P->range_off[k + 1]; ++r) {
+            for (int u = P->run_off[k]; u < P->run_off[k + 1]; ++u) {
                 const int e[2] = {P->range_e[k] & 255, P->range_e[k] >> 8};
-                cd v = 0;
-                for (int j = 0; j < 12; ++j) {
-                    const uint32_t op = P->prod_ops.at((size_t)(12 * r + j)), x = op & 0x7fff, y = op >> 15 & 0x7fff;
-                    if (x >= 2 * npair || y >= 2 * npair) return 1;
-                    const cd t = f.at((size_t)((s1 * npair + x % npair) * L.nxi + e[x / npair])) *
-                                 f.at((size_t)((s2 * npair + y % npair) * L.nxi + e[y / npair]));
-                    v += op >> 31 ? -t : t;
+                const auto &run = P->prod_runs.at((size_t)u);
+                if (run.n < 1 || run.n > mbc::PairPlan::kProdRun) return 1;
+                for (int t = 0; t < run.n; ++t) {
+                    const uint32_t rec = P->prod_rec.at(run.rec0 + (size_t)t);
+                    const int row = P->range_off[k] + (int)(rec >> 21 & 511);
+                    if (row >= P->range_off[k + 1]) return 1;
+                    cd v = 0;
+                    for (int q = 0; q < 3; ++q)
+                        for (int i = 0; i < 2; ++i) {
+                            const int64_t held = run.pair[q], other = rec >> (7 * q) & 127;
+                            if (held >= npair || other >= npair) return 1;
+                            auto F = [&](int s, int64_t p, int j) { return f.at((size_t)((s * npair + p) * L.nxi + e[j])); };
+                            const cd w = F(s1, held, i) * F(s2, other, 1 - i) + F(s1, other, i) * F(s2, held, 1 - i);
+                            v += (rec >> 30 == (uint32_t)q) != (i == 1) ? -w : w;
+                        }
+                    prod[base + (size_t)row] = v;
                 }
-                prod.push_back(v);
             }
     }
-    if (prod.size() != P->masks2.size() * (size_t)P->n_rows2) return 1;
     const int64_t brows = L.block_size / L.dim_snk;
     const int64_t pr = P->p_rows(brows), nr = P->n_rows(brows);
     std::vector<cd> ev((size_t)P->n_evals, 0);
