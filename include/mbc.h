@@ -386,7 +386,9 @@ typedef struct {
  * (a cudaStream_t; NULL = legacy default stream) and out is written in a
  * fixed reduction order (bitwise reproducible). Device scratch is owned by
  * the library, grown on demand and reused across calls; the first call per
- * list uploads it to the current device and caches it there.
+ * list uploads it to the current device and caches it there (operation arrays
+ * beyond 64 MB with the first call that runs the recursion on them: make that call
+ * before capturing one that forces it).
  * Returns MBC_ERR_INVALID_ARG for bad sizes/pointers, MBC_ERR_OOM when
  * device memory cannot be had, MBC_ERR_CUDA for a failed CUDA call.
  */

@@ -417,6 +417,166 @@ mbc_status upload_wave(const mbc_term_list *L, DeviceCache *c) {
     return MBC_OK;
 }
 
+// Tile shapes (row-side x gathered elements per unit) of the pair kernel: one
+// component, a few, all.
+constexpr int kPairShapes[3][2] = {{1, 1}, {2, 2}, {6, 2}};
+// Units per SM and tile: enough that the last ones finish together, few enough
+// that their partial sums stay small beside the products; a unit's work is at
+// least kPairUnitCost multiply-adds per site, so that its warps have a dozen rows
+// each for one copy of the gathered ones.
+constexpr int kPairUnitsPerSm = 8;
+constexpr int64_t kPairUnitCost = 8192;
+
+// Packs of a pair plan's rows (k_pair), group by group and side by side, and the
+// units: consecutive packs of about equal work for one tile of elements.
+struct PairLayout {
+    std::vector<PairPack> packs;
+    std::vector<PairRow> rows;
+    std::vector<uint32_t> cols;
+    std::vector<uint16_t> slot;
+    std::vector<PairUnit> units;
+    std::vector<int32_t> slot_off;
+};
+PairLayout pair_layout(const PairPlan &P, const int shape[2], int n_sm) {
+    PairLayout Q;
+    // cost of rows: entries x gathered elements (2 multiply-adds) + products (4)
+    auto cost = [&](int64_t nnz, int64_t rows, int64_t nr, int64_t ng) { return nnz * ng * 2 + rows * nr * ng * 4; };
+    int64_t total = 0, n_cols = 0;
+    for (const auto &g : P.groups)
+        for (int s = 0; s < 2; ++s)
+            total += cost(P.row_ptr[(size_t)g.row1[s]] - P.row_ptr[(size_t)g.row0[s]], g.row1[s] - g.row0[s],
+                          (int64_t)(s ? g.mn : g.mp).size(), (int64_t)(s ? g.mp : g.mn).size());
+    const int64_t target = std::max<int64_t>(kPairUnitCost, total / std::max(1, n_sm * kPairUnitsPerSm));
+    for (uint32_t c : P.col) n_cols = std::max<int64_t>(n_cols, (int64_t)c + 1);
+    std::vector<int32_t> seen((size_t)n_cols, -1);  // pack that holds a gathered row, its position
+    std::vector<uint16_t> pos((size_t)n_cols, 0);
+    Q.slot.resize(P.col.size());
+    for (size_t r = 0; r < P.row_id.size(); ++r)
+        Q.rows.push_back({P.row_id[r] | (uint32_t)(P.row_ptr[r + 1] - P.row_ptr[r]) << 24, (uint32_t)P.row_ptr[r]});
+    Q.slot_off.assign((size_t)P.n_evals + 1, 0);
+    std::vector<uint16_t> cls;
+    int32_t slot = 0;
+    for (const auto &g : P.groups) {
+        std::vector<int32_t> cut[2];  // unit bounds in packs, per side
+        for (int s = 0; s < 2; ++s) {
+            const auto &re = s ? g.mn : g.mp, &ge = s ? g.mp : g.mn;
+            const int64_t tr = std::min<int64_t>(shape[0], (int64_t)re.size()), tg = std::min<int64_t>(shape[1], (int64_t)ge.size());
+            cut[s].push_back((int32_t)Q.packs.size());
+            int64_t acc = 0;
+            for (int64_t r = g.row0[s]; r < g.row1[s];) {
+                PairPack pk{r, (int64_t)Q.cols.size(), 0, 0};
+                const int32_t id = (int32_t)Q.packs.size();
+                // rows while their gathered rows fit the pack and the unit is not full
+                for (; r < g.row1[s]; ++r) {
+                    const int64_t e0 = P.row_ptr[(size_t)r], e1 = P.row_ptr[(size_t)r + 1];
+                    int32_t fresh = 0;
+                    for (int64_t e = e0; e < e1; ++e) fresh += seen[P.col[(size_t)e]] != id;
+                    if (pk.n_rows > 0 && (pk.n_cols + fresh > kPackCols || acc >= target)) break;
+                    for (int64_t e = e0; e < e1; ++e) {
+                        const uint32_t c = P.col[(size_t)e];
+                        if (seen[c] != id) {
+                            seen[c] = id;
+                            pos[c] = (uint16_t)pk.n_cols++;
+                            Q.cols.push_back(c);
+                        }
+                        Q.slot[(size_t)e] = pos[c];
+                    }
+                    ++pk.n_rows;
+                    acc += cost(e1 - e0, 1, tr, tg);
+                }
+                // longest rows first: the warps' rows of a round are then of one length
+                std::stable_sort(Q.rows.begin() + pk.row0, Q.rows.begin() + pk.row0 + pk.n_rows,
+                                 [](const PairRow &a, const PairRow &b) { return a.n() > b.n(); });
+                Q.packs.push_back(pk);
+                if (acc >= target || r >= g.row1[s]) {
+                    cut[s].push_back((int32_t)Q.packs.size());
+                    acc = 0;
+                }
+            }
+        }
+        const int32_t n0 = (int32_t)cut[0].size() - 1, nc = n0 + (int32_t)cut[1].size() - 1;
+        const int32_t nb = (int32_t)g.mn.size(), na = (int32_t)g.mp.size();
+        for (int64_t ev = 0; ev < (int64_t)na * nb; ++ev) {
+            Q.slot_off[(size_t)(g.eval0 + ev)] = slot + (int32_t)ev * nc;
+            Q.slot_off[(size_t)(g.eval0 + ev) + 1] = slot + (int32_t)(ev + 1) * nc;
+        }
+        for (int s = 0; s < 2; ++s) {
+            const auto &re = s ? g.mn : g.mp, &ge = s ? g.mp : g.mn;
+            const int32_t sr = s ? nc : nb * nc, sg = s ? nb * nc : nc;
+            for (size_t a0 = 0; a0 < re.size(); a0 += (size_t)shape[0])
+                for (size_t b0 = 0; b0 < ge.size(); b0 += (size_t)shape[1])
+                    for (size_t k = 0; k + 1 < cut[s].size(); ++k) {
+                        PairUnit u;
+                        std::memset(&u, 0, sizeof(u));
+                        u.swap = s;
+                        u.pack0 = cut[s][k];
+                        u.pack1 = cut[s][k + 1];
+                        cls.push_back(P.row_class[(size_t)Q.packs[(size_t)u.pack0].row0]);
+                        u.nr = (int32_t)std::min<size_t>((size_t)shape[0], re.size() - a0);
+                        u.ng = (int32_t)std::min<size_t>((size_t)shape[1], ge.size() - b0);
+                        for (int i = 0; i < u.nr; ++i) u.re[i] = re[a0 + (size_t)i];
+                        for (int i = 0; i < u.ng; ++i) u.ge[i] = ge[b0 + (size_t)i];
+                        u.stride_r = sr;
+                        u.stride_g = sg;
+                        u.slot = slot + (int32_t)a0 * sr + (int32_t)b0 * sg + (s ? n0 : 0) + (int32_t)k;
+                        Q.units.push_back(u);
+                    }
+        }
+        slot += na * nb * nc;
+    }
+    // all groups' units of one colour content together: what they read (a few MB
+    // of a tile's products, 100 MB for 4He with all components) then stays in
+    // L2, where the groups one after the other sweep all of it
+    std::vector<size_t> order(Q.units.size());
+    for (size_t i = 0; i < order.size(); ++i) order[i] = i;
+    std::stable_sort(order.begin(), order.end(), [&](size_t a, size_t b) { return cls[a] < cls[b]; });
+    std::vector<PairUnit> sorted;
+    sorted.reserve(Q.units.size());
+    for (size_t i : order) sorted.push_back(Q.units[i]);
+    Q.units.swap(sorted);
+    return Q;
+}
+
+int sm_count(int device);
+
+// The list's device copy with its pair form (regime 0, one or two baryons per
+// species); c->pair stays empty where the list has none. Uploaded with the list's
+// first call whatever it asks for, so that later ones can be captured.
+mbc_status upload_pair(const mbc_term_list *L, DeviceCache *c) try {
+    const std::shared_ptr<const PairPlan> P = pair_plan(L);
+    if (!P) return MBC_OK;
+    mbc_status st = MBC_OK;
+    auto put = [&](auto **dst, const auto *src, size_t n) {
+        if (st == MBC_OK) st = upload(dst, src, n);
+    };
+    size_t most = 0;
+    for (const auto &g : P->groups) most = std::max({most, g.mp.size(), g.mn.size()});
+    c->pair_shape = most <= 1 ? 0 : most <= 2 ? 1 : 2;
+    const PairLayout Q = pair_layout(*P, kPairShapes[c->pair_shape], sm_count(c->device));
+    put(&c->d_prod_runs, P->prod_runs.data(), P->prod_runs.size());
+    put(&c->d_prod_rec, P->prod_rec.data(), P->prod_rec.size());
+    put(&c->d_prod_run_off, P->run_off.data(), P->run_off.size());
+    put(&c->d_masks2, P->masks2.data(), P->masks2.size());
+    put(&c->d_range_off, P->range_off.data(), P->range_off.size());
+    put(&c->d_range_e, P->range_e.data(), P->range_e.size());
+    put(&c->d_pair_packs, Q.packs.data(), Q.packs.size());
+    put(&c->d_pair_rows, Q.rows.data(), Q.rows.size());
+    put(&c->d_pair_cols, Q.cols.data(), Q.cols.size());
+    put(&c->d_pair_slot, Q.slot.data(), Q.slot.size());
+    put(&c->d_pair_val, P->val.data(), P->val.size());
+    put(&c->d_pair_comp_off, P->comp_off.data(), P->comp_off.size());
+    put(&c->d_pair_comp_eval, P->comp_eval.data(), P->comp_eval.size());
+    put(&c->d_pair_slot_off, Q.slot_off.data(), Q.slot_off.size());
+    put(&c->d_pair_units, Q.units.data(), Q.units.size());
+    if (st != MBC_OK) return st;
+    c->n_pair_units = (int32_t)Q.units.size();
+    c->pair_slots = Q.slot_off.back();
+    c->pair = P;
+    return MBC_OK;
+} catch (const std::bad_alloc &) {
+    return MBC_ERR_OOM;
+}
+
 DeviceCache *get_cache(const mbc_term_list *Lc, int device, mbc_status &st) {
     mbc_term_list *L = const_cast<mbc_term_list *>(Lc);
     std::lock_guard<std::mutex> g(L->dev_mu);
@@ -570,7 +730,7 @@ DeviceCache *get_cache(const mbc_term_list *Lc, int device, mbc_status &st) {
         c->max_stage = std::max(c->max_stage, s.n_z);
         op_bytes += s.x.size() * sizeof(uint32_t) + s.ys.size() * sizeof(uint16_t);
     }
-    if (op_bytes <= kEagerOpBytes && (st = upload_wave(L, c)) != MBC_OK) {
+    if ((st = upload_pair(L, c)) != MBC_OK || (op_bytes <= kEagerOpBytes && (st = upload_wave(L, c)) != MBC_OK)) {
         free_cache(c);
         return nullptr;
     }
@@ -585,166 +745,6 @@ DeviceCache *get_wave_cache(const mbc_term_list *L, int device, mbc_status &st) 
     std::lock_guard<std::mutex> g(const_cast<mbc_term_list *>(L)->dev_mu);
     st = upload_wave(L, c);
     return st == MBC_OK ? c : nullptr;
-}
-
-// Tile shapes (row-side x gathered elements per unit) of the pair kernel: one
-// component, a few, all.
-constexpr int kPairShapes[3][2] = {{1, 1}, {2, 2}, {6, 2}};
-// Units per SM and tile: enough that the last ones finish together, few enough
-// that their partial sums stay small beside the products; a unit's work is at
-// least kPairUnitCost multiply-adds per site, so that its warps have a dozen rows
-// each for one copy of the gathered ones.
-constexpr int kPairUnitsPerSm = 8;
-constexpr int64_t kPairUnitCost = 8192;
-
-// Packs of a pair plan's rows (k_pair), group by group and side by side, and the
-// units: consecutive packs of about equal work for one tile of elements.
-struct PairLayout {
-    std::vector<PairPack> packs;
-    std::vector<PairRow> rows;
-    std::vector<uint32_t> cols;
-    std::vector<uint16_t> slot;
-    std::vector<PairUnit> units;
-    std::vector<int32_t> slot_off;
-};
-PairLayout pair_layout(const PairPlan &P, const int shape[2], int n_sm) {
-    PairLayout Q;
-    // cost of rows: entries x gathered elements (2 multiply-adds) + products (4)
-    auto cost = [&](int64_t nnz, int64_t rows, int64_t nr, int64_t ng) { return nnz * ng * 2 + rows * nr * ng * 4; };
-    int64_t total = 0, n_cols = 0;
-    for (const auto &g : P.groups)
-        for (int s = 0; s < 2; ++s)
-            total += cost(P.row_ptr[(size_t)g.row1[s]] - P.row_ptr[(size_t)g.row0[s]], g.row1[s] - g.row0[s],
-                          (int64_t)(s ? g.mn : g.mp).size(), (int64_t)(s ? g.mp : g.mn).size());
-    const int64_t target = std::max<int64_t>(kPairUnitCost, total / std::max(1, n_sm * kPairUnitsPerSm));
-    for (uint32_t c : P.col) n_cols = std::max<int64_t>(n_cols, (int64_t)c + 1);
-    std::vector<int32_t> seen((size_t)n_cols, -1);  // pack that holds a gathered row, its position
-    std::vector<uint16_t> pos((size_t)n_cols, 0);
-    Q.slot.resize(P.col.size());
-    for (size_t r = 0; r < P.row_id.size(); ++r)
-        Q.rows.push_back({P.row_id[r] | (uint32_t)(P.row_ptr[r + 1] - P.row_ptr[r]) << 24, (uint32_t)P.row_ptr[r]});
-    Q.slot_off.assign((size_t)P.n_evals + 1, 0);
-    std::vector<uint16_t> cls;
-    int32_t slot = 0;
-    for (const auto &g : P.groups) {
-        std::vector<int32_t> cut[2];  // unit bounds in packs, per side
-        for (int s = 0; s < 2; ++s) {
-            const auto &re = s ? g.mn : g.mp, &ge = s ? g.mp : g.mn;
-            const int64_t tr = std::min<int64_t>(shape[0], (int64_t)re.size()), tg = std::min<int64_t>(shape[1], (int64_t)ge.size());
-            cut[s].push_back((int32_t)Q.packs.size());
-            int64_t acc = 0;
-            for (int64_t r = g.row0[s]; r < g.row1[s];) {
-                PairPack pk{r, (int64_t)Q.cols.size(), 0, 0};
-                const int32_t id = (int32_t)Q.packs.size();
-                // rows while their gathered rows fit the pack and the unit is not full
-                for (; r < g.row1[s]; ++r) {
-                    const int64_t e0 = P.row_ptr[(size_t)r], e1 = P.row_ptr[(size_t)r + 1];
-                    int32_t fresh = 0;
-                    for (int64_t e = e0; e < e1; ++e) fresh += seen[P.col[(size_t)e]] != id;
-                    if (pk.n_rows > 0 && (pk.n_cols + fresh > kPackCols || acc >= target)) break;
-                    for (int64_t e = e0; e < e1; ++e) {
-                        const uint32_t c = P.col[(size_t)e];
-                        if (seen[c] != id) {
-                            seen[c] = id;
-                            pos[c] = (uint16_t)pk.n_cols++;
-                            Q.cols.push_back(c);
-                        }
-                        Q.slot[(size_t)e] = pos[c];
-                    }
-                    ++pk.n_rows;
-                    acc += cost(e1 - e0, 1, tr, tg);
-                }
-                // longest rows first: the warps' rows of a round are then of one length
-                std::stable_sort(Q.rows.begin() + pk.row0, Q.rows.begin() + pk.row0 + pk.n_rows,
-                                 [](const PairRow &a, const PairRow &b) { return a.n() > b.n(); });
-                Q.packs.push_back(pk);
-                if (acc >= target || r >= g.row1[s]) {
-                    cut[s].push_back((int32_t)Q.packs.size());
-                    acc = 0;
-                }
-            }
-        }
-        const int32_t n0 = (int32_t)cut[0].size() - 1, nc = n0 + (int32_t)cut[1].size() - 1;
-        const int32_t nb = (int32_t)g.mn.size(), na = (int32_t)g.mp.size();
-        for (int64_t ev = 0; ev < (int64_t)na * nb; ++ev) {
-            Q.slot_off[(size_t)(g.eval0 + ev)] = slot + (int32_t)ev * nc;
-            Q.slot_off[(size_t)(g.eval0 + ev) + 1] = slot + (int32_t)(ev + 1) * nc;
-        }
-        for (int s = 0; s < 2; ++s) {
-            const auto &re = s ? g.mn : g.mp, &ge = s ? g.mp : g.mn;
-            const int32_t sr = s ? nc : nb * nc, sg = s ? nb * nc : nc;
-            for (size_t a0 = 0; a0 < re.size(); a0 += (size_t)shape[0])
-                for (size_t b0 = 0; b0 < ge.size(); b0 += (size_t)shape[1])
-                    for (size_t k = 0; k + 1 < cut[s].size(); ++k) {
-                        PairUnit u;
-                        std::memset(&u, 0, sizeof(u));
-                        u.swap = s;
-                        u.pack0 = cut[s][k];
-                        u.pack1 = cut[s][k + 1];
-                        cls.push_back(P.row_class[(size_t)Q.packs[(size_t)u.pack0].row0]);
-                        u.nr = (int32_t)std::min<size_t>((size_t)shape[0], re.size() - a0);
-                        u.ng = (int32_t)std::min<size_t>((size_t)shape[1], ge.size() - b0);
-                        for (int i = 0; i < u.nr; ++i) u.re[i] = re[a0 + (size_t)i];
-                        for (int i = 0; i < u.ng; ++i) u.ge[i] = ge[b0 + (size_t)i];
-                        u.stride_r = sr;
-                        u.stride_g = sg;
-                        u.slot = slot + (int32_t)a0 * sr + (int32_t)b0 * sg + (s ? n0 : 0) + (int32_t)k;
-                        Q.units.push_back(u);
-                    }
-        }
-        slot += na * nb * nc;
-    }
-    // all groups' units of one colour content together: what they read (a few MB
-    // of a tile's products, 100 MB for 4He with all components) then stays in
-    // L2, where the groups one after the other sweep all of it
-    std::vector<size_t> order(Q.units.size());
-    for (size_t i = 0; i < order.size(); ++i) order[i] = i;
-    std::stable_sort(order.begin(), order.end(), [&](size_t a, size_t b) { return cls[a] < cls[b]; });
-    std::vector<PairUnit> sorted;
-    sorted.reserve(Q.units.size());
-    for (size_t i : order) sorted.push_back(Q.units[i]);
-    Q.units.swap(sorted);
-    return Q;
-}
-
-int sm_count(int device);
-
-// The list's device copy with its pair form (regime 0, one or two baryons per
-// species); c->pair stays empty where the list has none. Built and uploaded
-// with the first call that can use it.
-mbc_status ensure_pair(const mbc_term_list *Lc, DeviceCache *c, bool mixed) {
-    const std::shared_ptr<const PairPlan> P = pair_plan(Lc);
-    if (!P || (mixed && !P->val_fp32)) return MBC_OK;
-    std::lock_guard<std::mutex> lock(const_cast<mbc_term_list *>(Lc)->dev_mu);
-    if (c->pair) return MBC_OK;
-    mbc_status st = MBC_OK;
-    auto put = [&](auto **dst, const auto *src, size_t n) {
-        if (st == MBC_OK && !*dst) st = upload(dst, src, n);
-    };
-    size_t most = 0;
-    for (const auto &g : P->groups) most = std::max({most, g.mp.size(), g.mn.size()});
-    c->pair_shape = most <= 1 ? 0 : most <= 2 ? 1 : 2;
-    const PairLayout Q = pair_layout(*P, kPairShapes[c->pair_shape], sm_count(c->device));
-    put(&c->d_prod_runs, P->prod_runs.data(), P->prod_runs.size());
-    put(&c->d_prod_rec, P->prod_rec.data(), P->prod_rec.size());
-    put(&c->d_prod_run_off, P->run_off.data(), P->run_off.size());
-    put(&c->d_masks2, P->masks2.data(), P->masks2.size());
-    put(&c->d_range_off, P->range_off.data(), P->range_off.size());
-    put(&c->d_range_e, P->range_e.data(), P->range_e.size());
-    put(&c->d_pair_packs, Q.packs.data(), Q.packs.size());
-    put(&c->d_pair_rows, Q.rows.data(), Q.rows.size());
-    put(&c->d_pair_cols, Q.cols.data(), Q.cols.size());
-    put(&c->d_pair_slot, Q.slot.data(), Q.slot.size());
-    put(&c->d_pair_val, P->val.data(), P->val.size());
-    put(&c->d_pair_comp_off, P->comp_off.data(), P->comp_off.size());
-    put(&c->d_pair_comp_eval, P->comp_eval.data(), P->comp_eval.size());
-    put(&c->d_pair_slot_off, Q.slot_off.data(), Q.slot_off.size());
-    put(&c->d_pair_units, Q.units.data(), Q.units.size());
-    if (st != MBC_OK) return st;
-    c->n_pair_units = (int32_t)Q.units.size();
-    c->pair_slots = Q.slot_off.back();
-    c->pair = P;
-    return MBC_OK;
 }
 
 // ---- scratch ---------------------------------------------------------------
@@ -1040,7 +1040,6 @@ bool has_pair(const DeviceCache *c, const mbc_tune *tune, bool mixed) {
 DeviceCache *get_large_cache(const mbc_term_list *L, int device, const mbc_tune *tune, bool mixed, mbc_status &st) {
     DeviceCache *c = get_cache(L, device, st);
     if (!c) return nullptr;
-    if (wants_pair(tune) && (st = ensure_pair(L, c, mixed)) != MBC_OK) return nullptr;
     return has_pair(c, tune, mixed) ? c : get_wave_cache(L, device, st);
 }
 

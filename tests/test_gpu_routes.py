@@ -122,6 +122,28 @@ def test_zero_momentum_without_phase_table(mbc):
         assert np.array_equal(one[..., 0, :], two[..., 0, :]), p
 
 
+def test_pair_form_captured_after_a_forced_recursion(mbc):
+    """A list's first call uploads what its other calls read: the default form is
+    captured after a warm call that forced the recursion (scratch grown by another
+    list of the same sizes)."""
+    import torch
+    dims, sp = (1, 5, 13), (0, 1, 0, 1)
+    field = torch.from_numpy(synth.field(47, 1, 1, dims, 0.3, eps=EPS)).cuda()
+    a, b = (mbc.build_term_list(2, 2, 4, spins=[(sp, sp)]) for _ in range(2))
+    st = torch.cuda.Stream()
+    out = torch.zeros((1, 1, 1, 1, 1), dtype=torch.complex128, device="cuda")
+    mbc.contract(field, [a], stream=st, out=out)
+    mbc.contract(field, [b], stream=st, out=out, tune={"regime": 2})
+    st.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        mbc.contract(field, [b], stream=st, out=out)
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, mbc.contract(field, [a], stream=st))
+
+
 def test_block_slices_on_two_relativistic_sources(mbc):
     """24-column tiles (triangular diquarks, entry slices) on pn, 5 sites."""
     from oracle import gamma, recursion
