@@ -23,7 +23,7 @@
 // the pipe) and its few warps' latencies. Whole calls on GB300 against the
 // recursion (8.5 M complex multiply-adds per site for one component, here 0.37 M
 // for the products and 0.31 M real-complex ones; 531 M for all 1296): one
-// component mixed, 16^3 x 4, 125.2 -> 8.7 ms; all, FP64, 64 sites, 233.7 -> 19.5
+// component mixed, 16^3 x 4, 125.2 -> 7.9 ms; all, FP64, 64 sites, 233.7 -> 19.5
 // ms; all, mixed, 512 sites, 210.1 -> 19.9 ms. With L2 gathers and rows in rank
 // order 12.1, 26.9 and 70.8; with rows staged through registers (one load's
 // latency per row and warp, 10 % of a pack's time) 9.35, 20.0 and 24.2.
