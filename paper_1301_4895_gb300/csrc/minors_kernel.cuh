@@ -183,8 +183,9 @@ __global__ void __launch_bounds__(32 * MinorRows<Tr>::kWarps, MinorRows<Tr>::kMx
                 const unsigned char *X = R + d.x_off * T::kRow, *Y = R + d.y_off * T::kRow;
                 unsigned char *Z = R + d.z_off * T::kRow;
                 const uint32_t *ops = P.zops + d.zop_off;
-                // k tells the order: 2 = two tile rows; 4 = two order-2 minors;
-                // 3, 5, 6 a tile row and the next lower order
+                // k tells the order: 2 from two tile rows; 3 and 5 from a tile row
+                // and the next lower order; 6 products make order 4 (two second-
+                // order minors) or order 6 (a tile row and order 5)
                 switch (d.k) {
                 case 2: minor_step<Tr, 2, true, true>(X, Y, Z, ops, d.n_z, low_off, warp); break;
                 case 3: minor_step<Tr, 3, true, false>(X, Y, Z, ops, d.n_z, low_off, warp); break;
