@@ -140,8 +140,9 @@ def test_pair_form_captured_after_a_forced_recursion(mbc):
         mbc.contract(field, [b], stream=st, out=out)
     out.zero_()
     g.replay()
-    torch.cuda.synchronize()
-    assert torch.equal(out, mbc.contract(field, [a], stream=st))
+    ref = mbc.contract(field, [a], stream=st)
+    torch.cuda.synchronize()  # ref is made on st, compared on the current stream
+    assert torch.equal(out, ref)
 
 
 def test_block_slices_on_two_relativistic_sources(mbc):
