@@ -1036,6 +1036,30 @@ bool has_pair(const DeviceCache *c, const mbc_tune *tune, bool mixed) {
     return wants_pair(tune) && c->pair && (!mixed || c->pair->val_fp32);
 }
 
+// Complex multiply-adds of a pair plan per site or item, without the blocks.
+double pair_ops(const PairPlan &P) {
+    double ops = 12.0 * P.masks2.size() * P.n_rows2;
+    for (const auto &g : P.groups)
+        for (int s = 0; s < 2; ++s)
+            ops += (double)(P.row_ptr[(size_t)g.row1[s]] - P.row_ptr[(size_t)g.row0[s]]) *
+                       (double)(s ? g.mp : g.mn).size() / 2 +
+                   (double)(g.row1[s] - g.row0[s]) * (double)(g.mp.size() * g.mn.size());
+    return ops;
+}
+
+// A mixed call with projected blocks contracts its items in FP64 where the pair
+// form is small: there are few items (one per slab and momentum), and FP32 blocks
+// and products are all that still rounds there, since the sites' roundings average
+// out: median error against FP64 of 4He rel on 8^3 sites 1.4e-8 -> 4.8e-9, of two
+// sources and sinks on 16^3 3.9e-8 -> 3.6e-9 (recursion in FP32: 1.3e-8 and 5.0e-8),
+// for 30 us of a call with 8 items (494 -> 526 us). kItemOps64: 4He with one
+// component has 0.5 M; lists of many components, whose items FP64 would hold up
+// (4He with all, 64 sites: 19.5 ms, FP32 2.5), keep FP32.
+constexpr double kItemOps64 = 2e6;
+bool items_fp64(const DeviceCache *c, const mbc_tune *tune, bool mixed) {
+    return mixed && has_pair(c, tune, true) && pair_ops(*c->pair) <= kItemOps64;
+}
+
 // The list's device copy with what its large route reads.
 DeviceCache *get_large_cache(const mbc_term_list *L, int device, const mbc_tune *tune, bool mixed, mbc_status &st) {
     DeviceCache *c = get_cache(L, device, st);
@@ -1532,8 +1556,9 @@ const void *project_kernel(int n_x) {
 
 // Momentum-projected blocks: per-site blocks summed over sites with the phase,
 // then the recursion once per (slab, momentum group) item on the wave kernels; a
-// group holds the n_sinks momenta of the list's sink functions.
-template <class Tr>
+// group holds the n_sinks momenta of the list's sink functions. Sum: the arithmetic
+// of the site sums; Tr: of the items.
+template <class Tr, class Sum>
 mbc_status run_projected(const mbc_term_list *L, const DeviceCache *c, const FieldDesc &F, const MomDesc &M,
                          const mbc_tune *tune, int device, cudaStream_t stream, char *scratch, int li, int n_lists,
                          int comp_max, double2 *out, int64_t n_slabs, const LargeSizes &ls, const ProjectSizes &pz) {
@@ -1541,7 +1566,7 @@ mbc_status run_projected(const mbc_term_list *L, const DeviceCache *c, const Fie
     const int nxi = L->nxi, nrow = 3 * L->dim, n_k = L->n_sinks;
     const int bs = (int)(L->block_size / n_k);  // one sink function: dirac_dim * C(nxi, 2) * nxi
     const int n_groups = M.n_mom / n_k;
-    const bool mx = sizeof(V) == sizeof(float2);
+    const bool mx = sizeof(V) == sizeof(float2), sum_mx = sizeof(typename Sum::V) == sizeof(float2);
     if (nxi != 6 && nxi != 12) return MBC_ERR_UNSUPPORTED;  // 3 x Dirac dimension x sources
     char *p = scratch;
     double2 *xtab = reinterpret_cast<double2 *>(p), *ytab = xtab + (size_t)F.lx * M.n_mom;
@@ -1607,9 +1632,8 @@ mbc_status run_projected(const mbc_term_list *L, const DeviceCache *c, const Fie
     int64_t n_ways = n_slabs * (nrow / 6) * n_chunks;
     const int64_t grid = (n_ways + proj_ways(nxi) - 1) / proj_ways(nxi);
     for (const ProjPass &ps : passes) {
-        using Sum = std::conditional_t<std::is_same<Tr, FP64Traits>::value, ProjSum64, ProjSumMx>;
         const void *kern = nxi == 6 ? project_kernel<Sum, 6>(ps.n_x) : project_kernel<Sum, 12>(ps.n_x);
-        const size_t smem = project_smem_bytes(nrow, nxi, ps.n_mom, mx);
+        const size_t smem = project_smem_bytes(nrow, nxi, ps.n_mom, sum_mx);
         int per_sm = 0;
         mbc_status pst = prepare_kernel(kern, device, proj_threads(nxi), smem, &per_sm);
         if (pst != MBC_OK) return pst;
@@ -1946,7 +1970,8 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
             if (L->pauli_forbidden || L->n_comp == 0) continue;
             cs[(size_t)li] = get_large_cache(L, device, opts->tune, mixed, st);
             if (!cs[(size_t)li]) return st;
-            lsz[(size_t)li] = wave_sizes(L, cs[(size_t)li], opts->tune, n_items_p, mixed);
+            lsz[(size_t)li] = wave_sizes(L, cs[(size_t)li], opts->tune, n_items_p,
+                                         mixed && !items_fp64(cs[(size_t)li], opts->tune, mixed));
             psz[(size_t)li] = project_sizes(L, F, M, n_slabs, device);
             need = std::max(need, psz[(size_t)li].bytes() + lsz[(size_t)li].buffers());
         }
@@ -1954,7 +1979,9 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
         if ((st = scratch_get(device, stream, need, &scr_p)) != MBC_OK) return st;
         for (int li = 0; li < n_lists; ++li) {
             if (!cs[(size_t)li]) continue;
-            auto run = mixed ? run_projected<MixedTraits> : run_projected<FP64Traits>;
+            auto run = !mixed ? run_projected<FP64Traits, ProjSum64>
+                       : items_fp64(cs[(size_t)li], opts->tune, mixed) ? run_projected<FP64Traits, ProjSumMx>
+                                                                       : run_projected<MixedTraits, ProjSumMx>;
             st = run(lists[li], cs[(size_t)li], F, M, opts->tune, device, stream, reinterpret_cast<char *>(scr_p), li,
                      n_lists, comp_max, reinterpret_cast<double2 *>(dev_out), n_slabs, lsz[(size_t)li], psz[(size_t)li]);
             if (st != MBC_OK) return st;
@@ -2163,12 +2190,7 @@ extern "C" mbc_status mbc_term_list_form(const mbc_term_list *L, int32_t sink_mo
         for (const auto &st : minor->steps) ops += (double)st.n_z * st.k;
     } else if (pair && (precision == MBC_FP64 || pair->val_fp32)) {
         kind = MBC_FORM_PAIR;
-        ops = blocks + 12.0 * pair->masks2.size() * pair->n_rows2;
-        for (const auto &g : pair->groups)
-            for (int s = 0; s < 2; ++s)
-                ops += (double)(pair->row_ptr[(size_t)g.row1[s]] - pair->row_ptr[(size_t)g.row0[s]]) *
-                           (double)(s ? g.mp : g.mn).size() / 2 +
-                       (double)(g.row1[s] - g.row0[s]) * (double)(g.mp.size() * g.mn.size());
+        ops = blocks + pair_ops(*pair);
     } else {
         ops = blocks + L->stats.n_l_total / 2.0;
         for (size_t m = 0; m < L->steps.size(); ++m)
