@@ -109,6 +109,26 @@ def test_projection_lines_and_passes(mbc, dims, n_p, n_n, D, spins):
                 parity.check(got[0, 0, t, :, : len(comps)], C, sc, p, what=f"lines {dims} ({n_p},{n_n}) t {t}")
 
 
+@pytest.mark.parametrize("spins", [
+    [((0, 1, 0, 2), (0, 1, 1, 3)), ((0, 2, 0, 1), (1, 3, 0, 1)), ((2, 3, 0, 1), (0, 1, 1, 3))],
+    [((0, 1, 0, 2), s) for s in ((0, 1, 0, 1), (0, 1, 0, 2), (0, 2, 0, 3), (0, 3, 1, 2), (1, 2, 1, 3))],
+])
+def test_projected_items_around_the_fp64_rule(mbc, spins):
+    """Mixed projected blocks whose pair form has 1.7 M and 2.3 M multiply-adds an
+    item: contracted in FP64 and in FP32."""
+    from oracle import projection
+    dims, moms = (1, 2, 3), ((0, 0, 0), (1, 1, 0))
+    tl = mbc.build_term_list(2, 2, 4, spins=spins)
+    assert (tl.form(mbc.SINK_BLOCK_MOMENTUM, 1)[1] <= 8 * 2e6) == (len(spins) == 3)
+    comps = tl.components()
+    plan = oracle_plan(2, 2, 4, comps)
+    for field, precs in legs(48, 1, 1, dims, 0.3, gauss=False):
+        C, sc = projection.projected_correlators(plan, field[0, 0], dims, moms)
+        for p in precs:
+            got = run(mbc, field, [tl], p, moms=moms, sink=mbc.SINK_BLOCK_MOMENTUM)[0, 0, 0, :, : len(comps)]
+            parity.check(got, C, sc, p, what=f"projected items, {len(spins)} components")
+
+
 def test_zero_momentum_without_phase_table(mbc):
     """Calls at zero momentum alone use no phase table: the same bits as the zero
     momentum of a call with others."""
