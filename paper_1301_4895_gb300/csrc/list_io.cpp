@@ -254,6 +254,7 @@ mbc_status mbc_load_term_list(const char *path, mbc_term_list **out) {
         delete L;
         return st;
     }
+    L->from_file = true;
     *out = L;
     return L->pauli_forbidden ? MBC_ERR_PAULI_FORBIDDEN : MBC_OK;
 }

@@ -83,6 +83,8 @@ struct mbc_term_list {
     std::shared_ptr<const mbc::PairPlan> pair;
     std::shared_ptr<const mbc::MirrorPlan> mirror;
     bool minor_tried = false, saturated_tried = false, pair_tried = false, mirror_tried = false;
+    // read from a file: its operations are checked before a plan replaces them
+    bool from_file = false, ops_checked = false, ops_complete = false;
 };
 
 namespace mbc {

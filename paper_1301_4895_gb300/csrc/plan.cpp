@@ -85,6 +85,8 @@ bool stage_key(const mbc_term_list &L, int m, int64_t z, PlanKey &key) {
 bool list_entries(const mbc_term_list &L, std::vector<std::vector<PlanEntry>> &comp) {
     comp.assign((size_t)L.n_comp, {});
     if (L.pauli_forbidden || (int)L.steps.size() != L.A - 1) return false;
+    for (double l : L.fin_l)
+        if (!std::isfinite(l)) return false;  // plans compare and merge equal values
     for (const auto &pt : L.parts) {
         if (pt.A < 1 || pt.A > L.A || pt.n_p < 0 || pt.n_n < 0 || pt.n_p + pt.n_n != pt.A) return false;
         for (int c = pt.c0; c < pt.c1; ++c)
@@ -96,6 +98,73 @@ bool list_entries(const mbc_term_list &L, std::vector<std::vector<PlanEntry>> &c
                     return false;
                 comp[(size_t)c].push_back({z, L.fin_l[(size_t)e]});
             }
+    }
+    return true;
+}
+
+bool complete_operations(const mbc_term_list &L) {
+    if ((L.dim != 2 && L.dim != 4) || L.nxi != 3 * L.dim * L.n_sources || L.dim_snk != L.dim * L.n_sinks ||
+        (int)L.steps.size() != L.A - 1 || L.A < 1)
+        return false;
+    std::vector<PlanKey> block[2], x;  // keys of the block (by species) and of the stage so far
+    for (int b : {MBC_PROTON, MBC_NEUTRON})
+        for (int64_t i = 0; i < L.block_size; ++i) block[b == MBC_NEUTRON].push_back(block_key(i, b, L.nxi));
+    x = block[L.path[0] == MBC_NEUTRON];
+    int n_p = L.path[0] != MBC_NEUTRON, n_n = 1 - n_p;
+    for (const Step &s : L.steps) {
+        const bool proton = s.baryon == MBC_PROTON;
+        const int xk[4] = {n_p, n_n, 2 * n_p + n_n, n_p + 2 * n_n};
+        (proton ? n_p : n_n) += 1;
+        const int zk[4] = {n_p, n_n, 2 * n_p + n_n, n_p + 2 * n_n};
+        if (s.k != binom_p(proton ? n_p : n_n, 1) * binom_p(zk[2], proton ? 2 : 1) * binom_p(zk[3], proton ? 1 : 2) ||
+            (int64_t)x.size() != s.n_x)
+            return false;
+        std::vector<PlanKey> z((size_t)s.n_z);
+        if (s.generated) {
+            // regenerated from the key: complete where both stages are dense
+            if (!s.zrank.empty() || !s.xmap.empty() || !std::equal(zk, zk + 4, s.zk) || !std::equal(xk, xk + 4, s.xk))
+                return false;
+            const int n[4] = {L.dim_snk, L.dim_snk, L.nxi, L.nxi};
+            const int64_t radix[3] = {binom_p(n[1], zk[1]), binom_p(n[2], zk[2]), binom_p(n[3], zk[3])};
+#pragma omp parallel for
+            for (int64_t i = 0; i < s.n_z; ++i)
+                z[(size_t)i] = {unrank(i / radix[2] / radix[1] / radix[0], zk[0], n[0]),
+                                unrank(i / radix[2] / radix[1] % radix[0], zk[1], n[1]),
+                                unrank(i / radix[2] % radix[1], zk[2], n[2]), unrank(i % radix[2], zk[3], n[3])};
+        } else {
+            std::atomic<bool> ok{true};
+            const std::vector<PlanKey> &f = block[!proton];
+#pragma omp parallel
+            {
+                std::vector<int64_t> seen;  // output whose operations name this block entry
+                try {
+                    seen.assign(f.size(), -1);
+                } catch (const std::bad_alloc &) {
+                    ok = false;
+                }
+#pragma omp for schedule(dynamic, 256)
+                for (int64_t i = 0; i < s.n_z; ++i)
+                    for (int64_t j = 0; ok && j < s.k; ++j) {
+                        const size_t o = (size_t)(i * s.k + j);
+                        const PlanKey &a = x[s.x[o]], &b = f[s.ys[o] & 0x7fff];
+                        PlanKey &k = z[(size_t)i];
+                        if (j == 0) {
+                            k = {a.dp | b.dp, a.dn | b.dn, a.u | b.u, a.d | b.d};
+                            if (__builtin_popcount(k.dp) != zk[0] || __builtin_popcount(k.dn) != zk[1] ||
+                                __builtin_popcount(k.u) != zk[2] || __builtin_popcount(k.d) != zk[3])
+                                ok = false;
+                        }
+                        const int neg = parity(a.dp, b.dp) ^ parity(a.dn, b.dn) ^ parity(a.u, b.u) ^ parity(a.d, b.d);
+                        if (!disjoint(a, b) || (a.dp | b.dp) != k.dp || (a.dn | b.dn) != k.dn || (a.u | b.u) != k.u ||
+                            (a.d | b.d) != k.d || seen[s.ys[o] & 0x7fff] == i || (s.ys[o] >> 15) != neg)
+                            ok = false;
+                        else
+                            seen[s.ys[o] & 0x7fff] = i;
+                    }
+            }
+            if (!ok) return false;
+        }
+        x.swap(z);
     }
     return true;
 }
@@ -675,12 +744,26 @@ std::shared_ptr<const PairPlan> make_pair_plan(const mbc_term_list &L) {
 
 }  // namespace
 
+namespace {
+// A plan stands in for the list's operations, so those of a file must be the
+// recursion's own, all of them (caller holds plan_mu).
+template <class P>
+std::shared_ptr<const P> replaces_ops(mbc_term_list *L, std::shared_ptr<const P> plan) {
+    if (!plan || !L->from_file) return plan;
+    if (!L->ops_checked) {
+        L->ops_complete = complete_operations(*L);
+        L->ops_checked = true;
+    }
+    return L->ops_complete ? plan : nullptr;
+}
+}  // namespace
+
 std::shared_ptr<const PairPlan> pair_plan(const mbc_term_list *Lc) {
     mbc_term_list *L = const_cast<mbc_term_list *>(Lc);
     std::lock_guard<std::mutex> g(L->plan_mu);
     if (!L->pair_tried) {
         try {
-            L->pair = make_pair_plan(*L);
+            L->pair = replaces_ops(L, make_pair_plan(*L));
             L->pair_tried = true;
         } catch (const std::bad_alloc &) {
             return nullptr;
@@ -694,7 +777,7 @@ std::shared_ptr<const SaturatedPlan> saturated_plan(const mbc_term_list *Lc) {
     std::lock_guard<std::mutex> g(L->plan_mu);
     if (!L->saturated_tried) {
         try {
-            L->saturated = make_saturated_plan(*L);
+            L->saturated = replaces_ops(L, make_saturated_plan(*L));
             L->saturated_tried = true;
         } catch (const std::bad_alloc &) {
             return nullptr;
@@ -733,7 +816,7 @@ std::shared_ptr<const MirrorPlan> mirror_plan(const mbc_term_list *Lc) {
     std::lock_guard<std::mutex> g(L->plan_mu);
     if (!L->mirror_tried) {
         try {
-            L->mirror = make_mirror_plan(*L);
+            L->mirror = replaces_ops(L, make_mirror_plan(*L));
             L->mirror_tried = true;
         } catch (const std::bad_alloc &) {
             return nullptr;
@@ -747,7 +830,7 @@ std::shared_ptr<const MinorPlan> minor_plan(const mbc_term_list *Lc) {
     std::lock_guard<std::mutex> g(L->plan_mu);
     if (!L->minor_tried) {
         try {
-            L->minor = make_minor_plan(*L);
+            L->minor = replaces_ops(L, make_minor_plan(*L));
             L->minor_tried = true;
         } catch (const std::bad_alloc &) {
             return nullptr;  // the list's own operations serve; tried again at the next use

@@ -24,9 +24,16 @@ struct PlanEntry {
 };
 
 // Contraction entries of every component with their keys, read back from the
-// operations (or ranks) of the list. False where the list's operations do not
-// define consistent keys (a file can hold anything that stays in bounds).
+// first operation (or the rank) of each output. False where those do not have the
+// component's numbers of quarks and baryons, or an L value is not finite.
 bool list_entries(const mbc_term_list &L, std::vector<std::vector<PlanEntry>> &comp);
+
+// True where every output of the list has all splits of its key, each once and
+// with its sign, so that a formula of the keys gives what the operations give.
+// A file can hold any operations that stay in bounds; the builder's are complete.
+// List-free steps with index tables are not looked through: false. 8Be's stored
+// operations (448 M) take 0.9 s on 8 cores, 4He's with one component 20 ms.
+bool complete_operations(const mbc_term_list &L);
 
 // The sink (or unit-propagator) tensor of k baryons of one species with the
 // given spin set: nonzero values of the ordered product of the G tensors as

@@ -19,6 +19,18 @@ def test_plans_match_the_recursion(tmp_path):
     assert res.returncode == 0 and res.stdout.strip().endswith("OK"), res.stdout + res.stderr
 
 
+def test_plans_of_lists_from_files(tmp_path):
+    """A list read from a file whose operations are not the recursion's keeps them:
+    no plan, made from the components' keys alone, stands in."""
+    if shutil.which("g++") is None:
+        pytest.skip("no host C++ compiler")
+    exe = str(tmp_path / "list_file_check")
+    src = os.path.join(ROOT, "tests", "host", "list_file_check.cpp")
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-fopenmp", "-I", os.path.join(ROOT, "include"), src, "-o", exe])
+    res = subprocess.run([exe, str(tmp_path / "list.bin")], capture_output=True, text=True, timeout=600)
+    assert res.returncode == 0 and res.stdout.strip().endswith("OK"), res.stdout + res.stderr
+
+
 @pytest.mark.parametrize("spec,kind", [
     (dict(n_p=2, n_n=2, dirac_dim=2), "minors"), (dict(n_p=1, n_n=1, dirac_dim=2), "recursion"),
     (dict(n_p=2, n_n=2, dirac_dim=2, list_free=True), "recursion"),
