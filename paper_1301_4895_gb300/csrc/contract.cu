@@ -935,13 +935,15 @@ mbc_status launch_small_batch(const SmallBatch &B, const FieldDesc &F, const Mom
 size_t align256(size_t n) { return (n + 255) & ~size_t(255); }
 
 // k_reduce_tiles with warps per output from the tiles a lane would add: several
-// where the outputs are too few to fill the SMs, at most one per FP64 unit (one
-// output of 512 tiles: 16 warps 9.0 us, 4 warps 6.0).
+// where a slab's outputs are too few to fill the SMs, at most one per FP64 unit (one
+// output of 512 tiles: 16 warps 9.0 us, 4 warps 6.0). The warps fix the order of the
+// sum, so they follow from one slab alone: a slab's result has the same bits in a
+// call of any number of them (sharded runs).
 mbc_status launch_reduce(const double2 *partial, int64_t n_slabs, int tiles_per_slab, int n_mom, int n_comp, int n_t,
                          int li, int n_lists, int comp_max, double2 *out, int nsm, cudaStream_t stream) {
-    const int64_t outs = n_slabs * n_mom * n_comp;
+    const int64_t slab_outs = (int64_t)n_mom * n_comp, outs = n_slabs * slab_outs;
     int warps = 1;
-    while (warps < 4 && tiles_per_slab > 16 * warps && outs * warps < 4LL * nsm) warps *= 2;
+    while (warps < 4 && tiles_per_slab > 16 * warps && slab_outs * warps < 4LL * nsm) warps *= 2;
     auto kern = warps == 1 ? k_reduce_tiles<1> : warps == 2 ? k_reduce_tiles<2> : k_reduce_tiles<4>;
     const int per_cta = 4 / warps;
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((outs + per_cta - 1) / per_cta, 65535));
@@ -1427,9 +1429,10 @@ mbc_status pair_wave(const mbc_term_list *L, const DeviceCache *c, int W, const 
         MBC_CUDA_TRY(cudaLaunchKernel(kern, dim3((unsigned)grid), dim3(threads), args, smem, stream));
     }
     note_launch();
-    // wide: too few CTAs of the other shape to fill the SMs, and the slots that a
-    // component sums on average make long chains for its four groups
-    const bool wide = (int64_t)L->n_comp * W < 32LL * nsm &&
+    // wide: too few CTAs of the other shape to fill the SMs in a wave of 64 sites, and
+    // the slots that a component sums on average make long chains for its four groups.
+    // The shape fixes the order of the sum, so the list alone decides, not the wave
+    const bool wide = (int64_t)L->n_comp * 64 < 32LL * nsm &&
                       c->pair_slots * (int64_t)P.comp_eval.size() >= 32 * P.n_evals * (int64_t)L->n_comp;
     auto *sum = wide ? k_pair_sum<8, 128> : k_pair_sum<32, 4>;
     sum<<<dim3((unsigned)L->n_comp, (unsigned)(W / (wide ? 8 : 32))), wide ? 1024 : 128, 0, stream>>>(
@@ -2076,10 +2079,9 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
     size_t large_bytes = 0;
     // 8Be: four warps per site where one would leave FP64 units idle (512 sites
     // mixed: 22 us against 36); half a warp per site from the lattice on where that
-    // fills them
+    // fills them. Both give the same bits
     const bool sat_few = n_slabs * v3 <= 16LL * sm_count(device);
-    const int sat_sites = sat_few ? 1 : kSatSites;
-    const int sat_tiles = (int)((v3 + sat_sites - 1) / sat_sites);  // per slab
+    const int sat_tiles = (int)((v3 + kSatSites - 1) / kSatSites);  // per slab
     for (int li : sat_ids)
         large_bytes = std::max(large_bytes, (size_t)(n_slabs * sat_tiles) * M.n_mom * lists[li]->n_comp * sizeof(double2));
     std::vector<LargeSizes> lsz((size_t)n_lists);
@@ -2129,7 +2131,7 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
             const unsigned grid = (unsigned)(n_slabs * sat_tiles);
             const double *coef = caches[(size_t)li]->d_sat_coef;
             if (sat_few)
-                k_saturated_few<<<grid, 128, 0, stream>>>(F, M, coef, lists[li]->n_comp, partial);
+                k_saturated_few<<<grid * kSatSites, 128, 0, stream>>>(F, M, coef, lists[li]->n_comp, sat_tiles, partial);
             else
                 k_saturated<<<grid, 16 * kSatSites, 0, stream>>>(F, M, coef, lists[li]->n_comp, sat_tiles, partial);
         }

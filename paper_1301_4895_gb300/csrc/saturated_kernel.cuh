@@ -6,13 +6,15 @@
 //
 // Half a warp owns a site, lane r < 12 holds row r in registers. A step picks
 // the pivot row by the largest |re| + |im| (compared on the high words), sends
-// it to the other rows by shuffles and eliminates; rows stay where they are,
-// the permutation's sign is counted. The kernel is bound by the FP64 units (a
+// it to the other rows by shuffles and eliminates; rows stay where they are (the
+// permutation's sign squares away). The kernel is bound by the FP64 units (a
 // warp's FP64 instruction takes one of the SM's four for 64 cycles) through
 // 12 dependent steps. Measured on GB300 against the recursion, whole calls: 64
 // sites FP64 198.0 ms -> 33 us, 512 sites mixed 156.1 ms -> 58 us, the kernels 17
 // and 22 us of it.
 #pragma once
+
+#include <cooperative_groups.h>
 
 #include "small_kernel.cuh"
 
@@ -35,13 +37,12 @@ __device__ __forceinline__ double2 pivot_factor(double2 a, double2 piv) {
     return make_double2(__fma_rn(a.x, piv.x, a.y * piv.y) * inv, __fma_rn(a.y, piv.x, -a.x * piv.y) * inv);
 }
 
-// det of the 12 x 12 matrix whose row (lane & 15) this lane holds
+// det, up to its sign, of the 12 x 12 matrix whose row (lane & 15) this lane holds.
+// The pivots are multiplied in the order of k_saturated_few's tree.
 __device__ __forceinline__ double2 det12(double2 (&a)[12]) {
     const int row = threadIdx.x & 15;
     const unsigned half = 0xffffu << (threadIdx.x & 16);
     unsigned left = 0xfffu;  // rows not yet used as pivots
-    unsigned odd = 0;
-    double2 det = make_double2(1.0, 0.0);
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
         // +1 keeps zero rows above the used ones; NaN compares above all
@@ -49,41 +50,27 @@ __device__ __forceinline__ double2 det12(double2 (&a)[12]) {
             (left >> row & 1u) ? (uint32_t)__double2hiint(fabs(a[k].x) + fabs(a[k].y)) + 1u : 0u;
         const uint32_t best = __reduce_max_sync(half, key);
         const int p = __ffs((__ballot_sync(half, key == best) >> (threadIdx.x & 16)) & 0xffffu) - 1;
-        odd ^= __popc(left & ((1u << p) - 1u)) & 1u;
         left &= ~(1u << p);
         const double2 piv = make_double2(__shfl_sync(half, a[k].x, p, 16), __shfl_sync(half, a[k].y, p, 16));
-        det = cmul(det, piv);
         const double2 f = pivot_factor(a[k], piv);
+        a[k] = piv;  // the column is done with: its place keeps the pivot
 #pragma unroll
         for (int j = k + 1; j < 12; ++j) {
             const double2 q = make_double2(__shfl_sync(half, a[j].x, p, 16), __shfl_sync(half, a[j].y, p, 16));
             if (left >> row & 1u) a[j] = cfms(f, q, a[j]);
         }
     }
-    return odd ? make_double2(-det.x, -det.y) : det;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) a[i] = cmul(cmul(a[i], a[i + 8]), a[i + 4]);
+    return cmul(cmul(a[0], a[2]), cmul(a[1], a[3]));
 }
 
-// partial[tile][mom][comp]: phase-weighted sums over the tile's sites in a
-// fixed order, scaled by the component's coefficient
-__global__ void __launch_bounds__(16 * kSatSites)
-    k_saturated(FieldDesc F, MomDesc M, const double *__restrict__ coef, int n_comp, int tiles_per_slab,
-                double2 *__restrict__ partial) {
-    __shared__ double2 d2[kSatSites], sum[kMaxMom];
-    const int64_t tile = blockIdx.x, slab = tile / tiles_per_slab;
-    const int site0 = (int)(tile % tiles_per_slab) * kSatSites, v3 = F.lx * F.ly * F.lz;
-    const int s = threadIdx.x >> 4, row = threadIdx.x & 15;
-    const bool live = site0 + s < v3;
-    double2 a[12];
-#pragma unroll
-    for (int j = 0; j < 12; ++j) a[j] = make_double2(0.0, 0.0);
-    if (live && row < 12) {
-        const int64_t base = slab / F.n_t * F.stride_cfg + (F.t0 + slab % F.n_t) * F.stride_t + (int64_t)(site0 + s) * 144;
-#pragma unroll
-        for (int j = 0; j < 12; ++j) a[j] = load_prop(F, base, row * 12 + j);
-    }
-    const double2 d = det12(a);
-    if (row == 0) d2[s] = live ? cmul(d, d) : make_double2(0.0, 0.0);
-    __syncthreads();
+// partial[tile][mom][comp]: phase-weighted sums over the tile's sites (d2: their
+// squared determinants) in a fixed order, scaled by the component's coefficient
+__device__ __forceinline__ void saturated_sums(const double2 *d2, double2 *sum, const FieldDesc &F, const MomDesc &M,
+                                               const double *coef, int n_comp, int64_t tile, int site0,
+                                               double2 *partial) {
+    const int v3 = F.lx * F.ly * F.lz;
     for (int q = threadIdx.x; q < M.n_mom; q += blockDim.x) {
         double re = 0.0, im = 0.0;
         for (int w = 0; w < kSatSites && site0 + w < v3; ++w) {
@@ -102,27 +89,53 @@ __global__ void __launch_bounds__(16 * kSatSites)
     }
 }
 
+__global__ void __launch_bounds__(16 * kSatSites)
+    k_saturated(FieldDesc F, MomDesc M, const double *__restrict__ coef, int n_comp, int tiles_per_slab,
+                double2 *__restrict__ partial) {
+    __shared__ double2 d2[kSatSites], sum[kMaxMom];
+    const int64_t tile = blockIdx.x, slab = tile / tiles_per_slab;
+    const int site0 = (int)(tile % tiles_per_slab) * kSatSites, v3 = F.lx * F.ly * F.lz;
+    const int s = threadIdx.x >> 4, row = threadIdx.x & 15;
+    const bool live = site0 + s < v3;
+    double2 a[12];
+#pragma unroll
+    for (int j = 0; j < 12; ++j) a[j] = make_double2(0.0, 0.0);
+    if (live && row < 12) {
+        const int64_t base = slab / F.n_t * F.stride_cfg + (F.t0 + slab % F.n_t) * F.stride_t + (int64_t)(site0 + s) * 144;
+#pragma unroll
+        for (int j = 0; j < 12; ++j) a[j] = load_prop(F, base, row * 12 + j);
+    }
+    const double2 d = det12(a);
+    if (row == 0) d2[s] = cmul(d, d);
+    __syncthreads();
+    saturated_sums(d2, sum, F, M, coef, n_comp, tile, site0, partial);
+}
+
 // The same elimination with a CTA of four warps per site, for lattices of few
 // sites: a warp's FP64 instructions run on one of the SM's four FP64 units, so
 // one warp per site leaves three idle. Lanes are rows, twice; warp w holds columns
 // w, w + 4 (upper half) and w + 8. The warp that owns a step's column finds the
 // pivot and writes the rows' factors to shared memory; every warp then fetches its
 // columns' pivot elements by shuffles and eliminates. 64 sites: 17 us, one warp
-// for two sites 30.
-__global__ void __launch_bounds__(128) k_saturated_few(FieldDesc F, MomDesc M, const double *__restrict__ coef,
-                                                       int n_comp, double2 *__restrict__ partial) {
-    __shared__ double2 fac[2][12], pivots[12], dd;
+// for two sites 30. The CTAs of a tile are a cluster whose first one sums the
+// sites: the operations and their order are k_saturated's, and so are the bits.
+__global__ void __launch_bounds__(128) __cluster_dims__(kSatSites, 1, 1)
+    k_saturated_few(FieldDesc F, MomDesc M, const double *__restrict__ coef, int n_comp, int tiles_per_slab,
+                    double2 *__restrict__ partial) {
+    __shared__ double2 fac[2][12], pivots[12], d2[kSatSites], sum[kMaxMom];
     __shared__ int prow[2];
+    const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
     const int v3 = F.lx * F.ly * F.lz;
-    const int64_t tile = blockIdx.x, slab = tile / v3;
-    const int site = (int)(tile % v3), lane = threadIdx.x & 31, w = threadIdx.x >> 5, half = lane >> 4, row = lane & 15;
+    const int64_t tile = blockIdx.x / kSatSites, slab = tile / tiles_per_slab;
+    const int site0 = (int)(tile % tiles_per_slab) * kSatSites, in_tile = blockIdx.x % kSatSites, site = site0 + in_tile;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, half = lane >> 4, row = lane & 15;
     double2 a[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};  // columns w + 4 half, w + 8 (lower half)
-    if (row < 12) {
+    if (site < v3 && row < 12) {
         const int64_t base = slab / F.n_t * F.stride_cfg + (F.t0 + slab % F.n_t) * F.stride_t + (int64_t)site * 144;
         a[0] = load_prop(F, base, row * 12 + w + 4 * half);
         if (half == 0) a[1] = load_prop(F, base, row * 12 + w + 8);
     }
-    unsigned left = 0xfffu, odd = 0;
+    unsigned left = 0xfffu;
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
         const int h = (k >> 2) & 1, q = k >> 3;  // column k: warp k % 4, half h, register q
@@ -142,7 +155,6 @@ __global__ void __launch_bounds__(128) k_saturated_few(FieldDesc F, MomDesc M, c
         }
         __syncthreads();  // double-buffered: a step's readers are done before the next but one writes
         const int p = prow[k & 1];
-        odd ^= __popc(left & ((1u << p) - 1u)) & 1u;
         left &= ~(1u << p);
         const double2 f = row < 12 ? fac[k & 1][row] : make_double2(0.0, 0.0);
 #pragma unroll
@@ -152,22 +164,17 @@ __global__ void __launch_bounds__(128) k_saturated_few(FieldDesc F, MomDesc M, c
             if (w + 4 * half + 8 * g > k && (left >> row & 1u)) a[g] = cfms(f, x, a[g]);
         }
     }
-    if (w == 0) {  // product of the pivots, in a fixed tree
+    cluster.sync();  // the first CTA has started (every pivot is written by now)
+    if (w == 0) {    // product of the pivots, in a fixed tree
         double2 d = lane < 12 ? pivots[lane] : make_double2(1.0, 0.0);
         for (int off = 8; off > 0; off >>= 1) {
             const double2 o = make_double2(__shfl_xor_sync(0xffffffffu, d.x, off), __shfl_xor_sync(0xffffffffu, d.y, off));
-            d = cmul(d, o);
+            if (off < 8 || lane < 4) d = cmul(d, o);  // four pivots have no partner eight further
         }
-        if (lane == 0) dd = cmul(d, d);  // the permutation's sign squares away
+        if (lane == 0) cluster.map_shared_rank(d2, 0)[in_tile] = cmul(d, d);
     }
-    __syncthreads();
-    for (int o = threadIdx.x; o < M.n_mom * n_comp; o += blockDim.x) {
-        const double2 ph = mom_phase(M.mom[o / n_comp], site % F.lx, (site / F.lx) % F.ly, site / (F.lx * F.ly), F.lx,
-                                     F.ly, F.lz);
-        const double c = __ldg(coef + o % n_comp);
-        partial[tile * (int64_t)(M.n_mom * n_comp) + o] =
-            make_double2(c * __fma_rn(ph.x, dd.x, -ph.y * dd.y), c * __fma_rn(ph.x, dd.y, ph.y * dd.x));
-    }
+    cluster.sync();  // the tile's determinants are in the first CTA
+    if (in_tile == 0) saturated_sums(d2, sum, F, M, coef, n_comp, tile, site0, partial);
 }
 
 }  // namespace mbc

@@ -178,3 +178,25 @@ def test_block_slices_on_two_relativistic_sources(mbc):
         for p in precs:
             got = run(mbc, field, [tl], p)[0, 0, 0, :, : len(comps)]
             parity.check(got, ref, scale[None, :], p, what="24 columns")
+
+
+@pytest.mark.parametrize("build,dims,nt,precs", [
+    # 8Be: 1,728 sites a slab by four warps a site, 5,184 by half a warp
+    (lambda m: [m.build_term_list(4, 4, 4, spins=[(BE8, BE8)], list_free=True)], (12, 12, 12), 3, (0, 1)),
+    # nonrelativistic lists in mixed precision: 64 tiles of 32 sites, 64 outputs a slab
+    (lambda m: [m.build_term_list(1, 1, 2), m.build_term_list(2, 1, 2), m.build_term_list(2, 2, 2)], (16, 16, 8), 6, (1,)),
+    # pair form: waves of 64 and of 1,024 sites; 18 tiles and 256 outputs a slab
+    (lambda m: [m.build_term_list(2, 2, 4, spins=[((0, 1, 0, 1), (0, 1, a, b)) for a in range(4) for b in range(a)])],
+     (4, 4, 4), 16, (0, 1)),
+    (lambda m: [m.build_term_list(1, 1, 4)], (9, 8, 8), 2, (0, 1)),
+])
+def test_a_slab_alone_and_among_others(mbc, build, dims, nt, precs):
+    """A slab's correlators have the same bits whether the call holds that slab alone,
+    as a rank of a sharded run may, or all of them."""
+    moms = ((0, 0, 0), (1, 0, 0), (0, 1, 0), (1, 1, 0))
+    field, lists = synth.field(49, 1, nt, dims, 0.1, eps=EPS), build(mbc)
+    for p in precs:
+        whole = run(mbc, field, lists, p, moms=moms)
+        for t in range(nt):
+            alone = run(mbc, field, lists, p, moms=moms, t0=t, t1=t + 1)
+            assert np.array_equal(alone[:, :, 0], whole[:, :, t]), (p, t)
