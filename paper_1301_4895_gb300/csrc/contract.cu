@@ -1628,7 +1628,7 @@ mbc_status run_projected(const mbc_term_list *L, const DeviceCache *c, const Fie
         const int64_t n = (int64_t)F.lx * D.n_mom + (int64_t)F.ly * F.lz * M.n_mom;
         note_launch();
         k_line_phases<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 4096)), 256, 0, stream>>>(
-            F, M, D, xtab, ytab);
+            F, M, D, sum_mx ? 1 : 0, xtab, ytab);
         MBC_CUDA_TRY(cudaGetLastError());
     }
     int n_dx = D.n_mom, n_g2_ = n_g2(L), n_chunks = pz.n_chunks, n_mom = M.n_mom, nrow_ = nrow;

@@ -22,8 +22,13 @@
 //                   layout of the wave kernels (MIXED: exact power-of-two scaling
 //                   per item);
 //   k_write_items   writes each item's contracted components to out.
-// FP64 throughout in the FP64 path (bound by its pipe); FP32 products with
-// compensated FP32 sums over a line and over the lines in the mixed path.
+// FP64 throughout in the FP64 path (bound by its pipe). The mixed path takes FP32
+// products and compensated FP32 sums along a line; a line's sum enters the momenta
+// in both words, with exact products and the line's phase in two words: rounded to one
+// word before and after that product, a line of near-identity sites cost up to a third
+// of the accuracy at momenta across the lines (median error of 4He rel at (0, 1, 0),
+// eps = 0.05: 16^3 9.1e-7 -> 6.4e-7, 5 x 7 x 9 1.6e-6 -> 6.8e-7; blocks weighted by one
+// FP32 phase per site 6.9e-7 and 1.4e-6), for 2 % of a call's time.
 #pragma once
 
 #include "large_kernel.cuh"
@@ -39,28 +44,46 @@ struct ProjPass {
     int32_t nx_of[kProjMoms], xcol[kProjMoms], trivial[kProjMoms];
 };
 
+// A phase table's entry in the mixed path: two FP32 words of a complex number.
+struct Phase32 {
+    float2 h, l;
+};
+static_assert(sizeof(Phase32) == sizeof(double2), "one table for both");
+
 // xtab[x][d] = e^{-2 pi i D.mom[d][0] x / Lx}; ytab[y + Ly z][q] = the (y, z) phase
-// of momentum q. Column d of xtab belongs to the d-th distinct n_x.
-__global__ void k_line_phases(FieldDesc F, MomDesc M, MomDesc D, double2 *xtab, double2 *ytab) {
+// of momentum q. Column d of xtab belongs to the d-th distinct n_x. words: entries as
+// Phase32.
+__global__ void k_line_phases(FieldDesc F, MomDesc M, MomDesc D, int words, double2 *xtab, double2 *ytab) {
+    auto put = [&](double2 *to, double2 v) {
+        if (words) {
+            const float2 h = make_float2((float)v.x, (float)v.y);
+            *reinterpret_cast<Phase32 *>(to) = Phase32{h, make_float2((float)(v.x - h.x), (float)(v.y - h.y))};
+        } else {
+            *to = v;
+        }
+    };
     const int nl = F.ly * F.lz;
     const int64_t total = (int64_t)F.lx * D.n_mom + (int64_t)nl * M.n_mom;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         if (i < (int64_t)F.lx * D.n_mom) {
             const int n[3] = {D.mom[i % D.n_mom][0], 0, 0};
-            xtab[i] = mom_phase(n, (int)(i / D.n_mom), 0, 0, F.lx, F.ly, F.lz);
+            put(xtab + i, mom_phase(n, (int)(i / D.n_mom), 0, 0, F.lx, F.ly, F.lz));
         } else {
             const int64_t k = i - (int64_t)F.lx * D.n_mom;
             const int q = (int)(k % M.n_mom), line = (int)(k / M.n_mom);
             const int n[3] = {0, M.mom[q][1], M.mom[q][2]};
-            ytab[k] = mom_phase(n, 0, line % F.ly, line / F.ly, F.lx, F.ly, F.lz);
+            put(ytab + k, mom_phase(n, 0, line % F.ly, line / F.ly, F.lx, F.ly, F.lz));
         }
     }
 }
 
-// Sums over sites: acc += ph x (or += x), and acc += ph times a line's sum.
+// Sums over a line's sites (acc += x, or ph x) and, Total, over the lines (acc += ph
+// times a line's sum). Phase: a phase table's entry, first() what a site multiplies by.
 struct ProjSum64 {
     using V = double2;
+    using Phase = double2;
     double re, im;
+    __device__ __forceinline__ static V first(Phase p) { return p; }
     __device__ __forceinline__ void zero() { re = im = 0.0; }
     __device__ __forceinline__ void add(V x) {
         re += x.x;
@@ -70,17 +93,35 @@ struct ProjSum64 {
         re = __fma_rn(ph.x, x.x, __fma_rn(-ph.y, x.y, re));
         im = __fma_rn(ph.x, x.y, __fma_rn(ph.y, x.x, im));
     }
-    __device__ __forceinline__ V line() const { return make_double2(re, im); }
-    __device__ __forceinline__ double2 value() const { return make_double2(re, im); }
+    struct Total;
+};
+struct ProjSum64::Total {
+    ProjSum64 s;
+    __device__ __forceinline__ void zero() { s.zero(); }
+    __device__ __forceinline__ void add(Phase ph, const ProjSum64 &line) { s.add(ph, make_double2(line.re, line.im)); }
+    __device__ __forceinline__ double2 value() const { return make_double2(s.re, s.im); }
 };
 struct ProjSumMx {
     using V = float2;
+    using Phase = Phase32;
     MixedTraits::Acc a;
+    __device__ __forceinline__ static V first(Phase p) { return p.h; }
     __device__ __forceinline__ void zero() { a.zero(); }
     __device__ __forceinline__ void add(V x) { f2_kahan(a.s, a.n, f2_pack(x.x, x.y)); }
     __device__ __forceinline__ void add(V ph, V x) { a.add_prod(ph, x); }
-    __device__ __forceinline__ V line() const { return a.store(); }
-    __device__ __forceinline__ double2 value() const { return a.value(); }
+    struct Total {
+        BlockAccMx b;
+        __device__ __forceinline__ void zero() { b.zero(); }
+        __device__ __forceinline__ void add(Phase ph, const ProjSumMx &line) {
+            const DiquarkMx y{f2_unpack(line.a.s), f2_unpack(line.a.n)};
+            b.add(ph.h, y);
+            b.l.x = __fmaf_rn(ph.l.x, y.h.x, __fmaf_rn(-ph.l.y, y.h.y, b.l.x));
+            b.l.y = __fmaf_rn(ph.l.x, y.h.y, __fmaf_rn(ph.l.y, y.h.x, b.l.y));
+        }
+        __device__ __forceinline__ double2 value() const {
+            return make_double2((double)b.h.x + (double)b.l.x, (double)b.h.y + (double)b.l.y);
+        }
+    };
 };
 
 // (j, s) pairs, i values per thread, threads of one way (a walk over one chunk)
@@ -109,9 +150,11 @@ __global__ void __launch_bounds__(proj_threads(NXI), 1)
     constexpr int B = proj_batch(sizeof(V) == 8);
     constexpr int I = proj_ipt(NXI), O = 2 * I;  // outputs of a thread: (spin, i)
     constexpr int kProjThreads = proj_threads(NXI);
-    static_assert(sizeof(Sum) == 16, "sums in shared memory");
+    using Total = typename Sum::Total;
+    using Phase = typename Sum::Phase;
+    static_assert(sizeof(Total) == 16, "sums in shared memory");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    Sum *out = reinterpret_cast<Sum *>(smem_raw) + threadIdx.x;  // [mom][O][thread]
+    Total *out = reinterpret_cast<Total *>(smem_raw) + threadIdx.x;  // [mom][O][thread]
     const int nent = nrow * NXI, per_way = B * (nent + 3 * NJS + kProjMoms);
     const int wy = threadIdx.x / WAY, tw = threadIdx.x % WAY;
     const int64_t way = (int64_t)blockIdx.x * WAYS + wy;
@@ -156,7 +199,7 @@ __global__ void __launch_bounds__(proj_threads(NXI), 1)
         }
         if (ph_lane && s0 + ph_b < c1) {
             const double2 v = __ldg(xtab + (int64_t)((s0 + ph_b) % F.lx) * n_dx + ph_col);
-            pre_ph = V{(R)v.x, (R)v.y};
+            pre_ph = Sum::first(*reinterpret_cast<const Phase *>(&v));
         }
     };
     // the thread's diquark entries: pair (x2, x3) = js, colours and sites in turn
@@ -233,12 +276,12 @@ __global__ void __launch_bounds__(proj_threads(NXI), 1)
                     for (int m = 0; m < ps.n_mom; ++m) {
                         if (ps.nx_of[m] != k) continue;
                         const double2 p = __ldg(yt + m);
-                        const V ph{(R)p.x, (R)p.y};
-                        Sum *t = out + m * O * kProjThreads;
+                        const Phase ph = *reinterpret_cast<const Phase *>(&p);
+                        Total *t = out + m * O * kProjThreads;
 #pragma unroll
                         for (int o = 0; o < O; ++o) {
-                            Sum v = t[o * kProjThreads];
-                            v.add(ph, line[k][o].line());
+                            Total v = t[o * kProjThreads];
+                            v.add(ph, line[k][o]);
                             t[o * kProjThreads] = v;
                         }
                     }
