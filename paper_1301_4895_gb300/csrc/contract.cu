@@ -390,6 +390,32 @@ bool plan_small(const mbc_term_list *L, const MinorPlan *minor, const MirrorPlan
     return true;
 }
 
+// Operation i of step m as the shared-memory kernels run it: operand indices and
+// sign, of the list's own steps (a pn list's kept outputs) or of its minor form's.
+struct SmallOp {
+    uint32_t x, y, neg;
+};
+SmallOp small_op(const mbc_term_list *L, const MinorPlan *minor, const MirrorPlan *mirror, size_t m, size_t i) {
+    if (minor) {
+        const auto &s = minor->steps[m];
+        return SmallOp{s.x[i], s.y[i], s.neg[i]};
+    }
+    const Step &s = L->steps[m];
+    if (mirror) i = (size_t)mirror->keep[i / (size_t)s.k] * (size_t)s.k + i % (size_t)s.k;
+    return SmallOp{s.x[i], s.ys[i] & 0x7fffu, (uint32_t)(s.ys[i] >> 15)};
+}
+
+// The lanes-are-sites kernels' operation words hold operand rows below 256 (all
+// nonrelativistic lists); mixed calls on other lists take the wave kernels.
+bool ls_rows(const mbc_term_list *L, const MinorPlan *minor, const MirrorPlan *mirror, const SmallPlan &P) {
+    for (int m = 0; m < P.n_steps; ++m)
+        for (size_t i = 0; i < (size_t)P.step[m].n_z * (size_t)P.step[m].k; ++i) {
+            const SmallOp o = small_op(L, minor, mirror, (size_t)m, i);
+            if (o.x >= 256 || o.y >= 256) return false;
+        }
+    return true;
+}
+
 // Operation arrays up to this size go to the device with the list's first use;
 // larger ones (8Be 2.7 GB, 4He with all components 3.2 GB) with the first call
 // that runs them, since other routes never read them.
@@ -629,20 +655,7 @@ DeviceCache *get_cache(const mbc_term_list *Lc, int device, mbc_status &st) {
         }
         // per step and part (outputs [0, n_main) with g lanes, the rest with
         // g2): [round j][z][sub], padded to a whole number of rounds
-        // operation i of step m: operand indices and sign, of the list's own
-        // steps or of the minor form's
-        struct Op {
-            uint32_t x, y, neg;
-        };
-        auto op_at = [&](size_t m, size_t i) {
-            if (minor) {
-                const auto &s = minor->steps[m];
-                return Op{s.x[i], s.y[i], s.neg[i]};
-            }
-            const Step &s = L->steps[m];
-            if (mirror) i = (size_t)mirror->keep[i / (size_t)s.k] * (size_t)s.k + i % (size_t)s.k;
-            return Op{s.x[i], s.ys[i] & 0x7fffu, (uint32_t)(s.ys[i] >> 15)};
-        };
+        auto op_at = [&](size_t m, size_t i) { return small_op(L, minor.get(), mirror.get(), m, i); };
         std::vector<uint32_t> packed;
         for (int m = 0; m < c->sp.n_steps; ++m) {
             SmallStepDesc &d = c->sp.step[m];
@@ -653,7 +666,7 @@ DeviceCache *get_cache(const mbc_term_list *Lc, int device, mbc_status &st) {
                 uint32_t *dst = packed.data() + off;
                 for (int64_t zl = 0; zl < n; ++zl)
                     for (int64_t j = 0; j < k; ++j) {
-                        const Op o = op_at((size_t)m, (size_t)((z_begin + zl) * k + j));
+                        const SmallOp o = op_at((size_t)m, (size_t)((z_begin + zl) * k + j));
                         dst[((j / g) * n + zl) * g + (j % g)] = o.x | o.y << 16 | o.neg << 31;
                     }
                 return off;
@@ -666,23 +679,20 @@ DeviceCache *get_cache(const mbc_term_list *Lc, int device, mbc_status &st) {
             return nullptr;
         }
         // lanes-are-sites layout: z-major, operands as byte offsets of their
-        // 256 B shared-memory rows (x << 8 | sign in bit 0 | y << 24), which
-        // needs every stage and block index below 256 (all nonrelativistic
-        // lists); otherwise the mixed path takes the wave kernels. Each
-        // output's terms are ordered positive first (stable), so the kernel
-        // adds the first ones and subtracts the rest and its operation
-        // records need no sign
+        // 256 B shared-memory rows (x << 8 | sign in bit 0 | y << 24; see
+        // ls_rows). Each output's terms are ordered positive first (stable),
+        // so the kernel adds the first ones and subtracts the rest and its
+        // operation records need no sign
         std::vector<uint32_t> zpk;
-        c->ls_ok = true;
+        c->ls_ok = ls_rows(L, minor.get(), mirror.get(), c->sp);
         for (int m = 0; m < c->sp.n_steps; ++m) {
             SmallStepDesc &d = c->sp.step[m];
             d.zop_off = (int64_t)zpk.size();
             for (int64_t z = 0; z < d.n_z; ++z)
                 for (uint32_t want = 0; want < 2; ++want)
                     for (int64_t j = 0; j < d.k; ++j) {
-                        const Op o = op_at((size_t)m, (size_t)(z * d.k + j));
+                        const SmallOp o = op_at((size_t)m, (size_t)(z * d.k + j));
                         if (o.neg != want) continue;
-                        if (o.x >= 256 || o.y >= 256) c->ls_ok = false;
                         zpk.push_back((o.x & 0xffu) << 8 | o.neg | (o.y & 0xffu) << 24);
                     }
         }
@@ -905,6 +915,13 @@ SmallLaunch size_small_batch(const std::vector<const DeviceCache *> &cs, const F
         comp_stride = std::max(comp_stride, c->sp.n_comp);
     }
     return size_small_tiles(site_stride, comp_stride, F, tune, mixed, cs[0]->sp.bilinear != 0, n_sm);
+}
+
+// A list alone takes the shared-memory kernels: its site buffers fit, and in mixed
+// precision its operation words hold its rows (ls_ok).
+bool small_route(int32_t site_entries, int32_t n_comp, bool ls_ok, const FieldDesc &F, const mbc_tune *tune, bool mixed,
+                 bool bilinear) {
+    return (!mixed || ls_ok) && size_small_tiles(site_entries, n_comp, F, tune, mixed, bilinear).ok;
 }
 
 mbc_status launch_small_batch(const SmallBatch &B, const FieldDesc &F, const MomDesc &M, const SmallLaunch &l,
@@ -2002,15 +2019,14 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
         if (L->pauli_forbidden || L->n_comp == 0) continue;  // identically zero
         caches[(size_t)li] = get_cache(L, device, st);
         if (!caches[(size_t)li]) return st;
-        if (regime == 0 && caches[(size_t)li]->d_sat_coef) {
+        const DeviceCache *c = caches[(size_t)li];
+        if (regime == 0 && c->d_sat_coef) {
             sat_ids.push_back(li);
             continue;
         }
-        bool small = caches[(size_t)li]->small_ok && (!mixed || caches[(size_t)li]->ls_ok) && regime != 2;
-        if (small) {  // the list alone must fit the shared-memory kernel
-            int32_t ss, cs;
-            small = size_small_batch({caches[(size_t)li]}, F, opts->tune, mixed, ss, cs).ok;
-        }
+        const bool small = c->small_ok && regime != 2 &&
+                           small_route((int32_t)c->site_entries, c->sp.n_comp, c->ls_ok, F, opts->tune, mixed,
+                                       c->sp.bilinear != 0);
         if (regime == 1 && !small) return MBC_ERR_UNSUPPORTED;
         if (!small && !get_large_cache(L, device, opts->tune, mixed, st)) return st;
         (small ? small_ids : large_ids).push_back(li);
@@ -2178,8 +2194,13 @@ extern "C" mbc_status mbc_term_list_form(const mbc_term_list *L, int32_t sink_mo
     int64_t entries = 0;
     std::vector<int> part_off;
     const std::shared_ptr<const MirrorPlan> mirror = mirror_plan(L);
+    FieldDesc one;  // the route does not depend on the lattice
+    std::memset(&one, 0, sizeof(one));
+    one.n_cfg = one.n_t = one.lx = one.ly = one.lz = 1;
+    const bool mixed = precision == MBC_MIXED;
     const bool small = point && !L->pauli_forbidden && plan_small(L, minor.get(), mirror.get(), sp, entries, part_off) &&
-                       (int64_t)(entries + L->n_comp) * 16 <= kSmemLimit;
+                       small_route((int32_t)entries, sp.n_comp, !mixed || ls_rows(L, minor.get(), mirror.get(), sp), one,
+                                   nullptr, mixed, minor != nullptr);
     const std::shared_ptr<const PairPlan> pair = small ? nullptr : pair_plan(L);
     if (L->pauli_forbidden || L->n_comp == 0) {
         ops = 0.0;
@@ -2190,7 +2211,7 @@ extern "C" mbc_status mbc_term_list_form(const mbc_term_list *L, int32_t sink_mo
         kind = MBC_FORM_MINORS;
         ops = (double)minor->terms.size();
         for (const auto &st : minor->steps) ops += (double)st.n_z * st.k;
-    } else if (pair && (precision == MBC_FP64 || pair->val_fp32)) {
+    } else if (pair && (!mixed || pair->val_fp32)) {
         kind = MBC_FORM_PAIR;
         ops = blocks + pair_ops(*pair);
     } else {

@@ -41,3 +41,13 @@ def test_form_of_a_list(spec, kind):
     tl = mbc.build_term_list(**spec)
     assert tl.form()[0] == kind and tl.form()[1] > 0
     assert tl.form(mbc.SINK_BLOCK_MOMENTUM)[0] == ("recursion" if spec.get("list_free") else "pair")
+
+
+def test_form_follows_the_precision():
+    """A relativistic pn list fits the FP64 shared-memory kernel, but not the operation
+    words of the mixed one: mixed calls take its pair form on the wave kernels."""
+    import paper_1301_4895_gb300 as mbc
+    tl = mbc.build_term_list(1, 1, 4, spins=[((0, 3), (1, 2))])
+    assert tl.form(0, mbc.FP64)[0] == "recursion" and tl.form(0, mbc.MIXED)[0] == "pair"
+    he3 = mbc.build_term_list(2, 1, 2)
+    assert he3.form(0, mbc.FP64) == he3.form(0, mbc.MIXED)
