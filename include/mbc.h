@@ -335,7 +335,8 @@ typedef struct {
     int32_t list_free;          /* large-stage step kernel: 0 regenerate the splits of
                                    list-free lists, read the arrays of the others;
                                    1 also regenerate the dense steps of lists with
-                                   arrays                                           */
+                                   arrays: lists with a pair form or a saturated one
+                                   take the recursion                               */
 } mbc_tune;
 
 /*

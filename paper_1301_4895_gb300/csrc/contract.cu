@@ -1048,11 +1048,11 @@ LargeSizes large_sizes(const mbc_term_list *L, const DeviceCache *c, const mbc_t
     return s;
 }
 
-// A list takes its pair form unless the call forces the wave kernels or asks
-// them to regenerate operations.
-bool wants_pair(const mbc_tune *tune) { return !tune || (tune->regime == 0 && tune->list_free == 0); }
+// A list takes its pair or saturated form unless the call forces other kernels or
+// asks the wave kernels to regenerate operations.
+bool wants_form(const mbc_tune *tune) { return !tune || (tune->regime == 0 && tune->list_free == 0); }
 bool has_pair(const DeviceCache *c, const mbc_tune *tune, bool mixed) {
-    return wants_pair(tune) && c->pair && (!mixed || c->pair->val_fp32);
+    return wants_form(tune) && c->pair && (!mixed || c->pair->val_fp32);
 }
 
 // Complex multiply-adds of a pair plan per site or item, without the blocks.
@@ -2020,7 +2020,7 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
         caches[(size_t)li] = get_cache(L, device, st);
         if (!caches[(size_t)li]) return st;
         const DeviceCache *c = caches[(size_t)li];
-        if (regime == 0 && c->d_sat_coef) {
+        if (wants_form(opts->tune) && c->d_sat_coef) {
             sat_ids.push_back(li);
             continue;
         }

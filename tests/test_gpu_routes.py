@@ -211,3 +211,36 @@ def test_mixed_projection_across_the_lines(mbc):
     field = synth.field(50, 2, 128, (5, 7, 9), 0.0, eps=EPS)
     exact, got = (run(mbc, field, [tl], p, moms=((0, 1, 0),), sink=mbc.SINK_BLOCK_MOMENTUM) for p in (0, 1))
     assert np.median(np.abs(got - exact) / np.abs(exact)) <= 1.0e-6
+
+
+def test_be8_recursion_on_request(mbc):
+    """8Be by its recursion: stored operations, the same regenerated on request (which
+    default tuning honours too), and a list-free list. On near-identity propagators,
+    against O3; the three perform the same operations."""
+    dims = (1, 2, 2)
+    field = synth.field(4, 1, 1, dims, 0.4, dtype=np.complex64, eps=EPS)
+    stored, free = (mbc.build_term_list(4, 4, 4, spins=[(BE8, BE8)], list_free=lf) for lf in (False, True))
+    ref, scale = oracle_slab(oracle_plan(4, 4, 4, [(BE8, BE8)]), field[0, 0], dims, [(0, 0, 0)])
+    for p in (0, 1):
+        a = run(mbc, field, [stored], p, tune={"regime": 2})
+        parity.check(a[0, 0, 0, :, :1], ref, scale[None, :], p, what="8Be recursion")
+        for tl, tune in ((stored, {"regime": 2, "list_free": 1}), (stored, {"list_free": 1}), (free, {"regime": 2})):
+            b = run(mbc, field, [tl], p, tune=tune)
+            if p == 0:
+                assert np.array_equal(a, b), tune
+            parity.check(b[0, 0, 0, :, :1], ref, scale[None, :], p, what=f"8Be recursion {tune}")
+
+
+@pytest.mark.parametrize("p", [0, 1])
+@pytest.mark.parametrize("dims", [(1, 2, 3), (14, 14, 13)])
+def test_saturated_form_is_fp64_in_both_precisions(mbc, dims, p):
+    """8Be's determinants of a permutation and of a random matrix, a few and many sites."""
+    n = int(np.prod(dims))
+    rng = np.random.default_rng(51)
+    S = np.zeros((n, 12, 12), dtype=np.complex128)
+    S[0] = np.eye(12)[rng.permutation(12)] * 1.5
+    S[n - 1] = rng.standard_normal((12, 12)) + 1j * rng.standard_normal((12, 12))
+    tl = mbc.build_term_list(4, 4, 4, spins=[(BE8, BE8)], list_free=True)
+    got = run(mbc, S.reshape((1, 1) + dims + (12, 12)), [tl], p)[0, 0, 0, 0, 0]
+    det2 = np.linalg.det(S[[0, n - 1]]) ** 2
+    assert abs(got - _be8_K() * np.sum(det2)) <= 1e-12 * _be8_K() * np.sum(np.abs(det2))
