@@ -1,16 +1,19 @@
 """Launch-shape autotuner for mbc_contract.
 
 For a set of term lists, a precision and a lattice geometry it times the
-candidate launch shapes of the kernels those lists use - sites per CTA of the
-FP64 shared-memory kernel, threads per CTA of the mixed one, wave size and
-outputs per warp item of the wave kernels - on a bounded sample of the
-caller's field (the first time slices of the first configuration), with
-CUDA events on the caller's stream, and keeps the fastest. Results are cached
-in a JSON file keyed by (lists, precision, geometry, storage type).
+library's own choice and other launch shapes of the kernels those lists use -
+sites per CTA of the FP64 shared-memory kernel, threads per CTA of the mixed
+one, wave size and outputs per warp item of the wave kernels - on a bounded
+sample of the caller's field (the first time slices of the first
+configuration), with CUDA events on the caller's stream, and keeps the
+fastest. Results are cached in a JSON file keyed by (lists and their forms,
+precision, geometry, storage type).
 
-The tuner only chooses ``mbc_tune`` fields; every candidate runs the same
-kernels on the same data, so all of them produce the same correlators up to
-rounding order.
+The tuner only chooses ``mbc_tune`` fields of the form that a list takes
+anyway, so all candidates produce the same correlators up to rounding. A field
+may change the kernel (``sites_per_cta``: one warp per site also where the
+minor form would take lanes as sites) or mean nothing to a form (the pair form
+reads ``wave_sites`` alone).
 """
 from __future__ import annotations
 
@@ -37,7 +40,8 @@ def _key(field, lists, precision) -> str:
     for tl in lists:
         st = tl.stats()
         specs.append([tl.spec["n_p"], tl.spec["n_n"], tl.spec["dirac_dim"], st["n_ops_total"], st["n_comp"]])
-    return json.dumps({"lists": specs, "precision": int(precision), "geom": list(field.shape[2:5]),
+    # forms: what an earlier library tuned for other kernels is not taken up
+    return json.dumps({"lists": specs, "forms": [tl.form(0, int(precision))[0] for tl in lists], "precision": int(precision), "geom": list(field.shape[2:5]),
                        "dtype": str(field.dtype)}, sort_keys=True)
 
 
@@ -45,10 +49,11 @@ def candidates(lists, precision):
     small = any(tl.spec["dirac_dim"] == 2 for tl in lists)  # nonrelativistic: shared-memory kernels
     large = any(tl.spec["dirac_dim"] == 4 for tl in lists)  # relativistic: wave kernels
     fp64 = precision == FP64
-    opt_small = [{"sites_per_cta": s} for s in (2, 4, 8, 12, 16, 20, 24, 32)] if fp64 else \
-        [{"threads_per_cta": t} for t in (256, 512, 768, 1024)]
-    if not small:
-        opt_small = [{}]
+    opt_small = [{}]  # the library's choice: the minor form with lanes as sites wherever that is the faster one
+    if small and fp64:
+        opt_small += [{"sites_per_cta": s} for s in (2, 4, 8, 12, 16, 20, 24, 32)]
+    elif any(tl.spec["dirac_dim"] == 2 and tl.form(0, precision)[0] != "minors" for tl in lists):
+        opt_small = [{"threads_per_cta": t} for t in (256, 512, 768, 1024)]  # 1024 is the default
     opt_large = [{}]
     if large:
         opt_large = [dict(w, **z, **o) for w, z, o in itertools.product(
@@ -56,6 +61,17 @@ def candidates(lists, precision):
             [{}, {"zchunk": 4}, {"zchunk": 32}], [{}, {"wave_order": 1}] if fp64 else [{}, {"wave_order": 3}])]
     for a, b in itertools.product(opt_small, opt_large):
         yield dict(a, **b)
+
+
+def _slices(shape, lists, precision, sample_slices, n_sm) -> int:
+    """Time slices of the timing sample. FP64 minor-form lists take another kernel on
+    few sites than on many (32 per SM), so their sample spans several rounds of it
+    where the field does; one where relativistic lists take most of the time."""
+    n = sample_slices
+    if precision == FP64 and any(tl.form(0, FP64)[0] == "minors" for tl in lists):
+        rounds = 1 if any(tl.spec["dirac_dim"] == 4 for tl in lists) else 8
+        n = max(n, -(-rounds * 32 * n_sm // (shape[2] * shape[3] * shape[4])))
+    return max(1, min(n, shape[1]))
 
 
 def _time(field, lists, precision, tune, t1, stream, reps):
@@ -75,7 +91,8 @@ def autotune(field, lists, precision: int = FP64, stream=None, reps: int = 2, sa
              use_cache: bool = True, verbose: bool = False) -> dict:
     """Best ``mbc_tune`` dict for these lists on this field (torch tensor on
     the device). The timing sample is configuration 0, time slices
-    [0, sample_slices)."""
+    [0, sample_slices), more where ``_slices`` says so."""
+    import torch
     key = _key(field, lists, precision)
     path = cache_path()
     if use_cache:
@@ -88,7 +105,8 @@ def autotune(field, lists, precision: int = FP64, stream=None, reps: int = 2, sa
             except (OSError, ValueError):
                 pass
     sub = field[:1]
-    t1 = max(1, min(sample_slices, field.shape[1]))
+    t1 = _slices(field.shape, lists, precision, sample_slices,
+                 torch.cuda.get_device_properties(field.device).multi_processor_count)
     best, best_ms = {}, float("inf")
     results = []
     for cand in candidates(lists, precision):

@@ -33,3 +33,29 @@ def test_item_orders_per_wave_step_kernel():
     rel = [mbc.build_term_list(1, 1, 4)]
     assert {c.get("wave_order", 0) for c in _cands(rel, mbc.FP64)} == {0, 1}
     assert {c.get("wave_order", 0) for c in _cands(rel, mbc.MIXED)} == {0, 3}
+
+
+def test_the_librarys_choice_is_a_candidate():
+    """FP64 minor-form lists leave their fast kernel where sites_per_cta is set, so the
+    candidates hold the library's own choice; in mixed precision the minor form reads
+    no field. pn, which runs the recursion there, keeps its shapes."""
+    he = [mbc.build_term_list(2, 1, 2), mbc.build_term_list(2, 2, 2)]
+    pn, rel = mbc.build_term_list(1, 1, 2), mbc.build_term_list(1, 1, 4)
+    for lists in (he, he + [pn], he + [rel]):
+        assert {} in _cands(lists, mbc.FP64)
+    assert _cands(he, mbc.MIXED) == [{}]
+    assert {c["threads_per_cta"] for c in _cands(he + [pn], mbc.MIXED)} == {256, 512, 768, 1024}
+
+
+def test_cache_key_and_sample_follow_the_form():
+    import json
+
+    import numpy as np
+    he, rel = [mbc.build_term_list(2, 1, 2)], [mbc.build_term_list(1, 1, 4)]
+    field = np.zeros((1, 2, 2, 2, 2, 12, 12), dtype=np.complex128)
+    assert json.loads(autotune._key(field, he, mbc.FP64))["forms"] == ["minors"]
+    shape = (1, 32, 16, 16, 16, 12, 12)
+    assert autotune._slices(shape, he, mbc.FP64, 1, 152) == 10  # 8 x 32 x 152 sites
+    assert autotune._slices(shape, he + rel, mbc.FP64, 1, 152) == 2
+    assert autotune._slices(shape, he, mbc.MIXED, 1, 152) == autotune._slices(shape, rel, mbc.FP64, 1, 152) == 1
+    assert autotune._slices((1, 4) + shape[2:], he, mbc.FP64, 1, 152) == 4

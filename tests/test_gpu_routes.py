@@ -244,3 +244,12 @@ def test_saturated_form_is_fp64_in_both_precisions(mbc, dims, p):
     got = run(mbc, S.reshape((1, 1) + dims + (12, 12)), [tl], p)[0, 0, 0, 0, 0]
     det2 = np.linalg.det(S[[0, n - 1]]) ** 2
     assert abs(got - _be8_K() * np.sum(det2)) <= 1e-12 * _be8_K() * np.sum(np.abs(det2))
+
+
+def test_autotune_keeps_the_fast_kernel(mbc):
+    """FP64 3He + 4He on 16^3 x 12: the library's choice (the minor form with lanes as
+    sites) is a fifth faster than every setting of sites_per_cta."""
+    import torch
+    from paper_1301_4895_gb300.autotune import autotune
+    field = torch.from_numpy(synth.field(52, 1, 12, (16, 16, 16), 0.1)).cuda()
+    assert autotune(field, [mbc.build_term_list(2, 1, 2), mbc.build_term_list(2, 2, 2)], use_cache=False) == {}
