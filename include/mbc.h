@@ -389,7 +389,8 @@ typedef struct {
  * the library, grown on demand and reused across calls; the first call per
  * list uploads it to the current device and caches it there (operation arrays
  * beyond 64 MB with the first call that runs the recursion on them: make that call
- * before capturing one that forces it).
+ * before capturing one that forces it). A list whose pair form's tables find no room
+ * then keeps the recursion on that device.
  * Returns MBC_ERR_INVALID_ARG for bad sizes/pointers, MBC_ERR_OOM when
  * device memory cannot be had, MBC_ERR_CUDA for a failed CUDA call.
  */

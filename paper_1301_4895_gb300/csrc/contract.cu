@@ -200,6 +200,29 @@ struct DeviceCache {
 
 namespace {
 
+// Free the pair form's tables (also a set that was cut short).
+void free_pair(DeviceCache *c) {
+    auto drop = [](auto *&p) {
+        cudaFree(p);
+        p = nullptr;
+    };
+    drop(c->d_prod_runs);
+    drop(c->d_prod_rec);
+    drop(c->d_prod_run_off);
+    drop(c->d_masks2);
+    drop(c->d_range_off);
+    drop(c->d_range_e);
+    drop(c->d_pair_packs);
+    drop(c->d_pair_rows);
+    drop(c->d_pair_cols);
+    drop(c->d_pair_slot);
+    drop(c->d_pair_val);
+    drop(c->d_pair_comp_off);
+    drop(c->d_pair_comp_eval);
+    drop(c->d_pair_units);
+    drop(c->d_pair_slot_off);
+}
+
 void free_cache(DeviceCache *c) {
     if (!c) return;
     int prev = -1;
@@ -208,21 +231,7 @@ void free_cache(DeviceCache *c) {
     cudaFree(c->d_small_ops);
     cudaFree(c->d_small_zops);
     cudaFree(c->d_sat_coef);
-    cudaFree(c->d_prod_runs);
-    cudaFree(c->d_prod_rec);
-    cudaFree(c->d_prod_run_off);
-    cudaFree(c->d_masks2);
-    cudaFree(c->d_range_off);
-    cudaFree(c->d_range_e);
-    cudaFree(c->d_pair_packs);
-    cudaFree(c->d_pair_rows);
-    cudaFree(c->d_pair_cols);
-    cudaFree(c->d_pair_slot);
-    cudaFree(c->d_pair_val);
-    cudaFree(c->d_pair_comp_off);
-    cudaFree(c->d_pair_comp_eval);
-    cudaFree(c->d_pair_units);
-    cudaFree(c->d_pair_slot_off);
+    free_pair(c);
     cudaFree(c->d_run_off);
     cudaFree(c->d_term_off);
     cudaFree(c->d_run_coef);
@@ -565,9 +574,10 @@ PairLayout pair_layout(const PairPlan &P, const int shape[2], int n_sm) {
 
 int sm_count(int device);
 
-// The list's device copy with its pair form (regime 0, one or two baryons per
-// species); c->pair stays empty where the list has none. Uploaded with the list's
-// first call whatever it asks for, so that later ones can be captured.
+// The tables of the list's pair form, with the list's first call whatever it asks for,
+// so that later calls can be captured. c->pair stays empty where the list has none, or
+// where the device has no room for the tables: the recursion serves then, and a call
+// that would not read them is not refused for them.
 mbc_status upload_pair(const mbc_term_list *L, DeviceCache *c) try {
     const std::shared_ptr<const PairPlan> P = pair_plan(L);
     if (!P) return MBC_OK;
@@ -594,13 +604,17 @@ mbc_status upload_pair(const mbc_term_list *L, DeviceCache *c) try {
     put(&c->d_pair_comp_eval, P->comp_eval.data(), P->comp_eval.size());
     put(&c->d_pair_slot_off, Q.slot_off.data(), Q.slot_off.size());
     put(&c->d_pair_units, Q.units.data(), Q.units.size());
-    if (st != MBC_OK) return st;
+    if (st != MBC_OK) {
+        free_pair(c);
+        return st == MBC_ERR_OOM ? MBC_OK : st;
+    }
     c->n_pair_units = (int32_t)Q.units.size();
     c->pair_slots = Q.slot_off.back();
     c->pair = P;
     return MBC_OK;
 } catch (const std::bad_alloc &) {
-    return MBC_ERR_OOM;
+    free_pair(c);
+    return MBC_OK;
 }
 
 DeviceCache *get_cache(const mbc_term_list *Lc, int device, mbc_status &st) {
@@ -740,7 +754,7 @@ DeviceCache *get_cache(const mbc_term_list *Lc, int device, mbc_status &st) {
         c->max_stage = std::max(c->max_stage, s.n_z);
         op_bytes += s.x.size() * sizeof(uint32_t) + s.ys.size() * sizeof(uint16_t);
     }
-    if ((st = upload_pair(L, c)) != MBC_OK || (op_bytes <= kEagerOpBytes && (st = upload_wave(L, c)) != MBC_OK)) {
+    if ((op_bytes <= kEagerOpBytes && (st = upload_wave(L, c)) != MBC_OK) || (st = upload_pair(L, c)) != MBC_OK) {
         free_cache(c);
         return nullptr;
     }

@@ -253,3 +253,30 @@ def test_autotune_keeps_the_fast_kernel(mbc):
     from paper_1301_4895_gb300.autotune import autotune
     field = torch.from_numpy(synth.field(52, 1, 12, (16, 16, 16), 0.1)).cuda()
     assert autotune(field, [mbc.build_term_list(2, 1, 2), mbc.build_term_list(2, 2, 2)], use_cache=False) == {}
+
+
+def test_no_room_for_the_pair_tables(mbc):
+    """With too little device memory left for a list's pair tables, a call that forces
+    the recursion, which does not read them, runs all the same."""
+    import torch
+    spins = [((0, 1, 0), (a, b, c)) for b in range(4) for a in range(b) for c in range(4)]
+    field = torch.from_numpy(synth.field(53, 1, 1, (1, 2, 2), 0.3, eps=EPS)).cuda()
+    out = torch.zeros((4, 1, 1, 1, 1, len(spins)), dtype=torch.complex128, device="cuda")
+    lists = [mbc.build_term_list(2, 1, 4, spins=spins) for _ in range(4)]
+
+    def call(i):  # bytes of device memory that it took
+        before = torch.cuda.mem_get_info()[0]
+        mbc.contract(field, [lists[i]], out=out[i], tune={"regime": 2})
+        torch.cuda.synchronize()
+        return before - torch.cuda.mem_get_info()[0]
+
+    call(0)  # scratch and kernels
+    copy = min(call(1), call(2))  # 8 MB of operations, then 9 MB of pair tables
+    filler = torch.empty(((torch.cuda.mem_get_info()[0] - copy + (4 << 20)) >> 21) << 21, dtype=torch.uint8, device="cuda")
+    try:
+        assert copy - (7 << 20) < torch.cuda.mem_get_info()[0] < copy - (1 << 20)
+        call(3)
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    assert torch.equal(out[3], out[0]) and torch.equal(out[1], out[0])
