@@ -1652,6 +1652,7 @@ mbc_status run_projected(const mbc_term_list *L, const DeviceCache *c, const Fie
                 ++ps.n_x;
             }
             ps.nx_of[m] = k;
+            ps.flat[m] = M.mom[q0 + m][1] % F.ly == 0 && M.mom[q0 + m][2] % F.lz == 0;
         }
         passes.push_back(ps);
     }
