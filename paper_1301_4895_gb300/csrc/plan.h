@@ -76,11 +76,12 @@ struct MinorPlan {
 };
 
 // The minor plan of a list, made once per list; nullptr where the list does
-// not qualify (several sources or sink functions, relativistic operators) or
-// where its own operations are fewer: 3He takes 2.4 K complex multiply-adds per
-// site as minors against 8.6 K (with both blocks), 4He 0.2 K against 13.6 K,
-// while pn's 7 K products exceed its recursion's 2.7 K. Measured on GB300, 3He
-// and 4He on 16^3 x 32 sites: FP64 18.42 -> 2.14 ms, mixed 2.05 -> 0.48 ms.
+// not qualify (several sources or sink functions, relativistic operators; more
+// than kMaxMinorRuns runs or kMaxMinorRows minors of an order) or where its own
+// operations are fewer, its block included: 3He takes 1,860 complex multiply-adds
+// per site as minors against 7,560, 4He 187 against 12,492, while pn's 6,784 exceed
+// its recursion's 4,176. Measured on GB300, 3He and 4He on 16^3 x 32 sites: FP64
+// 18.42 -> 2.12 ms, mixed 2.05 -> 0.46 ms.
 std::shared_ptr<const MinorPlan> minor_plan(const mbc_term_list *L);
 
 // Saturated form of a relativistic point-sink list: where every contracted

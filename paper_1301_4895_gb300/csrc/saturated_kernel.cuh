@@ -65,34 +65,39 @@ __device__ __forceinline__ double2 det12(double2 (&a)[12]) {
     return cmul(cmul(a[0], a[2]), cmul(a[1], a[3]));
 }
 
-// partial[tile][mom][comp]: phase-weighted sums over the tile's sites (d2: their
-// squared determinants) in a fixed order, scaled by the component's coefficient
-__device__ __forceinline__ void saturated_sums(const double2 *d2, double2 *sum, const FieldDesc &F, const MomDesc &M,
-                                               const double *coef, int n_comp, int64_t tile, int site0,
-                                               double2 *partial) {
-    const int v3 = F.lx * F.ly * F.lz;
+// What the sums over a tile's sites read: squared determinants and phases.
+struct SatTile {
+    double2 d2[kSatSites], ph[kSatSites][kMaxMom], sum[kMaxMom];
+};
+__device__ __forceinline__ double2 sat_phase(const FieldDesc &F, const MomDesc &M, int site, int q) {
+    return mom_phase(M.mom[q], site % F.lx, (site / F.lx) % F.ly, site / (F.lx * F.ly), F.lx, F.ly, F.lz);
+}
+
+// partial[tile][mom][comp]: phase-weighted sums over the tile's sites in a fixed
+// order, scaled by the component's coefficient
+__device__ __forceinline__ void saturated_sums(SatTile &T, const FieldDesc &F, const MomDesc &M, const double *coef,
+                                               int n_comp, int64_t tile, int site0, double2 *partial) {
+    const int n = min(kSatSites, F.lx * F.ly * F.lz - site0);
     for (int q = threadIdx.x; q < M.n_mom; q += blockDim.x) {
         double re = 0.0, im = 0.0;
-        for (int w = 0; w < kSatSites && site0 + w < v3; ++w) {
-            const int site = site0 + w;
-            const double2 ph = mom_phase(M.mom[q], site % F.lx, (site / F.lx) % F.ly, site / (F.lx * F.ly), F.lx, F.ly,
-                                         F.lz);
-            re = __fma_rn(ph.x, d2[w].x, __fma_rn(-ph.y, d2[w].y, re));
-            im = __fma_rn(ph.x, d2[w].y, __fma_rn(ph.y, d2[w].x, im));
+        for (int w = 0; w < n; ++w) {
+            const double2 ph = T.ph[w][q];
+            re = __fma_rn(ph.x, T.d2[w].x, __fma_rn(-ph.y, T.d2[w].y, re));
+            im = __fma_rn(ph.x, T.d2[w].y, __fma_rn(ph.y, T.d2[w].x, im));
         }
-        sum[q] = make_double2(re, im);
+        T.sum[q] = make_double2(re, im);
     }
     __syncthreads();
     for (int o = threadIdx.x; o < M.n_mom * n_comp; o += blockDim.x) {
         const double c = __ldg(coef + o % n_comp);
-        partial[tile * (int64_t)(M.n_mom * n_comp) + o] = make_double2(c * sum[o / n_comp].x, c * sum[o / n_comp].y);
+        partial[tile * (int64_t)(M.n_mom * n_comp) + o] = make_double2(c * T.sum[o / n_comp].x, c * T.sum[o / n_comp].y);
     }
 }
 
 __global__ void __launch_bounds__(16 * kSatSites)
     k_saturated(FieldDesc F, MomDesc M, const double *__restrict__ coef, int n_comp, int tiles_per_slab,
                 double2 *__restrict__ partial) {
-    __shared__ double2 d2[kSatSites], sum[kMaxMom];
+    __shared__ SatTile T;
     const int64_t tile = blockIdx.x, slab = tile / tiles_per_slab;
     const int site0 = (int)(tile % tiles_per_slab) * kSatSites, v3 = F.lx * F.ly * F.lz;
     const int s = threadIdx.x >> 4, row = threadIdx.x & 15;
@@ -105,10 +110,13 @@ __global__ void __launch_bounds__(16 * kSatSites)
 #pragma unroll
         for (int j = 0; j < 12; ++j) a[j] = load_prop(F, base, row * 12 + j);
     }
+    // phases: an FP64 sine and cosine each, so every thread takes some
+    for (int o = threadIdx.x; o < kSatSites * M.n_mom; o += blockDim.x)
+        if (site0 + o / M.n_mom < v3) T.ph[o / M.n_mom][o % M.n_mom] = sat_phase(F, M, site0 + o / M.n_mom, o % M.n_mom);
     const double2 d = det12(a);
-    if (row == 0) d2[s] = cmul(d, d);
+    if (row == 0) T.d2[s] = cmul(d, d);
     __syncthreads();
-    saturated_sums(d2, sum, F, M, coef, n_comp, tile, site0, partial);
+    saturated_sums(T, F, M, coef, n_comp, tile, site0, partial);
 }
 
 // The same elimination with a CTA of four warps per site, for lattices of few
@@ -122,7 +130,8 @@ __global__ void __launch_bounds__(16 * kSatSites)
 __global__ void __launch_bounds__(128) __cluster_dims__(kSatSites, 1, 1)
     k_saturated_few(FieldDesc F, MomDesc M, const double *__restrict__ coef, int n_comp, int tiles_per_slab,
                     double2 *__restrict__ partial) {
-    __shared__ double2 fac[2][12], pivots[12], d2[kSatSites], sum[kMaxMom];
+    __shared__ SatTile T;
+    __shared__ double2 fac[2][12], pivots[12];
     __shared__ int prow[2];
     const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
     const int v3 = F.lx * F.ly * F.lz;
@@ -165,16 +174,19 @@ __global__ void __launch_bounds__(128) __cluster_dims__(kSatSites, 1, 1)
         }
     }
     cluster.sync();  // the first CTA has started (every pivot is written by now)
-    if (w == 0) {    // product of the pivots, in a fixed tree
+    SatTile *first = cluster.map_shared_rank(&T, 0);
+    if (w > 0) {
+        for (int q = threadIdx.x - 32; q < M.n_mom && site < v3; q += 96) first->ph[in_tile][q] = sat_phase(F, M, site, q);
+    } else {  // product of the pivots, in a fixed tree
         double2 d = lane < 12 ? pivots[lane] : make_double2(1.0, 0.0);
         for (int off = 8; off > 0; off >>= 1) {
             const double2 o = make_double2(__shfl_xor_sync(0xffffffffu, d.x, off), __shfl_xor_sync(0xffffffffu, d.y, off));
             if (off < 8 || lane < 4) d = cmul(d, o);  // four pivots have no partner eight further
         }
-        if (lane == 0) cluster.map_shared_rank(d2, 0)[in_tile] = cmul(d, d);
+        if (lane == 0) first->d2[in_tile] = cmul(d, d);
     }
-    cluster.sync();  // the tile's determinants are in the first CTA
-    if (in_tile == 0) saturated_sums(d2, sum, F, M, coef, n_comp, tile, site0, partial);
+    cluster.sync();  // the tile's determinants and phases are in the first CTA
+    if (in_tile == 0) saturated_sums(T, F, M, coef, n_comp, tile, site0, partial);
 }
 
 }  // namespace mbc

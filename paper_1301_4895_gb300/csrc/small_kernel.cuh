@@ -13,8 +13,8 @@
 //   3. every step F^(m+1)[z] = sum_j s_j F^(m)[x_j] f[y_j] (eq. recr_F) over
 //      the z-major lists; g lanes share one z and combine by xor shuffles;
 //   4. the contraction with L (eq. C_final) into FP64;
-// Lists whose minor form (plan.h) takes fewer operations - 3He and 4He: 1.8 K
-// complex multiply-adds per site for both instead of 19.6 K - skip 2., build
+// Lists whose minor form (plan.h) takes fewer operations - 3He and 4He: 2.0 K
+// complex multiply-adds per site for both instead of 18.5 K - skip 2., build
 // minors of the tile in 3. (the same step code on other operands) and sum
 // signed products of two minors in 4.;
 // then the CTA multiplies each site's components by the momentum phases and

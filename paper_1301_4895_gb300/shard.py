@@ -70,7 +70,11 @@ def contract_sharded(field, lists, group=None, contract=None, **kw):
     configuration it touches, and the per-slab correlators are gathered in
     slab order. Returns, on every rank, the array a single call over the
     whole field returns: (n_cfg, n_lists, nt, n_mom / N_k, n_comp_max),
-    complex128. ``contract`` defaults to the library's contract (keyword
+    complex128 - bit for bit with point sinks, in mixed precision and for the
+    FP64 lists of the wave kernels (relativistic ones beyond pn), else up to
+    the order of the site sums: the FP64 shared-memory kernels choose their
+    tile, and momentum-projected blocks their chunks, by the sites of a call.
+    ``contract`` defaults to the library's contract (keyword
     arguments are passed on; t0 / t1 are taken here)."""
     if contract is None:
         from . import contract as contract
