@@ -965,17 +965,21 @@ mbc_status launch_small_batch(const SmallBatch &B, const FieldDesc &F, const Mom
 
 size_t align256(size_t n) { return (n + 255) & ~size_t(255); }
 
-// k_reduce_tiles with warps per output from the tiles a lane would add: several
+// k_reduce_tiles with parts per output from the tiles a lane would add: several
 // where a slab's outputs are too few to fill the SMs, at most one per FP64 unit (one
-// output of 512 tiles: 16 warps 9.0 us, 4 warps 6.0). The warps fix the order of the
+// output of 512 tiles: 16 warps 9.0 us, 4 warps 6.0). The parts fix the order of the
 // sum, so they follow from one slab alone: a slab's result has the same bits in a
-// call of any number of them (sharded runs).
+// call of any number of them (sharded runs). The call's outputs decide whether the
+// parts get a warp each.
 mbc_status launch_reduce(const double2 *partial, int64_t n_slabs, int tiles_per_slab, int n_mom, int n_comp, int n_t,
                          int li, int n_lists, int comp_max, double2 *out, int nsm, cudaStream_t stream) {
     const int64_t slab_outs = (int64_t)n_mom * n_comp, outs = n_slabs * slab_outs;
-    int warps = 1;
-    while (warps < 4 && tiles_per_slab > 16 * warps && slab_outs * warps < 4LL * nsm) warps *= 2;
-    auto kern = warps == 1 ? k_reduce_tiles<1> : warps == 2 ? k_reduce_tiles<2> : k_reduce_tiles<4>;
+    int parts = 1;
+    while (parts < 4 && tiles_per_slab > 16 * parts && slab_outs * parts < 4LL * nsm) parts *= 2;
+    const int warps = outs * parts < 8LL * nsm ? parts : 1;
+    auto kern = parts == 1 ? k_reduce_tiles<1, 1>
+                : parts == 2 ? (warps == 2 ? k_reduce_tiles<2, 2> : k_reduce_tiles<2, 1>)
+                             : (warps == 4 ? k_reduce_tiles<4, 4> : k_reduce_tiles<4, 1>);
     const int per_cta = 4 / warps;
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((outs + per_cta - 1) / per_cta, 65535));
     note_launch();

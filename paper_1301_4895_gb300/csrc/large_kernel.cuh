@@ -583,14 +583,15 @@ __global__ void __launch_bounds__(256) k_large_sitesum(FieldDesc F, WaveDesc wv,
     }
 }
 
-// Final reduction over the tiles of each slab: WARPS warps per output, the lower
-// half of a warp adds real parts, the upper half imaginary ones, lane by lane over
-// strided tiles with Neumaier compensation; a fixed xor tree combines the lanes'
-// (sum, compensation) pairs and the warps' in turn - a fixed order, so results are
-// bitwise reproducible. An FP64 instruction of a warp holds one of the SM's four
-// units for 64 cycles however many lanes use it, hence the split halves, four
-// warps per CTA, and several warps for outputs of many tiles. 128 outputs of 16
-// tiles: 3.3 us (8.9 with both parts in every lane and 8 warps per CTA).
+// Final reduction over the tiles of each slab: the lower half of a warp adds real
+// parts, the upper half imaginary ones, with Neumaier compensation. An output's tiles
+// go to PARTS x 16 partial sums (strided), a lane's partial sums are added in pairs,
+// the lanes' by a fixed xor tree - an order that PARTS and the tiles fix, so
+// results are bitwise reproducible, and the same whether the parts are taken by WARPS =
+// PARTS warps (few outputs) or by one. An FP64 instruction of a warp holds one of the
+// SM's four units for 64 cycles however many lanes use it, hence the split halves, four
+// warps per CTA, and several warps for outputs of many tiles. 128 outputs of 16 tiles:
+// 3.3 us (8.9 with both parts in every lane and 8 warps per CTA).
 // out[cfg][list][t - t0][mom][comp_stride].
 __device__ __forceinline__ void neumaier(double &s, double &c, double v) {
     const double t = s + v;
@@ -607,12 +608,13 @@ __device__ __forceinline__ void neumaier_pair(double &s, double &c, int off, int
     neumaier(s, c, b);
 }
 constexpr int kReduceThreads = 128;
-template <int WARPS>
+template <int PARTS, int WARPS>
 __global__ void __launch_bounds__(kReduceThreads)
     k_reduce_tiles(const double2 *__restrict__ partial, int64_t n_slabs, int tiles_per_slab, int n_mom, int n_comp,
                    int n_t, int list_idx, int n_lists, int comp_stride, double2 *out) {
+    static_assert(WARPS == 1 || WARPS == PARTS, "one part per warp, or all in one");
     constexpr int OUTS = 4 / WARPS;  // outputs per CTA
-    __shared__ double part_s[4][2], part_c[4][2];
+    __shared__ double part_s[4][32], part_c[4][32];
     const int64_t per_slab = (int64_t)n_mom * n_comp;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, im = lane >> 4;
     const int w = warp % WARPS;
@@ -622,34 +624,54 @@ __global__ void __launch_bounds__(kReduceThreads)
         const bool live = o < n_slabs * per_slab;
         const int64_t slab = live ? o / per_slab : 0;
         const int r = (int)(o % per_slab);
-        double s = 0.0, c = 0.0;
+        constexpr int MINE = PARTS / WARPS;  // parts of this warp: w, or all
+        double s[MINE], c[MINE];
+        auto at = [&](int tl) { return p[2 * ((slab * tiles_per_slab + tl) * per_slab + r) + im]; };
         int tl = w * 16 + (lane & 15);
-        if (live && tl < tiles_per_slab) {
-            s = p[2 * ((slab * tiles_per_slab + tl) * per_slab + r) + im];
-            for (tl += 16 * WARPS; tl < tiles_per_slab; tl += 16 * WARPS)
-                neumaier(s, c, p[2 * ((slab * tiles_per_slab + tl) * per_slab + r) + im]);
+#pragma unroll
+        for (int v = 0; v < MINE; ++v) {
+            s[v] = c[v] = 0.0;
+            if (live && tl + 16 * v < tiles_per_slab) s[v] = at(tl + 16 * v);
         }
-        for (int off = 8; off > 0; off >>= 1)
-            if (off < tiles_per_slab) neumaier_pair(s, c, off, lane);
+        if constexpr (MINE == 1) {
+            if (live)
+                for (tl += 16 * PARTS; tl < tiles_per_slab; tl += 16 * PARTS) neumaier(s[0], c[0], at(tl));
+        } else {  // the parts side by side: their chains overlap
+            for (int t0 = 16 * PARTS; live && t0 < tiles_per_slab; t0 += 16 * PARTS)
+#pragma unroll
+                for (int v = 0; v < MINE; ++v)
+                    if (t0 + tl + 16 * v < tiles_per_slab) neumaier(s[v], c[v], at(t0 + tl + 16 * v));
+        }
         if (WARPS > 1) {
-            if ((lane & 15) == 0) {
-                part_s[warp][im] = s;
-                part_c[warp][im] = c;
-            }
+            part_s[warp][lane] = s[0];
+            part_c[warp][lane] = c[0];
             __syncthreads();
-            if (w == 0) {
-                const int k = lane & 15;
-                s = k < WARPS ? part_s[warp + k][im] : 0.0;
-                c = k < WARPS ? part_c[warp + k][im] : 0.0;
-                for (int off = WARPS / 2; off > 0; off >>= 1) neumaier_pair(s, c, off, lane);
-            }
-            __syncthreads();  // read before the next output's
         }
+        if (w == 0) {
+            double a[PARTS], e[PARTS];
+#pragma unroll
+            for (int v = 0; v < PARTS; ++v) {
+                a[v] = WARPS > 1 ? part_s[(warp + v) & 3][lane] : s[v % MINE];
+                e[v] = WARPS > 1 ? part_c[(warp + v) & 3][lane] : c[v % MINE];
+            }
+#pragma unroll
+            for (int d = 1; d < PARTS; d *= 2)
+#pragma unroll
+                for (int v = 0; v + d < PARTS; v += 2 * d) {
+                    e[v] += e[v + d];
+                    neumaier(a[v], e[v], a[v + d]);
+                }
+            for (int off = 8; off > 0; off >>= 1)
+                if (off < tiles_per_slab) neumaier_pair(a[0], e[0], off, lane);
+            s[0] = a[0];
+            c[0] = e[0];
+        }
+        if (WARPS > 1) __syncthreads();  // read before the next output's
         if (live && w == 0 && (lane & 15) == 0) {
             const int cfg = (int)(slab / n_t), tt = (int)(slab % n_t);
             const int q = r / n_comp, cc = r % n_comp;
             const int64_t oi = ((((int64_t)cfg * n_lists + list_idx) * n_t + tt) * n_mom + q) * comp_stride + cc;
-            reinterpret_cast<double *>(out)[2 * oi + im] = s + c;
+            reinterpret_cast<double *>(out)[2 * oi + im] = s[0] + c[0];
         }
     }
 }
