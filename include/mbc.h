@@ -345,9 +345,12 @@ typedef struct {
  *                MBC_MIXED: per-site power-of-two input scaling, FP32 complex
  *                products with compensated FP32 accumulation of every sum,
  *                FP64 for the site/momentum sum. The contraction with L is FP64
- *                in the recursion and the minor form; the pair form, which mixed
- *                calls take only where every coefficient is exact in FP32, sums
- *                it compensated in FP32. 8Be's determinants are FP64 in both.
+ *                in the recursion. The minor form sums its products compensated in
+ *                FP32 and multiplies the sums by their coefficients in FP64; the
+ *                pair form, which mixed calls take only where every coefficient is
+ *                exact in FP32, sums the contraction compensated in FP32 too (median
+ *                errors of both forms below the recursion's). 8Be's determinants
+ *                are FP64 in both.
  *   n_mom, mom   n_mom >= 1 momenta, mom[3 * i + {0, 1, 2}] = (n_x, n_y, n_z)
  *                integers (host pointer, read during the call).
  *   t0, t1       time slices [t0, t1) are evaluated; t1 == 0 means nt.
