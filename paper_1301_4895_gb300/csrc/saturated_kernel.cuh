@@ -74,18 +74,23 @@ __device__ __forceinline__ double2 sat_phase(const FieldDesc &F, const MomDesc &
 }
 
 // partial[tile][mom][comp]: phase-weighted sums over the tile's sites in a fixed
-// order, scaled by the component's coefficient
+// tree, scaled by the component's coefficient; a lane takes a real or imaginary part
 __device__ __forceinline__ void saturated_sums(SatTile &T, const FieldDesc &F, const MomDesc &M, const double *coef,
                                                int n_comp, int64_t tile, int site0, double2 *partial) {
     const int n = min(kSatSites, F.lx * F.ly * F.lz - site0);
-    for (int q = threadIdx.x; q < M.n_mom; q += blockDim.x) {
-        double re = 0.0, im = 0.0;
-        for (int w = 0; w < n; ++w) {
-            const double2 ph = T.ph[w][q];
-            re = __fma_rn(ph.x, T.d2[w].x, __fma_rn(-ph.y, T.d2[w].y, re));
-            im = __fma_rn(ph.x, T.d2[w].y, __fma_rn(ph.y, T.d2[w].x, im));
+    for (int i = threadIdx.x; i < 2 * M.n_mom; i += blockDim.x) {
+        const bool im = i & 1;
+        double t[kSatSites];
+#pragma unroll
+        for (int w = 0; w < kSatSites; ++w) {
+            const double2 d = T.d2[w], ph = T.ph[w][i >> 1];
+            t[w] = w < n ? __fma_rn(ph.x, im ? d.y : d.x, (im ? ph.y : -ph.y) * (im ? d.x : d.y)) : 0.0;
         }
-        T.sum[q] = make_double2(re, im);
+#pragma unroll
+        for (int off = 1; off < kSatSites; off *= 2)
+#pragma unroll
+            for (int w = 0; w < kSatSites; w += 2 * off) t[w] += t[w + off];
+        reinterpret_cast<double *>(T.sum)[i] = t[0];
     }
     __syncthreads();
     for (int o = threadIdx.x; o < M.n_mom * n_comp; o += blockDim.x) {
