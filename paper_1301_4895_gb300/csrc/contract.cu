@@ -2165,10 +2165,21 @@ extern "C" mbc_status mbc_contract(const mbc_props *props, const mbc_term_list *
             note_launch();
             const unsigned grid = (unsigned)(n_slabs * sat_tiles);
             const double *coef = caches[(size_t)li]->d_sat_coef;
-            if (sat_few)
-                k_saturated_few<<<grid * kSatSites, 128, 0, stream>>>(F, M, coef, lists[li]->n_comp, sat_tiles, partial);
-            else
+            if (sat_few) {
+                cudaLaunchAttribute at[1];
+                at[0].id = cudaLaunchAttributeClusterDimension;
+                at[0].val.clusterDim.x = (unsigned)sat_cluster(v3);
+                at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+                cudaLaunchConfig_t cfg = {};
+                cfg.gridDim = dim3(grid * (unsigned)sat_cluster(v3));
+                cfg.blockDim = dim3(128);
+                cfg.stream = stream;
+                cfg.attrs = at;
+                cfg.numAttrs = 1;
+                MBC_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_saturated_few, F, M, coef, (int)lists[li]->n_comp, sat_tiles, partial));
+            } else {
                 k_saturated<<<grid, 16 * kSatSites, 0, stream>>>(F, M, coef, lists[li]->n_comp, sat_tiles, partial);
+            }
         }
         MBC_CUDA_TRY(cudaGetLastError());
         if ((st = reduce(li, partial, sat_tiles)) != MBC_OK) return st;

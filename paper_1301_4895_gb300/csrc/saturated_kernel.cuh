@@ -130,9 +130,11 @@ __global__ void __launch_bounds__(16 * kSatSites)
 // w, w + 4 (upper half) and w + 8. The warp that owns a step's column finds the
 // pivot and writes the rows' factors to shared memory; every warp then fetches its
 // columns' pivot elements by shuffles and eliminates. 64 sites: 17 us, one warp
-// for two sites 30. The CTAs of a tile are a cluster whose first one sums the
-// sites: the operations and their order are k_saturated's, and so are the bits.
-__global__ void __launch_bounds__(128) __cluster_dims__(kSatSites, 1, 1)
+// for two sites 30. The CTAs of a tile are a cluster (sat_cluster of them) whose first
+// one sums the sites: the operations and their order are k_saturated's, and so are
+// the bits.
+inline int sat_cluster(int64_t v3) { return v3 > 4 ? kSatSites : v3 > 2 ? 4 : v3 > 1 ? 2 : 1; }
+__global__ void __launch_bounds__(128)
     k_saturated_few(FieldDesc F, MomDesc M, const double *__restrict__ coef, int n_comp, int tiles_per_slab,
                     double2 *__restrict__ partial) {
     __shared__ SatTile T;
@@ -140,11 +142,13 @@ __global__ void __launch_bounds__(128) __cluster_dims__(kSatSites, 1, 1)
     __shared__ int prow[2];
     const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
     const int v3 = F.lx * F.ly * F.lz;
-    const int64_t tile = blockIdx.x / kSatSites, slab = tile / tiles_per_slab;
-    const int site0 = (int)(tile % tiles_per_slab) * kSatSites, in_tile = blockIdx.x % kSatSites, site = site0 + in_tile;
+    const int ctas = (int)cluster.num_blocks(), in_tile = (int)cluster.block_rank();
+    const int64_t tile = blockIdx.x / ctas, slab = tile / tiles_per_slab;
+    const int site0 = (int)(tile % tiles_per_slab) * kSatSites, site = site0 + in_tile;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, half = lane >> 4, row = lane & 15;
     double2 a[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};  // columns w + 4 half, w + 8 (lower half)
-    if (site < v3 && row < 12) {
+    const bool live = site < v3;  // a tile's last CTAs may have no site
+    if (live && row < 12) {
         const int64_t base = slab / F.n_t * F.stride_cfg + (F.t0 + slab % F.n_t) * F.stride_t + (int64_t)site * 144;
         a[0] = load_prop(F, base, row * 12 + w + 4 * half);
         if (half == 0) a[1] = load_prop(F, base, row * 12 + w + 8);
@@ -152,6 +156,7 @@ __global__ void __launch_bounds__(128) __cluster_dims__(kSatSites, 1, 1)
     unsigned left = 0xfffu;
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
+        if (!live) break;
         const int h = (k >> 2) & 1, q = k >> 3;  // column k: warp k % 4, half h, register q
         if (w == (k & 3) && half == h) {
             const unsigned mask = 0xffffu << (16 * h);
@@ -180,9 +185,9 @@ __global__ void __launch_bounds__(128) __cluster_dims__(kSatSites, 1, 1)
     }
     cluster.sync();  // the first CTA has started (every pivot is written by now)
     SatTile *first = cluster.map_shared_rank(&T, 0);
-    if (w > 0) {
-        for (int q = threadIdx.x - 32; q < M.n_mom && site < v3; q += 96) first->ph[in_tile][q] = sat_phase(F, M, site, q);
-    } else {  // product of the pivots, in a fixed tree
+    if (w > 0 && live) {
+        for (int q = threadIdx.x - 32; q < M.n_mom; q += 96) first->ph[in_tile][q] = sat_phase(F, M, site, q);
+    } else if (live) {  // product of the pivots, in a fixed tree
         double2 d = lane < 12 ? pivots[lane] : make_double2(1.0, 0.0);
         for (int off = 8; off > 0; off >>= 1) {
             const double2 o = make_double2(__shfl_xor_sync(0xffffffffu, d.x, off), __shfl_xor_sync(0xffffffffu, d.y, off));

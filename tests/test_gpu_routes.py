@@ -183,6 +183,8 @@ def test_block_slices_on_two_relativistic_sources(mbc):
 @pytest.mark.parametrize("build,dims,nt,precs", [
     # 8Be: 1,728 sites a slab by four warps a site, 5,184 by half a warp
     (lambda m: [m.build_term_list(4, 4, 4, spins=[(BE8, BE8)], list_free=True)], (12, 12, 12), 3, (0, 1)),
+    # clusters of four CTAs: 3 sites a slab
+    (lambda m: [m.build_term_list(4, 4, 4, spins=[(BE8, BE8)], list_free=True)], (1, 1, 3), 4, (0, 1)),
     # nonrelativistic lists in mixed precision: 64 tiles of 32 sites, 64 outputs a slab
     (lambda m: [m.build_term_list(1, 1, 2), m.build_term_list(2, 1, 2), m.build_term_list(2, 2, 2)], (16, 16, 8), 6, (1,)),
     # pair form: waves of 64 and of 1,024 sites; 18 tiles and 256 outputs a slab
