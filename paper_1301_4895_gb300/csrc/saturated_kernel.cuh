@@ -10,8 +10,8 @@
 // permutation's sign squares away). The kernel is bound by the FP64 units (a
 // warp's FP64 instruction takes one of the SM's four for 64 cycles) through
 // 12 dependent steps. Measured on GB300 against the recursion, whole calls: 64
-// sites FP64 198.0 ms -> 33 us, 512 sites mixed 156.1 ms -> 58 us, the kernels 17
-// and 22 us of it.
+// sites FP64 198.0 ms -> 27 us, 512 sites mixed 156.1 ms -> 55 us (host and launches
+// more than half of both), 16^3 sites FP64 86 us, with 4 momenta 91.
 #pragma once
 
 #include <cooperative_groups.h>
